@@ -1,402 +1,595 @@
-// General row kernel: one thread block per position, any V, dtype and strides.
-// All arithmetic is float64 and every pass re-reads the row from global
-// memory (L2 after the first pass).  It is the library's fallback for layouts
-// the bf16 streaming kernels do not serve (fp32 logits, odd strides, ragged V), their second tier
-// (rows they hand over through the row list), and the slow, careful path.  Steps follow the method's definition:
+// General row kernel: any V, dtype and strides, float64 arithmetic throughout.  It serves the layouts the bf16
+// kernels do not (fp32 logits, odd strides, ragged V), and it is their second tier (rows they hand over through
+// the row list).  Steps follow the method's definition:
 //   log-softmax x2 -> lambda (Eqs. "bridge", "trust_region") -> TV and the
 //   maximal coupling (Eqs. "accept", "residual") -> routed loss (Eqs.
 //   "k1_loss_token", "teacher_mode_loss") -> gradient (Eq. "general_objective").
-// In list mode (the second tier of the bf16 kernels: usually a handful of rows) a short list is routed with a
-// row spread over a cluster of 8 thread blocks, which add up their block totals through distributed shared
-// memory: one block per row leaves a row of 151,936 elements 1.3 ms on a single SM, a cluster 0.47 ms.  A
-// long list keeps one block per row (18 clusters are fewer than 148 blocks).  The host does not know the
-// list's length when it launches, so both forms are launched and each returns at once unless the length
-// is in its range.
-#include "saki_common.cuh"
+//
+// What bounds it: the float64 pipe (64 lanes per clock and SM; a warp instruction occupies its scheduler's half of
+// it for two clocks).  Hence:
+//   - 2^y costs eight float64 operations: y is split by a magic-number addition into n + i/256 + r, 2^(i/256) comes
+//     from a table in shared memory and 2^r from its Taylor polynomial (|r| <= 1/512: the first dropped term is
+//     4e-17).  The table is stored 16 times over, one copy per 64-bit bank, so a half-warp's lookups never conflict;
+//   - three passes over the row: "sums" (two exponentials), one or two evaluations of KL with its first four
+//     derivatives (one exponential each: the root of the fourth-order model, as in the bf16 kernels, here accepted
+//     when the dropped terms move lambda by less than 1e-10), "final" (two exponentials; total variation, draw
+//     weights and the gradient in one pass).  The row's maxima come out of pass "sums" itself: every warp runs
+//     under shifts fixed from its first elements (whole powers of two, so warps combine exactly) and repeats its
+//     part with the true maxima if they turn out so much larger that its sums could have overflowed;
+//   - the moments of the logit difference that only feed the first guess of lambda are float32.
+// A warp owns a contiguous segment of the row in every pass (the residual draw is in index order), a row is owned by
+// one block or by a cluster of blocks that add up their warps' partial sums through distributed shared memory.
+#include "saki_device.cuh"
 #include <cooperative_groups.h>
-#include <math_constants.h>
+#include <atomic>
 
 namespace cg = cooperative_groups;
 
 namespace saki {
 
-constexpr int GT = 512;        // threads per block
+namespace {
+
+constexpr int GT = 256;        // threads per block
 constexpr int GW = GT / 32;    // warps per block
-
-__device__ __forceinline__ double warp_sum(double v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
-// Sum NV doubles over the block (CS == 1) or over the cluster's CS blocks; every thread gets the same totals
-// (summed in a fixed order: by block rank, then by warp, so results are reproducible).  `sh` is the same
-// shared-memory array in every block of the cluster.
-template <int NV, int CS>
-__device__ __forceinline__ void block_sum(double (&v)[NV], double* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int k = 0; k < NV; ++k) v[k] = warp_sum(v[k]);
-  if (lane == 0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) sh[k * GW + warp] = v[k];
-  }
-  if constexpr (CS == 1) {
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      double a = 0.0;
-#pragma unroll
-      for (int w = 0; w < GW; ++w) a += sh[k * GW + w];
-      v[k] = a;
-    }
-    __syncthreads();
-  } else {
-    cg::cluster_group cl = cg::this_cluster();
-    cl.sync();
-#pragma unroll
-    for (int k = 0; k < NV; ++k) v[k] = 0.0;
-    for (int r = 0; r < CS; ++r) {
-      const double* rs = cl.map_shared_rank(sh, r);
-#pragma unroll
-      for (int k = 0; k < NV; ++k) {
-        double a = 0.0;
-#pragma unroll
-        for (int w = 0; w < GW; ++w) a += rs[k * GW + w];
-        v[k] += a;
-      }
-    }
-    cl.sync();
-  }
-}
+constexpr int MAX_CS = 8;      // blocks per row, at most
+constexpr int TAB = 256, COPIES = 16;
+constexpr int NPART = 12;      // doubles a warp leaves per phase
 
 struct Shared {
-  double red[4 * GW];
-  double warp_tot[GW];
-  float fmax_s[GW], fmax_t[GW];
-  int arg_t[GW];
-  int token;
-  int finite;
-  double wt_all[GW * 8];   // every warp's draw weight of the cluster, in segment order
+  double tab[TAB * COPIES];
+  double part[2][GW][NPART];   // alternates from phase to phase: one barrier per phase is enough
+  double bc[32];               // scalars broadcast to the block
+  double sub[GW];
+};
+enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G_LO, G_HI, G_ITER, G_AM, G_OWNER, G_BEFORE,
+       G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_COUNT };
+static_assert(G_COUNT <= 32, "broadcast area too small");
+enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
+enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
+
+struct Exp2 {
+  uint32_t base;   // shared-memory address of this lane's copy of the table
+  // 2^y for y <= ~1000; y below -1000 counts as -1000 (clamped through the high word: an unsigned minimum)
+  __device__ __forceinline__ double operator()(double y) const {
+    const uint32_t hi = min((uint32_t)__double2hiint(y), 0xC08F4000u);
+    y = __hiloint2double((int)hi, __double2loint(y));
+    const double M = 26388279066624.0;                       // 1.5 * 2^44: the low word of y + M is round(256 y)
+    const double t = y + M;
+    const double r = y - (t - M);
+    const int k = __double2loint(t);
+    double T;
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(T) : "r"(base + (((uint32_t)k << 7) & 0x7f80u)));
+    // Taylor coefficients of 2^r: ln2^i / i!
+    double q = fma(r, 9.618129107628477e-03, 5.550410866482158e-02);
+    q = fma(r, q, 2.402265069591007e-01);
+    q = fma(r, q, 6.931471805599453e-01);
+    T = __hiloint2double(__double2hiint(T) + ((k << 12) & 0xfff00000), __double2loint(T));
+    return fma(T * r, q, T);
+  }
 };
 
-// CS: blocks per row (1, or a cluster of CS blocks that share the row element by element)
+__device__ __forceinline__ double pow2_down(double n) {      // 2^n for whole n <= 0; 0 below -1000
+  return n < -1000.0 ? 0.0 : __longlong_as_double((long long)(1023 + (int)n) << 52);
+}
+
+// float64 to bf16, one rounding to nearest even: through a float rounded to odd
+__device__ __forceinline__ __nv_bfloat16 to_bf16(double v) {
+  float f = __double2float_rz(v);
+  if ((double)f != v) f = __uint_as_float(__float_as_uint(f) | 1u);
+  return __float2bfloat16_rn(f);
+}
+template <typename T> __device__ __forceinline__ void put(T* g, int64_t i, double v);
+template <> __device__ __forceinline__ void put<float>(float* g, int64_t i, double v) { g[i] = (float)v; }
+template <> __device__ __forceinline__ void put<__nv_bfloat16>(__nv_bfloat16* g, int64_t i, double v) { g[i] = to_bf16(v); }
+
+// Runs body(v, s, t) over the elements v = lo + lane, lo + lane + 32, ... < hi: four at a time, the loads of the next
+// four issued before the current ones are used (the row comes from L2 in all passes but the first).
+template <typename T, typename F>
+__device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* __restrict__ t, int lo, int hi, int lane, F&& body) {
+  constexpr int U = 4;
+  const int full = lo + (hi - lo) / (32 * U) * (32 * U);
+  int v = lo + lane;
+  float a[U], b[U];
+  if (lo < full) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) { a[u] = ld_as_float(s, v + 32 * u); b[u] = ld_as_float(t, v + 32 * u); }
+#pragma unroll 1
+    for (; v < full; v += 32 * U) {
+      float na[U], nb[U];
+      const bool more = v + 32 * U < full;
+#pragma unroll
+      for (int u = 0; u < U; ++u) { na[u] = more ? ld_as_float(s, v + 32 * (U + u)) : 0.f; nb[u] = more ? ld_as_float(t, v + 32 * (U + u)) : 0.f; }
+#pragma unroll
+      for (int u = 0; u < U; ++u) body(v + 32 * u, a[u], b[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) { a[u] = na[u]; b[u] = nb[u]; }
+    }
+  }
+#pragma unroll 1
+  for (; v < hi; v += 32) body(v, ld_as_float(s, v), ld_as_float(t, v));
+}
+
+// The scalars between the passes, on one warp per block (all lanes alike).
+__device__ __noinline__ double first_guess(double m1, double m2, double m3, double m4, double rtau, double kl1, double eps) {
+  const double var = m2 - m1 * m1, m1s = m1 * m1;
+  const double c3 = m3 - 3.0 * m1 * m2 + 2.0 * m1 * m1s;
+  const double c4 = m4 - 4.0 * m3 * m1 - 3.0 * m2 * m2 + 12.0 * m2 * m1s - 6.0 * m1s * m1s;
+  const float rt = (float)rtau, vd = fmaxf((float)var * rt * rt, 1e-30f), k3 = (float)c3 * rt * rt * rt, k4 = (float)c4 * (rt * rt) * (rt * rt);
+  const float e2 = 2.f * (float)eps;
+  float b = sqrtf(__fdividef(e2, vd));
+#pragma unroll 1
+  for (int it = 0; it < 3; ++it) {
+    const float bb = fminf(b, 1.f);
+    const float den = vd + (2.f / 3.f) * bb * k3 + 0.25f * bb * bb * k4;
+    if (den > 0.25f * vd) b = sqrtf(__fdividef(e2, den));
+  }
+  if (b > 0.45f) b = anchored_guess(b, vd, k3, k4, (float)kl1, (float)eps);
+  if (!(b > 1e-7f)) b = 1e-7f;
+  if (!(b < 0.98f)) b = 0.98f;
+  return (double)b;
+}
+
+// One evaluation at beta: v[k] = sum p exp(beta d) d^k.  Returns true when lambda is settled (bc[G_LAM], bc[G_LOGZ], bc[G_KL]).
+__device__ __noinline__ bool solve_step(double* bc, const double* v, double eps) {
+  const double beta = bc[G_BETA], r0 = 1.0 / v[0], L = log(v[0]);
+  const double m1 = v[1] * r0, m2 = v[2] * r0, m3 = v[3] * r0, m4 = v[4] * r0, m1s = m1 * m1;
+  const double var = fmax(m2 - m1s, 0.0), k3 = m3 - 3.0 * m2 * m1 + 2.0 * m1s * m1;
+  const double k4 = m4 - 4.0 * m3 * m1 - 3.0 * m2 * m2 + 12.0 * m2 * m1s - 6.0 * m1s * m1s;
+  const double kl = beta * m1 - L, slope = beta * var;
+  const double c2 = 0.5 * (beta * k3 + var), c3 = beta * k4 * (1.0 / 6.0) + k3 * (1.0 / 3.0), c4 = 0.125 * k4;
+  double lo = bc[G_LO], hi = bc[G_HI];
+  if (kl <= eps) lo = fmax(lo, beta); else hi = fmin(hi, beta);
+  const int iter = (int)bc[G_ITER] + 1;
+  // root of the fourth-order model of KL(beta + h) - eps
+  const double f0 = eps - kl;
+  double h = f0 / slope;
+  bool ok = slope > 0.0;
+#pragma unroll 1
+  for (int it = 0; it < 20 && ok; ++it) {
+    const double pv = h * (slope + h * (c2 + h * (c3 + h * c4))) - f0;
+    const double dv = slope + h * (2.0 * c2 + h * (3.0 * c3 + h * (4.0 * c4)));
+    if (!(dv > 0.25 * slope)) { ok = false; break; }
+    const double dh = pv / dv;
+    h -= dh;
+    if (fabs(dh) <= 1e-15 * fabs(beta)) break;
+  }
+  if (!ok) h = f0 / slope;                                   // the model bends over: Newton's step
+  double nb = beta + h;
+  bool bisected = false;
+  if (!(nb > lo && nb < hi)) {
+    // a step that is nothing but rounding may end on the wrong side of the bracket; a real one is halved
+    if (fabs(h) < 1e-13) nb = fmin(fmax(nb, lo), hi);
+    else { nb = 0.5 * (lo + hi); bisected = true; }
+  }
+  h = nb - beta;
+  const double h2 = h * h;
+  const double trunc = fmax(fabs(c4), fmax(fabs(c3), 0.5 * fabs(c2))) * h2 * h2;
+  const bool done = (ok && !bisected && trunc <= 1e-10 * slope) || fabs(h) < 1e-13 || hi - lo < 1e-15 || iter >= 100;
+  __syncwarp();                                              // every lane has read the state
+  if (done) {
+    bc[G_LAM] = nb;
+    bc[G_LOGZ] = L + h * (m1 + h * (0.5 * var + h * ((1.0 / 6.0) * k3 + h * (1.0 / 24.0) * k4)));
+    bc[G_KL] = kl + h * (slope + h * (c2 + h * (c3 + h * c4)));
+  } else {
+    bc[G_BETA] = nb; bc[G_LO] = lo; bc[G_HI] = hi; bc[G_ITER] = (double)iter;
+  }
+  __syncwarp();
+  return done;
+}
+
+}  // namespace
+
+// CS: blocks per row (1, or a cluster of CS blocks).
 template <typename T, int CS>
-__global__ void __launch_bounds__(GT) general_kernel(const RowParams P) {
+__global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
   __shared__ Shared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = P.V;
-  const double tau = (double)P.temperature;
-  const double eps = (double)P.eps;
   int crank = 0;
   if constexpr (CS > 1) crank = (int)cg::this_cluster().block_rank();
-  const int ET = GT * CS, e0 = crank * GT + tid;     // the cluster's threads take the elements e0, e0 + ET, ...
+  constexpr int NWC = GW * CS;                               // warps of the row, in index order of their segments
+  const int gw = crank * GW + warp;
 
   const int64_t n_work = P.from_list ? (int64_t)*P.redo_count : P.n_rows;
-  // list mode is launched twice: a cluster per row for a short list, a block per row for a long one
-  if (P.from_list && P.list_max > 0 && (n_work < P.list_min || n_work > P.list_max)) return;
+  if ((int64_t)(blockIdx.x / CS) >= n_work) return;          // the whole cluster: nothing to do (an empty row list, as a rule)
+  for (int i = tid; i < TAB; i += GT) {
+    const double e = exp2((double)i * (1.0 / TAB));
+#pragma unroll 1
+    for (int c = 0; c < COPIES; ++c) sh.tab[i * COPIES + ((c + lane) & (COPIES - 1))] = e;
+  }
+  __syncthreads();
+  Exp2 ex2;
+  ex2.base = smem_addr(sh.tab) + (uint32_t)(lane & (COPIES - 1)) * 8u;
+
+  const double rtau = 1.0 / (double)P.temperature, c = INV_LN2 * rtau, eps = (double)P.eps;
+  const int seg = (((V + NWC - 1) / NWC) + 31) & ~31;        // whole steps of 32 elements
+  const int seg0 = min(V, gw * seg), seg1 = min(V, seg0 + seg);
+  int ph = 0;
+  double* const bc = sh.bc;
+
+  // all warps' partial sums of a phase are in place
+  auto phase_barrier = [&]() {
+    if constexpr (CS == 1) __syncthreads(); else cg::this_cluster().sync();
+  };
+  // the record of warp w of the row (its segment order)
+  auto part_of = [&](int w) -> const double* {
+    if constexpr (CS == 1) return sh.part[ph][w];
+    else return cg::this_cluster().map_shared_rank(&sh.part[ph][w % GW][0], w / GW);
+  };
+
   for (int64_t item = blockIdx.x / CS; item < n_work; item += gridDim.x / CS) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;   // list mode: rows handed over by the float32 kernels
     const int64_t b = row / P.K1;
     const int j = (int)(row - b * P.K1);
-    const T* s = (const T*)P.s + b * P.s_seq + (int64_t)j * P.s_pos;
-    const T* t = (const T*)P.t + b * P.t_seq + (int64_t)j * P.t_pos;
+    const T* const s = (const T*)P.s + b * P.s_seq + (int64_t)j * P.s_pos;
+    const T* const t = (const T*)P.t + b * P.t_seq + (int64_t)j * P.t_pos;
     const bool bonus = P.spec && (j == P.K1 - 1);
     int x = 0;
     if (!bonus) x = P.spec ? P.proposal[b * P.prop_ld + j] : P.proposal[row];
     const uint64_t rid = P.row_offset + (uint64_t)row;
     const bool masked = (P.mask != nullptr) && (P.mask[row] == 0);
-    T* g = P.dlogits ? (T*)P.dlogits + row * P.ld_g : nullptr;
+    T* const g = P.dlogits ? (T*)P.dlogits + row * P.ld_g : nullptr;
+    const float d0 = ld_as_float(t, 0) - ld_as_float(s, 0);  // the logit difference is taken about this one: no offset of hundreds in its moments
 
-    // ---- pass 0: maxima, teacher argmax (lowest index among ties), finiteness
-    float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
-    int am = 0x7fffffff;
-    int finite = 1;
-    for (int v = e0; v < V; v += ET) {
-      const float a = ld_as_float(s, v), c = ld_as_float(t, v);
-      finite &= (isfinite(a) && isfinite(c)) ? 1 : 0;
-      ms = fmaxf(ms, a);
-      if (c > mt) { mt = c; am = v; }
-    }
+    // ---- pass "sums"
+    {
+      float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
+      for (int v = seg0 + lane, u = 0; v < seg1 && u < 4; v += 32, ++u) { ms = fmaxf(ms, ld_as_float(s, v)); mt = fmaxf(mt, ld_as_float(t, v)); }
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
-      const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
-      const int oam = __shfl_xor_sync(0xffffffffu, am, o);
-      if (omt > mt || (omt == mt && oam < am)) { mt = omt; am = oam; }
-    }
-    if (lane == 0) { sh.fmax_s[warp] = ms; sh.fmax_t[warp] = mt; sh.arg_t[warp] = am; }
-    finite = __syncthreads_and(finite);
-    if constexpr (CS == 1) {
-      ms = sh.fmax_s[0]; mt = sh.fmax_t[0]; am = sh.arg_t[0];
+      for (int o = 16; o > 0; o >>= 1) { ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o)); mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o)); }
+      double ks = 0.0, kt = 0.0, ss, st, n1;
+      float m1, m2, m3, m4;
+      int am, inf;
+      const double dd0 = (double)d0;
+      bool again = false;
+#pragma unroll 1
+      for (int pass = 0; pass < 2; ++pass) {
+        if (seg0 < seg1) { ks = -ceil(c * (double)ms); kt = -ceil(c * (double)mt); }
+        ss = st = n1 = 0.0; m1 = m2 = m3 = m4 = 0.f;
+        am = 0x7fffffff; inf = 0;
+        float xs = -CUDART_INF_F, xt = -CUDART_INF_F;
+        for_elements(s, t, seg0, seg1, lane, [&](int v, float a, float bt) {
+          const double es = ex2(fma(c, (double)a, ks)), et = ex2(fma(c, (double)bt, kt));
+          const double d = ((double)bt - (double)a) - dd0;
+          ss += es; st += et; n1 = fma(et, d, n1);
+          const float df = (bt - a) - d0, ef = (float)es;
+          const float w1 = ef * df, q = df * df, w2 = ef * q;
+          m1 += w1; m2 += w2; m3 = fmaf(w1, q, m3); m4 = fmaf(w2, q, m4);
+          inf = max(inf, max(__float_as_int(a) & 0x7fffffff, __float_as_int(bt) & 0x7fffffff));
+          xs = fmaxf(xs, a);
+          if (bt > xt) { xt = bt; am = v; }
+        });
 #pragma unroll
-      for (int w = 1; w < GW; ++w) {
-        ms = fmaxf(ms, sh.fmax_s[w]);
-        if (sh.fmax_t[w] > mt || (sh.fmax_t[w] == mt && sh.arg_t[w] < am)) { mt = sh.fmax_t[w]; am = sh.arg_t[w]; }
+        for (int o = 16; o > 0; o >>= 1) {
+          xs = fmaxf(xs, __shfl_xor_sync(0xffffffffu, xs, o));
+          const float oxt = __shfl_xor_sync(0xffffffffu, xt, o);
+          const int oam = __shfl_xor_sync(0xffffffffu, am, o);
+          if (oxt > xt || (oxt == xt && oam < am)) { xt = oxt; am = oam; }
+        }
+        again = fma(c, (double)xs, ks) > 900.0 || fma(c, (double)xt, kt) > 900.0;   // 2^y left its range: once more under the true maxima
+        ms = xs; mt = xt;
+        if (!again) break;
       }
-      __syncthreads();
-    } else {
-      cg::cluster_group cl = cg::this_cluster();
-      if (tid == 0) sh.finite = finite;
-      cl.sync();
-      ms = -CUDART_INF_F; mt = -CUDART_INF_F; am = 0x7fffffff; finite = 1;
-      for (int r = 0; r < CS; ++r) {
-        const Shared* rs = cl.map_shared_rank(&sh, r);
-        finite &= rs->finite;
-        for (int w = 0; w < GW; ++w) {
-          ms = fmaxf(ms, rs->fmax_s[w]);
-          const float omt = rs->fmax_t[w];
-          const int oam = rs->arg_t[w];
-          if (omt > mt || (omt == mt && oam < am)) { mt = omt; am = oam; }
+      ss = warp_sum(ss); st = warp_sum(st); n1 = warp_sum(n1);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        m1 += __shfl_xor_sync(0xffffffffu, m1, o); m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+        m3 += __shfl_xor_sync(0xffffffffu, m3, o); m4 += __shfl_xor_sync(0xffffffffu, m4, o);
+      }
+      inf = __any_sync(0xffffffffu, inf >= 0x7f800000);
+      if (lane == 0) {
+        double* const p = sh.part[ph][warp];
+        p[PA_KS] = ks; p[PA_KT] = kt; p[PA_SS] = ss; p[PA_ST] = st; p[PA_N1] = n1;
+        p[PA_M1] = (double)m1; p[PA_M2] = (double)m2; p[PA_M3] = (double)m3; p[PA_M4] = (double)m4;
+        p[PA_MS] = (double)ms; p[PA_MT] = (double)mt; p[PA_AM] = inf ? -1.0 : (double)am;
+      }
+    }
+    phase_barrier();
+    // the coupling decision and the constants of pass "final" (warp 0, once lambda is known)
+    auto decide_row = [&](uint32_t status) {
+      const double lam = bc[G_LAM], lse_s = -LN2 * bc[G_KP], lse_t = bc[G_LSE_T];
+      double lp_x = 0.0, lT_x = 0.0, acc = 1.0;
+      int corrected = 0, tok = -1;
+      if (!bonus) {
+        lp_x = (double)ld_as_float(s, x) / (double)P.temperature - lse_s;
+        lT_x = (double)ld_as_float(t, x) / (double)P.temperature - lse_t;
+        if (lam > 0.0) {
+          acc = exp(fmin(0.0, lam * (lT_x - lp_x) - bc[G_LOGZ]));
+          corrected = (scalar_uniform(P.seed, rid, STAGE_ACCEPT) < acc) ? 0 : 1;
         }
       }
-      cl.sync();
+      double loss = 0.0, coef = 0.0;                         // gradient = coef (p - onehot(tok)) / tau
+      if (masked) status |= SAKI_ROW_MASKED;
+      else if (!bonus) {
+        if (!corrected) { loss = (lp_x - lT_x) * lp_x; coef = -(lp_x - lT_x); tok = x; }
+        else { coef = 1.0; tok = (int)bc[G_AM]; }            // (the loss, -log p(v*), is filled in when the row is written)
+      }
+      __syncwarp();
+      bc[G_STATUS] = (double)status; bc[G_CORR] = (double)corrected; bc[G_TOK] = (double)tok;
+      bc[G_SC] = (double)P.grad_scale * coef * rtau;
+      bc[G_ACC] = acc; bc[G_LPX] = lp_x; bc[G_LTX] = lT_x; bc[G_LOSS] = loss; bc[G_MODE] = (double)G_FINAL;
+    };
+    if (warp == 0) {
+      double S = 0.0, St = 0.0, N1 = 0.0, M1 = 0.0, M2 = 0.0, M3 = 0.0, M4 = 0.0, ms = -CUDART_INF, mt = -CUDART_INF, am = 2147483647.0;
+      bool finite = true;
+      for (int w = lane; w < NWC; w += 32) {
+        const double* const p = part_of(w);
+        if (p[PA_AM] < 0.0) finite = false;
+        ms = fmax(ms, p[PA_MS]);
+        if (p[PA_MT] > mt || (p[PA_MT] == mt && p[PA_AM] < am)) { mt = p[PA_MT]; am = p[PA_AM]; }
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        ms = fmax(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+        const double omt = __shfl_xor_sync(0xffffffffu, mt, o), oam = __shfl_xor_sync(0xffffffffu, am, o);
+        if (omt > mt || (omt == mt && oam < am)) { mt = omt; am = oam; }
+      }
+      finite = __all_sync(0xffffffffu, finite);
+      const double ks = -ceil(c * ms), kt = -ceil(c * mt);
+      for (int w = lane; w < NWC; w += 32) {
+        const double* const p = part_of(w);
+        if (!(p[PA_MS] > -CUDART_INF)) continue;             // an empty segment
+        const double fs = pow2_down(ks - p[PA_KS]), ft = pow2_down(kt - p[PA_KT]);
+        S += fs * p[PA_SS]; St += ft * p[PA_ST]; N1 += ft * p[PA_N1];
+        M1 += fs * p[PA_M1]; M2 += fs * p[PA_M2]; M3 += fs * p[PA_M3]; M4 += fs * p[PA_M4];
+      }
+      S = warp_sum(S); St = warp_sum(St); N1 = warp_sum(N1);
+      M1 = warp_sum(M1); M2 = warp_sum(M2); M3 = warp_sum(M3); M4 = warp_sum(M4);
+      uint32_t status = 0;
+      if (!finite) status = SAKI_ROW_NONFINITE;
+      else if (!bonus && (x < 0 || x >= V)) status = SAKI_ROW_BAD_ID;
+      bc[G_AM] = am;
+      if (status) { bc[G_STATUS] = (double)status; bc[G_MODE] = (double)G_FLAG; }
+      else {
+        const double lse_s = log(S) - ks * LN2, lse_t = log(St) - kt * LN2, cc = lse_t - lse_s;
+        bc[G_KP] = -INV_LN2 * lse_s; bc[G_CC] = cc; bc[G_LSE_T] = lse_t;
+        const double kl1 = (N1 / St + (double)d0) * rtau - cc;                // KL(T || p)
+        const bool endpoint = !(eps > 0.0) || kl1 <= eps;
+        bc[G_LOGZ] = 0.0; bc[G_STATUS] = 0.0;
+        bc[G_LAM] = !(eps > 0.0) ? 0.0 : 1.0; bc[G_KL] = !(eps > 0.0) ? 0.0 : kl1;
+        __syncwarp();
+        if (endpoint) decide_row(!(eps > 0.0) ? SAKI_ROW_EPS_ZERO : SAKI_ROW_SATURATED);
+        else {
+          const double rS = 1.0 / S;
+          double beta = first_guess(M1 * rS, M2 * rS, M3 * rS, M4 * rS, rtau, kl1, eps);
+          if (P.from_list && P.redo_guess) {     // the float32 kernel's value of lambda, good to ~1e-5: one evaluation from here
+            const double g0 = (double)P.redo_guess[item];
+            if (g0 > 0.0 && g0 < 1.0) beta = g0;
+          }
+          bc[G_BETA] = beta; bc[G_LO] = 0.0; bc[G_HI] = 1.0; bc[G_ITER] = 0.0; bc[G_MODE] = (double)G_SOLVE;
+        }
+      }
     }
+    __syncthreads();
+    ph ^= 1;
 
-    uint32_t status = 0;
-    if (!finite) status = SAKI_ROW_NONFINITE;
-    else if (!bonus && (x < 0 || x >= V)) status = SAKI_ROW_BAD_ID;
-    if (status) {   // flagged row: zero outputs, zero gradient row
+    if ((int)bc[G_MODE] == G_FLAG) {   // flagged row: zero outputs, zero gradient row
       if (tid == 0 && crank == 0) {
-        write_row(P.out, row, zero_row(status), !P.spec);
+        write_row(P.out, row, zero_row((uint32_t)bc[G_STATUS]), !P.spec);
         atomicAdd(P.flagged, 1ull);
       }
-      if (g) for (int v = e0; v < V; v += ET) st_from_float(g, v, 0.f);
+      if (g) for (int v = seg0 + lane; v < seg1; v += 32) st_from_float(g, v, 0.f);
       continue;
     }
 
-    // ---- pass 1: log-sum-exp of both rows
-    const double zms = (double)ms / tau, zmt = (double)mt / tau;
-    double acc2[2] = {0.0, 0.0};
-    for (int v = e0; v < V; v += ET) {
-      acc2[0] += exp((double)ld_as_float(s, v) / tau - zms);
-      acc2[1] += exp((double)ld_as_float(t, v) / tau - zmt);
-    }
-    block_sum<2, CS>(acc2, sh.red);
-    const double lse_s = zms + log(acc2[0]), lse_t = zmt + log(acc2[1]);
-
-    // ---- lambda
-    double lam = 0.0, Lam = 0.0;   // Lam = log Z(lambda) = log sum p exp(lambda d)
-    if (!(eps > 0.0)) {
-      status |= SAKI_ROW_EPS_ZERO;
-    } else {
-      // pass 2: KL(T||p) and the variance of d under p (initial guess)
-      double a3[3] = {0.0, 0.0, 0.0};
-      for (int v = e0; v < V; v += ET) {
-        const double lp = (double)ld_as_float(s, v) / tau - lse_s;
-        const double lT = (double)ld_as_float(t, v) / tau - lse_t;
-        const double d = lT - lp, p = exp(lp);
-        a3[0] += exp(lT) * d;
-        a3[1] += p * d;
-        a3[2] += p * d * d;
+    // ---- pass "solve": one evaluation of KL(q_beta || p) and its derivatives
+    const double kp = bc[G_KP], cc = bc[G_CC];
+    while ((int)bc[G_MODE] == G_SOLVE) {
+      const double bi = bc[G_BETA] * INV_LN2;
+      double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
+      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) {
+        const double sd = (double)a, d = fma((double)bt - sd, rtau, -cc);
+        const double e = ex2(fma(bi, d, fma(c, sd, kp)));
+        const double w1 = e * d, q = d * d, w2 = e * q;
+        a0 += e; a1 += w1; a2 += w2; a3 = fma(w1, q, a3); a4 = fma(w2, q, a4);
+      });
+      a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3); a4 = warp_sum(a4);
+      if (lane == 0) {
+        double* const p = sh.part[ph][warp];
+        p[0] = a0; p[1] = a1; p[2] = a2; p[3] = a3; p[4] = a4;
       }
-      block_sum<3, CS>(a3, sh.red);
-      if (a3[0] <= eps) {
-        lam = 1.0;
-        status |= SAKI_ROW_SATURATED;
-      } else {
-        // KL(q_beta||p) is increasing in beta with slope beta Var_q(d):
-        // Newton on KL(beta) = eps, kept inside a bisection bracket.
-        const double varp = a3[2] - a3[1] * a3[1];
-        double lo = 0.0, hi = 1.0;
-        double beta = sqrt(2.0 * eps / fmax(varp, 1e-300));
-        if (!(beta > 0.0 && beta < 1.0)) beta = 0.5;
-        if (P.from_list && P.redo_guess) {       // the float32 kernel's value of lambda, good to ~1e-5: two steps from here
-          const double g0 = (double)P.redo_guess[item];
-          if (g0 > 0.0 && g0 < 1.0) beta = g0;
+      phase_barrier();
+      if (warp == 0) {
+        double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        for (int w = lane; w < NWC; w += 32) {
+          const double* const p = part_of(w);
+#pragma unroll
+          for (int k = 0; k < 5; ++k) v[k] += p[k];
         }
-        for (int it = 0; it < 100; ++it) {
-          double a[3] = {0.0, 0.0, 0.0};
-          for (int v = e0; v < V; v += ET) {
-            const double lp = (double)ld_as_float(s, v) / tau - lse_s;
-            const double lT = (double)ld_as_float(t, v) / tau - lse_t;
-            const double d = lT - lp, e = exp(lp + beta * d);
-            a[0] += e;
-            a[1] += e * d;
-            a[2] += e * d * d;
-          }
-          block_sum<3, CS>(a, sh.red);
-          const double E = a[1] / a[0], var = a[2] / a[0] - E * E;
-          const double kl = beta * E - log(a[0]);
-          if (kl <= eps) lo = beta; else hi = beta;
-          if (hi - lo < 1e-15) break;
-          const double step = (eps - kl) / (beta * var);
-          // at the root to rounding: stop here (a step that small can fall outside the bracket, and the
-          // bisection that would follow costs some thirty more passes for nothing)
-          if (fabs(step) < 1e-13) { beta = fmin(fmax(beta + step, lo), hi); break; }
-          double nb = beta + step;
-          if (!(nb > lo && nb < hi)) nb = 0.5 * (lo + hi);
-          beta = nb;
-        }
-        lam = beta;
-      }
-      // log Z at the final coefficient
-      double z1[1] = {0.0};
-      for (int v = e0; v < V; v += ET) {
-        const double lp = (double)ld_as_float(s, v) / tau - lse_s;
-        const double lT = (double)ld_as_float(t, v) / tau - lse_t;
-        z1[0] += exp(lp + lam * (lT - lp));
-      }
-      block_sum<1, CS>(z1, sh.red);
-      Lam = log(z1[0]);
-    }
-
-    // ---- TV, KL at lambda; partial sums kept per warp segment in index order
-    const int NWC = GW * CS;                              // warps of the cluster, in index order of their segments
-    const int seg = (V + NWC - 1) / NWC;
-    const int gw = crank * GW + warp;
-    const int seg0 = min(V, gw * seg), seg1 = min(V, seg0 + seg);
-    double tv = 0.0, kl = 0.0, tv_true = 0.0;
-    if (lam > 0.0 || bonus) {
-      double part = 0.0, klp[2] = {0.0, 0.0};   // klp[1]: TV of a bonus row (its draw weights are q)
-      for (int v = seg0 + lane; v < seg1; v += 32) {
-        const double lp = (double)ld_as_float(s, v) / tau - lse_s;
-        const double lT = (double)ld_as_float(t, v) / tau - lse_t;
-        const double lq = lp + lam * (lT - lp) - Lam;
-        const double q = exp(lq);
-        const double r = fmax(q - exp(lp), 0.0);
-        part += bonus ? q : r;
-        klp[0] += q * (lq - lp);
-        klp[1] += r;
-      }
-      part = warp_sum(part);
-      if (lane == 0) sh.warp_tot[warp] = part;
-      block_sum<2, CS>(klp, sh.red);   // its first barrier publishes warp_tot (to the cluster)
-      kl = klp[0];
-      tv_true = klp[1];
-      if (tid < NWC) {                 // every warp's weight of the cluster, in segment order, into this block's copy
-        if constexpr (CS == 1) sh.wt_all[tid] = sh.warp_tot[tid];
-        else sh.wt_all[tid] = cg::this_cluster().map_shared_rank(&sh, tid / GW)->warp_tot[tid % GW];
+#pragma unroll
+        for (int k = 0; k < 5; ++k) v[k] = warp_sum(v[k]);
+        if (solve_step(bc, v, eps)) decide_row(0u);
       }
       __syncthreads();
-      for (int w = 0; w < NWC; ++w) tv += sh.wt_all[w];
+      ph ^= 1;
     }
 
-    // ---- the coupling decision (every thread computes the same scalars)
-    double lp_x = 0.0, lT_x = 0.0, acc_p = 1.0;
-    int corrected = 0;
-    if (!bonus) {
-      lp_x = (double)ld_as_float(s, x) / tau - lse_s;
-      lT_x = (double)ld_as_float(t, x) / tau - lse_t;
-      if (lam > 0.0) {
-        acc_p = exp(fmin(0.0, lam * (lT_x - lp_x) - Lam));
-        const double u = scalar_uniform(P.seed, rid, STAGE_ACCEPT);
-        corrected = (u < acc_p) ? 0 : 1;
+    // ---- pass "final": total variation, draw weights (of a bonus row: q itself) and the gradient
+    const double li = bc[G_LAM] * INV_LN2, iz = exp(-bc[G_LOGZ]);
+    const bool corrected = bc[G_CORR] != 0.0, draw = corrected || bonus;
+    // p, and r = [q - p]_+ of an element
+    auto residual = [&](float a, float bt, double& p, double& e) {
+      const double sd = (double)a, d = fma((double)bt - sd, rtau, -cc), lp = fma(c, sd, kp);
+      p = ex2(lp);
+      e = ex2(fma(li, d, lp));
+      const double r = fma(e, iz, -p);
+      const int neg = __double2hiint(r) >> 31;               // max(r, 0) without the float64 pipe
+      return __hiloint2double(__double2hiint(r) & ~neg, __double2loint(r) & ~neg);
+    };
+    double tv = 0.0, wq = 0.0;
+    if (g) {
+      const double sc = bc[G_SC];
+      const int tok = (int)bc[G_TOK];
+      for_elements(s, t, seg0, seg1, lane, [&](int v, float a, float bt) {
+        double p, e;
+        tv += residual(a, bt, p, e);
+        double gv = sc * p;
+        if (v == tok) gv = sc * (p - 1.0);
+        put(g, v, gv);
+      });
+    } else if (bonus) {
+      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) { double p, e; tv += residual(a, bt, p, e); wq += e; });
+    } else if (li > 0.0) {
+      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) { double p, e; tv += residual(a, bt, p, e); });
+    }
+    tv = warp_sum(tv);
+    if (bonus) wq = warp_sum(wq);
+    if (lane == 0) { sh.part[ph][warp][0] = tv; sh.part[ph][warp][1] = bonus ? wq : tv; }
+    phase_barrier();
+    if (warp == 0) {   // the total, and for a draw the warp that owns the inverse-CDF target
+      double tvs = 0.0, wa[2] = {0.0, 0.0};
+      constexpr int PER = NWC > 32 ? 2 : 1;                  // consecutive warps per lane: index order
+#pragma unroll
+      for (int q = 0; q < PER; ++q) {
+        const int w = lane * PER + q;
+        if (w < NWC) { const double* const p = part_of(w); tvs += p[0]; wa[q] = p[1]; }
       }
+      tvs = warp_sum(tvs);
+      int owner = 0;
+      if (draw) {
+        double inc = wa[0] + wa[1];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const double up = __shfl_up_sync(0xffffffffu, inc, o);
+          if (lane >= o) inc += up;
+        }
+        const double target = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL) * __shfl_sync(0xffffffffu, inc, 31);
+        const unsigned hit = __ballot_sync(0xffffffffu, inc > target), pos = __ballot_sync(0xffffffffu, wa[0] + wa[1] > 0.0);
+        // rounding left no crossing: the last index with positive weight
+        const int ol = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
+        double before = inc - (wa[0] + wa[1]);
+        int q = 0;
+        if (PER == 2 && (hit ? !(before + wa[0] > target) : wa[1] > 0.0)) { q = 1; before += wa[0]; }
+        before = __shfl_sync(0xffffffffu, before, ol);
+        owner = ol * PER + __shfl_sync(0xffffffffu, q, ol);
+        bc[G_OWNER] = (double)owner; bc[G_BEFORE] = before; bc[G_TARGET] = target; bc[G_LAST] = hit ? 0.0 : 1.0;
+      }
+      bc[G_TV] = tvs;
     }
     int y = x;
-    if (corrected || bonus) {
-      // inverse CDF in index order: smallest index whose running sum exceeds u * total
-      const double u = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
-      const double target = u * tv;
-      int owner = -1;
-      double before = 0.0;
-      for (int w = 0; w < NWC; ++w) {
-        if (before + sh.wt_all[w] > target) { owner = w; break; }
-        before += sh.wt_all[w];
-      }
-      bool take_last = false;
-      if (owner < 0) {   // rounding left no crossing: last index with positive weight
-        take_last = true;
-        before = 0.0;
-        for (int w = NWC - 1; w >= 0; --w) if (sh.wt_all[w] > 0.0) { owner = w; break; }
-        if (owner < 0) owner = 0;
-      }
-      if (tid == 0) sh.token = -1;
+    bool writer = tid == 0 && crank == 0;
+    if (draw) {        // (all threads of the block agree)
       __syncthreads();
-      if (gw == owner) {
-        double running = before;
-        int last_pos = -1, found = -1;
-        for (int v0 = owner * seg; v0 < V && found < 0; v0 += 32) {
-          const int v = v0 + lane;
-          double r = 0.0;
-          if (v < V) {
-            const double lp = (double)ld_as_float(s, v) / tau - lse_s;
-            const double lT = (double)ld_as_float(t, v) / tau - lse_t;
-            const double q = exp(lp + lam * (lT - lp) - Lam);
-            r = bonus ? q : fmax(q - exp(lp), 0.0);
-          }
-          double inc = r;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            const double up = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += up;
-          }
-          const unsigned pos = __ballot_sync(0xffffffffu, r > 0.0);
-          const unsigned hit = take_last ? 0u : __ballot_sync(0xffffffffu, (running + inc > target) && v < V);
-          if (pos) last_pos = v0 + 31 - __clz(pos);
-          if (hit) found = v0 + __ffs(hit) - 1;
-          running += __shfl_sync(0xffffffffu, inc, 31);
+      const int owner = (int)bc[G_OWNER];
+      writer = false;
+      if (owner / GW == crank) {
+        // the owner's segment once more, an eighth per warp; the warp whose part holds the target walks it
+        const double target = bc[G_TARGET];
+        bool last = bc[G_LAST] != 0.0;
+        const int o0 = min(V, owner * seg), o1 = min(V, o0 + seg), sl = (((o1 - o0 + GW - 1) / GW) + 31) & ~31;
+        auto weight = [&](int v) {
+          double p, e;
+          const double r = residual(ld_as_float(s, v), ld_as_float(t, v), p, e);
+          return bonus ? e : r;
+        };
+        double w = 0.0;
+        for (int v = o0 + warp * sl + lane; v < min(o1, o0 + (warp + 1) * sl); v += 32) w += weight(v);
+        w = warp_sum(w);
+        if (lane == 0) sh.sub[warp] = w;
+        __syncthreads();
+        double running = bc[G_BEFORE], at = running;
+        int mine = -1, lastpos = 0;
+        double lastat = running;
+        for (int k = 0; k < GW; ++k) {
+          const double wk = sh.sub[k];
+          if (wk > 0.0) { lastpos = k; lastat = running; }
+          if (mine < 0 && !last && running + wk > target) { mine = k; at = running; }
+          running += wk;
         }
-        if (found < 0) found = (last_pos >= 0) ? last_pos : (V - 1);
-        if (lane == 0) sh.token = found;
-      }
-      if constexpr (CS == 1) {
-        __syncthreads();
-        y = sh.token;
-        __syncthreads();
-      } else {             // the owning warp's block holds the token
-        cg::cluster_group cl = cg::this_cluster();
-        cl.sync();
-        y = cl.map_shared_rank(&sh, owner / GW)->token;
-        cl.sync();
+        if (mine < 0) { mine = lastpos; at = lastat; last = true; }
+        if (warp == mine) {
+          int last_pos = -1, found = -1;
+          const int e1 = min(o1, o0 + (mine + 1) * sl);
+          for (int v0 = o0 + mine * sl; v0 < e1 && found < 0; v0 += 32) {
+            const int v = v0 + lane;
+            const double r = v < e1 ? weight(v) : 0.0;
+            double inc = r;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const double up = __shfl_up_sync(0xffffffffu, inc, o);
+              if (lane >= o) inc += up;
+            }
+            const unsigned pos = __ballot_sync(0xffffffffu, r > 0.0);
+            const unsigned hit = last ? 0u : __ballot_sync(0xffffffffu, at + inc > target && v < e1);
+            if (pos) last_pos = v0 + 31 - __clz(pos);
+            if (hit) found = v0 + __ffs(hit) - 1;
+            at += __shfl_sync(0xffffffffu, inc, 31);
+          }
+          if (found < 0) found = last_pos >= 0 ? last_pos : V - 1;
+          y = found;
+          writer = lane == 0;
+        }
       }
     }
-
-    // ---- routed loss and gradient coefficients
-    const double lp_v = (double)ld_as_float(s, am) / tau - lse_s;   // log p(v*)
-    double loss = 0.0, coef = 0.0;   // gradient = coef * (p - onehot(tok)) / tau
-    int tok = 0;
-    if (masked) {
-      status |= SAKI_ROW_MASKED;
-    } else if (!bonus) {
-      if (!corrected) { loss = (lp_x - lT_x) * lp_x; coef = -(lp_x - lT_x); tok = x; }
-      else { loss = -lp_v; coef = 1.0; tok = am; }
-    }
-    if (tid == 0 && crank == 0) {
+    if (writer) {
+      const double lam = bc[G_LAM], lse_s = -LN2 * kp, lse_t = bc[G_LSE_T], Lam = bc[G_LOGZ], tau = (double)P.temperature;
+      const double lp_x = bc[G_LPX], lT_x = bc[G_LTX];
       RowResult r;
-      r.corrected = corrected; r.token = y; r.vstar = am;
-      r.lambda = (float)lam; r.kl = (float)(lam > 0.0 ? kl : 0.0);
-      r.tv = (float)((lam > 0.0) ? (bonus ? tv_true : tv) : 0.0);
-      r.accept = bonus ? 0.f : (float)acc_p;
+      r.status = (uint32_t)bc[G_STATUS];
+      r.corrected = corrected ? 1 : 0; r.token = y; r.vstar = (int)bc[G_AM];
+      r.lambda = (float)lam; r.kl = (float)bc[G_KL];
+      r.tv = lam > 0.0 ? (float)bc[G_TV] : 0.f;
+      r.accept = bonus ? 0.f : (float)bc[G_ACC];
       r.logp_x = (float)lp_x; r.logT_x = (float)lT_x;
       r.logq_x = bonus ? 0.f : (float)(lp_x + lam * (lT_x - lp_x) - Lam);
-      const double lp_y = (double)ld_as_float(s, y) / tau - lse_s;
-      const double lT_y = (double)ld_as_float(t, y) / tau - lse_t;
-      r.logp_y = (float)lp_y;
+      const double lp_y = (double)ld_as_float(s, y) / tau - lse_s, lT_y = (double)ld_as_float(t, y) / tau - lse_t;
+      r.logp_y = (float)lp_y; r.logT_y = (float)lT_y;
       r.logq_y = (float)(lp_y + lam * (lT_y - lp_y) - Lam);
-      r.logT_y = (float)lT_y;
-      r.loss = (float)loss;
-      r.status = status;
+      r.loss = (float)bc[G_LOSS];
+      if (corrected && !masked) r.loss = (float)-((double)ld_as_float(s, r.vstar) / tau - lse_s);
       write_row(P.out, row, r, !P.spec);
     }
-    if (g) {
-      const double sc = (double)P.grad_scale * coef / tau;
-      for (int v = e0; v < V; v += ET) {
-        const double p = exp((double)ld_as_float(s, v) / tau - lse_s);
-        const double gv = sc * (p - (v == tok ? 1.0 : 0.0));
-        if constexpr (sizeof(T) == 2) g[v] = __double2bfloat16(gv);
-        else g[v] = (float)gv;
-      }
-    }
+    ph ^= 1;
   }
   if constexpr (CS > 1) cg::this_cluster().sync();   // no block leaves while a peer may still read its shared memory
 }
 
-constexpr int LIST_CS = 8;   // blocks per row in list mode
-
-template <typename T>
-static cudaError_t launch_list(const RowParams& p, int sms, cudaStream_t st) {
+template <typename T, int CS>
+static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t st) {
+  // blocks (clusters) that are resident at once: the grid, so that none starts after the others have finished
+  static std::atomic<int> fit_of[64];
+  int fit = dev < 64 ? fit_of[dev].load(std::memory_order_relaxed) : 0;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)((sms / LIST_CS) * LIST_CS), 1, 1);
   cfg.blockDim = dim3(GT, 1, 1);
-  cfg.dynamicSmemBytes = 0;
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = LIST_CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, general_kernel<T, LIST_CS>, p);
+  at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
+  if (fit <= 0) {
+    int n = 0;
+    cudaError_t e;
+    if (CS > 1) {
+      cfg.gridDim = dim3(CS, 1, 1);
+      e = cudaOccupancyMaxActiveClusters(&n, general_kernel<T, CS>, &cfg);
+    } else {
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, general_kernel<T, CS>, GT, 0);
+      n *= sms;
+    }
+    if (e != cudaSuccess) return e;
+    fit = n > 0 ? n : 1;
+    if (dev < 64) fit_of[dev].store(fit, std::memory_order_relaxed);
+  }
+  cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit ? p.n_rows : fit)), 1, 1);
+  return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p);
+}
+
+template <typename T>
+static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
+  // Blocks per row.  In list mode (a handful of rows as a rule; the host does not know their number) always the most;
+  // otherwise so many that few rows still fill the chip, each block keeping 1024 elements or more (below that the
+  // barriers of a cluster cost more than its blocks save), and that the rows in flight stay in L2 between the passes.
+  int cs = 1;
+  const int64_t in_flight = 3 * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
+  while (cs < MAX_CS && p.V >= 2048 * cs &&
+         (p.from_list || p.n_rows * cs < in_flight || in_flight / cs * row_bytes > (64 << 20)))
+    cs *= 2;
+  switch (cs) {
+    case 1: return launch_cs<T, 1>(p, dev, sms, st);
+    case 2: return launch_cs<T, 2>(p, dev, sms, st);
+    case 4: return launch_cs<T, 4>(p, dev, sms, st);
+    default: return launch_cs<T, 8>(p, dev, sms, st);
+  }
 }
 
 cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* n_launches) {
@@ -405,20 +598,7 @@ cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* 
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (n_launches) *n_launches += 1;
-  RowParams q = p;
-  q.list_min = 0; q.list_max = 0;
-  if (p.from_list && sms >= LIST_CS) {   // the rows the bf16 kernels handed over: a cluster per row while they are few
-    q.list_min = 0; q.list_max = 3 * (sms / LIST_CS);
-    cudaError_t e = dtype == SAKI_BF16 ? launch_list<__nv_bfloat16>(q, sms, st) : launch_list<float>(q, sms, st);
-    if (e != cudaSuccess) return e;
-    if (n_launches) *n_launches += 1;
-    q.list_min = q.list_max + 1; q.list_max = 0x7fffffff;
-  }
-  const int64_t cap = (int64_t)sms * (p.from_list ? 1 : 3);
-  const int grid = (int)(p.n_rows < cap ? p.n_rows : cap);
-  if (dtype == SAKI_BF16) general_kernel<__nv_bfloat16, 1><<<grid, GT, 0, st>>>(q);
-  else general_kernel<float, 1><<<grid, GT, 0, st>>>(q);
-  return cudaGetLastError();
+  return dtype == SAKI_BF16 ? launch_t<__nv_bfloat16>(p, dev, sms, st) : launch_t<float>(p, dev, sms, st);
 }
 
 }  // namespace saki
