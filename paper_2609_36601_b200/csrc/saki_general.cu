@@ -12,7 +12,7 @@
 //     4e-17).  The table is stored 16 times over, one copy per 64-bit bank, so a half-warp's lookups never conflict;
 //   - three passes over the row: "sums" (two exponentials), one or two evaluations of KL with its first four
 //     derivatives (one exponential each: the root of the fourth-order model, as in the bf16 kernels, here accepted
-//     when the dropped terms move lambda by less than 1e-10), "final" (two exponentials; total variation, draw
+//     when the dropped terms move lambda by less than about 1e-11), "final" (two exponentials; total variation, draw
 //     weights and the gradient in one pass).  The row's maxima come out of pass "sums" itself: every warp runs
 //     under shifts fixed from its first elements (whole powers of two, so warps combine exactly) and repeats its
 //     part with the true maxima if they turn out so much larger that its sums could have overflowed;
@@ -31,6 +31,9 @@ namespace {
 
 constexpr int GT = 256;        // threads per block
 constexpr int GW = GT / 32;    // warps per block
+// Blocks per SM: more of them hide one another's serial steps, fewer have the registers to interleave elements.
+// Measured (2 / 3 / 4): bf16 rows of 32003 0.275 / 0.280 / 0.309 ms, fp32 rows of 151936 0.784 / 0.786 / 0.734 ms.
+template <typename T> constexpr int BLOCKS_PER_SM = sizeof(T) == 4 ? 4 : 3;
 constexpr int MAX_CS = 8;      // blocks per row, at most
 constexpr int TAB = 256, COPIES = 16;
 constexpr int NPART = 12;      // doubles a warp leaves per phase
@@ -40,6 +43,9 @@ struct Shared {
   double part[2][GW][NPART];   // alternates from phase to phase: one barrier per phase is enough
   double bc[32];               // scalars broadcast to the block
   double sub[GW];
+  alignas(16) unsigned char answer[16];
+  uint64_t bar;
+  int next[2];
 };
 enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G_LO, G_HI, G_ITER, G_AM, G_OWNER, G_BEFORE,
        G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_COUNT };
@@ -47,8 +53,14 @@ static_assert(G_COUNT <= 32, "broadcast area too small");
 enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
 
+// The entry of 2^(i/256) has i << 12 taken off its high word: adding the low word of y + M, shifted by 12, then puts
+// the exponent in and the index back in one addition.
+// The coefficients are read from the constant bank (as operands: three 64-bit immediates cost two moves each per
+// exponential once registers are short, and a float64 operation on three register operands runs at two thirds of the rate).
+__constant__ double EXP2_COEF[4] = {9.618129107628477e-03, 5.550410866482158e-02, 2.402265069591007e-01, 6.931471805599453e-01};   // ln2^i / i!, i = 4..1
 struct Exp2 {
-  uint32_t base;   // shared-memory address of this lane's copy of the table
+  uint32_t lane8;   // this lane's copy of the table: byte offset among the 16 copies of an entry
+  const double* tab;
   // 2^y for y <= ~1000; y below -1000 counts as -1000 (clamped through the high word: an unsigned minimum)
   __device__ __forceinline__ double operator()(double y) const {
     const uint32_t hi = min((uint32_t)__double2hiint(y), 0xC08F4000u);
@@ -57,56 +69,105 @@ struct Exp2 {
     const double t = y + M;
     const double r = y - (t - M);
     const int k = __double2loint(t);
-    double T;
-    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(T) : "r"(base + (((uint32_t)k << 7) & 0x7f80u)));
-    // Taylor coefficients of 2^r: ln2^i / i!
-    double q = fma(r, 9.618129107628477e-03, 5.550410866482158e-02);
-    q = fma(r, q, 2.402265069591007e-01);
-    q = fma(r, q, 6.931471805599453e-01);
-    T = __hiloint2double(__double2hiint(T) + ((k << 12) & 0xfff00000), __double2loint(T));
+    double T = *(const double*)((const char*)tab + ((((uint32_t)k << 7) & 0x7f80u) | lane8));
+    double q = fma(r, EXP2_COEF[0], EXP2_COEF[1]);
+    q = fma(r, q, EXP2_COEF[2]);
+    q = fma(r, q, EXP2_COEF[3]);
+    T = __hiloint2double(__double2hiint(T) + (k << 12), __double2loint(T));
     return fma(T * r, q, T);
   }
 };
+
+// Dynamic rows: a block (cluster) that is done takes over the work of one that has not started yet, by cancelling its
+// launch.  The answer arrives in shared memory and completes an mbarrier.
+__device__ __forceinline__ void steal_request(void* answer, uint64_t* bar) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the last answer has been read
+  mbar_expect_tx(bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(smem_addr(answer)), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ int steal_answer(const void* answer) {   // first block index of the cancelled cluster, or -1
+  uint32_t ok, x;
+  asm volatile("{\n\t.reg .b128 h;\n\t.reg .pred p;\n\tld.shared.b128 h, [%2];\n\t"
+               "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\tselp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t"
+               "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n\t}"
+               : "=r"(ok), "=r"(x) : "r"(smem_addr(answer)) : "memory");
+  return ok ? (int)x : -1;
+}
 
 __device__ __forceinline__ double pow2_down(double n) {      // 2^n for whole n <= 0; 0 below -1000
   return n < -1000.0 ? 0.0 : __longlong_as_double((long long)(1023 + (int)n) << 52);
 }
 
-// float64 to bf16, one rounding to nearest even: through a float rounded to odd
-__device__ __forceinline__ __nv_bfloat16 to_bf16(double v) {
-  float f = __double2float_rz(v);
-  if ((double)f != v) f = __uint_as_float(__float_as_uint(f) | 1u);
-  return __float2bfloat16_rn(f);
+// float64 to float, ready to be rounded to bf16: truncated, with the last bit set if anything was dropped (rounded to
+// odd), so that the second rounding is the only one.  (The low 29 bits of a float64 do not fit a normal float.)
+__device__ __forceinline__ float to_odd(double v) {
+  return __uint_as_float(__float_as_uint(__double2float_rz(v)) | (uint32_t)((__double2loint(v) << 3) != 0));
 }
-template <typename T> __device__ __forceinline__ void put(T* g, int64_t i, double v);
-template <> __device__ __forceinline__ void put<float>(float* g, int64_t i, double v) { g[i] = (float)v; }
-template <> __device__ __forceinline__ void put<__nv_bfloat16>(__nv_bfloat16* g, int64_t i, double v) { g[i] = to_bf16(v); }
 
-// Runs body(v, s, t) over the elements v = lo + lane, lo + lane + 32, ... < hi: four at a time, the loads of the next
-// four issued before the current ones are used (the row comes from L2 in all passes but the first).
-template <typename T, typename F>
-__device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* __restrict__ t, int lo, int hi, int lane, F&& body) {
-  constexpr int U = 4;
-  const int full = lo + (hi - lo) / (32 * U) * (32 * U);
-  int v = lo + lane;
-  float a[U], b[U];
-  if (lo < full) {
+// Sixteen bytes of a row: eight bf16 or four fp32 elements.
+template <typename T> struct Chunk;
+template <> struct Chunk<__nv_bfloat16> {
+  static constexpr int W = 8;
+  uint32_t r[4];
+  __device__ __forceinline__ float get(int i) const { return __uint_as_float((i & 1) ? r[i >> 1] & 0xffff0000u : r[i >> 1] << 16); }
+  __device__ __forceinline__ void set2(int i, double a, double b) { r[i >> 1] = pack_bf16x2(to_odd(a), to_odd(b)); }
+  static __device__ __forceinline__ void put(__nv_bfloat16* g, double v) { *g = __float2bfloat16_rn(to_odd(v)); }
+};
+template <> struct Chunk<float> {
+  static constexpr int W = 4;
+  uint32_t r[4];
+  __device__ __forceinline__ float get(int i) const { return __uint_as_float(r[i]); }
+  __device__ __forceinline__ void set2(int i, double a, double b) { r[i] = __float_as_uint((float)a); r[i + 1] = __float_as_uint((float)b); }
+  static __device__ __forceinline__ void put(float* g, double v) { *g = (float)v; }
+};
+template <typename T> __device__ __forceinline__ Chunk<T> load_chunk(const T* p, bool vec) {
+  Chunk<T> c;
+  if (vec) {
+    const uint4 q = __ldg((const uint4*)p);
+    c.r[0] = q.x; c.r[1] = q.y; c.r[2] = q.z; c.r[3] = q.w;
+  } else {   // a row whose 16-byte boundaries are not the student row's
 #pragma unroll
-    for (int u = 0; u < U; ++u) { a[u] = ld_as_float(s, v + 32 * u); b[u] = ld_as_float(t, v + 32 * u); }
+    for (int i = 0; i < 4; ++i) {
+      if constexpr (sizeof(T) == 4) c.r[i] = __float_as_uint(p[i]);
+      else c.r[i] = (uint32_t)__bfloat16_as_ushort(p[2 * i]) | ((uint32_t)__bfloat16_as_ushort(p[2 * i + 1]) << 16);
+    }
+  }
+  return c;
+}
+
+// A warp's part of the row: the chunks [c0, c1) of the 16-byte chunks that start `head` elements into the row (the
+// student row's first 16-byte boundary); the first warp also takes the elements before them, the last one those after.
+struct Part { int c0, c1, head, x0, x1; };     // x0, x1: the extra elements (x0 == x1: none)
+
+// The chunks and extra elements of a warp's part: chunk(first element, s, t) and element(v, s, t).  The next chunk is on
+// its way while one is worked on (eight elements take a warp longer than a trip to memory).
+template <typename T, typename FC, typename FE>
+__device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* __restrict__ t, bool tvec, const Part& pt, int lane,
+                                             FC&& chunk, FE&& element) {
+  constexpr int W = Chunk<T>::W;
+  int k = pt.c0 + lane;
+  if (k < pt.c1) {
+    Chunk<T> a = load_chunk(s + pt.head + k * W, true), b = load_chunk(t + pt.head + k * W, tvec);
 #pragma unroll 1
-    for (; v < full; v += 32 * U) {
-      float na[U], nb[U];
-      const bool more = v + 32 * U < full;
-#pragma unroll
-      for (int u = 0; u < U; ++u) { na[u] = more ? ld_as_float(s, v + 32 * (U + u)) : 0.f; nb[u] = more ? ld_as_float(t, v + 32 * (U + u)) : 0.f; }
-#pragma unroll
-      for (int u = 0; u < U; ++u) body(v + 32 * u, a[u], b[u]);
-#pragma unroll
-      for (int u = 0; u < U; ++u) { a[u] = na[u]; b[u] = nb[u]; }
+    for (; k < pt.c1; k += 32) {
+      const int n = min(k + 32, pt.c1 - 1);
+      const Chunk<T> na = load_chunk(s + pt.head + n * W, true), nb = load_chunk(t + pt.head + n * W, tvec);
+      chunk(pt.head + k * W, a, b);
+      a = na; b = nb;
     }
   }
 #pragma unroll 1
-  for (; v < hi; v += 32) body(v, ld_as_float(s, v), ld_as_float(t, v));
+  for (int v = pt.x0 + lane; v < pt.x1; v += 32) element(v, ld_as_float(s, v), ld_as_float(t, v));
+}
+template <typename T, typename FE>
+__device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* __restrict__ t, bool tvec, const Part& pt, int lane,
+                                             FE&& element) {
+  for_elements(s, t, tvec, pt, lane,
+    [&](int v, const Chunk<T>& a, const Chunk<T>& b) {
+#pragma unroll
+      for (int i = 0; i < Chunk<T>::W; ++i) element(v + i, a.get(i), b.get(i));
+    }, element);
 }
 
 // The scalars between the passes, on one warp per block (all lanes alike).
@@ -162,9 +223,9 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
     else { nb = 0.5 * (lo + hi); bisected = true; }
   }
   h = nb - beta;
-  const double h2 = h * h;
-  const double trunc = fmax(fabs(c4), fmax(fabs(c3), 0.5 * fabs(c2))) * h2 * h2;
-  const bool done = (ok && !bisected && trunc <= 1e-10 * slope) || fabs(h) < 1e-13 || hi - lo < 1e-15 || iter >= 100;
+  // the first dropped term moves lambda by (k5 / k2) h^4 / 24; with D a scale of d under q, that is D^3 h^4 / 24
+  const double rv = 1.0 / var, D2 = fmax(var, fmax(k3 * rv * k3 * rv, fabs(k4) * rv)), h2 = h * h;
+  const bool done = (ok && !bisected && D2 * sqrt(D2) * h2 * h2 <= 2e-10) || fabs(h) < 1e-13 || hi - lo < 1e-15 || iter >= 100;
   __syncwarp();                                              // every lane has read the state
   if (done) {
     bc[G_LAM] = nb;
@@ -181,7 +242,7 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
 
 // CS: blocks per row (1, or a cluster of CS blocks).
 template <typename T, int CS>
-__global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
+__global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const RowParams P, const int steal, const double rtau, const double c) {
   __shared__ Shared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = P.V;
@@ -193,17 +254,20 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
   const int64_t n_work = P.from_list ? (int64_t)*P.redo_count : P.n_rows;
   if ((int64_t)(blockIdx.x / CS) >= n_work) return;          // the whole cluster: nothing to do (an empty row list, as a rule)
   for (int i = tid; i < TAB; i += GT) {
-    const double e = exp2((double)i * (1.0 / TAB));
+    double e = exp2((double)i * (1.0 / TAB));
+    e = __hiloint2double(__double2hiint(e) - (i << 12), __double2loint(e));
 #pragma unroll 1
     for (int c = 0; c < COPIES; ++c) sh.tab[i * COPIES + ((c + lane) & (COPIES - 1))] = e;
   }
+  if (tid == 0) {
+    mbar_init(&sh.bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
   __syncthreads();
   Exp2 ex2;
-  ex2.base = smem_addr(sh.tab) + (uint32_t)(lane & (COPIES - 1)) * 8u;
+  ex2.tab = sh.tab; ex2.lane8 = (uint32_t)(lane & (COPIES - 1)) * 8u;
 
-  const double rtau = 1.0 / (double)P.temperature, c = INV_LN2 * rtau, eps = (double)P.eps;
-  const int seg = (((V + NWC - 1) / NWC) + 31) & ~31;        // whole steps of 32 elements
-  const int seg0 = min(V, gw * seg), seg1 = min(V, seg0 + seg);
+  const double eps = (double)P.eps;     // (rtau = 1 / tau, c = log2(e) / tau)
   int ph = 0;
   double* const bc = sh.bc;
 
@@ -217,7 +281,9 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
     else return cg::this_cluster().map_shared_rank(&sh.part[ph][w % GW][0], w / GW);
   };
 
-  for (int64_t item = blockIdx.x / CS; item < n_work; item += gridDim.x / CS) {
+  const int64_t stride = gridDim.x / CS;
+  int turn = 0, nxt = -1;
+  for (int64_t item = blockIdx.x / CS; item >= 0 && item < n_work; item = steal ? (int64_t)nxt : item + stride) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;   // list mode: rows handed over by the float32 kernels
     const int64_t b = row / P.K1;
     const int j = (int)(row - b * P.K1);
@@ -226,39 +292,73 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
     const bool bonus = P.spec && (j == P.K1 - 1);
     int x = 0;
     if (!bonus) x = P.spec ? P.proposal[b * P.prop_ld + j] : P.proposal[row];
+    // the proposal's logits, for the scalar phase
+    const int xc = min(max(x, 0), V - 1);
+    const float sx = ld_as_float(s, xc), tx = ld_as_float(t, xc);
     const uint64_t rid = P.row_offset + (uint64_t)row;
     const bool masked = (P.mask != nullptr) && (P.mask[row] == 0);
     T* const g = P.dlogits ? (T*)P.dlogits + row * P.ld_g : nullptr;
+    // this warp's part of the row
+    constexpr int CW = Chunk<T>::W;
+    const int head = min(V, (int)(((16u - (uint32_t)((uintptr_t)s & 15u)) & 15u) / sizeof(T)));
+    const int nck = (V - head) / CW, cseg = (nck + NWC - 1) / NWC;
+    Part pt;
+    pt.head = head; pt.c0 = min(nck, gw * cseg); pt.c1 = min(nck, pt.c0 + cseg);
+    pt.x0 = gw == 0 ? 0 : V; pt.x1 = gw == 0 ? head : V;
+    if (gw == NWC - 1) pt.x0 = head + nck * CW;
+    const bool tvec = ((uintptr_t)(t + head) & 15u) == 0, gvec = ((uintptr_t)(g + head) & 15u) == 0;
+    auto part_begin = [&](int w) { return w == 0 ? 0 : head + min(nck, w * cseg) * CW; };
+    auto part_end = [&](int w) { return w == NWC - 1 ? V : head + min(nck, (w + 1) * cseg) * CW; };
+    if (steal && tid == 0 && crank == 0) steal_request(sh.answer, &sh.bar);
     const float d0 = ld_as_float(t, 0) - ld_as_float(s, 0);  // the logit difference is taken about this one: no offset of hundreds in its moments
 
     // ---- pass "sums"
     {
       float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
+      const int seg0 = part_begin(gw), seg1 = part_end(gw);
       for (int v = seg0 + lane, u = 0; v < seg1 && u < 4; v += 32, ++u) { ms = fmaxf(ms, ld_as_float(s, v)); mt = fmaxf(mt, ld_as_float(t, v)); }
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) { ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o)); mt = fmaxf(mt, __shfl_xor_sync(0xffffffffu, mt, o)); }
       double ks = 0.0, kt = 0.0, ss, st, n1;
       float m1, m2, m3, m4;
-      int am, inf;
-      const double dd0 = (double)d0;
+      int am;
       bool again = false;
 #pragma unroll 1
       for (int pass = 0; pass < 2; ++pass) {
         if (seg0 < seg1) { ks = -ceil(c * (double)ms); kt = -ceil(c * (double)mt); }
         ss = st = n1 = 0.0; m1 = m2 = m3 = m4 = 0.f;
-        am = 0x7fffffff; inf = 0;
+        am = 0x7fffffff;
         float xs = -CUDART_INF_F, xt = -CUDART_INF_F;
-        for_elements(s, t, seg0, seg1, lane, [&](int v, float a, float bt) {
-          const double es = ex2(fma(c, (double)a, ks)), et = ex2(fma(c, (double)bt, kt));
-          const double d = ((double)bt - (double)a) - dd0;
-          ss += es; st += et; n1 = fma(et, d, n1);
-          const float df = (bt - a) - d0, ef = (float)es;
-          const float w1 = ef * df, q = df * df, w2 = ef * q;
-          m1 += w1; m2 += w2; m3 = fmaf(w1, q, m3); m4 = fmaf(w2, q, m4);
-          inf = max(inf, max(__float_as_int(a) & 0x7fffffff, __float_as_int(bt) & 0x7fffffff));
-          xs = fmaxf(xs, a);
-          if (bt > xt) { xt = bt; am = v; }
-        });
+        float2 f1 = {0.f, 0.f}, f2 = f1, f3 = f1, f4 = f1;
+        const float2 nd0 = make_float2(-d0, -d0);
+        auto pair = [&](float a0, float b0, float a1, float b1) {
+          const double s0 = (double)a0, s1 = (double)a1, t0 = (double)b0, t1 = (double)b1;
+          const double es0 = ex2(fma(c, s0, ks)), es1 = ex2(fma(c, s1, ks)), et0 = ex2(fma(c, t0, kt)), et1 = ex2(fma(c, t1, kt));
+          ss += es0; ss += es1; st += et0; st += et1;
+          n1 = fma(et0, t0 - s0, n1); n1 = fma(et1, t1 - s1, n1);
+          const float2 d = fadd2(fadd2(make_float2(b0, b1), make_float2(-a0, -a1)), nd0), e = make_float2((float)es0, (float)es1);
+          const float2 w1 = fmul2(e, d), q = fmul2(d, d);
+          f1 = fadd2(f1, w1); f2 = ffma2(e, q, f2); f3 = ffma2(w1, q, f3); f4 = ffma2(fmul2(e, q), q, f4);
+        };
+        for_elements(s, t, tvec, pt, lane,
+          [&](int v, const Chunk<T>& a, const Chunk<T>& bt) {
+            float cx = bt.get(0);
+#pragma unroll
+            for (int i = 0; i < CW; i += 2) {
+              pair(a.get(i), bt.get(i), a.get(i + 1), bt.get(i + 1));
+              xs = fmaxf(fmaxf(xs, a.get(i)), a.get(i + 1)); cx = fmaxf(fmaxf(cx, bt.get(i)), bt.get(i + 1));
+            }
+            if (cx > xt) { xt = cx; am = v; }                // (the chunk; its element is found at the end)
+          },
+          [&](int v, float a, float bt) {
+            const double s0 = (double)a, t0 = (double)bt, es = ex2(fma(c, s0, ks)), et = ex2(fma(c, t0, kt));
+            ss += es; st += et; n1 = fma(et, t0 - s0, n1);
+            const float d = (bt - a) - d0, e = (float)es, q = d * d;
+            f1.x += e * d; f2.x += e * q; f3.x += e * d * q; f4.x += e * q * q;
+            xs = fmaxf(xs, a);
+            if (bt > xt) { xt = bt; am = v; }
+          });
+        m1 = f1.x + f1.y; m2 = f2.x + f2.y; m3 = f3.x + f3.y; m4 = f4.x + f4.y;
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
           xs = fmaxf(xs, __shfl_xor_sync(0xffffffffu, xs, o));
@@ -266,7 +366,12 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
           const int oam = __shfl_xor_sync(0xffffffffu, am, o);
           if (oxt > xt || (oxt == xt && oam < am)) { xt = oxt; am = oam; }
         }
-        again = fma(c, (double)xs, ks) > 900.0 || fma(c, (double)xt, kt) > 900.0;   // 2^y left its range: once more under the true maxima
+        {                                                    // the first element of that value in its chunk
+          const int v = am + lane;
+          const unsigned same = __ballot_sync(0xffffffffu, am < V && lane < CW && v < V && ld_as_float(t, min(v, V - 1)) == xt);
+          if (same) am += __ffs(same) - 1;
+        }
+        again = fma(c, (double)xs, ks) > 300.0 || fma(c, (double)xt, kt) > 300.0;   // 2^y left its range: once more under the true maxima
         ms = xs; mt = xt;
         if (!again) break;
       }
@@ -276,7 +381,8 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
         m1 += __shfl_xor_sync(0xffffffffu, m1, o); m2 += __shfl_xor_sync(0xffffffffu, m2, o);
         m3 += __shfl_xor_sync(0xffffffffu, m3, o); m4 += __shfl_xor_sync(0xffffffffu, m4, o);
       }
-      inf = __any_sync(0xffffffffu, inf >= 0x7f800000);
+      // a logit that is not finite leaves n1 so (an exponential is never 0 and the difference is then infinite or NaN)
+      const bool inf = !(fabs(n1) + ss + st < CUDART_INF);
       if (lane == 0) {
         double* const p = sh.part[ph][warp];
         p[PA_KS] = ks; p[PA_KT] = kt; p[PA_SS] = ss; p[PA_ST] = st; p[PA_N1] = n1;
@@ -284,15 +390,25 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
         p[PA_MS] = (double)ms; p[PA_MT] = (double)mt; p[PA_AM] = inf ? -1.0 : (double)am;
       }
     }
+    if (steal && tid == 0 && crank == 0) {     // the next row, decided while pass "sums" ran
+      const bool there = mbar_wait_bounded(&sh.bar, (uint32_t)(turn & 1));
+      const int first = there ? steal_answer(sh.answer) : -1;
+      sh.next[turn & 1] = first < 0 ? -1 : first / CS;
+    }
     phase_barrier();
+    if (steal) {
+      if constexpr (CS == 1) nxt = sh.next[turn & 1];
+      else nxt = *cg::this_cluster().map_shared_rank(&sh.next[turn & 1], 0);
+      ++turn;
+    }
     // the coupling decision and the constants of pass "final" (warp 0, once lambda is known)
     auto decide_row = [&](uint32_t status) {
       const double lam = bc[G_LAM], lse_s = -LN2 * bc[G_KP], lse_t = bc[G_LSE_T];
       double lp_x = 0.0, lT_x = 0.0, acc = 1.0;
       int corrected = 0, tok = -1;
       if (!bonus) {
-        lp_x = (double)ld_as_float(s, x) / (double)P.temperature - lse_s;
-        lT_x = (double)ld_as_float(t, x) / (double)P.temperature - lse_t;
+        lp_x = (double)sx / (double)P.temperature - lse_s;
+        lT_x = (double)tx / (double)P.temperature - lse_t;
         if (lam > 0.0) {
           acc = exp(fmin(0.0, lam * (lT_x - lp_x) - bc[G_LOGZ]));
           corrected = (scalar_uniform(P.seed, rid, STAGE_ACCEPT) < acc) ? 0 : 1;
@@ -343,7 +459,7 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
       else {
         const double lse_s = log(S) - ks * LN2, lse_t = log(St) - kt * LN2, cc = lse_t - lse_s;
         bc[G_KP] = -INV_LN2 * lse_s; bc[G_CC] = cc; bc[G_LSE_T] = lse_t;
-        const double kl1 = (N1 / St + (double)d0) * rtau - cc;                // KL(T || p)
+        const double kl1 = N1 / St * rtau - cc;               // KL(T || p)
         const bool endpoint = !(eps > 0.0) || kl1 <= eps;
         bc[G_LOGZ] = 0.0; bc[G_STATUS] = 0.0;
         bc[G_LAM] = !(eps > 0.0) ? 0.0 : 1.0; bc[G_KL] = !(eps > 0.0) ? 0.0 : kl1;
@@ -368,7 +484,7 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
         write_row(P.out, row, zero_row((uint32_t)bc[G_STATUS]), !P.spec);
         atomicAdd(P.flagged, 1ull);
       }
-      if (g) for (int v = seg0 + lane; v < seg1; v += 32) st_from_float(g, v, 0.f);
+      if (g) for (int v = part_begin(gw) + lane; v < part_end(gw); v += 32) st_from_float(g, v, 0.f);
       continue;
     }
 
@@ -377,7 +493,7 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
     while ((int)bc[G_MODE] == G_SOLVE) {
       const double bi = bc[G_BETA] * INV_LN2;
       double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
-      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) {
+      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) {
         const double sd = (double)a, d = fma((double)bt - sd, rtau, -cc);
         const double e = ex2(fma(bi, d, fma(c, sd, kp)));
         const double w1 = e * d, q = d * d, w2 = e * q;
@@ -407,30 +523,44 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
     // ---- pass "final": total variation, draw weights (of a bonus row: q itself) and the gradient
     const double li = bc[G_LAM] * INV_LN2, iz = exp(-bc[G_LOGZ]);
     const bool corrected = bc[G_CORR] != 0.0, draw = corrected || bonus;
-    // p, and r = [q - p]_+ of an element
-    auto residual = [&](float a, float bt, double& p, double& e) {
+    // p = p_v, e = Z q_v; returns q - p
+    auto diff = [&](float a, float bt, double& p, double& e) {
       const double sd = (double)a, d = fma((double)bt - sd, rtau, -cc), lp = fma(c, sd, kp);
       p = ex2(lp);
       e = ex2(fma(li, d, lp));
-      const double r = fma(e, iz, -p);
-      const int neg = __double2hiint(r) >> 31;               // max(r, 0) without the float64 pipe
-      return __hiloint2double(__double2hiint(r) & ~neg, __double2loint(r) & ~neg);
+      return fma(e, iz, -p);
     };
     double tv = 0.0, wq = 0.0;
     if (g) {
       const double sc = bc[G_SC];
       const int tok = (int)bc[G_TOK];
-      for_elements(s, t, seg0, seg1, lane, [&](int v, float a, float bt) {
+      auto grad = [&](float a, float bt) {
         double p, e;
-        tv += residual(a, bt, p, e);
-        double gv = sc * p;
-        if (v == tok) gv = sc * (p - 1.0);
-        put(g, v, gv);
-      });
+        const double r = diff(a, bt, p, e);
+        if (__double2hiint(r) >= 0) tv += r;                 // (the sign, without the float64 pipe)
+        return sc * p;
+      };
+      auto at_token = [&]() { return sc * (ex2(fma(c, (double)ld_as_float(s, tok), kp)) - 1.0); };
+      for_elements(s, t, tvec, pt, lane,
+        [&](int v, const Chunk<T>& a, const Chunk<T>& bt) {
+          Chunk<T> o;
+#pragma unroll
+          for (int i = 0; i < CW; i += 2) {
+            const double g0 = grad(a.get(i), bt.get(i)), g1 = grad(a.get(i + 1), bt.get(i + 1));
+            o.set2(i, g0, g1);
+          }
+          if (gvec) *(uint4*)(g + v) = make_uint4(o.r[0], o.r[1], o.r[2], o.r[3]);
+          else {
+#pragma unroll
+            for (int i = 0; i < CW; ++i) st_from_float(g, v + i, o.get(i));
+          }
+          if ((unsigned)(tok - v) < (unsigned)CW) Chunk<T>::put(g + tok, at_token());
+        },
+        [&](int v, float a, float bt) { const double gv = grad(a, bt); Chunk<T>::put(g + v, v == tok ? at_token() : gv); });
     } else if (bonus) {
-      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) { double p, e; tv += residual(a, bt, p, e); wq += e; });
+      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, e; const double r = diff(a, bt, p, e); if (__double2hiint(r) >= 0) tv += r; wq += e; });
     } else if (li > 0.0) {
-      for_elements(s, t, seg0, seg1, lane, [&](int, float a, float bt) { double p, e; tv += residual(a, bt, p, e); });
+      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, e; const double r = diff(a, bt, p, e); if (__double2hiint(r) >= 0) tv += r; });
     }
     tv = warp_sum(tv);
     if (bonus) wq = warp_sum(wq);
@@ -476,11 +606,11 @@ __global__ void __launch_bounds__(GT, 3) general_kernel(const RowParams P) {
         // the owner's segment once more, an eighth per warp; the warp whose part holds the target walks it
         const double target = bc[G_TARGET];
         bool last = bc[G_LAST] != 0.0;
-        const int o0 = min(V, owner * seg), o1 = min(V, o0 + seg), sl = (((o1 - o0 + GW - 1) / GW) + 31) & ~31;
+        const int o0 = part_begin(owner), o1 = part_end(owner), sl = (((o1 - o0 + GW - 1) / GW) + 31) & ~31;
         auto weight = [&](int v) {
           double p, e;
-          const double r = residual(ld_as_float(s, v), ld_as_float(t, v), p, e);
-          return bonus ? e : r;
+          const double r = diff(ld_as_float(s, v), ld_as_float(t, v), p, e);
+          return bonus ? e : fmax(r, 0.0);
         };
         double w = 0.0;
         for (int v = o0 + warp * sl + lane; v < min(o1, o0 + (warp + 1) * sl); v += 32) w += weight(v);
@@ -570,19 +700,24 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
     fit = n > 0 ? n : 1;
     if (dev < 64) fit_of[dev].store(fit, std::memory_order_relaxed);
   }
-  cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit ? p.n_rows : fit)), 1, 1);
-  return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p);
+  // One cluster per row where the hardware can be asked for the next one (a row's solve takes one evaluation or two,
+  // and the rows do not divide evenly); in list mode, and for more rows than a grid may have blocks, a fixed stride.
+  const bool steal = !p.from_list && p.n_rows > fit && p.n_rows <= (1 << 27);
+  const double rtau = 1.0 / (double)p.temperature;
+  cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit || steal ? p.n_rows : fit)), 1, 1);
+  return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p, (int)steal, rtau, INV_LN2 * rtau);
 }
 
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
   // Blocks per row.  In list mode (a handful of rows as a rule; the host does not know their number) always the most;
   // otherwise so many that few rows still fill the chip, each block keeping 1024 elements or more (below that the
-  // barriers of a cluster cost more than its blocks save), and that the rows in flight stay in L2 between the passes.
+  // barriers of a cluster cost more than its blocks save), and that the rows in flight stay in L2 between the passes
+  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).
   int cs = 1;
-  const int64_t in_flight = 3 * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
+  const int64_t in_flight = BLOCKS_PER_SM<T> * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
   while (cs < MAX_CS && p.V >= 2048 * cs &&
-         (p.from_list || p.n_rows * cs < in_flight || in_flight / cs * row_bytes > (64 << 20)))
+         (p.from_list || p.n_rows * cs < in_flight || in_flight / cs * row_bytes > (150 << 20)))
     cs *= 2;
   switch (cs) {
     case 1: return launch_cs<T, 1>(p, dev, sms, st);
