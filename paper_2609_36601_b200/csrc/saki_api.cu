@@ -336,48 +336,6 @@ __global__ void spec_resolve_kernel(int64_t B, int K, saki_out o, int32_t* n_acc
   }
 }
 
-// ---- proposal utility: Gumbel-max with per-element Philox noise ----
-template <typename T>
-__global__ void __launch_bounds__(256) proposal_kernel(const T* logits, int64_t ld, int64_t N, int V, double tau,
-                                                        uint64_t seed, uint64_t row_offset, int32_t* out) {
-  __shared__ double skey[8];
-  __shared__ int sidx[8];
-  for (int64_t row = blockIdx.x; row < N; row += gridDim.x) {
-    const T* s = logits + row * ld;
-    const uint64_t rid = row_offset + (uint64_t)row;
-    double best = -INFINITY;
-    int bi = 0x7fffffff;
-    for (int blk = threadIdx.x; blk * 4 < V; blk += blockDim.x) {
-      uint32_t w[4];
-      philox4x32_10((uint32_t)rid, (uint32_t)(rid >> 32), STAGE_PROPOSE, (uint32_t)blk, (uint32_t)seed,
-                    (uint32_t)(seed >> 32), w);
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int v = blk * 4 + k;
-        if (v < V) {
-          const double u = ((double)w[k] + 0.5) * (1.0 / 4294967296.0);
-          const double key = (double)ld_as_float(s, v) / tau - log(-log(u));
-          if (key > best) { best = key; bi = v; }
-        }
-      }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
-      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-    }
-    if ((threadIdx.x & 31) == 0) { skey[threadIdx.x >> 5] = best; sidx[threadIdx.x >> 5] = bi; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < 8; ++w)
-        if (skey[w] > best || (skey[w] == best && sidx[w] < bi)) { best = skey[w]; bi = sidx[w]; }
-      out[row] = bi;
-    }
-    __syncthreads();
-  }
-}
-
 // ---- host-buffer entry: staged, double-buffered ----
 struct HostStage {
   std::mutex mu;
@@ -593,17 +551,9 @@ SAKI_API int saki_sample_proposal(const void* logits, int64_t ld, int64_t N, int
   unsigned long long* flagged = nullptr;
   rc = device_ready(&flagged);
   if (rc) return rc;
-  const int grid = (int)std::min<int64_t>(N, 148 * 8);
-  cudaStream_t st = (cudaStream_t)cuda_stream;
-  if (dtype == SAKI_BF16)
-    proposal_kernel<__nv_bfloat16><<<grid, 256, 0, st>>>((const __nv_bfloat16*)logits, ld, N, V, (double)temperature,
-                                                         seed, row_offset, out);
-  else
-    proposal_kernel<float><<<grid, 256, 0, st>>>((const float*)logits, ld, N, V, (double)temperature, seed,
-                                                 row_offset, out);
-  g_launches += 1;
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = launch_propose(logits, ld, N, V, dtype, temperature, seed, row_offset, out, (cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(e, "proposal kernel launch");
+  g_launches += 1;
   return SAKI_OK;
 }
 

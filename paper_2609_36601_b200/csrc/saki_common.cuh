@@ -171,6 +171,8 @@ bool rowsm_can_serve(const RowParams& p, int dtype);
 cudaError_t launch_meta_general(const MetaParams& p, int dtype, cudaStream_t st, int* n_launches);
 cudaError_t launch_meta_stream(const MetaParams& p, cudaStream_t st, int* n_launches, bool* served);
 bool meta_stream_can_serve(const MetaParams& p, int dtype);
+cudaError_t launch_propose(const void* logits, int64_t ld, int64_t N, int V, int dtype, float tau, uint64_t seed,
+                           uint64_t row_offset, int32_t* out, cudaStream_t st);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t st, int* n_launches);
 cudaError_t launch_vshard_partial(const saki_vshard_in& in, int stage, const double* state, double* partial, void* dlogits,
                                   int64_t ld_g, float grad_scale, bool allow_fast, cudaStream_t st);

@@ -64,3 +64,28 @@ def test_maximum_far_above_the_first_elements(drop):
         d[k][:, low] -= drop
     d["proposal"][:] = peaks[:4].to(torch.int32)
     _check(d, w, list(range(4)))
+
+
+@pytest.mark.parametrize("V,N,dtype,off", [(2, 5, "f32", 0), (5, 3, "bf16", 1), (1023, 4, "bf16", 3), (1024, 700, "f32", 0),
+                                           (8191, 3, "bf16", 0), (8192, 3, "bf16", 2), (40003, 3, "f32", 1)])
+@pytest.mark.parametrize("scale", [1.0, 40.0])
+def test_proposal_edges(V, N, dtype, off, scale):
+    """Gumbel-max by float32 bounds: partial last Philox block, unaligned rows, one block and a cluster per row, peaked
+    rows (scale 40: the winner's Gumbel term is small, where the bound is loose)."""
+    w = synth.Workload("t", N, V, dtype, 0.1, 1.0, V > 100, 500 + V, 23)
+    s = _shift((synth.generate(w, DEV)["s"].float() * scale).to(w.torch_dtype), off)
+    x = P.sample_proposal(s, 0.75, 23, row_offset=(1 << 32) - 2).cpu().numpy()
+    rows = list(range(N)) if N < 10 else list(range(0, N, 41))
+    ref, gaps = O.sample_proposal(to_np64(s), 0.75, 23, row_offset=(1 << 32) - 2, rows=rows)
+    assert np.array_equal(x[rows][gaps >= 1e-12], ref[gaps >= 1e-12])     # float64 keys: a few ulp of ~100
+
+
+def test_proposal_of_unusual_logits():
+    """NaN and -inf are never drawn, +inf is (the first), a row of nothing else gives 0x7fffffff."""
+    s = torch.randn(5, 9000, device=DEV)
+    s[0, 5:] = float("-inf"); s[1, 7000] = s[1, 8000] = float("inf"); s[2, :] = float("nan"); s[3, ::2] = float("nan")
+    s[4] = 3e38 + 0 * s[4]
+    x = P.sample_proposal(s, 0.5, 1).cpu().numpy()
+    ref, _ = O.sample_proposal(to_np64(s[4:5]), 0.5, 1, row_offset=4)
+    assert x[0] < 5 and x[1] == 7000 and x[2] == 0x7fffffff and x[3] % 2 == 1
+    assert x[4] == ref[0]
