@@ -241,8 +241,10 @@ SAKI_API int saki_select_tm(const saki_select_in* in, uint8_t* selected, int32_t
  *      still solving (each wave moves to the root of a fourth-order model: two waves as a rule)
  *   2  shares of TV(p, q) and KL(q || p); the combine decides acceptance (Eq. "accept"), the routed loss
  *      (Eqs. "k1_loss_token", "teacher_mode_loss") and which rank owns the residual draw (Eq. "residual")
- *   3  the gradient slice (Eq. "general_objective": dlogits_slice [N, V_local], same dtype, may be NULL) and,
- *      on the owning rank, the drawn token; the combine writes the per-position outputs
+ *   3  on the owning rank, the drawn token; the combine writes the per-position outputs
+ *   The gradient slice (Eq. "general_objective": dlogits_slice [N, V_local], same dtype) is written by the partial call
+ *   of stage 2 or of stage 3 that is given it (NULL: not wanted): at stage 2 it comes out of the pass over the slice that
+ *   is made there anyway, at stage 3 it takes a pass of its own
  * Arithmetic: bf16 slices that start on 16-byte boundaries (V_local, v0 and the strides multiples of 8) with
  * eps >= 0.02 are reduced with the per-element arithmetic of the unsharded bf16 kernels (float32 elements,
  * float64 sums and scalars; a row that float32 cannot resolve goes on in float64, decided in the combine);
@@ -275,6 +277,12 @@ typedef struct {
 } saki_vshard_in;
 SAKI_API int saki_vshard_partial(const saki_vshard_in* in, int stage, const double* state, double* partial,
                                  void* dlogits_slice, int64_t ld_g, float grad_scale, void* cuda_stream);
+/* The same for the n slices a process holds (several ranks' slices on one device; same rows, dtype and arguments but
+ * for the slice): `in`, `partial`, `dlogits_slice` (may be NULL) and `ld_g` are HOST arrays of n entries.  One kernel
+ * launch per stage and 16 slices instead of one per slice. */
+SAKI_API int saki_vshard_partial_group(const saki_vshard_in* in, int n, int stage, const double* state,
+                                       double* const* partial, void* const* dlogits_slice, const int64_t* ld_g,
+                                       float grad_scale, void* cuda_stream);
 SAKI_API int saki_vshard_combine(const saki_vshard_in* in, int stage, const double* gathered, double* state,
                                  const saki_out* out, uint32_t* n_solving, void* cuda_stream);
 SAKI_API int saki_vshard_combine_host(const saki_vshard_in* in, int stage, const double* gathered, double* state,

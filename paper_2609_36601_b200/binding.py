@@ -21,7 +21,7 @@ ROW_SATURATED, ROW_EPS_ZERO, ROW_MASKED, ROW_NONFINITE, ROW_BAD_ID, ROW_TIMEOUT,
 _FLOAT_FIELDS = ("lambda", "kl", "tv", "accept_prob", "logp_x", "logq_x", "logT_x", "logp_y", "logq_y", "logT_y", "loss")
 EXPORTS = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc", "saki_route_host",
            "saki_route_bwd_from_meta", "saki_select_tm", "saki_spec_verify",
-           "saki_vshard_partial", "saki_vshard_combine", "saki_vshard_combine_host",
+           "saki_vshard_partial", "saki_vshard_partial_group", "saki_vshard_combine", "saki_vshard_combine_host",
            "saki_lmhead_scratch_bytes", "saki_lmhead_lse",
            "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_redo_count",
            "saki_set_spec_early_out", "saki_spec_positions_routed", "saki_solve_evaluations", "saki_set_wait_limit", "saki_set_phase_clock", "saki_phase_cycles",
@@ -134,6 +134,9 @@ def load_library(path: str | None = None):
     lib.saki_vshard_partial.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64,
                                         C.c_float, C.c_void_p]
     lib.saki_vshard_partial.restype = C.c_int
+    lib.saki_vshard_partial_group.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_int, C.c_void_p, C.POINTER(C.c_void_p),
+                                              C.POINTER(C.c_void_p), C.POINTER(C.c_int64), C.c_float, C.c_void_p]
+    lib.saki_vshard_partial_group.restype = C.c_int
     lib.saki_vshard_combine.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_void_p, C.c_void_p, C.POINTER(SakiOut),
                                         C.c_void_p, C.c_void_p]
     lib.saki_vshard_combine.restype = C.c_int
@@ -363,6 +366,28 @@ def vshard_partial(si: SakiVshardIn, stage: int, state, partial, dlogits=None, g
     _raise(lib, lib.saki_vshard_partial(C.byref(si), stage, state.data_ptr() if state is not None else None,
                                         partial.data_ptr(), dlogits.data_ptr() if dlogits is not None else None, ld_g,
                                         grad_scale, _stream_ptr(stream)))
+
+
+class VshardGroup:
+    """The slices of several ranks on one device as one argument list of saki_vshard_partial_group: `sis` their argument
+    records, `partials` and `dlogits` (or None) one tensor per slice."""
+
+    def __init__(self, sis, partials, dlogits=None):
+        n = len(sis)
+        self.n, self.sis = n, (SakiVshardIn * n)(*sis)
+        self.partials = (C.c_void_p * n)(*(p.data_ptr() for p in partials))
+        self.dlogits = self.ld_g = None
+        if dlogits is not None:
+            self.dlogits = (C.c_void_p * n)(*(g.data_ptr() for g in dlogits))
+            self.ld_g = (C.c_int64 * n)(*(g.stride(0) if g.shape[0] > 1 else max(1, g.shape[1]) for g in dlogits))
+
+    def partial(self, stage: int, state, with_grad=False, grad_scale=1.0, stream=None):
+        """saki_vshard_partial_group: every slice's partial vectors of one stage (and its gradient slice)."""
+        lib = load_library()
+        grad = with_grad and self.dlogits is not None
+        _raise(lib, lib.saki_vshard_partial_group(self.sis, self.n, stage, state.data_ptr() if state is not None else None,
+                                                  self.partials, self.dlogits if grad else None, self.ld_g if grad else None,
+                                                  grad_scale, _stream_ptr(stream)))
 
 
 def vshard_combine(si: SakiVshardIn, stage: int, gathered, state, out=None, n_solving=None, stream=None):

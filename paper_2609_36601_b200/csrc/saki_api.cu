@@ -412,24 +412,42 @@ static int vshard_check(const saki_vshard_in* in, int stage) {
   return SAKI_OK;
 }
 
+static int vshard_partials(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
+                           void* const* dlogits, const int64_t* ld_g, float grad_scale, void* cuda_stream) {
+  g_err[0] = 0;
+  if (n < 0) return fail(SAKI_ERR_INVALID_ARG, "negative number of slices");
+  if (n > 0 && (!in || !partial || (dlogits && !ld_g))) return fail(SAKI_ERR_INVALID_ARG, "NULL argument array");
+  for (int k = 0; k < n; ++k) {
+    const int rc = vshard_check(in + k, stage);
+    if (rc) return rc;
+    if (in[k].N != in[0].N || in[k].dtype != in[0].dtype) return fail(SAKI_ERR_INVALID_ARG, "the slices of one call have the same rows and dtype");
+  }
+  if (n == 0 || in[0].N == 0) return SAKI_OK;
+  for (int k = 0; k < n; ++k) {
+    if (in[k].V_local > 0 && (!in[k].student_logits || !in[k].teacher_logits)) return fail(SAKI_ERR_INVALID_ARG, "NULL logits pointer");
+    if (in[k].ld_s < in[k].V_local || in[k].ld_t < in[k].V_local) return fail(SAKI_ERR_INVALID_ARG, "row stride smaller than the slice");
+    if (!partial[k] || (stage > 0 && !state)) return fail(SAKI_ERR_INVALID_ARG, "NULL partial or state pointer");
+    if (dlogits && dlogits[k] && (ld_g[k] < in[k].V_local || !std::isfinite(grad_scale))) return fail(SAKI_ERR_INVALID_ARG, "bad gradient stride or scale");
+  }
+  unsigned long long* flagged = nullptr;
+  int rc = device_ready(&flagged);
+  if (rc) return rc;
+  int launches = 0;
+  cudaError_t e = launch_vshard_partial(in, n, stage, state, partial, dlogits, ld_g, grad_scale, g_kernel.load() != 1, &launches,
+                                        (cudaStream_t)cuda_stream);
+  if (e != cudaSuccess) return cuda_fail(e, "vocabulary-sharded partial kernel launch");
+  g_launches += (uint64_t)launches;
+  return SAKI_OK;
+}
+
 SAKI_API int saki_vshard_partial(const saki_vshard_in* in, int stage, const double* state, double* partial,
                                  void* dlogits_slice, int64_t ld_g, float grad_scale, void* cuda_stream) {
-  g_err[0] = 0;
-  int rc = vshard_check(in, stage);
-  if (rc) return rc;
-  if (in->N == 0) return SAKI_OK;
-  if (in->V_local > 0 && (!in->student_logits || !in->teacher_logits)) return fail(SAKI_ERR_INVALID_ARG, "NULL logits pointer");
-  if (in->ld_s < in->V_local || in->ld_t < in->V_local) return fail(SAKI_ERR_INVALID_ARG, "row stride smaller than the slice");
-  if (!partial || (stage > 0 && !state)) return fail(SAKI_ERR_INVALID_ARG, "NULL partial or state pointer");
-  if (dlogits_slice && (ld_g < in->V_local || !std::isfinite(grad_scale))) return fail(SAKI_ERR_INVALID_ARG, "bad gradient stride or scale");
-  unsigned long long* flagged = nullptr;
-  rc = device_ready(&flagged);
-  if (rc) return rc;
-  cudaError_t e = launch_vshard_partial(*in, stage, state, partial, stage == 3 ? dlogits_slice : nullptr, ld_g, grad_scale,
-                                        g_kernel.load() != 1, (cudaStream_t)cuda_stream);
-  if (e != cudaSuccess) return cuda_fail(e, "vocabulary-sharded partial kernel launch");
-  g_launches += 1;
-  return SAKI_OK;
+  return vshard_partials(in, 1, stage, state, &partial, dlogits_slice ? &dlogits_slice : nullptr, &ld_g, grad_scale, cuda_stream);
+}
+
+SAKI_API int saki_vshard_partial_group(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
+                                       void* const* dlogits_slice, const int64_t* ld_g, float grad_scale, void* cuda_stream) {
+  return vshard_partials(in, n, stage, state, partial, dlogits_slice, ld_g, grad_scale, cuda_stream);
 }
 
 SAKI_API int saki_vshard_combine(const saki_vshard_in* in, int stage, const double* gathered, double* state,

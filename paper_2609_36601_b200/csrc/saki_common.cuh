@@ -174,8 +174,9 @@ bool meta_stream_can_serve(const MetaParams& p, int dtype);
 cudaError_t launch_propose(const void* logits, int64_t ld, int64_t N, int V, int dtype, float tau, uint64_t seed,
                            uint64_t row_offset, int32_t* out, cudaStream_t st);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t st, int* n_launches);
-cudaError_t launch_vshard_partial(const saki_vshard_in& in, int stage, const double* state, double* partial, void* dlogits,
-                                  int64_t ld_g, float grad_scale, bool allow_fast, cudaStream_t st);
+cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
+                                  void* const* dlogits, const int64_t* ld_g, float grad_scale, bool allow_fast, int* n_launches,
+                                  cudaStream_t st);
 cudaError_t launch_vshard_combine(const saki_vshard_in& in, int stage, const double* gathered, double* state, const saki_out& out,
                                   unsigned int* n_solving, bool allow_fast, cudaStream_t st);
 int64_t lmhead_scratch_bytes(int64_t N, int32_t V);

@@ -5,8 +5,9 @@
 // its key, and only those whose bound reaches the best exact key are evaluated in float64, so the result is the argmax of
 // the float64 keys.  The bound: with v = 1 - u, -log u >= v + v^2/2, so the Gumbel term is at most -log(v + v^2/2), nearly
 // exact where it is large (v small); v is taken from the upper 23 bits of the word, rounded down.  Per element that
-// leaves a quarter of a Philox block (ten rounds of two wide multiplications and two xors: the integer pipe is the
-// bound), one lg2 and a few float operations; the row is read once.
+// leaves a quarter of a Philox block (ten rounds of two wide multiplications and two xors) and about eight more
+// instructions, half of them shared by the elements of a packed pair or of a group of eight: the integer pipe is the
+// bound.  The row is read once.  (The kernel works with minus the bound, in units of log 2: the smallest counts.)
 #include "saki_device.cuh"
 #include <cooperative_groups.h>
 
@@ -17,35 +18,56 @@ namespace saki {
 namespace {
 
 constexpr int PT = 256, PWARPS = PT / 32, PROPOSE_CS = 8;
+constexpr int G = 8;       // elements of a group: two Philox blocks, the unit that is bounded and remembered
+
+// The Philox key of every round: row-invariant, and an operand from the constant bank instead of two additions a round.
+struct Keys { uint32_t k0[10], k1[10]; };
 
 struct ProposeShared {
-  float ub[PWARPS];
-  int blk[PWARPS];
+  float lb[PWARPS];
+  int grp[PWARPS];
   double key[PWARPS];
   int idx[PWARPS];
   double block_key;      // read by the other blocks of the cluster
   int block_idx;
-  float block_ub;
-  int block_blk;
+  float block_lb;
+  int block_grp;
 };
 
-template <typename T> struct Quad { float x[4]; };
-
-// the four logits of Philox block blk (past the row's end: -inf)
-template <typename T> __device__ __forceinline__ Quad<T> load_quad(const T* s, int blk, int V, bool vec) {
-  Quad<T> q;
-  if (vec && blk * 4 + 4 <= V) {
-    if constexpr (sizeof(T) == 2) {
-      const uint2 r = __ldg((const uint2*)(s + blk * 4));
-      const float2 a = unpack_bf16x2(r.x), b = unpack_bf16x2(r.y);
-      q.x[0] = a.x; q.x[1] = a.y; q.x[2] = b.x; q.x[3] = b.y;
-    } else {
-      const float4 r = __ldg((const float4*)(s + blk * 4));
-      q.x[0] = r.x; q.x[1] = r.y; q.x[2] = r.z; q.x[3] = r.w;
+// The eight logits of a group, as stored (past the row's end: -inf).
+template <typename T> struct Raw;
+template <> struct Raw<__nv_bfloat16> {
+  uint32_t r[4];
+  __device__ __forceinline__ float2 pair(int i) const { return unpack_bf16x2(r[i]); }
+  __device__ __forceinline__ void set(const float* x) {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = pack_bf16x2(x[2 * i], x[2 * i + 1]);
+  }
+};
+template <> struct Raw<float> {
+  float r[8];
+  __device__ __forceinline__ float2 pair(int i) const { return make_float2(r[2 * i], r[2 * i + 1]); }
+  __device__ __forceinline__ void set(const float* x) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) r[i] = x[i];
+  }
+};
+template <typename T> __device__ __forceinline__ Raw<T> load_raw(const T* s, int grp, int V, bool vec) {
+  Raw<T> q;
+  if (vec && grp * G + G <= V) {
+    const uint4* const p = (const uint4*)(s + grp * G);
+    const uint4 a = __ldg(p);
+    if constexpr (sizeof(T) == 2) { q.r[0] = a.x; q.r[1] = a.y; q.r[2] = a.z; q.r[3] = a.w; }
+    else {
+      const uint4 b = __ldg(p + 1);
+      q.r[0] = __uint_as_float(a.x); q.r[1] = __uint_as_float(a.y); q.r[2] = __uint_as_float(a.z); q.r[3] = __uint_as_float(a.w);
+      q.r[4] = __uint_as_float(b.x); q.r[5] = __uint_as_float(b.y); q.r[6] = __uint_as_float(b.z); q.r[7] = __uint_as_float(b.w);
     }
   } else {
+    float x[G];
 #pragma unroll
-    for (int k = 0; k < 4; ++k) q.x[k] = blk * 4 + k < V ? ld_as_float(s, blk * 4 + k) : -CUDART_INF_F;
+    for (int k = 0; k < G; ++k) x[k] = grp * G + k < V ? ld_as_float(s, grp * G + k) : -CUDART_INF_F;
+    q.set(x);
   }
   return q;
 }
@@ -55,113 +77,153 @@ __device__ __forceinline__ float lg2f(float x) {
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// upper bound of the largest of a block's four keys, in units of log 2
-template <typename T> __device__ __forceinline__ float bound(const Quad<T>& q, const uint32_t* w, float c) {
-  float m = -CUDART_INF_F;
+__device__ __forceinline__ void philox_keys(uint64_t rid, uint32_t blk, const Keys& K, uint32_t (&w)[4]) {
+  uint32_t c0 = (uint32_t)rid, c1 = (uint32_t)(rid >> 32), c2 = STAGE_PROPOSE, c3 = blk;
 #pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    const float v = 1.99999988079071f - __uint_as_float(0x3f800000u | (w[k] >> 9));    // 1 - u, rounded down; may be 0
-    m = fmaxf(m, fmaf(q.x[k], c, -lg2f(fmaf(v, 0.5f * v, v))));
+  for (int r = 0; r < 10; ++r) {
+    const uint64_t p0 = (uint64_t)0xD2511F53u * c0, p1 = (uint64_t)0xCD9E8D57u * c2;
+    c0 = (uint32_t)(p1 >> 32) ^ c1 ^ K.k0[r]; c1 = (uint32_t)p1;
+    c2 = (uint32_t)(p0 >> 32) ^ c3 ^ K.k1[r]; c3 = (uint32_t)p0;
+  }
+  w[0] = c0; w[1] = c1; w[2] = c2; w[3] = c3;
+}
+// lower bound of minus a group's largest key, in units of log 2 (nc = -log2(e) / tau)
+template <typename T> __device__ __forceinline__ float lower(const Raw<T>& q, int grp, uint64_t rid, const Keys& K, float nc) {
+  float m = CUDART_INF_F;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    uint32_t w[4];
+    philox_keys(rid, (uint32_t)(2 * grp + h), K, w);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      // 1 - u, rounded down (0x7f : w) >> 9 is the float in [1, 2) with the word's upper 23 bits; may be 0
+      const float2 f = make_float2(-__uint_as_float(__funnelshift_r(w[2 * k], 0x7fu, 9)), -__uint_as_float(__funnelshift_r(w[2 * k + 1], 0x7fu, 9)));
+      const float2 v = fadd2(splat(1.99999988079071f), f), l = ffma2(v, fmul2(v, splat(0.5f)), v);
+      const float2 d = ffma2(q.pair(2 * h + k), splat(nc), make_float2(lg2f(l.x), lg2f(l.y)));
+      m = fminf(fminf(m, d.x), d.y);
+    }
   }
   return m;
 }
 __device__ __forceinline__ void better(double& key, int& idx, double k, int i) {
   if (k > key || (k == key && i < idx)) { key = k; idx = i; }
 }
-// the exact keys of a block's elements
+// a group's exact keys, one per lane (lanes 0 to 7 of the warp): each lane keeps its best
 template <typename T>
-__device__ __noinline__ void exact_keys(const T* s, int blk, int V, double tau, uint64_t rid, uint64_t seed, double& key, int& idx) {
-  uint32_t w[4];
-  philox4x32_10((uint32_t)rid, (uint32_t)(rid >> 32), STAGE_PROPOSE, (uint32_t)blk, (uint32_t)seed, (uint32_t)(seed >> 32), w);
-#pragma unroll 1
-  for (int k = 0; k < 4; ++k) {
-    const int v = blk * 4 + k;
-    if (v >= V) break;
+__device__ __noinline__ void exact_keys(const T* s, int grp, int V, double tau, uint64_t rid, uint64_t seed, double& key, int& idx) {
+  const int lane = threadIdx.x & 31, v = grp * G + lane;
+  if (lane < G && v < V) {
+    uint32_t w[4];
+    philox4x32_10((uint32_t)rid, (uint32_t)(rid >> 32), STAGE_PROPOSE, (uint32_t)(v >> 2), (uint32_t)seed, (uint32_t)(seed >> 32), w);
+    const int k = v & 3;
     const double u = ((double)(k == 0 ? w[0] : k == 1 ? w[1] : k == 2 ? w[2] : w[3]) + 0.5) * (1.0 / 4294967296.0);
     const double e = (double)ld_as_float(s, v) / tau - log(-log(u));
     if (e > -CUDART_INF) better(key, idx, e, v);
   }
 }
+__device__ __forceinline__ void warp_better(double& key, int& idx) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    const double ok = __shfl_xor_sync(0xffffffffu, key, o);
+    const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
+    better(key, idx, ok, oi);
+  }
+}
 
 // CS: blocks per row (1, or a cluster that shares the row)
 template <typename T, int CS>
-__global__ void __launch_bounds__(PT, 4) propose_kernel(const T* logits, int64_t ld, int64_t N, int V, double tau, float c,
-                                                        uint64_t seed, uint64_t row_offset, int32_t* out) {
+__global__ void __launch_bounds__(PT, 4) propose_kernel(const T* logits, int64_t ld, int64_t N, int V, double tau, float nc,
+                                                        const Keys K, uint64_t seed, uint64_t row_offset, int32_t* out) {
   __shared__ ProposeShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   int crank = 0;
   if constexpr (CS > 1) crank = (int)cg::this_cluster().block_rank();
-  const int first = crank * PT + tid, step = PT * CS, nblk = (V + 3) / 4;
+  const int first = crank * PT + tid, step = PT * CS, ngrp = (V + G - 1) / G;
   for (int64_t row = blockIdx.x / CS; row < N; row += gridDim.x / CS) {
     const T* const s = logits + row * ld;
-    const bool vec = ((uintptr_t)s & (4 * sizeof(T) - 1)) == 0;
+    const bool vec = ((uintptr_t)s & 15) == 0;
     const uint64_t rid = row_offset + (uint64_t)row;
-    // the two best blocks of this thread by their bounds, and the third best bound
-    float b1 = -CUDART_INF_F, b2 = b1, b3 = b1;
+    // the two best groups of this thread by their bounds, and the third best bound
+    float b1 = CUDART_INF_F, b2 = b1, b3 = b1;
     int i1 = 0, i2 = 0;
-    Quad<T> next = load_quad(s, min(first, nblk - 1), V, vec);
+    auto note = [&](float m, int grp) {
+      b3 = fminf(b3, fmaxf(b2, m));
+      const bool g1 = m < b1, g2 = m < b2;
+      i2 = g1 ? i1 : (g2 ? grp : i2); b2 = g1 ? b1 : (g2 ? m : b2);
+      i1 = g1 ? grp : i1; b1 = g1 ? m : b1;
+    };
+    // two groups at a time, the logits of the next two on their way
+    constexpr int U = 2;
+    Raw<T> next[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) next[u] = load_raw(s, min(first + u * step, ngrp - 1), V, vec);
 #pragma unroll 1
-    for (int blk = first; blk < nblk; blk += step) {
-      const Quad<T> q = next;
-      next = load_quad(s, min(blk + step, nblk - 1), V, vec);
-      uint32_t w[4];
-      philox4x32_10((uint32_t)rid, (uint32_t)(rid >> 32), STAGE_PROPOSE, (uint32_t)blk, (uint32_t)seed, (uint32_t)(seed >> 32), w);
-      const float m = bound(q, w, c);
-      b3 = fmaxf(b3, fminf(b2, m));
-      const bool g1 = m > b1, g2 = m > b2;
-      i2 = g1 ? i1 : (g2 ? blk : i2); b2 = g1 ? b1 : (g2 ? m : b2);
-      i1 = g1 ? blk : i1; b1 = g1 ? m : b1;
+    for (int g0 = first; g0 < ngrp; g0 += U * step) {
+      Raw<T> raw[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        raw[u] = next[u];
+        next[u] = load_raw(s, min(g0 + (U + u) * step, ngrp - 1), V, vec);
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int grp = g0 + u * step;
+        if (grp < ngrp) note(lower(raw[u], grp, rid, K, nc), grp);
+      }
     }
-    // the block with the largest bound: its exact keys set the bar
+    // the group with the best bound: its exact keys set the bar
     float mb = b1;
     int mi = i1;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
       const float ob = __shfl_xor_sync(0xffffffffu, mb, o);
       const int oi = __shfl_xor_sync(0xffffffffu, mi, o);
-      if (ob > mb) { mb = ob; mi = oi; }
+      if (ob < mb) { mb = ob; mi = oi; }
     }
-    if (lane == 0) { sh.ub[warp] = mb; sh.blk[warp] = mi; }
+    if (lane == 0) { sh.lb[warp] = mb; sh.grp[warp] = mi; }
     __syncthreads();
+    mb = sh.lb[0]; mi = sh.grp[0];
 #pragma unroll
-    for (int w = 0; w < PWARPS; ++w) if (sh.ub[w] > mb) { mb = sh.ub[w]; mi = sh.blk[w]; }
+    for (int w = 1; w < PWARPS; ++w) if (sh.lb[w] < mb) { mb = sh.lb[w]; mi = sh.grp[w]; }
     if constexpr (CS > 1) {
-      if (tid == 0) { sh.block_ub = mb; sh.block_blk = mi; }
+      if (tid == 0) { sh.block_lb = mb; sh.block_grp = mi; }
       cg::cluster_group cl = cg::this_cluster();
       cl.sync();
       for (int r = 0; r < CS; ++r) {
         const ProposeShared* const rs = cl.map_shared_rank(&sh, r);
-        if (rs->block_ub > mb) { mb = rs->block_ub; mi = rs->block_blk; }
+        if (rs->block_lb < mb) { mb = rs->block_lb; mi = rs->block_grp; }
       }
     }
     double key = -CUDART_INF;
     int idx = 0x7fffffff;
-    if (mb > -CUDART_INF_F) {
+    // the warp evaluates the groups its lanes ask for, one after the other
+    auto evaluate = [&](bool wanted, int grp) {
+      for (unsigned m = __ballot_sync(0xffffffffu, wanted); m; m &= m - 1)
+        exact_keys(s, __shfl_sync(0xffffffffu, grp, __ffs(m) - 1), V, tau, rid, seed, key, idx);
+    };
+    float thr = CUDART_INF_F;
+    const bool bounded = mb < CUDART_INF_F;
+    if (bounded) {
       double bar = -CUDART_INF;
       int bi = 0x7fffffff;
-      exact_keys(s, mi, V, tau, rid, seed, bar, bi);                    // (every thread alike)
+      exact_keys(s, mi, V, tau, rid, seed, bar, bi);                    // (every warp alike)
+      warp_better(bar, bi);
       // rounding of a bound: ~1e-7 of the scaled logit (the Gumbel term is within 33 of zero), and of lg2
-      const float fb = (float)(bar * INV_LN2), thr = fb - (1e-4f + 1e-6f * (fminf(fabsf(fb), 1e30f) + 64.f));
-      if (!(b1 < thr)) exact_keys(s, i1, V, tau, rid, seed, key, idx);
-      if (!(b2 < thr) && b2 > -CUDART_INF_F) exact_keys(s, i2, V, tau, rid, seed, key, idx);
-      if (!(b3 < thr) && b3 > -CUDART_INF_F) {                          // a third: every block of this thread that reaches the bar
+      const float fb = -(float)(bar * INV_LN2);
+      thr = fb + (1e-4f + 1e-6f * (fminf(fabsf(fb), 1e30f) + 64.f));
+      evaluate(!(b1 > thr), i1);
+      evaluate(!(b2 > thr) && b2 < CUDART_INF_F, i2);
+    }
+    // a third group of a thread reaches the bar, or there is no bound at all (NaN or -inf logits only, or logits beyond
+    // float32's range once scaled): every group again
+    if (__any_sync(0xffffffffu, !bounded || (!(b3 > thr) && b3 < CUDART_INF_F))) {
 #pragma unroll 1
-        for (int blk = first; blk < nblk; blk += step) {
-          uint32_t w[4];
-          philox4x32_10((uint32_t)rid, (uint32_t)(rid >> 32), STAGE_PROPOSE, (uint32_t)blk, (uint32_t)seed, (uint32_t)(seed >> 32), w);
-          if (!(bound(load_quad(s, blk, V, vec), w, c) < thr)) exact_keys(s, blk, V, tau, rid, seed, key, idx);
-        }
+      for (int g0 = first - lane; g0 < ngrp; g0 += step) {
+        const int grp = min(g0 + lane, ngrp - 1);
+        evaluate(!bounded || !(lower(load_raw(s, grp, V, vec), grp, rid, K, nc) > thr), grp);
       }
-    } else {          // no finite bound (NaN or -inf logits only, or logits beyond float32's range once scaled)
-#pragma unroll 1
-      for (int blk = first; blk < nblk; blk += step) exact_keys(s, blk, V, tau, rid, seed, key, idx);
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const double ok = __shfl_xor_sync(0xffffffffu, key, o);
-      const int oi = __shfl_xor_sync(0xffffffffu, idx, o);
-      better(key, idx, ok, oi);
-    }
+    warp_better(key, idx);
     if (lane == 0) { sh.key[warp] = key; sh.idx[warp] = idx; }
     __syncthreads();
     if (tid == 0) {
@@ -187,19 +249,31 @@ __global__ void __launch_bounds__(PT, 4) propose_kernel(const T* logits, int64_t
 template <typename T>
 cudaError_t launch(const void* logits, int64_t ld, int64_t N, int V, float tau, uint64_t seed, uint64_t row_offset, int32_t* out,
                    int sms, cudaStream_t st) {
-  const float c = (float)(INV_LN2 / (double)tau);
-  // A row per cluster of 8 while that does not ask for more blocks than fit, and a block keeps a few hundred elements.
-  const bool split = N * PROPOSE_CS <= 4 * (int64_t)sms && V >= 8192;
+  const float nc = -(float)(INV_LN2 / (double)tau);
+  Keys K;
+  for (int r = 0; r < 10; ++r) {
+    K.k0[r] = (uint32_t)seed + (uint32_t)r * 0x9E3779B9u;
+    K.k1[r] = (uint32_t)(seed >> 32) + (uint32_t)r * 0xBB67AE85u;
+  }
+  // Blocks per row: so many that they fill the chip, and two where a whole row per block would divide unevenly among the
+  // SMs, each keeping 1024 elements or more.
+  int cs = 1;
+  while (cs < PROPOSE_CS && (N * cs < 2 * (int64_t)sms || (cs == 1 && N < 4 * (int64_t)sms)) && V >= 2048 * cs) cs *= 2;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(PT, 1, 1);
   cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = PROPOSE_CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = split ? 1 : 0;
-  cfg.gridDim = dim3((unsigned)(split ? N * PROPOSE_CS : (N < (1 << 30) ? N : (1 << 30))), 1, 1);
-  if (split) return cudaLaunchKernelEx(&cfg, propose_kernel<T, PROPOSE_CS>, (const T*)logits, ld, N, V, (double)tau, c, seed, row_offset, out);
-  return cudaLaunchKernelEx(&cfg, propose_kernel<T, 1>, (const T*)logits, ld, N, V, (double)tau, c, seed, row_offset, out);
+  at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = cs > 1 ? 1 : 0;
+  cfg.gridDim = dim3((unsigned)((N < (1 << 27) ? N : (1 << 27)) * cs), 1, 1);
+  auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, (const T*)logits, ld, N, V, (double)tau, nc, K, seed, row_offset, out); };
+  switch (cs) {
+    case 1: return go(propose_kernel<T, 1>);
+    case 2: return go(propose_kernel<T, 2>);
+    case 4: return go(propose_kernel<T, 4>);
+    default: return go(propose_kernel<T, 8>);
+  }
 }
 
 }  // namespace

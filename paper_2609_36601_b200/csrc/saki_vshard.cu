@@ -58,6 +58,27 @@ __host__ __device__ inline void vs_cumulants(double a0, double a1, double a2, do
 // the order of (k5 / k2) step^4 / 24
 constexpr double VS_SETTLE_STEP = 3e-3;
 
+// The coupling decision and the gradient's coefficient of a row whose lambda is settled: they need no further sums, so
+// the gradient can be written by the pass that takes the shares of TV.
+__host__ __device__ inline void vs_decide(const VsConsts& c, int64_t i, double* st) {
+  const double lam = st[VS_LAM];
+  const double lp_x = st[VS_SX] / c.tau - st[VS_LSE_S], lT_x = st[VS_TX] / c.tau - st[VS_LSE_T];
+  double acc = 1.0;
+  int corrected = 0;
+  if (lam > 0.0) {
+    acc = exp(fmin(0.0, lam * (lT_x - lp_x) - st[VS_LOGZ]));
+    corrected = (scalar_uniform(c.seed, c.row_offset + (uint64_t)i, STAGE_ACCEPT) < acc) ? 0 : 1;
+  }
+  const bool masked = c.mask != nullptr && c.mask[i] == 0;
+  double loss = 0.0, coef = 0.0;
+  int tok = -1;
+  if (!masked) {
+    if (!corrected) { loss = (lp_x - lT_x) * lp_x; coef = -(lp_x - lT_x); tok = c.proposal[i]; }
+    else { coef = 1.0; tok = (int)st[VS_VSTAR]; }         // (the loss, -log p(v*), when the slices have sent s[v*])
+  }
+  st[VS_ACC] = acc; st[VS_CORR] = (double)corrected; st[VS_COEF] = coef; st[VS_TOK] = (double)tok; st[VS_LOSS] = loss;
+}
+
 // ---------------------------------------------------------------- the combine steps (host and device)
 // `part`: [world][N][SAKI_VSHARD_PARTIALS] gathered partials; row i of rank r at part[(r * N + i) * P].
 __host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const double* part, double* st) {
@@ -87,11 +108,16 @@ __host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const
   }
   const double lse_s = ms / c.tau + log(Ss), lse_t = mt / c.tau + log(St);
   st[VS_LSE_S] = lse_s; st[VS_LSE_T] = lse_t; st[VS_SX] = sx; st[VS_TX] = tx;
-  if (!(c.eps > 0.0)) { st[VS_STATUS] = (double)SAKI_ROW_EPS_ZERO; st[VS_MODE] = VS_SETTLED; return; }   // lambda = 0, log Z = 0
+  if (!(c.eps > 0.0)) {                                  // lambda = 0, log Z = 0
+    st[VS_STATUS] = (double)SAKI_ROW_EPS_ZERO; st[VS_MODE] = VS_SETTLED;
+    vs_decide(c, i, st);
+    return;
+  }
   const double cc = lse_t - lse_s;                       // d = delta - cc with delta = (t - s) / tau
   const double kl1 = Td / St - cc;                       // KL(T || p)
   if (kl1 <= c.eps) {                                    // teacher endpoint: q = T, log Z(1) = 0
     st[VS_LAM] = 1.0; st[VS_STATUS] = (double)SAKI_ROW_SATURATED; st[VS_MODE] = VS_SETTLED;
+    vs_decide(c, i, st);
     return;
   }
   // First guess: d KL(q_beta||p) / d beta = beta Var_{q_beta}(d) and the variance under q_beta is
@@ -179,6 +205,7 @@ __host__ __device__ inline int vs_combine_b(const VsConsts& c, int64_t i, const 
   st[VS_LAM] = beta + h;
   st[VS_LOGZ] = logZ + h * (E + h * (0.5 * k2 + h * (k3 / 6.0 + h * k4 / 24.0)));   // log Z along beta: the cumulant series of d under q_beta
   st[VS_MODE] = VS_SETTLED;
+  vs_decide(c, i, st);
   return 0;
 }
 
@@ -191,17 +218,11 @@ __host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const
     const double* p = part + ((int64_t)r * c.N + i) * P;
     tv += p[0]; kl += p[1]; sv += p[2];
   }
-  const double lam = st[VS_LAM], logZ = st[VS_LOGZ];
   const int x = c.proposal[i];
   const uint64_t rid = c.row_offset + (uint64_t)i;
-  const double lp_x = st[VS_SX] / c.tau - st[VS_LSE_S], lT_x = st[VS_TX] / c.tau - st[VS_LSE_T];
-  double acc = 1.0;
-  int corrected = 0;
-  if (lam > 0.0) {
-    acc = exp(fmin(0.0, lam * (lT_x - lp_x) - logZ));
-    corrected = (scalar_uniform(c.seed, rid, STAGE_ACCEPT) < acc) ? 0 : 1;
-  } else { tv = 0.0; kl = 0.0; }
-  st[VS_SV] = sv; st[VS_TV] = tv; st[VS_KL] = kl; st[VS_ACC] = acc; st[VS_CORR] = (double)corrected;
+  const bool corrected = st[VS_CORR] != 0.0;
+  if (!(st[VS_LAM] > 0.0)) { tv = 0.0; kl = 0.0; }
+  st[VS_SV] = sv; st[VS_TV] = tv; st[VS_KL] = kl;
   st[VS_OWNER] = -1.0; st[VS_Y] = (double)x; st[VS_SY] = st[VS_SX]; st[VS_TY] = st[VS_TX];
   if (corrected) {        // inverse CDF in index order: slices are contiguous, so rank order is index order
     const double target = scalar_uniform(c.seed, rid, STAGE_RESIDUAL) * tv;
@@ -220,14 +241,8 @@ __host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const
     }
     st[VS_OWNER] = (double)owner; st[VS_BEFORE] = before; st[VS_TARGET] = target; st[VS_TAKE_LAST] = take_last;
   }
-  const bool masked = c.mask != nullptr && c.mask[i] == 0;
-  uint32_t status = (uint32_t)st[VS_STATUS];
-  double loss = 0.0, coef = 0.0;
-  int tok = -1;
-  if (masked) status |= SAKI_ROW_MASKED;
-  else if (!corrected) { loss = (lp_x - lT_x) * lp_x; coef = -(lp_x - lT_x); tok = x; }
-  else { loss = -(sv / c.tau - st[VS_LSE_S]); coef = 1.0; tok = (int)st[VS_VSTAR]; }
-  st[VS_STATUS] = (double)status; st[VS_LOSS] = loss; st[VS_COEF] = coef; st[VS_TOK] = (double)tok;
+  if (c.mask != nullptr && c.mask[i] == 0) st[VS_STATUS] = (double)((uint32_t)st[VS_STATUS] | SAKI_ROW_MASKED);
+  else if (corrected) st[VS_LOSS] = -(sv / c.tau - st[VS_LSE_S]);
 }
 
 // the drawn token and the per-position outputs
@@ -286,7 +301,15 @@ struct VsSlice {
   int32_t V_local, v0, rank;
   double tau;
   const int32_t* proposal;
+  double* partial;
+  void* dlogits;         // stages C and D; NULL: not wanted
+  int64_t ld_g;
+  int32_t fast;          // the float32 kernels can read this slice
 };
+// The slices of one launch (blockIdx.y): one for a rank of a distributed call, all of them where a process holds several
+// ranks' slices (one launch per stage instead of one per rank: a slice of a thousand rows keeps the chip busy for 20 us).
+constexpr int VS_GROUP = 16;
+struct VsGroup { VsSlice s[VS_GROUP]; };
 
 // The residual draw on the rank that owns the inverse-CDF target (all threads of the block call; NW warps).
 // Every warp adds up the residual weights of its contiguous segment; the warp whose segment holds the target
@@ -344,22 +367,37 @@ __device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double r
 }
 
 template <typename T>
-__global__ void __launch_bounds__(VT) vs_partial_kernel(const VsSlice S, const int stage, const double* state, double* partial,
-                                                        void* dlogits, const int64_t ld_g, const double grad_scale,
-                                                        const bool only_flagged) {
+__global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ VsGroup Gr, const int stage, const double* state,
+                                                        const double grad_scale) {
+  const VsSlice& S = Gr.s[blockIdx.y];
+  double* const partial = S.partial;
+  void* const dlogits = S.dlogits;
+  const int64_t ld_g = S.ld_g;
+  const bool only_flagged = S.fast != 0;     // the float32 kernel has the other rows
   __shared__ double red[7 * VW];
   __shared__ float smax[2][VW];
   __shared__ int sarg[VW];
   __shared__ int stoken;
+  __shared__ unsigned char marks[VT];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
-  for (int64_t row = blockIdx.x; row < S.N; row += gridDim.x) {
+  if (only_flagged && stage == 0) return;    // no row is marked for float64 before the first combine
+  // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
+  // rule none is marked, and a block is done after one load)
+  for (int64_t base = blockIdx.x; base < S.N; base += (int64_t)gridDim.x * VT) {
+    const int64_t mine_row = base + (int64_t)tid * gridDim.x;
+    if (only_flagged) {
+      const bool marked = mine_row < S.N && state[mine_row * SAKI_VSHARD_STATE + VS_F64] != 0.0;
+      marks[tid] = marked ? 1 : 0;
+      if (!__syncthreads_or(marked)) continue;
+    }
+  for (int64_t row = base; row < S.N && row < base + (int64_t)gridDim.x * VT; row += gridDim.x) {
     const T* s = (const T*)S.s + row * S.ld_s;
     const T* t = (const T*)S.t + row * S.ld_t;
     double* out = partial + row * SAKI_VSHARD_PARTIALS;
     const double* st = state ? state + row * SAKI_VSHARD_STATE : nullptr;
-    if (only_flagged && !(st != nullptr && st[VS_F64] != 0.0)) continue;   // the float32 kernel has this row
+    if (only_flagged && !marks[(row - base) / gridDim.x]) continue;   // the float32 kernel has this row
     if (stage == 0) {
       // ---- stage A: maxima and argmax, then the sums under this slice's own shifts
       float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
@@ -446,25 +484,8 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const VsSlice S, const i
         out[2] = (live && vs >= 0 && vs < Vl) ? (double)ld_as_float(s, vs) : 0.0;
       }
     } else {
-      // ---- stage D: the gradient slice; on the owning rank the residual draw
+      // ---- stage D: on the owning rank the residual draw
       const int mode = (int)st[VS_MODE];
-      T* g = dlogits ? (T*)dlogits + row * ld_g : nullptr;
-      if (g) {
-        const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
-        const double lse_s = st[VS_LSE_S];
-        const int tok = mode == VS_FLAGGED ? -1 : (int)st[VS_TOK] - S.v0;
-        for (int v = tid; v < Vl; v += VT) {
-          double gv = 0.0;
-          if (sc != 0.0) gv = sc * (exp((double)ld_as_float(s, v) * rtau - lse_s) - (v == tok ? 1.0 : 0.0));
-          if constexpr (sizeof(T) == 2) {
-            // float64 -> bf16, round to nearest even: through a float rounded to odd (truncate, and keep in the
-            // last bit whether anything was cut off), which the second rounding cannot mistake for a tie
-            float f = __double2float_rz(gv);
-            if ((double)f != gv) f = __uint_as_float(__float_as_uint(f) | 1u);
-            g[v] = __float2bfloat16_rn(f);
-          } else g[v] = (float)gv;
-        }
-      }
       if (tid == 0) stoken = -1;
       __syncthreads();
       const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
@@ -480,6 +501,28 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const VsSlice S, const i
       }
       __syncthreads();
     }
+    if (stage >= 2 && dlogits) {
+      // ---- the gradient slice (with stage C, or with stage D)
+      const int mode = (int)st[VS_MODE];
+      T* g = (T*)dlogits + row * ld_g;
+      {
+        const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
+        const double lse_s = st[VS_LSE_S];
+        const int tok = mode == VS_FLAGGED ? -1 : (int)st[VS_TOK] - S.v0;
+        for (int v = tid; v < Vl; v += VT) {
+          double gv = 0.0;
+          if (sc != 0.0) gv = sc * (exp((double)ld_as_float(s, v) * rtau - lse_s) - (v == tok ? 1.0 : 0.0));
+          if constexpr (sizeof(T) == 2) {
+            // float64 -> bf16, round to nearest even: through a float rounded to odd (truncate, and keep in the
+            // last bit whether anything was cut off), which the second rounding cannot mistake for a tie
+            float f = __double2float_rz(gv);
+            if ((double)f != gv) f = __uint_as_float(__float_as_uint(f) | 1u);
+            g[v] = __float2bfloat16_rn(f);
+          } else g[v] = (float)gv;
+        }
+      }
+    }
+  }
   }
 }
 
@@ -636,8 +679,12 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(FT) vs_fast_kernel(const VsSlice S, const double* state, double* partial, void* dlogits,
-                                                     const int64_t ld_g, const double grad_scale) {
+__global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale) {
+  const VsSlice& S = Gr.s[blockIdx.y];
+  if (!S.fast) return;
+  double* const partial = S.partial;
+  void* const dlogits = S.dlogits;
+  const int64_t ld_g = S.ld_g;
   __shared__ double red[7 * FW];
   __shared__ float smax[2][FW];
   __shared__ int sarg[FW];
@@ -658,6 +705,39 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const VsSlice S, const doub
     double* out = partial + row * SAKI_VSHARD_PARTIALS;
     const double* st = state ? state + row * SAKI_VSHARD_STATE : nullptr;
     if (STAGE > 0 && st[VS_F64] != 0.0) continue;
+    __nv_bfloat16* const g = STAGE >= 2 && dlogits ? (__nv_bfloat16*)dlogits + row * ld_g : nullptr;
+    // the gradient slice on its own (a row without a TV pass, or a caller that asks for it at stage D)
+    auto gradient_only = [&]() {
+        const double sc = (int)st[VS_MODE] == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
+        if (sc == 0.0) {
+          for (int c = tid; c < n_chunks; c += FT) *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(0, 0, 0, 0);
+        } else {
+          const float msf = (float)st[VS_MS];
+          const double kp2 = (st[VS_LSE_S] - st[VS_MS] * rtau) * VF_LOG2E;
+          const float kpi = floorf((float)kp2 - 1e-3f);
+          const float kgf = (float)(sc * exp2((double)kpi - kp2)), scf = (float)sc;     // gradient entry = e_p * kgf (- sc at the token)
+          const float2 kpp = splat(-kpi), kgg = splat(kgf), nms = splat(-msf);
+          const int tok = (int)st[VS_TOK] - S.v0;
+          const int tok_c = (tok >= 0 && tok < Vl) ? (tok >> 3) : -1;
+          for (int c = tid; c < n_chunks; c += FT) {
+            const uint4 s4 = vf_ld(s + (size_t)c * 8);
+            const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w};
+            float gv[8];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float2 ep = ex2f2(ffma2(fadd2(unpack_bf16x2(sw[i]), nms), cc, kpp));
+              const float2 v = fmul2(ep, kgg);
+              gv[2 * i] = v.x; gv[2 * i + 1] = v.y;
+            }
+            if (c == tok_c) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) if (i == (tok & 7)) gv[i] -= scf;
+            }
+            *reinterpret_cast<uint4*>(g + (size_t)c * 8) =
+                make_uint4(pack_bf16x2(gv[0], gv[1]), pack_bf16x2(gv[2], gv[3]), pack_bf16x2(gv[4], gv[5]), pack_bf16x2(gv[6], gv[7]));
+          }
+        }
+    };
     if (STAGE == 0) {
       // ---- stage A, first sweep: the slice's maxima, and the first chunk that holds the teacher's
       uint32_t run_s = VF_FILLER;
@@ -787,7 +867,8 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
         out[0] = a[0]; out[1] = a[1] * rtau; out[2] = a[2] * r2; out[3] = a[3] * r2 * rtau; out[4] = a[4] * r2 * r2;
       }
     } else if (STAGE == 2) {
-      // ---- stage C: the slice's share of TV and KL(q||p); the student's logit at the teacher's argmax
+      // ---- stage C: the slice's share of TV and KL(q||p); the student's logit at the teacher's argmax; the gradient
+      // slice (the row's coefficient has been known since its lambda settled)
       const bool live = (int)st[VS_MODE] == VS_SETTLED;
       const double lam = st[VS_LAM];
       double a[3] = {0.0, 0.0, 0.0};
@@ -809,16 +890,23 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
         fq = exp2((double)kqi - kq2);
         const float2 cll = splat(cl), ccll = splat(ccl), kpp = splat(-kpi), kqq = splat(-kqi), nrho = splat(-(float)(fp / fq));
         const float2 nms = splat(-msf), nmt = splat(-mtf);
+        // the gradient entry is e_p * kgf (- sc at the token)
+        const double sc = grad_scale * st[VS_COEF] * rtau;
+        const float kgf = (float)(sc * fp), scf = (float)sc;
+        const float2 kgg = splat(kgf);
+        const int tok = (int)st[VS_TOK] - S.v0, tok_c = (tok >= 0 && tok < Vl) ? (tok >> 3) : -1;
         float2 R = splat(0.f), Sq = splat(0.f), Sqd = splat(0.f);
 #pragma unroll 2
         for (int c = tid; c < n_chunks; c += FT) {
           const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
           const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
+          float2 gv[4];
 #pragma unroll
           for (int i = 0; i < 4; ++i) {
             const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
             const float2 d = ffma2(sf, neg1, tf);
             const float2 ep = ex2f2(ffma2(sf, cc, kpp));
+            gv[i] = fmul2(ep, kgg);
             const float2 eq = ex2f2(ffma2(tf, cll, ffma2(sf, ccll, kqq)));
             float2 r = ffma2(ep, nrho, eq);          // (q_i - p_i) / fq
             r.x = fmaxf(r.x, 0.f); r.y = fmaxf(r.y, 0.f);
@@ -826,9 +914,17 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
             Sq = fadd2(Sq, eq);
             Sqd = ffma2(eq, d, Sqd);
           }
+          if (g) {
+            if (c == tok_c) {
+#pragma unroll
+              for (int i = 0; i < 8; ++i) if (i == (tok & 7)) { if (i & 1) gv[i >> 1].y -= scf; else gv[i >> 1].x -= scf; }
+            }
+            *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(pack_bf16x2(gv[0].x, gv[0].y), pack_bf16x2(gv[1].x, gv[1].y),
+                                                                      pack_bf16x2(gv[2].x, gv[2].y), pack_bf16x2(gv[3].x, gv[3].y));
+          }
         }
         a[0] = vf_tot(R); a[1] = vf_tot(Sq); a[2] = vf_tot(Sqd);
-      }
+      } else if (g) gradient_only();
       vf_block_sum<3>(a, red);
       if (tid == 0) {
         for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
@@ -841,40 +937,9 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
         out[2] = (live && vs >= 0 && vs < Vl) ? (double)__bfloat162float(s[vs]) : 0.0;
       }
     } else {
-      // ---- stage D: the gradient slice; on the owning rank the residual draw
+      // ---- stage D: on the owning rank the residual draw; the gradient slice, if stage C has not written it
       const int mode = (int)st[VS_MODE];
-      __nv_bfloat16* g = dlogits ? (__nv_bfloat16*)dlogits + row * ld_g : nullptr;
-      if (g) {
-        const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
-        if (sc == 0.0) {
-          for (int c = tid; c < n_chunks; c += FT) *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(0, 0, 0, 0);
-        } else {
-          const float msf = (float)st[VS_MS];
-          const double kp2 = (st[VS_LSE_S] - st[VS_MS] * rtau) * VF_LOG2E;
-          const float kpi = floorf((float)kp2 - 1e-3f);
-          const float kgf = (float)(sc * exp2((double)kpi - kp2)), scf = (float)sc;     // gradient entry = e_p * kgf (- sc at the token)
-          const float2 kpp = splat(-kpi), kgg = splat(kgf), nms = splat(-msf);
-          const int tok = (int)st[VS_TOK] - S.v0;
-          const int tok_c = (tok >= 0 && tok < Vl) ? (tok >> 3) : -1;
-          for (int c = tid; c < n_chunks; c += FT) {
-            const uint4 s4 = vf_ld(s + (size_t)c * 8);
-            const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w};
-            float gv[8];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              const float2 ep = ex2f2(ffma2(fadd2(unpack_bf16x2(sw[i]), nms), cc, kpp));
-              const float2 v = fmul2(ep, kgg);
-              gv[2 * i] = v.x; gv[2 * i + 1] = v.y;
-            }
-            if (c == tok_c) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i) if (i == (tok & 7)) gv[i] -= scf;
-            }
-            *reinterpret_cast<uint4*>(g + (size_t)c * 8) =
-                make_uint4(pack_bf16x2(gv[0], gv[1]), pack_bf16x2(gv[2], gv[3]), pack_bf16x2(gv[4], gv[5]), pack_bf16x2(gv[6], gv[7]));
-          }
-        }
-      }
+      if (g) gradient_only();
       if (tid == 0) stoken = -1;
       __syncthreads();
       const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
@@ -910,33 +975,51 @@ static bool vshard_fast_call(const saki_vshard_in& in, bool allow_fast) {
   return allow_fast && in.dtype == SAKI_BF16 && in.eps >= 0.02f;   // below, KL needs the float64 sums (or a quadrature)
 }
 
-cudaError_t launch_vshard_partial(const saki_vshard_in& in, int stage, const double* state, double* partial, void* dlogits,
-                                  int64_t ld_g, float grad_scale, bool allow_fast, cudaStream_t st) {
-  VsSlice S;
-  S.s = in.student_logits; S.t = in.teacher_logits; S.ld_s = in.ld_s; S.ld_t = in.ld_t; S.N = in.N;
-  S.V_local = in.V_local; S.v0 = in.v0; S.rank = in.rank; S.tau = (double)in.temperature; S.proposal = in.proposal;
+cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
+                                  void* const* dlogits, const int64_t* ld_g, float grad_scale, bool allow_fast, int* n_launches,
+                                  cudaStream_t st) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
-  const bool fast = vshard_fast_call(in, allow_fast) && in.V_local % 8 == 0 && in.ld_s % 8 == 0 && in.ld_t % 8 == 0 &&
-                    al16(in.student_logits) && al16(in.teacher_logits) && (!dlogits || (al16(dlogits) && ld_g % 8 == 0));
-  if (fast) {
-    const int fgrid = (int)(in.N < 8LL * sms ? in.N : 8LL * sms);
+  for (int i0 = 0; i0 < n; i0 += VS_GROUP) {
+    const int m = n - i0 < VS_GROUP ? n - i0 : VS_GROUP;
+    VsGroup Gr;
+    int n_fast = 0;
+    for (int k = 0; k < m; ++k) {
+      const saki_vshard_in& a = in[i0 + k];
+      VsSlice& S = Gr.s[k];
+      S.s = a.student_logits; S.t = a.teacher_logits; S.ld_s = a.ld_s; S.ld_t = a.ld_t; S.N = a.N;
+      S.V_local = a.V_local; S.v0 = a.v0; S.rank = a.rank; S.tau = (double)a.temperature; S.proposal = a.proposal;
+      S.partial = partial[i0 + k];
+      S.dlogits = stage >= 2 && dlogits ? dlogits[i0 + k] : nullptr;
+      S.ld_g = S.dlogits ? ld_g[i0 + k] : 0;
+      S.fast = vshard_fast_call(a, allow_fast) && a.V_local % 8 == 0 && a.ld_s % 8 == 0 && a.ld_t % 8 == 0 && al16(S.s) &&
+               al16(S.t) && (!S.dlogits || (al16(S.dlogits) && S.ld_g % 8 == 0));
+      n_fast += S.fast;
+    }
+    const int64_t N = in[i0].N;
     const double gs = (double)grad_scale;
-    if (stage == 0) vs_fast_kernel<0><<<fgrid, FT, 0, st>>>(S, state, partial, dlogits, ld_g, gs);
-    else if (stage == 1) vs_fast_kernel<1><<<fgrid, FT, 0, st>>>(S, state, partial, dlogits, ld_g, gs);
-    else if (stage == 2) vs_fast_kernel<2><<<fgrid, FT, 0, st>>>(S, state, partial, dlogits, ld_g, gs);
-    else vs_fast_kernel<3><<<fgrid, FT, 0, st>>>(S, state, partial, dlogits, ld_g, gs);
+    if (n_fast > 0) {
+      const dim3 grid((unsigned)(N < 8LL * sms ? N : 8LL * sms), (unsigned)m, 1);
+      if (stage == 0) vs_fast_kernel<0><<<grid, FT, 0, st>>>(Gr, state, gs);
+      else if (stage == 1) vs_fast_kernel<1><<<grid, FT, 0, st>>>(Gr, state, gs);
+      else if (stage == 2) vs_fast_kernel<2><<<grid, FT, 0, st>>>(Gr, state, gs);
+      else vs_fast_kernel<3><<<grid, FT, 0, st>>>(Gr, state, gs);
+      *n_launches += 1;
+      cudaError_t e = cudaGetLastError();
+      if (e != cudaSuccess) return e;
+    }
+    if (n_fast == m && stage == 0) continue;           // no row is marked for float64 before the first combine
+    const int64_t blocks = (3LL * sms + m - 1) / m;
+    const dim3 grid((unsigned)(N < blocks ? N : blocks), (unsigned)m, 1);
+    if (in[i0].dtype == SAKI_BF16) vs_partial_kernel<__nv_bfloat16><<<grid, VT, 0, st>>>(Gr, stage, state, gs);
+    else vs_partial_kernel<float><<<grid, VT, 0, st>>>(Gr, stage, state, gs);
+    *n_launches += 1;
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess || stage == 0) return e;          // no row is marked for float64 before the first combine
+    if (e != cudaSuccess) return e;
   }
-  const int grid = (int)(in.N < 3LL * sms ? in.N : 3LL * sms);
-  if (in.dtype == SAKI_BF16)
-    vs_partial_kernel<__nv_bfloat16><<<dim3(grid, 1, 1), VT, 0, st>>>(S, stage, state, partial, dlogits, ld_g, (double)grad_scale, fast);
-  else
-    vs_partial_kernel<float><<<dim3(grid, 1, 1), VT, 0, st>>>(S, stage, state, partial, dlogits, ld_g, (double)grad_scale, false);
-  return cudaGetLastError();
+  return cudaSuccess;
 }
 
 static VsConsts consts_of(const saki_vshard_in& in, bool allow_fast) {
@@ -950,7 +1033,7 @@ static VsConsts consts_of(const saki_vshard_in& in, bool allow_fast) {
 cudaError_t launch_vshard_combine(const saki_vshard_in& in, int stage, const double* gathered, double* state, const saki_out& out,
                                   unsigned int* n_solving, bool allow_fast, cudaStream_t st) {
   const VsConsts c = consts_of(in, allow_fast);
-  const int th = 128;
+  const int th = 32;           // one thread per row, a chain of float64 scalars: spread over the SMs
   vs_combine_kernel<<<(unsigned)((in.N + th - 1) / th), th, 0, st>>>(c, stage, gathered, state, out, n_solving);
   return cudaGetLastError();
 }
