@@ -42,12 +42,16 @@ static int device_ready(unsigned long long** flagged) {
   int dev = -1;
   cudaError_t e = cudaGetDevice(&dev);
   if (e != cudaSuccess) return fail(SAKI_ERR_UNSUPPORTED, "no CUDA device: %s", cudaGetErrorString(e));
+  // looked up once per device (a call of a few rows spends as long in these queries as in a launch)
+  static std::atomic<unsigned long long*> known[64];
+  if (dev < 64 && (*flagged = known[dev].load(std::memory_order_acquire)) != nullptr) return SAKI_OK;
   int major = 0;
   e = cudaDeviceGetAttribute(&major, cudaDevAttrComputeCapabilityMajor, dev);
   if (e != cudaSuccess) return cuda_fail(e, "cudaDeviceGetAttribute");
   if (major != 10) return fail(SAKI_ERR_UNSUPPORTED, "device compute capability %d.x: this library is built for sm_100a only", major);
   e = cudaGetSymbolAddress((void**)flagged, g_flagged_rows);
   if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress");
+  if (dev < 64) known[dev].store(*flagged, std::memory_order_release);
   return SAKI_OK;
 }
 
@@ -89,10 +93,12 @@ static int redo_scratch(int64_t n_rows, cudaStream_t st, int32_t** list, unsigne
   if (b.cap < n_rows) {
     if (b.list) g_retired.emplace_back(dev, b.list);   // an earlier call on this stream may still be running on it
     b = RedoBuf();
-    const int64_t cap = std::max<int64_t>(n_rows, 1 << 16);
-    // row ids, 64 words of counters, and as many words again (block verification: one per sequence)
-    cudaError_t e = cudaMalloc((void**)&b.list, (size_t)(2 * cap + 64) * sizeof(int32_t));
+    const int64_t cap = (std::max<int64_t>(n_rows, 1 << 16) + 63) & ~(int64_t)63;
+    // row ids, the counters, and as many words again (block verification: one per sequence)
+    cudaError_t e = cudaMalloc((void**)&b.list, (size_t)(2 * cap + CNT_WORDS) * sizeof(int32_t));
     if (e != cudaSuccess) { b = RedoBuf(); return cuda_fail(e, "cudaMalloc (redo list)"); }
+    e = cudaMemsetAsync(b.list + cap, 0, CNT_WORDS * sizeof(int32_t), st);
+    if (e != cudaSuccess) { cudaFree(b.list); b = RedoBuf(); return cuda_fail(e, "cudaMemsetAsync (redo list)"); }
     b.cap = cap;
   }
   *list = b.list;
@@ -101,14 +107,14 @@ static int redo_scratch(int64_t n_rows, cudaStream_t st, int32_t** list, unsigne
 }
 // the calling thread's last routing call's counters, or NULL if there are none (any more)
 static unsigned int* last_counters() {
-  return g_last_redo_generation == g_redo_generation.load() ? g_last_redo_count : nullptr;
+  return g_last_redo_generation == g_redo_generation.load() && g_last_redo_count ? g_last_redo_count + CNT_LAST : nullptr;
 }
 
 // Fixed scratch of saki_route_fwd_bwd_noalloc: the redo list of the two-tier routing for callers that must
 // not allocate.  SAKI_NOALLOC_MAX_ROWS row ids plus the counter; every device that loads the library holds
 // these 4 MB until the process exits.
 #define SAKI_NOALLOC_MAX_ROWS (1 << 20)
-static __device__ __align__(256) int32_t g_noalloc_scratch[SAKI_NOALLOC_MAX_ROWS + 64];
+static __device__ __align__(256) int32_t g_noalloc_scratch[SAKI_NOALLOC_MAX_ROWS + CNT_WORDS];
 static std::mutex g_noalloc_mu;
 static int32_t* g_noalloc_ptr[64] = {nullptr};   // device address of the array, per device ordinal
 
@@ -169,12 +175,13 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
       if (rc) return rc;
       // the words behind the counters (one per row; block verification keeps its sequences' stops there) take
       // what the float32 kernel made of lambda for the rows it hands over
-      if (!p.spec) p.redo_guess = (float*)(p.redo_count + 64);
+      if (!p.spec) p.redo_guess = (float*)(p.redo_count + CNT_WORDS);
     }
-    // the counter, the three statistics words after it, and the phase clock's sums
-    e = cudaMemsetAsync(p.redo_count, 0, (8 + 2 * SAKI_PHASE_COUNTERS) * sizeof(unsigned int), st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
-    p.phase_cycles = g_phase_clock.load() ? (unsigned long long*)(p.redo_count + 8) : nullptr;
+    if (scratch_list) {   // shared by all callers of the device: whatever a call that was cut short may have left
+      e = cudaMemsetAsync(p.redo_count, 0, CNT_LIVE * sizeof(unsigned int), st);
+      if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
+    }
+    p.phase_cycles = g_phase_clock.load() ? (unsigned long long*)(p.redo_count + CNT_PHASES) : nullptr;
     g_last_redo_count = p.redo_count;
     g_last_redo_generation = g_redo_generation.load();
   }
@@ -195,8 +202,8 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
     if (p.spec && (cudaGetDevice(&dev_now) != cudaSuccess ||
                    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev_now) != cudaSuccess)) sms = 0;
     if (p.spec && g_spec_early_out.load() && !scratch_list && sms > 0 && p.n_rows / p.K1 >= 2 * (int64_t)sms) {
-      p.seq_next = p.redo_count + 1;
-      p.seq_stop = (int*)(p.redo_count + 64);
+      p.seq_next = p.redo_count + CNT_TICKET;
+      p.seq_stop = (int*)(p.redo_count + CNT_WORDS);
       e = cudaMemsetAsync(p.seq_stop, 0x7f, (size_t)(p.n_rows / p.K1) * sizeof(int), st);   // "no stop yet": above any position
       if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     }
@@ -213,7 +220,10 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
   if (served) {   // second tier: the rows the float32 kernel handed over
     p.from_list = 1;
     e = launch_general(p, dtype, st, &launches);
-    if (e != cudaSuccess) return cuda_fail(e, "general kernel launch (redo list)");
+    if (e != cudaSuccess) {
+      cudaMemsetAsync(p.redo_count, 0, CNT_LIVE * sizeof(unsigned int), st);   // the kernel that would have cleared them is missing
+      return cuda_fail(e, "general kernel launch (redo list)");
+    }
   } else {
     e = launch_general(p, dtype, st, &launches);
     if (e != cudaSuccess) return cuda_fail(e, "general kernel launch");
@@ -301,8 +311,6 @@ static int meta_impl(const saki_meta_in* in, const saki_meta_out* out, void* dlo
     scratch_lock.lock();         // until the kernels that use the list are launched
     rc = redo_scratch(p.n_rows, st, &p.redo_list, &p.redo_count);
     if (rc) return rc;
-    e = cudaMemsetAsync(p.redo_count, 0, (8 + 2 * SAKI_PHASE_COUNTERS) * sizeof(unsigned int), st);
-    if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     g_last_redo_count = p.redo_count;
     g_last_redo_generation = g_redo_generation.load();
     e = launch_meta_stream(p, st, &launches, &served);
@@ -310,7 +318,10 @@ static int meta_impl(const saki_meta_in* in, const saki_meta_out* out, void* dlo
     if (served) { used = 4; p.from_list = 1; }
   }
   e = launch_meta_general(p, in->dtype, st, &launches);
-  if (e != cudaSuccess) return cuda_fail(e, "general backward kernel launch");
+  if (e != cudaSuccess) {
+    if (p.from_list) cudaMemsetAsync(p.redo_count, 0, CNT_LIVE * sizeof(unsigned int), st);
+    return cuda_fail(e, "general backward kernel launch");
+  }
   g_launches += (uint64_t)launches;
   g_last_kernel = used;
   return SAKI_OK;
@@ -319,6 +330,7 @@ static int meta_impl(const saki_meta_in* in, const saki_meta_out* out, void* dlo
 // ---- block verification: per-sequence first-rejection resolve (Section 3.5) ----
 __global__ void spec_resolve_kernel(int64_t B, int K, saki_out o, int32_t* n_accept, int32_t* next_token,
                                     uint8_t* next_is_corr) {
+  wait_for_predecessor();
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
   const int K1 = K + 1;
@@ -550,10 +562,9 @@ SAKI_API int saki_spec_verify(const saki_spec_in* in, const saki_spec_out* out, 
   rc = dispatch_rows(p, in->dtype, st);
   if (rc) return rc;
   const int th = 128;
-  spec_resolve_kernel<<<(unsigned)((in->B + th - 1) / th), th, 0, st>>>(in->B, in->K, p.out, out->n_accept,
-                                                                        out->next_token, out->next_is_correction);
+  cudaError_t e = launch_pdl(spec_resolve_kernel, (int)((in->B + th - 1) / th), th, 0, st, true, in->B, in->K, p.out,
+                             out->n_accept, out->next_token, out->next_is_correction);
   g_launches += 1;
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail(e, "resolve kernel launch");
   return SAKI_OK;
 }
@@ -731,7 +742,7 @@ SAKI_API int saki_solve_evaluations(void* cuda_stream, uint64_t* n_passes) {
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   unsigned int h = 0;
-  e = cudaMemcpy(&h, counters + 3, sizeof(h), cudaMemcpyDeviceToHost);
+  e = cudaMemcpy(&h, counters + CNT_EVALS, sizeof(h), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   *n_passes = h;
   return SAKI_OK;
@@ -749,7 +760,7 @@ SAKI_API int saki_phase_cycles(void* cuda_stream, uint64_t* cycles) {
   if (!counters) return SAKI_OK;
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
-  e = cudaMemcpy(cycles, counters + 8, SAKI_PHASE_COUNTERS * sizeof(uint64_t), cudaMemcpyDeviceToHost);
+  e = cudaMemcpy(cycles, counters + CNT_PHASES, SAKI_PHASE_COUNTERS * sizeof(uint64_t), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   return SAKI_OK;
 }
@@ -765,7 +776,7 @@ SAKI_API int saki_spec_positions_routed(void* cuda_stream, uint64_t* n_positions
   cudaError_t e = cudaStreamSynchronize((cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(e, "cudaStreamSynchronize");
   unsigned int h = 0;
-  e = cudaMemcpy(&h, counters + 2, sizeof(h), cudaMemcpyDeviceToHost);
+  e = cudaMemcpy(&h, counters + CNT_ROUTED, sizeof(h), cudaMemcpyDeviceToHost);
   if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy");
   *n_positions = h;
   return SAKI_OK;

@@ -64,6 +64,7 @@ static_assert(OFF_MBAR % 8 == 0 && OFF_SCR % 16 == 0, "alignment");
 template <int CS>
 __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const int n_clusters) {
   extern __shared__ __align__(128) unsigned char smem[];
+  launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const unsigned rank = cg::this_cluster().block_rank();
   const int cluster_id = blockIdx.x / CS;

@@ -40,8 +40,7 @@ struct RowParams {
   float grad_scale;
   unsigned long long* flagged;         // device counter of flagged rows
   int32_t* redo_list;                  // scratch: rows the float32 kernels hand to the float64 kernel
-  unsigned int* redo_count;            // scratch: their number (zeroed before the launch, with the three words
-                                       // after it: [1], [2] see seq_next; [3] evaluation passes of the row-per-SM kernel)
+  unsigned int* redo_count;            // scratch: the call's counters (CNT_*), zero before the first kernel of the call
   float* redo_guess;                   // scratch or NULL: what the float32 kernel made of lambda for each row of redo_list (< 0: nothing)
   int32_t from_list;                   // general kernel only: route the rows of redo_list
 
@@ -52,6 +51,55 @@ struct RowParams {
                                        // [1] positions routed (both zeroed before the launch); NULL: rows in static order
   int* seq_stop;                       // [n_rows / K1] position of each sequence's first stop (>= K1 before the launch)
 };
+
+// The counters of a two-tier call.  They are zero whenever no call is under way: the call's last kernel, the list-mode
+// one, copies them to the words from CNT_LAST on (what saki_redo_count and its kin read) and clears them, so that a call
+// needs no memset of its own and a captured call can be replayed.
+enum { CNT_REDO = 0,      // rows on the redo list
+       CNT_TICKET, CNT_ROUTED,                 // see seq_next
+       CNT_EVALS,         // evaluation passes of the row-per-SM kernel
+       CNT_DONE,          // blocks of the list-mode kernel that have finished
+       CNT_PHASES = 8,    // SAKI_PHASE_COUNTERS 64-bit sums
+       CNT_LIVE = CNT_PHASES + 2 * SAKI_PHASE_COUNTERS,
+       CNT_LAST = 64, CNT_WORDS = 128 };
+static_assert(CNT_LIVE <= CNT_LAST, "the counters of a call and of the last one overlap");
+
+#ifdef __CUDACC__
+// Programmatic dependent launch: a kernel lets the next one on the stream be set up while it runs, and that one waits
+// here, before it touches memory, until everything in front of it has finished.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// Called by every block of the list-mode kernel, all threads, when it is done.
+__device__ __forceinline__ void close_counters(unsigned int* c) {
+  __shared__ bool last;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    last = atomicAdd(c + CNT_DONE, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (last) {
+    for (int i = threadIdx.x; i < CNT_LIVE; i += blockDim.x) {
+      c[CNT_LAST + i] = *(volatile unsigned int*)(c + i);
+      c[i] = 0u;
+    }
+  }
+}
+// A launch that may (pdl) be set up while the kernel in front of it runs: the kernel starts with wait_for_predecessor.
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t st, bool pdl, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid, 1, 1);
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+#endif
 
 // Parameters of the metadata-driven backward kernels (saki_route_bwd_from_meta).
 struct MetaParams {

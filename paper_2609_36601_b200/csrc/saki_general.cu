@@ -7,9 +7,7 @@
 //
 // What bounds it: the float64 pipe (64 lanes per clock and SM; a warp instruction occupies its scheduler's half of
 // it for two clocks).  Hence:
-//   - 2^y costs eight float64 operations: y is split by a magic-number addition into n + i/256 + r, 2^(i/256) comes
-//     from a table in shared memory and 2^r from its Taylor polynomial (|r| <= 1/512: the first dropped term is
-//     4e-17).  The table is stored 16 times over, one copy per 64-bit bank, so a half-warp's lookups never conflict;
+//   - 2^y costs eight float64 operations (saki_exp2.cuh);
 //   - three passes over the row: "sums" (two exponentials), one or two evaluations of KL with its first four
 //     derivatives (one exponential each: the root of the fourth-order model, as in the bf16 kernels, here accepted
 //     when the dropped terms move lambda by less than about 1e-11), "final" (two exponentials; total variation, draw
@@ -19,8 +17,9 @@
 //   - the moments of the logit difference that only feed the first guess of lambda are float32.
 // A warp owns a contiguous segment of the row in every pass (the residual draw is in index order), a row is owned by
 // one block or by a cluster of blocks that add up their warps' partial sums through distributed shared memory.
-#include "saki_device.cuh"
+#include "saki_exp2.cuh"
 #include <cooperative_groups.h>
+#include <algorithm>
 #include <atomic>
 
 namespace cg = cooperative_groups;
@@ -35,11 +34,10 @@ constexpr int GW = GT / 32;    // warps per block
 // Measured (2 / 3 / 4): bf16 rows of 32003 0.275 / 0.280 / 0.309 ms, fp32 rows of 151936 0.784 / 0.786 / 0.734 ms.
 template <typename T> constexpr int BLOCKS_PER_SM = sizeof(T) == 4 ? 4 : 3;
 constexpr int MAX_CS = 8;      // blocks per row, at most
-constexpr int TAB = 256, COPIES = 16;
 constexpr int NPART = 12;      // doubles a warp leaves per phase
 
 struct Shared {
-  double tab[TAB * COPIES];
+  double tab[EXP2_TAB * EXP2_COPIES];
   double part[2][GW][NPART];   // alternates from phase to phase: one barrier per phase is enough
   double bc[32];               // scalars broadcast to the block
   double sub[GW];
@@ -52,31 +50,6 @@ enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G
 static_assert(G_COUNT <= 32, "broadcast area too small");
 enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
-
-// The entry of 2^(i/256) has i << 12 taken off its high word: adding the low word of y + M, shifted by 12, then puts
-// the exponent in and the index back in one addition.
-// The coefficients are read from the constant bank (as operands: three 64-bit immediates cost two moves each per
-// exponential once registers are short, and a float64 operation on three register operands runs at two thirds of the rate).
-__constant__ double EXP2_COEF[4] = {9.618129107628477e-03, 5.550410866482158e-02, 2.402265069591007e-01, 6.931471805599453e-01};   // ln2^i / i!, i = 4..1
-struct Exp2 {
-  uint32_t lane8;   // this lane's copy of the table: byte offset among the 16 copies of an entry
-  const double* tab;
-  // 2^y for y <= ~1000; y below -1000 counts as -1000 (clamped through the high word: an unsigned minimum)
-  __device__ __forceinline__ double operator()(double y) const {
-    const uint32_t hi = min((uint32_t)__double2hiint(y), 0xC08F4000u);
-    y = __hiloint2double((int)hi, __double2loint(y));
-    const double M = 26388279066624.0;                       // 1.5 * 2^44: the low word of y + M is round(256 y)
-    const double t = y + M;
-    const double r = y - (t - M);
-    const int k = __double2loint(t);
-    double T = *(const double*)((const char*)tab + ((((uint32_t)k << 7) & 0x7f80u) | lane8));
-    double q = fma(r, EXP2_COEF[0], EXP2_COEF[1]);
-    q = fma(r, q, EXP2_COEF[2]);
-    q = fma(r, q, EXP2_COEF[3]);
-    T = __hiloint2double(__double2hiint(T) + (k << 12), __double2loint(T));
-    return fma(T * r, q, T);
-  }
-};
 
 // Dynamic rows: a block (cluster) that is done takes over the work of one that has not started yet, by cancelling its
 // launch.  The answer arrives in shared memory and completes an mbarrier.
@@ -97,12 +70,6 @@ __device__ __forceinline__ int steal_answer(const void* answer) {   // first blo
 
 __device__ __forceinline__ double pow2_down(double n) {      // 2^n for whole n <= 0; 0 below -1000
   return n < -1000.0 ? 0.0 : __longlong_as_double((long long)(1023 + (int)n) << 52);
-}
-
-// float64 to float, ready to be rounded to bf16: truncated, with the last bit set if anything was dropped (rounded to
-// odd), so that the second rounding is the only one.  (The low 29 bits of a float64 do not fit a normal float.)
-__device__ __forceinline__ float to_odd(double v) {
-  return __uint_as_float(__float_as_uint(__double2float_rz(v)) | (uint32_t)((__double2loint(v) << 3) != 0));
 }
 
 // Sixteen bytes of a row: eight bf16 or four fp32 elements.
@@ -251,21 +218,20 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   constexpr int NWC = GW * CS;                               // warps of the row, in index order of their segments
   const int gw = crank * GW + warp;
 
-  const int64_t n_work = P.from_list ? (int64_t)*P.redo_count : P.n_rows;
-  if ((int64_t)(blockIdx.x / CS) >= n_work) return;          // the whole cluster: nothing to do (an empty row list, as a rule)
-  for (int i = tid; i < TAB; i += GT) {
-    double e = exp2((double)i * (1.0 / TAB));
-    e = __hiloint2double(__double2hiint(e) - (i << 12), __double2loint(e));
-#pragma unroll 1
-    for (int c = 0; c < COPIES; ++c) sh.tab[i * COPIES + ((c + lane) & (COPIES - 1))] = e;
+  if (P.from_list) wait_for_predecessor();
+  launch_dependents();
+  const int64_t n_work = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
+  if ((int64_t)(blockIdx.x / CS) >= n_work) {                // the whole cluster: nothing to do (an empty row list, as a rule)
+    if (P.from_list) close_counters(P.redo_count);
+    return;
   }
+  exp2_table(sh.tab, tid, GT);
   if (tid == 0) {
     mbar_init(&sh.bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncthreads();
-  Exp2 ex2;
-  ex2.tab = sh.tab; ex2.lane8 = (uint32_t)(lane & (COPIES - 1)) * 8u;
+  const Exp2 ex2(sh.tab, lane);
 
   const double eps = (double)P.eps;     // (rtau = 1 / tau, c = log2(e) / tau)
   int ph = 0;
@@ -672,6 +638,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
     ph ^= 1;
   }
   if constexpr (CS > 1) cg::this_cluster().sync();   // no block leaves while a peer may still read its shared memory
+  if (P.from_list) close_counters(P.redo_count);
 }
 
 template <typename T, int CS>
@@ -682,15 +649,18 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(GT, 1, 1);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = CS > 1 ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = p.from_list ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = CS; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = CS > 1 ? 2 : 1;
   if (fit <= 0) {
     int n = 0;
     cudaError_t e;
     if (CS > 1) {
       cfg.gridDim = dim3(CS, 1, 1);
+      at[0].val.programmaticStreamSerializationAllowed = 0;
       e = cudaOccupancyMaxActiveClusters(&n, general_kernel<T, CS>, &cfg);
     } else {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, general_kernel<T, CS>, GT, 0);
@@ -704,6 +674,8 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
   // and the rows do not divide evenly); in list mode, and for more rows than a grid may have blocks, a fixed stride.
   const bool steal = !p.from_list && p.n_rows > fit && p.n_rows <= (1 << 27);
   const double rtau = 1.0 / (double)p.temperature;
+  at[0].val.programmaticStreamSerializationAllowed = p.from_list ? 1 : 0;
+  if (p.from_list) fit = std::min(fit, std::max(1, sms / CS));     // as a rule they only find the list empty
   cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit || steal ? p.n_rows : fit)), 1, 1);
   return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p, (int)steal, rtau, INV_LN2 * rtau);
 }

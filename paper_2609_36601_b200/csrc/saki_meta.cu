@@ -78,7 +78,8 @@ __device__ __forceinline__ double block_max_d(double v, double* sh) {
 template <typename T>
 __global__ void __launch_bounds__(MG_THREADS) meta_general_kernel(const MetaParams P) {
   __shared__ double sh[MG_THREADS / 32];
-  const int64_t n_items = P.from_list ? (int64_t)*P.redo_count : P.n_rows;
+  if (P.from_list) wait_for_predecessor();
+  const int64_t n_items = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
   for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;
     const T* s = (const T*)P.s + row * P.ld_s;
@@ -115,15 +116,15 @@ __global__ void __launch_bounds__(MG_THREADS) meta_general_kernel(const MetaPara
     }
     if (threadIdx.x == 0) meta_write(P, row, (float)(-(double)m.coef * logp), (float)logp, 0u);
   }
+  if (P.from_list) close_counters(P.redo_count);
 }
 
 cudaError_t launch_meta_general(const MetaParams& p, int dtype, cudaStream_t st, int* n_launches) {
   if (p.n_rows <= 0) return cudaSuccess;
-  const int grid = (int)std::min<int64_t>(p.n_rows, p.from_list ? 1184 : (1 << 20));
-  if (dtype == SAKI_BF16) meta_general_kernel<__nv_bfloat16><<<grid, MG_THREADS, 0, st>>>(p);
-  else meta_general_kernel<float><<<grid, MG_THREADS, 0, st>>>(p);
+  const int grid = (int)std::min<int64_t>(p.n_rows, p.from_list ? 148 : (1 << 20));   // a list is empty as a rule
   ++*n_launches;
-  return cudaGetLastError();
+  return dtype == SAKI_BF16 ? launch_pdl(meta_general_kernel<__nv_bfloat16>, grid, MG_THREADS, 0, st, p.from_list != 0, p)
+                            : launch_pdl(meta_general_kernel<float>, grid, MG_THREADS, 0, st, p.from_list != 0, p);
 }
 
 // ---------------------------------------------------------------- streaming kernel (bf16)
@@ -224,6 +225,7 @@ template <int MW>
 __global__ void __launch_bounds__(MW * 32, MW_FULL / MW) meta_stream_kernel(const MetaParams P) {
   constexpr int MOFF_RED = moff_red(MW), MOFF_BC = moff_bc(MW);
   extern __shared__ __align__(128) unsigned char msm[];
+  launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   double* red = (double*)(msm + MOFF_RED);

@@ -278,6 +278,7 @@ __device__ __forceinline__ void for_each_chunk(const Seg& sg, int lane, const ui
 template <bool SPEC>
 __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams P) {
   extern __shared__ __align__(128) unsigned char smem[];
+  launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31;
   const bool spec = SPEC && P.spec != 0;
   const int K1c = SPEC ? P.K1 : 1;             // positions per sequence

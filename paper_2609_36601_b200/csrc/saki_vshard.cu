@@ -19,7 +19,7 @@
 //   stage D  the gradient slice, and on the owning rank the residual draw; the last combine writes the outputs
 // Two families of slice kernels: float64 throughout (one block of 16 warps per row; any dtype, any alignment),
 // and, further down, float32 per element for aligned bf16 slices.
-#include "saki_device.cuh"
+#include "saki_exp2.cuh"
 #include <math_constants.h>
 #include <cmath>
 
@@ -315,7 +315,7 @@ struct VsGroup { VsSlice s[VS_GROUP]; };
 // Every warp adds up the residual weights of its contiguous segment; the warp whose segment holds the target
 // (segments in index order) walks it 32 elements at a time.  float64, whichever kernel family calls.
 template <typename T, int NW>
-__device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double rtau, const double* st, double* red, int* stoken) {
+__device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double rtau, const double* st, double* red, int* stoken, const Exp2& ex2) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const double lam = st[VS_LAM], lse_s = st[VS_LSE_S], lse_t = st[VS_LSE_T], logZ = st[VS_LOGZ];
   const double target = st[VS_TARGET];
@@ -323,9 +323,10 @@ __device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double r
   const int seg = (Vl + NW - 1) / NW, v_lo = min(Vl, warp * seg), v_hi = min(Vl, v_lo + seg);
   auto weight = [&](int v) {
     const double lp = (double)ld_as_float(s, v) * rtau - lse_s, lT = (double)ld_as_float(t, v) * rtau - lse_t;
-    return fmax(exp(lp + lam * (lT - lp) - logZ) - exp(lp), 0.0);
+    return fmax(ex2((lp + lam * (lT - lp) - logZ) * INV_LN2) - ex2(lp * INV_LN2), 0.0);
   };
   double wsum = 0.0;
+#pragma unroll 4
   for (int v = v_lo + lane; v < v_hi; v += 32) wsum += weight(v);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
@@ -379,6 +380,9 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   __shared__ int sarg[VW];
   __shared__ int stoken;
   __shared__ unsigned char marks[VT];
+  __shared__ double tab[EXP2_TAB * EXP2_COPIES];
+  bool table = false;
+  const Exp2 ex2(tab, threadIdx.x & 31);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
@@ -392,6 +396,11 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       marks[tid] = marked ? 1 : 0;
       if (!__syncthreads_or(marked)) continue;
     }
+    if (!table) {
+      exp2_table(tab, tid, VT);
+      __syncthreads();
+      table = true;
+    }
   for (int64_t row = base; row < S.N && row < base + (int64_t)gridDim.x * VT; row += gridDim.x) {
     const T* s = (const T*)S.s + row * S.ld_s;
     const T* t = (const T*)S.t + row * S.ld_t;
@@ -402,6 +411,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       // ---- stage A: maxima and argmax, then the sums under this slice's own shifts
       float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
       int am = 0x7fffffff, finite = 1;
+#pragma unroll 4
       for (int v = tid; v < Vl; v += VT) {
         const float a = ld_as_float(s, v), c = ld_as_float(t, v);
         finite &= (isfinite(a) && isfinite(c)) ? 1 : 0;
@@ -426,9 +436,10 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       double a[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
       if (finite && Vl > 0) {
         const double zms = (double)ms * rtau, zmt = (double)mt * rtau;
-        for (int v = tid; v < Vl; v += VT) {
+  #pragma unroll 4
+      for (int v = tid; v < Vl; v += VT) {
           const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
-          const double es = exp(zs - zms), et = exp(zt - zmt), dl = zt - zs, ed = es * dl, ed2 = ed * dl;
+          const double es = ex2((zs - zms) * INV_LN2), et = ex2((zt - zmt) * INV_LN2), dl = zt - zs, ed = es * dl, ed2 = ed * dl;
           a[0] += es; a[1] += et; a[2] += et * dl; a[3] += ed; a[4] += ed2; a[5] += ed2 * dl; a[6] += ed2 * dl * dl;
         }
       }
@@ -449,9 +460,10 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       if ((int)st[VS_MODE] == VS_SOLVING) {
         const double beta = st[VS_BETA];
         const double kb = ((1.0 - beta) * st[VS_MS] + beta * st[VS_MT]) * rtau;
-        for (int v = tid; v < Vl; v += VT) {
+  #pragma unroll 4
+      for (int v = tid; v < Vl; v += VT) {
           const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
-          const double dl = zt - zs, e = exp(zs + beta * dl - kb), ed = e * dl, ed2 = ed * dl;
+          const double dl = zt - zs, e = ex2((zs + beta * dl - kb) * INV_LN2), ed = e * dl, ed2 = ed * dl;
           a[0] += e; a[1] += ed; a[2] += ed2; a[3] += ed2 * dl; a[4] += ed2 * dl * dl;
         }
       }
@@ -469,10 +481,11 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
         const double lse_s = st[VS_LSE_S], lse_t = st[VS_LSE_T], logZ = st[VS_LOGZ];
         // per-warp segments in index order, summed in warp order: close to the index-order sum of the definition
         const int seg = (Vl + VW - 1) / VW, v_lo = warp * seg, v_hi = min(Vl, v_lo + seg);
+#pragma unroll 4
         for (int v = v_lo + lane; v < v_hi; v += 32) {
           const double lp = (double)ld_as_float(s, v) * rtau - lse_s, lT = (double)ld_as_float(t, v) * rtau - lse_t;
-          const double lq = lp + lam * (lT - lp) - logZ, q = exp(lq);
-          a[0] += fmax(q - exp(lp), 0.0);
+          const double lq = lp + lam * (lT - lp) - logZ, q = ex2(lq * INV_LN2);
+          a[0] += fmax(q - ex2(lp * INV_LN2), 0.0);
           a[1] += q * (lq - lp);
         }
       }
@@ -489,7 +502,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       if (tid == 0) stoken = -1;
       __syncthreads();
       const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
-      if (mine) vs_draw<T, VW>(s, t, Vl, rtau, st, red, &stoken);
+      if (mine) vs_draw<T, VW>(s, t, Vl, rtau, st, red, &stoken, ex2);
       __syncthreads();
       if (tid == 0) {
         for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
@@ -509,15 +522,12 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
         const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
         const double lse_s = st[VS_LSE_S];
         const int tok = mode == VS_FLAGGED ? -1 : (int)st[VS_TOK] - S.v0;
-        for (int v = tid; v < Vl; v += VT) {
+  #pragma unroll 4
+      for (int v = tid; v < Vl; v += VT) {
           double gv = 0.0;
-          if (sc != 0.0) gv = sc * (exp((double)ld_as_float(s, v) * rtau - lse_s) - (v == tok ? 1.0 : 0.0));
+          if (sc != 0.0) gv = sc * (ex2(((double)ld_as_float(s, v) * rtau - lse_s) * INV_LN2) - (v == tok ? 1.0 : 0.0));
           if constexpr (sizeof(T) == 2) {
-            // float64 -> bf16, round to nearest even: through a float rounded to odd (truncate, and keep in the
-            // last bit whether anything was cut off), which the second rounding cannot mistake for a tie
-            float f = __double2float_rz(gv);
-            if ((double)f != gv) f = __uint_as_float(__float_as_uint(f) | 1u);
-            g[v] = __float2bfloat16_rn(f);
+            g[v] = __float2bfloat16_rn(to_odd(gv));
           } else g[v] = (float)gv;
         }
       }
@@ -827,8 +837,7 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
     } else if (STAGE == 1) {
       // ---- stage B: one evaluation at the row's current beta, under the row's shift (its maxima: no factor)
       if ((int)st[VS_MODE] != VS_SOLVING) {        // (block-uniform)
-        if (tid < SAKI_VSHARD_PARTIALS) out[tid] = 0.0;
-        continue;
+        continue;                                  // (its partial is not read)
       }
       const double beta = st[VS_BETA];
       float cb = (float)(c64 * beta);
