@@ -188,10 +188,15 @@ def alloc_outputs(n: int, device):
     return _alloc_out(n, device)
 
 
-def _alloc_out(n: int, device, pinned=False):
+def _alloc_out(n: int, device, pinned=False, packed=True):
     kw = dict(device=device)
     if pinned:
         kw = dict(device="cpu", pin_memory=True)
+    if not packed:
+        out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw)}
+        out.update((f, torch.empty(n, dtype=torch.int32, **kw)) for f in ("token", "teacher_top1", "row_status"))
+        out.update((f, torch.empty(n, dtype=torch.float32, **kw)) for f in _FLOAT_FIELDS)
+        return out
     # one allocation per dtype, a row of it per field: fifteen separate ones took longer than a small call's kernels
     token, top1, status = torch.empty((3, n), dtype=torch.int32, **kw).unbind(0)
     out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw), "token": token, "teacher_top1": top1, "row_status": status}
@@ -459,7 +464,8 @@ def spec_verify(s, t, draft, eps, temperature=1.0, seed=0, seq_offset=0, stream=
     if s.dim() != 3 or t.shape != s.shape or t.dtype != s.dtype or s.stride(2) != 1 or t.stride(2) != 1:
         raise SakiError(1, "logits must be [B,K+1,V] with unit stride along V")
     B, K1, V = s.shape
-    per = _alloc_out(B * K1, s.device)
+    # one tensor per field: `loss` is not written here and keeps whatever its memory held
+    per = _alloc_out(B * K1, s.device, packed=False)
     res = {"n_accept": torch.empty(B, dtype=torch.int32, device=s.device),
            "next_token": torch.empty(B, dtype=torch.int32, device=s.device),
            "next_is_correction": torch.empty(B, dtype=torch.uint8, device=s.device), "per_pos": per}

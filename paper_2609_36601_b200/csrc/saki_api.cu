@@ -189,7 +189,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
   // row per cluster of 8 blocks, than on one SM each: 32 clusters fit at once, and at V = 151936 a call of
   // up to 32 rows takes 32 to 40 us there against 62 us (V = 65536: 28 to 34 against 33 to 39; at V = 32000
   // the row-per-SM kernel is the faster one at every size).
-  if (fast && which == 0 && p.n_rows <= 32 && p.V >= 65536 && eps_ok && cluster_can_serve(p, dtype)) {
+  if (fast && which == 0 && p.call_rows <= 32 && p.V >= 65536 && eps_ok && cluster_can_serve(p, dtype)) {
     e = launch_cluster(p, st, &launches, &served);
     if (e != cudaSuccess) return cuda_fail(e, "cluster kernel launch");
     if (served) used = 2;
@@ -207,7 +207,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
       e = cudaMemsetAsync(p.seq_stop, 0x7f, (size_t)(p.n_rows / p.K1) * sizeof(int), st);   // "no stop yet": above any position
       if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     }
-    e = launch_rowsm(p, st, &launches, &served);
+    e = launch_rowsm(p, which == 0, st, &launches, &served);
     p.seq_next = nullptr; p.seq_stop = nullptr;
     if (e != cudaSuccess) return cuda_fail(e, "row-per-SM kernel launch");
     if (served) used = 3;
@@ -234,7 +234,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
 }
 
 static int route_impl(const saki_in* in, const saki_out* out, void* dlogits, int64_t ld_g, float grad_scale,
-                      bool bwd, void* stream, bool fixed_scratch = false) {
+                      bool bwd, void* stream, bool fixed_scratch = false, int64_t call_rows = 0) {
   g_err[0] = 0;
   if (!in || !out) return fail(SAKI_ERR_INVALID_ARG, "NULL argument struct");
   if (fixed_scratch && in->N > SAKI_NOALLOC_MAX_ROWS)
@@ -259,6 +259,7 @@ static int route_impl(const saki_in* in, const saki_out* out, void* dlogits, int
   p.s = in->student_logits; p.t = in->teacher_logits;
   p.s_seq = in->ld_s; p.s_pos = 0; p.t_seq = in->ld_t; p.t_pos = 0;
   p.n_rows = in->N; p.V = in->V; p.K1 = 1; p.spec = 0;
+  p.call_rows = call_rows > 0 ? call_rows : in->N;
   p.proposal = in->proposal; p.prop_ld = 0; p.mask = in->mask;
   p.eps = in->eps; p.temperature = in->temperature; p.seed = in->seed; p.row_offset = in->row_offset;
   p.out = *out;
@@ -348,13 +349,21 @@ __global__ void spec_resolve_kernel(int64_t B, int K, saki_out o, int32_t* n_acc
   }
 }
 
-// ---- host-buffer entry: staged, double-buffered ----
+// ---- host-buffer entry ----
+// The rows go through the GPU in chunks on HOST_BUFS streams, so that the link carries logits in and gradients out at the
+// same time while a third chunk is being routed.  What a call keeps per position (proposals, mask, outputs) is moved once
+// for all chunks, the outputs through a pinned buffer (a copy per field and chunk costs more than its bytes).
+constexpr int HOST_BUFS = 3;
 struct HostStage {
   std::mutex mu;
   int dev = -1;
-  cudaStream_t st[2] = {nullptr, nullptr};
-  void* buf[2] = {nullptr, nullptr};
-  size_t cap[2] = {0, 0};
+  cudaStream_t st[HOST_BUFS] = {nullptr};
+  cudaEvent_t ev[HOST_BUFS] = {nullptr};
+  void* buf[HOST_BUFS] = {nullptr};
+  size_t cap[HOST_BUFS] = {0};
+  void* pos = nullptr;       // device: per-position arrays of the whole call
+  void* pos_host = nullptr;  // pinned: the outputs among them
+  size_t pos_cap = 0, pos_host_cap = 0;
 };
 static HostStage g_stage;
 
@@ -551,7 +560,7 @@ SAKI_API int saki_spec_verify(const saki_spec_in* in, const saki_spec_out* out, 
   memset(&p, 0, sizeof(p));
   p.s = in->student_logits; p.t = in->teacher_logits;
   p.s_seq = in->ss_seq; p.s_pos = in->ss_pos; p.t_seq = in->ts_seq; p.t_pos = in->ts_pos;
-  p.K1 = in->K + 1; p.n_rows = in->B * p.K1; p.V = in->V; p.spec = 1;
+  p.K1 = in->K + 1; p.n_rows = p.call_rows = in->B * p.K1; p.V = in->V; p.spec = 1;
   p.proposal = in->draft; p.prop_ld = in->draft_ld; p.mask = nullptr;
   p.eps = in->eps; p.temperature = in->temperature; p.seed = in->seed;
   p.row_offset = in->seq_offset * (uint64_t)p.K1;
@@ -623,31 +632,29 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
   cudaGetDevice(&dev);
   cudaError_t e;
   if (g_stage.dev != dev) {   // (re)create the staging streams on this device
-    for (int k = 0; k < 2; ++k) {
+    g_stage.dev = -1;
+    if (g_stage.pos) { cudaFree(g_stage.pos); g_stage.pos = nullptr; g_stage.pos_cap = 0; }
+    for (int k = 0; k < HOST_BUFS; ++k) {
       if (g_stage.buf[k]) { cudaFree(g_stage.buf[k]); g_stage.buf[k] = nullptr; g_stage.cap[k] = 0; }
       if (g_stage.st[k]) { cudaStreamDestroy(g_stage.st[k]); g_stage.st[k] = nullptr; }
+      if (g_stage.ev[k]) { cudaEventDestroy(g_stage.ev[k]); g_stage.ev[k] = nullptr; }
       e = cudaStreamCreateWithFlags(&g_stage.st[k], cudaStreamNonBlocking);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g_stage.ev[k], cudaEventDisableTiming);
       if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
     }
     g_stage.dev = dev;
   }
   const size_t es = in->dtype == SAKI_BF16 ? 2 : 4;
   const size_t Vp = align_up((size_t)in->V, 16);   // padded device row stride: rows stay 16-byte aligned
-  // rows per chunk: about 192 MB of logits per buffer
-  int64_t chunk = (int64_t)std::max<size_t>(1, (size_t)192 << 20) / (int64_t)(2 * Vp * es);
-  chunk = std::max<int64_t>(1, std::min<int64_t>(chunk, in->N));
   const size_t row_bytes = Vp * es;
-  // device layout of one chunk
-  size_t off = 0;
-  auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return o; };
-  const size_t o_s = take(chunk * row_bytes), o_t = take(chunk * row_bytes);
-  const size_t o_g = dlogits ? take(chunk * row_bytes) : 0;
-  const size_t o_prop = take(chunk * 4), o_mask = take(chunk);
-  const size_t o_corr = take(chunk), o_tok = take(chunk * 4), o_top = take(chunk * 4), o_stat = take(chunk * 4);
-  size_t o_f[11];
-  for (int k = 0; k < 11; ++k) o_f[k] = take(chunk * 4);
-  const size_t total = off;
-  for (int k = 0; k < 2; ++k) {
+  const int64_t N = in->N;
+  // Chunks of a twelfth of the call's logits: what is not overlapped is the first chunk's way in and the last one's way
+  // out.  At least 2 MB (a copy of 1 MB takes as long as the calls that issue it), at most 32 MB (nothing is gained
+  // beyond).  512 rows of 32000 (66 MB in, 33 MB out): __HOST__.
+  const int64_t chunk_bytes = std::min<int64_t>(32 << 20, std::max<int64_t>(2 << 20, N * 2 * (int64_t)row_bytes / 12));
+  const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(N, chunk_bytes / (2 * (int64_t)row_bytes)));
+  const size_t total = (size_t)chunk * row_bytes * (dlogits ? 3 : 2);
+  for (int k = 0; k < HOST_BUFS; ++k) {
     if (g_stage.cap[k] < total) {
       if (g_stage.buf[k]) cudaFree(g_stage.buf[k]);
       g_stage.buf[k] = nullptr; g_stage.cap[k] = 0;
@@ -656,58 +663,83 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
       g_stage.cap[k] = total;
     }
   }
-  float* const host_f[11] = {out->lambda, out->kl, out->tv, out->accept_prob, out->logp_x,
-                             out->logq_x, out->logT_x, out->logp_y, out->logq_y, out->logT_y, out->loss};
+  // per-position arrays: the 15 outputs first (copied back as one block), then proposals and mask
+  struct Field { void* host; size_t size, off; };
+  Field f[15] = {{out->token, 4, 0}, {out->teacher_top1, 4, 0}, {out->row_status, 4, 0}, {out->lambda, 4, 0}, {out->kl, 4, 0},
+                 {out->tv, 4, 0}, {out->accept_prob, 4, 0}, {out->logp_x, 4, 0}, {out->logq_x, 4, 0}, {out->logT_x, 4, 0},
+                 {out->logp_y, 4, 0}, {out->logq_y, 4, 0}, {out->logT_y, 4, 0}, {out->loss, 4, 0}, {out->corrected, 1, 0}};
+  size_t off = 0;
+  for (Field& x : f)
+    if (x.host) { x.off = off; off += align_up((size_t)N * x.size, 16); }
+  const size_t out_bytes = off, o_prop = off, o_mask = o_prop + align_up((size_t)N * 4, 16), pos_bytes = o_mask + (size_t)N;
+  if (g_stage.pos_cap < pos_bytes) {
+    if (g_stage.pos) cudaFree(g_stage.pos);
+    g_stage.pos = nullptr; g_stage.pos_cap = 0;
+    e = cudaMalloc(&g_stage.pos, pos_bytes);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc (staging)");
+    g_stage.pos_cap = pos_bytes;
+  }
+  if (g_stage.pos_host_cap < out_bytes) {
+    if (g_stage.pos_host) cudaFreeHost(g_stage.pos_host);
+    g_stage.pos_host = nullptr; g_stage.pos_host_cap = 0;
+    e = cudaMallocHost(&g_stage.pos_host, out_bytes);
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMallocHost (staging)");
+    g_stage.pos_host_cap = out_bytes;
+  }
+  char* const pos = (char*)g_stage.pos;
+  auto field = [&](int q, int64_t r0) -> void* { return f[q].host ? pos + f[q].off + (size_t)r0 * f[q].size : nullptr; };
+  // rows whose strides agree are one piece
+  auto copy_rows = [&](void* dst, size_t dpitch, const void* src, size_t spitch, int64_t n, cudaMemcpyKind kind, cudaStream_t st) {
+    const size_t width = (size_t)in->V * es;
+    if (dpitch == width && spitch == width) return cudaMemcpyAsync(dst, src, width * (size_t)n, kind, st);
+    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, (size_t)n, kind, st);
+  };
   int result = SAKI_OK;
+  e = cudaMemcpyAsync(pos + o_prop, in->proposal, (size_t)N * 4, cudaMemcpyHostToDevice, g_stage.st[0]);
+  if (e == cudaSuccess && in->mask) e = cudaMemcpyAsync(pos + o_mask, in->mask, (size_t)N, cudaMemcpyHostToDevice, g_stage.st[0]);
+  if (e == cudaSuccess) e = cudaEventRecord(g_stage.ev[0], g_stage.st[0]);
+  for (int k = 1; k < HOST_BUFS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(g_stage.st[k], g_stage.ev[0], 0);
+  if (e != cudaSuccess) result = cuda_fail(e, "host-to-device copy");
   int k = 0;
-  for (int64_t r0 = 0; r0 < in->N && result == SAKI_OK; r0 += chunk, k ^= 1) {
-    const int64_t n = std::min<int64_t>(chunk, in->N - r0);
-    char* base = (char*)g_stage.buf[k];
-    cudaStream_t st = g_stage.st[k];
-    const char* hs = (const char*)in->student_logits + (size_t)r0 * in->ld_s * es;
-    const char* ht = (const char*)in->teacher_logits + (size_t)r0 * in->ld_t * es;
-    e = cudaMemcpy2DAsync(base + o_s, row_bytes, hs, in->ld_s * es, in->V * es, n, cudaMemcpyHostToDevice, st);
+  for (int64_t r0 = 0; r0 < N && result == SAKI_OK; r0 += chunk, k = (k + 1) % HOST_BUFS) {
+    const int64_t n = std::min<int64_t>(chunk, N - r0);
+    const bool last = r0 + n == N;
+    char* const b_s = (char*)g_stage.buf[k];
+    char* const b_t = b_s + (size_t)chunk * row_bytes;
+    char* const b_g = b_t + (size_t)chunk * row_bytes;
+    cudaStream_t st = g_stage.st[k];             // (its previous chunk is in front of this one: the buffer is free by then)
+    e = copy_rows(b_s, row_bytes, (const char*)in->student_logits + (size_t)r0 * in->ld_s * es, in->ld_s * es, n, cudaMemcpyHostToDevice, st);
     if (e == cudaSuccess)
-      e = cudaMemcpy2DAsync(base + o_t, row_bytes, ht, in->ld_t * es, in->V * es, n, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = cudaMemcpyAsync(base + o_prop, in->proposal + r0, n * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && in->mask) e = cudaMemcpyAsync(base + o_mask, in->mask + r0, n, cudaMemcpyHostToDevice, st);
+      e = copy_rows(b_t, row_bytes, (const char*)in->teacher_logits + (size_t)r0 * in->ld_t * es, in->ld_t * es, n, cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) { result = cuda_fail(e, "host-to-device copy"); break; }
     saki_in din = *in;
-    din.student_logits = base + o_s; din.teacher_logits = base + o_t; din.ld_s = din.ld_t = (int64_t)Vp;
-    din.N = n; din.proposal = (const int32_t*)(base + o_prop);
-    din.mask = in->mask ? (const uint8_t*)(base + o_mask) : nullptr;
+    din.student_logits = b_s; din.teacher_logits = b_t; din.ld_s = din.ld_t = (int64_t)Vp;
+    din.N = n; din.proposal = (const int32_t*)(pos + o_prop) + r0;
+    din.mask = in->mask ? (const uint8_t*)(pos + o_mask) + r0 : nullptr;
     din.row_offset = in->row_offset + (uint64_t)r0;
     saki_out dout;
-    dout.corrected = (uint8_t*)(base + o_corr); dout.token = (int32_t*)(base + o_tok);
-    dout.teacher_top1 = (int32_t*)(base + o_top); dout.row_status = (uint32_t*)(base + o_stat);
-    float** df[11] = {&dout.lambda, &dout.kl, &dout.tv, &dout.accept_prob, &dout.logp_x,
-                      &dout.logq_x, &dout.logT_x, &dout.logp_y, &dout.logq_y, &dout.logT_y, &dout.loss};
-    for (int q = 0; q < 11; ++q) *df[q] = (float*)(base + o_f[q]);
-    result = route_impl(&din, &dout, dlogits ? base + o_g : nullptr, (int64_t)Vp, grad_scale, dlogits != nullptr, st);
+    dout.token = (int32_t*)field(0, r0); dout.teacher_top1 = (int32_t*)field(1, r0); dout.row_status = (uint32_t*)field(2, r0);
+    float** const df[11] = {&dout.lambda, &dout.kl, &dout.tv, &dout.accept_prob, &dout.logp_x, &dout.logq_x, &dout.logT_x,
+                            &dout.logp_y, &dout.logq_y, &dout.logT_y, &dout.loss};
+    for (int q = 0; q < 11; ++q) *df[q] = (float*)field(3 + q, r0);
+    dout.corrected = (uint8_t*)field(14, r0);
+    result = route_impl(&din, &dout, dlogits ? b_g : nullptr, (int64_t)Vp, grad_scale, dlogits != nullptr, st, false, N);
     if (result != SAKI_OK) break;
-    e = cudaMemcpyAsync(out->corrected + r0, dout.corrected, n, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(out->token + r0, dout.token, n * 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && out->teacher_top1)
-      e = cudaMemcpyAsync(out->teacher_top1 + r0, dout.teacher_top1, n * 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && out->row_status)
-      e = cudaMemcpyAsync(out->row_status + r0, dout.row_status, n * 4, cudaMemcpyDeviceToHost, st);
-    for (int q = 0; q < 11 && e == cudaSuccess; ++q)
-      if (host_f[q]) e = cudaMemcpyAsync(host_f[q] + r0, *df[q], n * 4, cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess && dlogits)
-      e = cudaMemcpy2DAsync((char*)dlogits + (size_t)r0 * ld_g * es, ld_g * es, base + o_g, row_bytes, in->V * es, n,
-                            cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) { result = cuda_fail(e, "device-to-host copy"); break; }
-    // the other buffer is reused two chunks later: its stream must have drained by then
-    if (r0 + chunk < in->N) {
-      e = cudaStreamSynchronize(g_stage.st[k ^ 1]);
-      if (e != cudaSuccess) { result = cuda_fail(e, "cudaStreamSynchronize"); break; }
+    e = cudaEventRecord(g_stage.ev[k], st);
+    if (last) {                                  // every chunk's outputs, in front of the last gradient
+      for (int q = 0; q < HOST_BUFS && e == cudaSuccess; ++q) if (q != k && r0 > 0) e = cudaStreamWaitEvent(st, g_stage.ev[q], 0);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(g_stage.pos_host, pos, out_bytes, cudaMemcpyDeviceToHost, st);
     }
+    if (e == cudaSuccess && dlogits)
+      e = copy_rows((char*)dlogits + (size_t)r0 * ld_g * es, ld_g * es, b_g, row_bytes, n, cudaMemcpyDeviceToHost, st);
+    if (e != cudaSuccess) { result = cuda_fail(e, "device-to-host copy"); break; }
   }
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < HOST_BUFS; ++q) {
     e = cudaStreamSynchronize(g_stage.st[q]);
     if (e != cudaSuccess && result == SAKI_OK) result = cuda_fail(e, "cudaStreamSynchronize");
   }
+  if (result == SAKI_OK)
+    for (const Field& x : f) if (x.host) memcpy(x.host, (const char*)g_stage.pos_host + x.off, (size_t)N * x.size);
   return result;
 }
 

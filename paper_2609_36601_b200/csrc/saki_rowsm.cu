@@ -27,7 +27,21 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
   return true;
 }
 
-cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
+// by_rows: a call that leaves SMs idle takes the variant with the most threads per row that still holds all its rows at
+// once (a row's passes are then a half or a quarter as long).  Measured, forward, us, 1 / 2 / 4 CTAs per SM: V = 49152,
+// 8 rows 28.8 / 30.8 / 37.1, 148 rows 28.8 / 32.5 / 38.9, 296 rows 49.5 / 39.7 / 44.9, 592 rows 86.9 / 71.0 / 67.5;
+// V = 16384, 8 rows 20.6 / 20.6 / 22.9, 296 rows 32.5 / 23.4 / 26.7, 592 rows 53.2 / 38.5 / 32.8; below V = 8192 no
+// difference.  Not where saki_set_kernel pins the kernel: then the variant goes by V alone, and pieces of a batch agree
+// with the whole to the bit.
+cudaError_t launch_rowsm(const RowParams& p, bool by_rows, cudaStream_t st, int* n_launches, bool* served) {
+  if (by_rows && p.V >= 8192) {
+    int dev = 0, sms = 148;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (p.call_rows <= sms) return full_sm::launch(p, st, n_launches, served);
+    if (p.call_rows <= 2 * sms && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);
+    if (p.call_rows <= 4 * sms && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
+  }
   if (p.V <= QUARTER_MAX_V && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
   if (p.V <= HALF_MAX_V && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);
   return full_sm::launch(p, st, n_launches, served);

@@ -6,9 +6,12 @@
 // One block per trajectory.  A position's key is a 64-bit integer that orders like
 // (tier, float64 key value): bit 63 is the tier (0: weighted key, or any key in Random mode; 1: the
 // uniform of a zero-TV position, used by the fill), the rest are the bits of the non-negative double.
-// The m-th smallest key is found by an 8-pass radix select over the keys, which are recomputed in
-// every pass (a Philox call and a logarithm: the whole call touches N scalars, nothing is worth
-// storing); equal keys go to the lower index by an ordered count.
+// The m-th smallest key is found by a radix select, a byte per pass; equal keys go to the lower index by an
+// ordered count.  The call touches N scalars, so what counts is the chain of steps in a block: the keys (a
+// Philox call and a logarithm each) are formed once and kept in shared memory (a trajectory of more than KEEP
+// positions recomputes them in every pass), the bin that holds the m-th key is found by a warp's scan of the
+// histogram, and the passes stop as soon as a bin is chosen as a whole (after three of the eight as a rule).
+// 16 trajectories of 512: __SEL__.
 #include "saki_common.cuh"
 #include <math_constants.h>
 
@@ -46,66 +49,89 @@ __device__ __forceinline__ int block_sum_i(int v, int* sh) {
   return a;
 }
 
+constexpr int KEEP = 4096;     // keys in shared memory (32 KB)
+
 __global__ void __launch_bounds__(ST) select_kernel(const SelectParams P) {
-  __shared__ int hist[256];
+  __shared__ unsigned long long keys[KEEP];
+  __shared__ int hist[256];      // ST == 256 bins
   __shared__ int sh[ST / 32 + 1];
-  __shared__ int pick[2];        // the chosen digit of a pass and the count below it
+  __shared__ int pick[3];        // the chosen bin of a pass, the count below it, the count in it
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int64_t b = blockIdx.x; b < P.B; b += gridDim.x) {
     const int64_t lo = P.seq_start[b], hi = P.seq_start[b + 1];
-    // m = corrected valid positions of the trajectory
+    const bool keep = hi - lo <= KEEP;
+    // the keys, and m = corrected valid positions of the trajectory
     int cnt = 0;
-    for (int64_t i = lo + threadIdx.x; i < hi; i += ST) cnt += (sel_valid(P, i) && P.corrected[i] != 0) ? 1 : 0;
+    for (int64_t i = lo + tid; i < hi; i += ST) {
+      if (keep) {
+        const unsigned long long k = sel_key(P, i);
+        keys[i - lo] = k;
+        cnt += (k != KEY_INVALID && P.corrected[i] != 0) ? 1 : 0;
+      } else cnt += (sel_valid(P, i) && P.corrected[i] != 0) ? 1 : 0;
+    }
+    auto key = [&](int64_t i) { return keep ? keys[i - lo] : sel_key(P, i); };
     const int m = block_sum_i(cnt, sh);
-    if (threadIdx.x == 0 && P.m) P.m[b] = m;
+    if (tid == 0 && P.m) P.m[b] = m;
     if (m == 0) {
-      for (int64_t i = lo + threadIdx.x; i < hi; i += ST) P.selected[i] = 0;
+      for (int64_t i = lo + tid; i < hi; i += ST) P.selected[i] = 0;
       continue;
     }
-    // radix select of the m-th smallest key: after the passes, `prefix` is that key and `below` the
-    // number of keys smaller than it
-    unsigned long long prefix = 0ull;
+    // radix select of the m-th smallest key: after the passes, the keys below `prefix` (`below` of them) are chosen, and
+    // of those that agree with it on `high_mask` the first m - below
+    unsigned long long prefix = 0ull, high_mask = 0ull;
     int below = 0;
-    for (int pass = 0; pass < 8; ++pass) {
-      const int shift = 56 - 8 * pass;
-      const unsigned long long high_mask = pass == 0 ? 0ull : (~0ull << (shift + 8));
-      hist[threadIdx.x] = 0;               // ST == 256 bins
+    for (int shift = 56; shift >= 0; shift -= 8) {
+      hist[tid] = 0;
       __syncthreads();
-      for (int64_t i = lo + threadIdx.x; i < hi; i += ST) {
-        const unsigned long long k = sel_key(P, i);
+      for (int64_t i = lo + tid; i < hi; i += ST) {
+        const unsigned long long k = key(i);
         if ((k & high_mask) == prefix) atomicAdd(&hist[(int)((k >> shift) & 0xffull)], 1);
       }
       __syncthreads();
-      if (threadIdx.x == 0) {
-        int acc = below, dgt = 0;
-        for (; dgt < 255; ++dgt) {
-          if (acc + hist[dgt] >= m) break;
-          acc += hist[dgt];
+      if (warp == 0) {           // eight bins per lane
+        int h[8], sum = 0;
+#pragma unroll
+        for (int q = 0; q < 8; ++q) { h[q] = hist[lane * 8 + q]; sum += h[q]; }
+        int acc = sum;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const int up = __shfl_up_sync(0xffffffffu, acc, o);
+          if (lane >= o) acc += up;
         }
-        pick[0] = dgt; pick[1] = acc;
+        const unsigned reach = __ballot_sync(0xffffffffu, below + acc >= m);      // (the last lane's does)
+        if (lane == __ffs(reach) - 1) {
+          int a = below + acc - sum, q = 0;
+#pragma unroll
+          for (int z = 0; z < 7; ++z) if (q == z && a + h[z] < m) { a += h[z]; ++q; }
+          int in_bin = 0;
+#pragma unroll
+          for (int z = 0; z < 8; ++z) if (q == z) in_bin = h[z];
+          pick[0] = lane * 8 + q; pick[1] = a; pick[2] = in_bin;
+        }
       }
       __syncthreads();
       prefix |= (unsigned long long)pick[0] << shift;
+      high_mask |= 0xffull << shift;
       below = pick[1];
-      __syncthreads();
+      if (below + pick[2] == m) break;       // the whole bin is chosen
     }
-    // keys below the threshold are chosen; of the keys equal to it, the first (m - below) in index order
     int need = m - below;
     for (int64_t base = lo; base < hi; base += ST) {
-      const int64_t i = base + threadIdx.x;
-      const unsigned long long k = i < hi ? sel_key(P, i) : KEY_INVALID;
-      const bool eq = (i < hi) && (k == prefix) && (k != KEY_INVALID);
-      // ordered rank of this thread among the equal keys of the chunk
+      const int64_t i = base + tid;
+      const unsigned long long k = i < hi ? key(i) : KEY_INVALID;
+      const bool eq = (k & high_mask) == prefix && k != KEY_INVALID;
+      // ordered rank of this thread among the chunk's keys of the bin
       const unsigned bal = __ballot_sync(0xffffffffu, eq);
-      const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
       __syncthreads();
       if (lane == 0) sh[warp] = __popc(bal);
       __syncthreads();
       int before = 0, total = 0;
       for (int w = 0; w < ST / 32; ++w) { if (w < warp) before += sh[w]; total += sh[w]; }
       const int rank = before + __popc(bal & ((1u << lane) - 1u));
-      if (i < hi) P.selected[i] = (k < prefix || (eq && rank < need)) ? 1 : 0;
+      if (i < hi) P.selected[i] = ((k & high_mask) < prefix || (eq && rank < need)) ? 1 : 0;
       need = max(0, need - total);
     }
+    __syncthreads();
   }
 }
 
