@@ -350,15 +350,16 @@ __global__ void spec_resolve_kernel(int64_t B, int K, saki_out o, int32_t* n_acc
 }
 
 // ---- host-buffer entry ----
-// The rows go through the GPU in chunks on HOST_BUFS streams, so that the link carries logits in and gradients out at the
-// same time while a third chunk is being routed.  What a call keeps per position (proposals, mask, outputs) is moved once
-// for all chunks, the outputs through a pinned buffer (a copy per field and chunk costs more than its bytes).
+// The rows go through the GPU in chunks: one stream brings logits in, without a gap, one routes, one takes the gradient out
+// while later chunks come in.  What a call keeps per position (proposals, mask, outputs) is moved once for all chunks, the
+// outputs through a pinned buffer (a copy per field and chunk costs more than its bytes).
 constexpr int HOST_BUFS = 3;
+enum { HS_IN = 0, HS_RUN, HS_OUT, HS_STREAMS };
 struct HostStage {
   std::mutex mu;
   int dev = -1;
-  cudaStream_t st[HOST_BUFS] = {nullptr};
-  cudaEvent_t ev[HOST_BUFS] = {nullptr};
+  cudaStream_t st[HS_STREAMS] = {nullptr};
+  cudaEvent_t in[HOST_BUFS] = {nullptr}, run[HOST_BUFS] = {nullptr}, out[HOST_BUFS] = {nullptr};   // chunk is in / routed / out
   void* buf[HOST_BUFS] = {nullptr};
   size_t cap[HOST_BUFS] = {0};
   void* pos = nullptr;       // device: per-position arrays of the whole call
@@ -636,10 +637,15 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
     if (g_stage.pos) { cudaFree(g_stage.pos); g_stage.pos = nullptr; g_stage.pos_cap = 0; }
     for (int k = 0; k < HOST_BUFS; ++k) {
       if (g_stage.buf[k]) { cudaFree(g_stage.buf[k]); g_stage.buf[k] = nullptr; g_stage.cap[k] = 0; }
-      if (g_stage.st[k]) { cudaStreamDestroy(g_stage.st[k]); g_stage.st[k] = nullptr; }
-      if (g_stage.ev[k]) { cudaEventDestroy(g_stage.ev[k]); g_stage.ev[k] = nullptr; }
-      e = cudaStreamCreateWithFlags(&g_stage.st[k], cudaStreamNonBlocking);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g_stage.ev[k], cudaEventDisableTiming);
+      for (cudaEvent_t* ev : {&g_stage.in[k], &g_stage.run[k], &g_stage.out[k]}) {
+        if (*ev) { cudaEventDestroy(*ev); *ev = nullptr; }
+        e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaEventCreate");
+      }
+    }
+    for (cudaStream_t& st : g_stage.st) {
+      if (st) { cudaStreamDestroy(st); st = nullptr; }
+      e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
       if (e != cudaSuccess) return cuda_fail(e, "cudaStreamCreate");
     }
     g_stage.dev = dev;
@@ -648,11 +654,19 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
   const size_t Vp = align_up((size_t)in->V, 16);   // padded device row stride: rows stay 16-byte aligned
   const size_t row_bytes = Vp * es;
   const int64_t N = in->N;
-  // Chunks of a twelfth of the call's logits: what is not overlapped is the first chunk's way in and the last one's way
-  // out.  At least 2 MB (a copy of 1 MB takes as long as the calls that issue it), at most 32 MB (nothing is gained
-  // beyond).  512 rows of 32000 (66 MB in, 33 MB out): __HOST__.
-  const int64_t chunk_bytes = std::min<int64_t>(32 << 20, std::max<int64_t>(2 << 20, N * 2 * (int64_t)row_bytes / 12));
-  const int64_t chunk = std::max<int64_t>(1, std::min<int64_t>(N, chunk_bytes / (2 * (int64_t)row_bytes)));
+  // A chunk is half of what is left, between 4 and 32 MB of logits.  The gradient is half of the logits, so a chunk's way
+  // out takes as long as the next one's way in, and only the last, short chunk is routed and taken out with nothing beside
+  // it.  Copies are few because each costs some 5 us beyond its bytes, more where both directions are busy: 512 rows of
+  // 32000 (66 MB in: 1.21 ms, 33 MB out: 0.60 ms; 1.27 ms both at once in one piece each) took 1.94 ms in one chunk, 1.51
+  // to 1.60 ms in twelve, 1.74 ms in eight, 1.55 ms with the gradient stored into host memory by the kernels.
+  const int64_t pair_bytes = 2 * (int64_t)row_bytes;
+  auto chunk_rows = [&](int64_t left) {
+    const int64_t bytes = std::min<int64_t>(32 << 20, std::max<int64_t>(4 << 20, left * pair_bytes / 2));
+    const int64_t n = std::max<int64_t>(1, bytes / pair_bytes);
+    return left * pair_bytes <= (6 << 20) ? left : std::min(left, n);     // (no crumbs)
+  };
+  int64_t chunk = 0;
+  for (int64_t r0 = 0, n = 0; r0 < N && r0 < 8 * std::max<int64_t>(1, chunk); r0 += n) { n = chunk_rows(N - r0); chunk = std::max(chunk, n); }
   const size_t total = (size_t)chunk * row_bytes * (dlogits ? 3 : 2);
   for (int k = 0; k < HOST_BUFS; ++k) {
     if (g_stage.cap[k] < total) {
@@ -694,24 +708,27 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
     if (dpitch == width && spitch == width) return cudaMemcpyAsync(dst, src, width * (size_t)n, kind, st);
     return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, (size_t)n, kind, st);
   };
+  cudaStream_t const s_in = g_stage.st[HS_IN], s_run = g_stage.st[HS_RUN], s_out = g_stage.st[HS_OUT];
   int result = SAKI_OK;
-  e = cudaMemcpyAsync(pos + o_prop, in->proposal, (size_t)N * 4, cudaMemcpyHostToDevice, g_stage.st[0]);
-  if (e == cudaSuccess && in->mask) e = cudaMemcpyAsync(pos + o_mask, in->mask, (size_t)N, cudaMemcpyHostToDevice, g_stage.st[0]);
-  if (e == cudaSuccess) e = cudaEventRecord(g_stage.ev[0], g_stage.st[0]);
-  for (int k = 1; k < HOST_BUFS && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(g_stage.st[k], g_stage.ev[0], 0);
-  if (e != cudaSuccess) result = cuda_fail(e, "host-to-device copy");
-  int k = 0;
-  for (int64_t r0 = 0; r0 < N && result == SAKI_OK; r0 += chunk, k = (k + 1) % HOST_BUFS) {
-    const int64_t n = std::min<int64_t>(chunk, N - r0);
-    const bool last = r0 + n == N;
+  auto ok = [&](cudaError_t err, const char* what) {
+    if (err != cudaSuccess && result == SAKI_OK) result = cuda_fail(err, what);
+  };
+  ok(cudaMemcpyAsync(pos + o_prop, in->proposal, (size_t)N * 4, cudaMemcpyHostToDevice, s_in), "host-to-device copy");
+  if (in->mask) ok(cudaMemcpyAsync(pos + o_mask, in->mask, (size_t)N, cudaMemcpyHostToDevice, s_in), "host-to-device copy");
+  int64_t i = 0;                                     // chunk number
+  for (int64_t r0 = 0, n = 0; r0 < N && result == SAKI_OK; r0 += n, ++i) {
+    const int k = (int)(i % HOST_BUFS);
+    n = chunk_rows(N - r0);
     char* const b_s = (char*)g_stage.buf[k];
     char* const b_t = b_s + (size_t)chunk * row_bytes;
     char* const b_g = b_t + (size_t)chunk * row_bytes;
-    cudaStream_t st = g_stage.st[k];             // (its previous chunk is in front of this one: the buffer is free by then)
-    e = copy_rows(b_s, row_bytes, (const char*)in->student_logits + (size_t)r0 * in->ld_s * es, in->ld_s * es, n, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess)
-      e = copy_rows(b_t, row_bytes, (const char*)in->teacher_logits + (size_t)r0 * in->ld_t * es, in->ld_t * es, n, cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) { result = cuda_fail(e, "host-to-device copy"); break; }
+    if (i >= HOST_BUFS) ok(cudaStreamWaitEvent(s_in, g_stage.run[k], 0), "cudaStreamWaitEvent");   // the buffer's last rows are routed
+    ok(copy_rows(b_s, row_bytes, (const char*)in->student_logits + (size_t)r0 * in->ld_s * es, in->ld_s * es, n, cudaMemcpyHostToDevice, s_in), "host-to-device copy");
+    ok(copy_rows(b_t, row_bytes, (const char*)in->teacher_logits + (size_t)r0 * in->ld_t * es, in->ld_t * es, n, cudaMemcpyHostToDevice, s_in), "host-to-device copy");
+    ok(cudaEventRecord(g_stage.in[k], s_in), "cudaEventRecord");
+    ok(cudaStreamWaitEvent(s_run, g_stage.in[k], 0), "cudaStreamWaitEvent");
+    if (dlogits && i >= HOST_BUFS) ok(cudaStreamWaitEvent(s_run, g_stage.out[k], 0), "cudaStreamWaitEvent");
+    if (result != SAKI_OK) break;
     saki_in din = *in;
     din.student_logits = b_s; din.teacher_logits = b_t; din.ld_s = din.ld_t = (int64_t)Vp;
     din.N = n; din.proposal = (const int32_t*)(pos + o_prop) + r0;
@@ -723,21 +740,17 @@ SAKI_API int saki_route_host(const saki_in* in, const saki_out* out, void* dlogi
                             &dout.logp_y, &dout.logq_y, &dout.logT_y, &dout.loss};
     for (int q = 0; q < 11; ++q) *df[q] = (float*)field(3 + q, r0);
     dout.corrected = (uint8_t*)field(14, r0);
-    result = route_impl(&din, &dout, dlogits ? b_g : nullptr, (int64_t)Vp, grad_scale, dlogits != nullptr, st, false, N);
+    result = route_impl(&din, &dout, dlogits ? b_g : nullptr, (int64_t)Vp, grad_scale, dlogits != nullptr, s_run, false, N);
     if (result != SAKI_OK) break;
-    e = cudaEventRecord(g_stage.ev[k], st);
-    if (last) {                                  // every chunk's outputs, in front of the last gradient
-      for (int q = 0; q < HOST_BUFS && e == cudaSuccess; ++q) if (q != k && r0 > 0) e = cudaStreamWaitEvent(st, g_stage.ev[q], 0);
-      if (e == cudaSuccess) e = cudaMemcpyAsync(g_stage.pos_host, pos, out_bytes, cudaMemcpyDeviceToHost, st);
+    ok(cudaEventRecord(g_stage.run[k], s_run), "cudaEventRecord");
+    if (dlogits) {
+      ok(cudaStreamWaitEvent(s_out, g_stage.run[k], 0), "cudaStreamWaitEvent");
+      ok(copy_rows((char*)dlogits + (size_t)r0 * ld_g * es, ld_g * es, b_g, row_bytes, n, cudaMemcpyDeviceToHost, s_out), "device-to-host copy");
+      ok(cudaEventRecord(g_stage.out[k], s_out), "cudaEventRecord");
     }
-    if (e == cudaSuccess && dlogits)
-      e = copy_rows((char*)dlogits + (size_t)r0 * ld_g * es, ld_g * es, b_g, row_bytes, n, cudaMemcpyDeviceToHost, st);
-    if (e != cudaSuccess) { result = cuda_fail(e, "device-to-host copy"); break; }
   }
-  for (int q = 0; q < HOST_BUFS; ++q) {
-    e = cudaStreamSynchronize(g_stage.st[q]);
-    if (e != cudaSuccess && result == SAKI_OK) result = cuda_fail(e, "cudaStreamSynchronize");
-  }
+  if (result == SAKI_OK) ok(cudaMemcpyAsync(g_stage.pos_host, pos, out_bytes, cudaMemcpyDeviceToHost, s_run), "device-to-host copy");
+  for (cudaStream_t st : g_stage.st) ok(cudaStreamSynchronize(st), "cudaStreamSynchronize");
   if (result == SAKI_OK)
     for (const Field& x : f) if (x.host) memcpy(x.host, (const char*)g_stage.pos_host + x.off, (size_t)N * x.size);
   return result;
