@@ -331,6 +331,7 @@ static int meta_impl(const saki_meta_in* in, const saki_meta_out* out, void* dlo
 // ---- block verification: per-sequence first-rejection resolve (Section 3.5) ----
 __global__ void spec_resolve_kernel(int64_t B, int K, saki_out o, int32_t* n_accept, int32_t* next_token,
                                     uint8_t* next_is_corr) {
+  launch_dependents();
   wait_for_predecessor();
   const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (b >= B) return;
@@ -572,7 +573,7 @@ SAKI_API int saki_spec_verify(const saki_spec_in* in, const saki_spec_out* out, 
   rc = dispatch_rows(p, in->dtype, st);
   if (rc) return rc;
   const int th = 128;
-  cudaError_t e = launch_pdl(spec_resolve_kernel, (int)((in->B + th - 1) / th), th, 0, st, true, in->B, in->K, p.out,
+  cudaError_t e = launch_pdl(spec_resolve_kernel, dim3((unsigned)((in->B + th - 1) / th)), th, 0, st, true, in->B, in->K, p.out,
                              out->n_accept, out->next_token, out->next_is_correction);
   g_launches += 1;
   if (e != cudaSuccess) return cuda_fail(e, "resolve kernel launch");

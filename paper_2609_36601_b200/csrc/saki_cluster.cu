@@ -130,6 +130,7 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   cg::this_cluster().sync();   // every CTA's barriers exist before any peer signals them
+  wait_for_predecessor();
   if (tid == 0 && cluster_id < P.n_rows) issue(cluster_id);
   uint32_t phase = 0, xph0 = 0, xph1 = 0, mph0 = 0, mph1 = 0;
   int parity = 0, rb = 0;
@@ -530,9 +531,11 @@ static cudaError_t launch_cs(const RowParams& p, cudaStream_t st) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
   cfg.attrs = at; cfg.numAttrs = 1;
   int n_clusters;
@@ -552,6 +555,7 @@ static cudaError_t launch_cs(const RowParams& p, cudaStream_t st) {
   }
   if ((int64_t)n_clusters > p.n_rows) n_clusters = (int)p.n_rows;
   cfg.gridDim = dim3(CS * n_clusters);
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, p, n_clusters);
 }
 

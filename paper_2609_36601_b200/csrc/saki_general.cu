@@ -218,8 +218,10 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   constexpr int NWC = GW * CS;                               // warps of the row, in index order of their segments
   const int gw = crank * GW + warp;
 
-  if (P.from_list) wait_for_predecessor();
-  launch_dependents();
+  if (P.from_list) {
+    wait_for_predecessor();
+    launch_dependents();
+  }
   const int64_t n_work = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
   if ((int64_t)(blockIdx.x / CS) >= n_work) {                // the whole cluster: nothing to do (an empty row list, as a rule)
     if (P.from_list) close_counters(P.redo_count);
@@ -232,6 +234,10 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   }
   __syncthreads();
   const Exp2 ex2(sh.tab, lane);
+  if (!P.from_list) {
+    launch_dependents();
+    wait_for_predecessor();
+  }
 
   const double eps = (double)P.eps;     // (rtau = 1 / tau, c = log2(e) / tau)
   int ph = 0;
@@ -651,7 +657,6 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
   cfg.stream = st;
   cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = p.from_list ? 1 : 0;
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = CS; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   cfg.attrs = at; cfg.numAttrs = CS > 1 ? 2 : 1;
@@ -674,7 +679,7 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
   // and the rows do not divide evenly); in list mode, and for more rows than a grid may have blocks, a fixed stride.
   const bool steal = !p.from_list && p.n_rows > fit && p.n_rows <= (1 << 27);
   const double rtau = 1.0 / (double)p.temperature;
-  at[0].val.programmaticStreamSerializationAllowed = p.from_list ? 1 : 0;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
   if (p.from_list) fit = std::min(fit, std::max(1, sms / CS));     // as a rule they only find the list empty
   cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit || steal ? p.n_rows : fit)), 1, 1);
   return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p, (int)steal, rtau, INV_LN2 * rtau);

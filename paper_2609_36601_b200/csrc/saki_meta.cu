@@ -78,7 +78,7 @@ __device__ __forceinline__ double block_max_d(double v, double* sh) {
 template <typename T>
 __global__ void __launch_bounds__(MG_THREADS) meta_general_kernel(const MetaParams P) {
   __shared__ double sh[MG_THREADS / 32];
-  if (P.from_list) wait_for_predecessor();
+  wait_for_predecessor();
   const int64_t n_items = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
   for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;
@@ -123,8 +123,8 @@ cudaError_t launch_meta_general(const MetaParams& p, int dtype, cudaStream_t st,
   if (p.n_rows <= 0) return cudaSuccess;
   const int grid = (int)std::min<int64_t>(p.n_rows, p.from_list ? 148 : (1 << 20));   // a list is empty as a rule
   ++*n_launches;
-  return dtype == SAKI_BF16 ? launch_pdl(meta_general_kernel<__nv_bfloat16>, grid, MG_THREADS, 0, st, p.from_list != 0, p)
-                            : launch_pdl(meta_general_kernel<float>, grid, MG_THREADS, 0, st, p.from_list != 0, p);
+  return dtype == SAKI_BF16 ? launch_pdl(meta_general_kernel<__nv_bfloat16>, dim3((unsigned)grid), MG_THREADS, 0, st, true, p)
+                            : launch_pdl(meta_general_kernel<float>, dim3((unsigned)grid), MG_THREADS, 0, st, true, p);
 }
 
 // ---------------------------------------------------------------- streaming kernel (bf16)
@@ -226,6 +226,7 @@ __global__ void __launch_bounds__(MW * 32, MW_FULL / MW) meta_stream_kernel(cons
   constexpr int MOFF_RED = moff_red(MW), MOFF_BC = moff_bc(MW);
   extern __shared__ __align__(128) unsigned char msm[];
   launch_dependents();
+  wait_for_predecessor();
   const int tid = threadIdx.x, lane = tid & 31;
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);
   double* red = (double*)(msm + MOFF_RED);
@@ -419,8 +420,7 @@ static cudaError_t launch_meta_stream_as(const MetaParams& p, cudaStream_t st) {
     }
   }
   const int grid = (int)std::min<int64_t>(p.n_rows, (int64_t)cached_sms * (MW_FULL / MW));
-  meta_stream_kernel<MW><<<grid, MW * 32, msmem_bytes(MW), st>>>(p);
-  return cudaGetLastError();
+  return launch_pdl(meta_stream_kernel<MW>, dim3((unsigned)grid), MW * 32, msmem_bytes(MW), st, true, p);
 }
 
 cudaError_t launch_meta_stream(const MetaParams& p, cudaStream_t st, int* n_launches, bool* served) {

@@ -136,6 +136,8 @@ __global__ void __launch_bounds__(PT, 4) propose_kernel(const T* logits, int64_t
                                                         const Keys K, uint64_t seed, uint64_t row_offset, int32_t* out) {
   __shared__ ProposeShared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  launch_dependents();
+  wait_for_predecessor();
   int crank = 0;
   if constexpr (CS > 1) crank = (int)cg::this_cluster().block_rank();
   const int first = crank * PT + tid, step = PT * CS, ngrp = (V + G - 1) / G;
@@ -262,10 +264,12 @@ cudaError_t launch(const void* logits, int64_t ld, int64_t N, int V, float tau, 
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(PT, 1, 1);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = (unsigned)cs; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = cs > 1 ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cs; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = cs > 1 ? 2 : 1;
   cfg.gridDim = dim3((unsigned)((N < (1 << 27) ? N : (1 << 27)) * cs), 1, 1);
   auto go = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, (const T*)logits, ld, N, V, (double)tau, nc, K, seed, row_offset, out); };
   switch (cs) {

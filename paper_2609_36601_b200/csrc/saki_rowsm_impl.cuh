@@ -414,6 +414,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     seqres[0] = n_tickets; seqres[1] = 0; seqres[2] = 0; seqres[3] = 1;
   }
   __syncthreads();
+  wait_for_predecessor();
   const __nv_bfloat16 *n_s = nullptr, *n_t = nullptr;   // the rows of the CTA's next position, if any
   const int64_t first_row = dyn ? ticket_row((int)blockIdx.x) : (int64_t)blockIdx.x;   // grid <= n_rows
   if (first_row < P.n_rows) {
@@ -915,9 +916,8 @@ cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* s
   }
   const int64_t ctas = (int64_t)cached_sms * CTAS_PER_SM;
   const int grid = (int)(p.n_rows < ctas ? p.n_rows : ctas);
-  if (p.spec) rowsm_kernel<true><<<grid, RT, RSMEM_BYTES, st>>>(p);
-  else rowsm_kernel<false><<<grid, RT, RSMEM_BYTES, st>>>(p);
-  cudaError_t e = cudaGetLastError();
+  const cudaError_t e = p.spec ? launch_pdl(rowsm_kernel<true>, dim3((unsigned)grid), RT, RSMEM_BYTES, st, true, p)
+                               : launch_pdl(rowsm_kernel<false>, dim3((unsigned)grid), RT, RSMEM_BYTES, st, true, p);
   if (e == cudaSuccess) { *served = true; if (n_launches) *n_launches += 1; }
   return e;
 }

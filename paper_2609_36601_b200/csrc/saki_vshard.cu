@@ -386,6 +386,8 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
+  launch_dependents();
+  wait_for_predecessor();
   if (only_flagged && stage == 0) return;    // no row is marked for float64 before the first combine
   // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
   // rule none is marked, and a block is done after one load)
@@ -691,6 +693,8 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
 template <int STAGE>
 __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale) {
   const VsSlice& S = Gr.s[blockIdx.y];
+  launch_dependents();
+  wait_for_predecessor();
   if (!S.fast) return;
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
@@ -969,6 +973,8 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
 
 __global__ void vs_combine_kernel(const VsConsts C, const int stage, const double* part, double* state, const saki_out o,
                                   unsigned int* n_solving) {
+  launch_dependents();
+  wait_for_predecessor();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= C.N) return;
   double* st = state + i * SAKI_VSHARD_STATE;
@@ -1011,21 +1017,17 @@ cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, co
     const double gs = (double)grad_scale;
     if (n_fast > 0) {
       const dim3 grid((unsigned)(N < 8LL * sms ? N : 8LL * sms), (unsigned)m, 1);
-      if (stage == 0) vs_fast_kernel<0><<<grid, FT, 0, st>>>(Gr, state, gs);
-      else if (stage == 1) vs_fast_kernel<1><<<grid, FT, 0, st>>>(Gr, state, gs);
-      else if (stage == 2) vs_fast_kernel<2><<<grid, FT, 0, st>>>(Gr, state, gs);
-      else vs_fast_kernel<3><<<grid, FT, 0, st>>>(Gr, state, gs);
+      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, FT, 0, st, true, Gr, state, gs); };
+      cudaError_t e = stage == 0 ? go(vs_fast_kernel<0>) : stage == 1 ? go(vs_fast_kernel<1>) : stage == 2 ? go(vs_fast_kernel<2>) : go(vs_fast_kernel<3>);
       *n_launches += 1;
-      cudaError_t e = cudaGetLastError();
       if (e != cudaSuccess) return e;
     }
     if (n_fast == m && stage == 0) continue;           // no row is marked for float64 before the first combine
     const int64_t blocks = (3LL * sms + m - 1) / m;
     const dim3 grid((unsigned)(N < blocks ? N : blocks), (unsigned)m, 1);
-    if (in[i0].dtype == SAKI_BF16) vs_partial_kernel<__nv_bfloat16><<<grid, VT, 0, st>>>(Gr, stage, state, gs);
-    else vs_partial_kernel<float><<<grid, VT, 0, st>>>(Gr, stage, state, gs);
+    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, VT, 0, st, true, Gr, stage, state, gs); };
+    cudaError_t e = in[i0].dtype == SAKI_BF16 ? go(vs_partial_kernel<__nv_bfloat16>) : go(vs_partial_kernel<float>);
     *n_launches += 1;
-    cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
@@ -1043,8 +1045,7 @@ cudaError_t launch_vshard_combine(const saki_vshard_in& in, int stage, const dou
                                   unsigned int* n_solving, bool allow_fast, cudaStream_t st) {
   const VsConsts c = consts_of(in, allow_fast);
   const int th = 32;           // one thread per row, a chain of float64 scalars: spread over the SMs
-  vs_combine_kernel<<<(unsigned)((in.N + th - 1) / th), th, 0, st>>>(c, stage, gathered, state, out, n_solving);
-  return cudaGetLastError();
+  return launch_pdl(vs_combine_kernel, dim3((unsigned)((in.N + th - 1) / th)), th, 0, st, true, c, stage, gathered, state, out, n_solving);
 }
 
 // the same combine on HOST buffers (a caller without a GPU at hand, and the multi-process tests of the exchange)
