@@ -1,4 +1,5 @@
-"""Thin ctypes binding of the C-ABI library: argument marshalling only.
+"""Thin binding of the C-ABI library: argument marshalling only, by ctypes, and for the entry points of a decoding or
+training step by the compiled module `_saki_torch` (the same work, without the interpreter's share of it).
 
 Every function takes torch tensors (device memory and streams are torch's),
 passes raw pointers, sizes and strides to the library, and returns torch
@@ -14,6 +15,9 @@ import torch
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libsaki.so")
 _lib = None
+_fast = None          # the module _saki_torch, bound to the library
+_BOUND = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc", "saki_route_bwd_from_meta", "saki_select_tm",
+          "saki_spec_verify", "saki_sample_proposal", "saki_vshard_partial_group", "saki_vshard_combine", "saki_last_error")
 
 SAKI_F32, SAKI_BF16 = 0, 1
 ROW_SATURATED, ROW_EPS_ZERO, ROW_MASKED, ROW_NONFINITE, ROW_BAD_ID, ROW_TIMEOUT, ROW_NOT_COMPUTED = 1, 2, 4, 8, 16, 32, 64
@@ -101,7 +105,7 @@ class SakiSpecOut(C.Structure):
 
 def load_library(path: str | None = None):
     """Loads libsaki.so (built in-tree by `python -m paper_2609_36601_b200.build`)."""
-    global _lib
+    global _lib, _fast
     if _lib is not None and path is None:
         return _lib
     p = path or LIB_PATH
@@ -160,8 +164,20 @@ def load_library(path: str | None = None):
               "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_redo_count",
               "saki_version"):
         getattr(lib, f).restype = C.c_int
-    _lib = lib
+    try:
+        from . import _saki_torch
+    except ImportError as e:
+        raise SakiError(-1, f"_saki_torch: {e}: build it with `python -m paper_2609_36601_b200.build`") from e
+    _saki_torch.bind(SakiError, *(C.cast(getattr(lib, f), C.c_void_p).value for f in _BOUND))
+    _lib, _fast = lib, _saki_torch
     return lib
+
+
+def _tensors():
+    """The module _saki_torch, bound to the loaded library."""
+    if _fast is None:
+        load_library()
+    return _fast
 
 
 def _raise(lib, rc):
@@ -183,21 +199,18 @@ def _stream_ptr(stream) -> int:
     return int(stream.cuda_stream)
 
 
+def _handle(stream):
+    """For _saki_torch: None (torch's current stream) or the stream's handle."""
+    return None if stream is None else int(stream.cuda_stream)
+
+
 def alloc_outputs(n: int, device):
     """Preallocated per-position output tensors for the calls that take `out=`."""
-    return _alloc_out(n, device)
+    return _tensors().alloc_outputs(n, device)
 
 
-def _alloc_out(n: int, device, pinned=False, packed=True):
-    kw = dict(device=device)
-    if pinned:
-        kw = dict(device="cpu", pin_memory=True)
-    if not packed:
-        out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw)}
-        out.update((f, torch.empty(n, dtype=torch.int32, **kw)) for f in ("token", "teacher_top1", "row_status"))
-        out.update((f, torch.empty(n, dtype=torch.float32, **kw)) for f in _FLOAT_FIELDS)
-        return out
-    # one allocation per dtype, a row of it per field: fifteen separate ones took longer than a small call's kernels
+def _alloc_pinned(n: int):
+    kw = dict(device="cpu", pin_memory=True)
     token, top1, status = torch.empty((3, n), dtype=torch.int32, **kw).unbind(0)
     out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw), "token": token, "teacher_top1": top1, "row_status": status}
     out.update(zip(_FLOAT_FIELDS, torch.empty((len(_FLOAT_FIELDS), n), dtype=torch.float32, **kw).unbind(0)))
@@ -210,12 +223,6 @@ def _out_struct(out: dict) -> SakiOut:
         t = out.get(name)
         setattr(so, name, t.data_ptr() if t is not None else None)
     return so
-
-
-def _vec_check(v, dtype, n, dev, name):
-    if v.dtype != dtype or v.shape != (n,) or v.device != dev or not v.is_contiguous():
-        raise ValueError(f"{name} must be a contiguous {dtype} tensor of length N on the logits' device")
-    return v
 
 
 def _check_rows(s, t):
@@ -236,63 +243,22 @@ def _in_struct(s, t, proposal, mask, eps, temperature, seed, row_offset) -> Saki
 
 def route_fwd(s, t, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=None, out=None, stream=None):
     """saki_route_fwd on device tensors; returns the dict of per-position output tensors."""
-    lib = load_library()
-    _check_rows(s, t)
-    out = out if out is not None else _alloc_out(s.shape[0], s.device)
-    si, so = _in_struct(s, t, proposal, mask, eps, temperature, seed, row_offset), _out_struct(out)
-    _raise(lib, lib.saki_route_fwd(C.byref(si), C.byref(so), _stream_ptr(stream)))
-    return out
+    return (_fast or _tensors()).route(0, s, t, proposal, eps, temperature, seed, row_offset, mask, 1.0, out, None, _handle(stream))
 
 
 def route_fwd_bwd(s, t, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=None, grad_scale=1.0,
                   out=None, dlogits=None, stream=None):
     """saki_route_fwd_bwd on device tensors; returns (outputs dict, dlogits)."""
-    lib = load_library()
-    _check_rows(s, t)
-    out = out if out is not None else _alloc_out(s.shape[0], s.device)
-    if dlogits is None:
-        dlogits = torch.empty_like(s)
-    ld_g = dlogits.stride(0) if dlogits.shape[0] > 1 else dlogits.shape[1]
-    si, so = _in_struct(s, t, proposal, mask, eps, temperature, seed, row_offset), _out_struct(out)
-    _raise(lib, lib.saki_route_fwd_bwd(C.byref(si), C.byref(so), dlogits.data_ptr(), ld_g, grad_scale,
-                                       _stream_ptr(stream)))
-    return out, dlogits
+    return (_fast or _tensors()).route(1, s, t, proposal, eps, temperature, seed, row_offset, mask, grad_scale, out, dlogits,
+                                       _handle(stream))
 
 
 def route_bwd_from_meta(s, corrected, proposal, teacher_top1, advantage, temperature=1.0, mask=None,
                         rollout_status=None, grad_scale=1.0, dlogits=None, stream=None):
     """saki_route_bwd_from_meta on device tensors: loss and gradient of the routed objective for the
     current student logits `s`, from the rollout's metadata.  Returns (outputs dict, dlogits)."""
-    lib = load_library()
-    if s.dim() != 2 or s.stride(1) != 1:
-        raise ValueError("logits must be [N,V] with unit stride along V")
-    n, dev = s.shape[0], s.device
-    if dlogits is None:
-        dlogits = torch.empty_like(s)
-    ld_g = dlogits.stride(0) if dlogits.shape[0] > 1 else dlogits.shape[1]
-    out = {"loss": torch.empty(n, dtype=torch.float32, device=dev),
-           "logp_tok": torch.empty(n, dtype=torch.float32, device=dev),
-           "row_status": torch.empty(n, dtype=torch.int32, device=dev)}
-    keep = [_vec_check(corrected, torch.uint8, n, dev, "corrected"),
-            _vec_check(proposal, torch.int32, n, dev, "proposal"),
-            _vec_check(teacher_top1, torch.int32, n, dev, "teacher_top1"),
-            _vec_check(advantage, torch.float32, n, dev, "advantage")]
-    mi = SakiMetaIn()
-    mi.student_logits = s.data_ptr()
-    mi.ld_s = s.stride(0) if n > 1 else s.shape[1]
-    mi.N, mi.V, mi.dtype = n, s.shape[1], _dtype_code(s)
-    mi.corrected, mi.proposal, mi.teacher_top1, mi.advantage = (t.data_ptr() for t in keep)
-    if mask is not None:
-        keep.append(_vec_check(mask, torch.uint8, n, dev, "mask"))
-        mi.mask = keep[-1].data_ptr()
-    if rollout_status is not None:
-        keep.append(_vec_check(rollout_status, torch.int32, n, dev, "rollout_status"))
-        mi.rollout_status = keep[-1].data_ptr()
-    mi.temperature = temperature
-    mo = SakiMetaOut(out["loss"].data_ptr(), out["logp_tok"].data_ptr(), out["row_status"].data_ptr())
-    _raise(lib, lib.saki_route_bwd_from_meta(C.byref(mi), C.byref(mo), dlogits.data_ptr(), ld_g, grad_scale,
-                                             _stream_ptr(stream)))
-    return out, dlogits
+    return (_fast or _tensors()).meta(s, corrected, proposal, teacher_top1, advantage, temperature, mask, rollout_status, grad_scale,
+                                      dlogits, _handle(stream))
 
 
 SELECT_RANDOM, SELECT_TV_WEIGHTED = 0, 1
@@ -301,28 +267,7 @@ SELECT_RANDOM, SELECT_TV_WEIGHTED = 0, 1
 def select_tm(seq_start, corrected, tv, mode, seed=0, row_offset=0, mask=None, rollout_status=None, stream=None):
     """saki_select_tm on device tensors: the placement controls (Random-TM, TV-Weighted-TM).  `seq_start`
     is the int64 [B+1] tensor of trajectory boundaries.  Returns (selected uint8 [N], m int32 [B])."""
-    lib = load_library()
-    dev = corrected.device
-    n, nb = corrected.shape[0], seq_start.shape[0] - 1
-    if seq_start.dtype != torch.int64 or seq_start.device != dev or not seq_start.is_contiguous():
-        raise ValueError("seq_start must be a contiguous int64 tensor on the same device")
-    keep = [_vec_check(corrected, torch.uint8, n, dev, "corrected")]
-    si = SakiSelectIn()
-    si.N, si.B, si.seq_start, si.corrected = n, nb, seq_start.data_ptr(), corrected.data_ptr()
-    if tv is not None:
-        keep.append(_vec_check(tv, torch.float32, n, dev, "tv"))
-        si.tv = tv.data_ptr()
-    if mask is not None:
-        keep.append(_vec_check(mask, torch.uint8, n, dev, "mask"))
-        si.mask = mask.data_ptr()
-    if rollout_status is not None:
-        keep.append(_vec_check(rollout_status, torch.int32, n, dev, "rollout_status"))
-        si.rollout_status = rollout_status.data_ptr()
-    si.mode, si.seed, si.row_offset = mode, seed, row_offset
-    selected = torch.empty(n, dtype=torch.uint8, device=dev)
-    m = torch.empty(max(nb, 0), dtype=torch.int32, device=dev)
-    _raise(lib, lib.saki_select_tm(C.byref(si), selected.data_ptr(), m.data_ptr(), _stream_ptr(stream)))
-    return selected, m
+    return (_fast or _tensors()).select(seq_start, corrected, tv, mode, seed, row_offset, mask, rollout_status, _handle(stream))
 
 
 def route_fwd_bwd_noalloc(s, t, proposal, eps, out, dlogits, temperature=1.0, seed=0, row_offset=0, mask=None,
@@ -330,13 +275,8 @@ def route_fwd_bwd_noalloc(s, t, proposal, eps, out, dlogits, temperature=1.0, se
     """saki_route_fwd_bwd_noalloc: the variant for callers that cannot allocate device memory.  The caller
     passes every buffer (`out`: dict of preallocated output tensors, `dlogits`); the library's own scratch
     is a fixed device array, so nothing is allocated on the way (at most 1,048,576 rows per call)."""
-    lib = load_library()
-    _check_rows(s, t)
-    ld_g = dlogits.stride(0) if dlogits.shape[0] > 1 else dlogits.shape[1]
-    si, so = _in_struct(s, t, proposal, mask, eps, temperature, seed, row_offset), _out_struct(out)
-    _raise(lib, lib.saki_route_fwd_bwd_noalloc(C.byref(si), C.byref(so), dlogits.data_ptr(), ld_g, grad_scale,
-                                               _stream_ptr(stream)))
-    return out, dlogits
+    return (_fast or _tensors()).route(2, s, t, proposal, eps, temperature, seed, row_offset, mask, grad_scale, out, dlogits,
+                                       _handle(stream))
 
 
 def vshard_in(s_loc, t_loc, v0, V, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=None, rank=0, world=1,
@@ -369,28 +309,6 @@ def vshard_partial(si: SakiVshardIn, stage: int, state, partial, dlogits=None, g
     _raise(lib, lib.saki_vshard_partial(C.byref(si), stage, state.data_ptr() if state is not None else None,
                                         partial.data_ptr(), dlogits.data_ptr() if dlogits is not None else None, ld_g,
                                         grad_scale, _stream_ptr(stream)))
-
-
-class VshardGroup:
-    """The slices of several ranks on one device as one argument list of saki_vshard_partial_group: `sis` their argument
-    records, `partials` and `dlogits` (or None) one tensor per slice."""
-
-    def __init__(self, sis, partials, dlogits=None):
-        n = len(sis)
-        self.n, self.sis = n, (SakiVshardIn * n)(*sis)
-        self.partials = (C.c_void_p * n)(*(p.data_ptr() for p in partials))
-        self.dlogits = self.ld_g = None
-        if dlogits is not None:
-            self.dlogits = (C.c_void_p * n)(*(g.data_ptr() for g in dlogits))
-            self.ld_g = (C.c_int64 * n)(*(g.stride(0) if g.shape[0] > 1 else max(1, g.shape[1]) for g in dlogits))
-
-    def partial(self, stage: int, state, with_grad=False, grad_scale=1.0, stream=None):
-        """saki_vshard_partial_group: every slice's partial vectors of one stage (and its gradient slice)."""
-        lib = load_library()
-        grad = with_grad and self.dlogits is not None
-        _raise(lib, lib.saki_vshard_partial_group(self.sis, self.n, stage, state.data_ptr() if state is not None else None,
-                                                  self.partials, self.dlogits if grad else None, self.ld_g if grad else None,
-                                                  grad_scale, _stream_ptr(stream)))
 
 
 def vshard_combine(si: SakiVshardIn, stage: int, gathered, state, out=None, n_solving=None, stream=None):
@@ -448,7 +366,7 @@ def route_host(s, t, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=
     _check_rows(s, t)
     if s.is_cuda:
         raise SakiError(1, "route_host takes host tensors")
-    out = out if out is not None else _alloc_out(s.shape[0], "cpu", pinned=True)
+    out = out if out is not None else _alloc_pinned(s.shape[0])
     if backward and dlogits is None:
         dlogits = torch.empty(s.shape, dtype=s.dtype, pin_memory=True)
     ld_g = (dlogits.stride(0) if dlogits.shape[0] > 1 else dlogits.shape[1]) if backward else 0
@@ -460,37 +378,12 @@ def route_host(s, t, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=
 
 def spec_verify(s, t, draft, eps, temperature=1.0, seed=0, seq_offset=0, stream=None):
     """saki_spec_verify on device tensors s, t: [B,K+1,V], draft: [B,K] int32."""
-    lib = load_library()
-    if s.dim() != 3 or t.shape != s.shape or t.dtype != s.dtype or s.stride(2) != 1 or t.stride(2) != 1:
-        raise SakiError(1, "logits must be [B,K+1,V] with unit stride along V")
-    B, K1, V = s.shape
-    # one tensor per field: `loss` is not written here and keeps whatever its memory held
-    per = _alloc_out(B * K1, s.device, packed=False)
-    res = {"n_accept": torch.empty(B, dtype=torch.int32, device=s.device),
-           "next_token": torch.empty(B, dtype=torch.int32, device=s.device),
-           "next_is_correction": torch.empty(B, dtype=torch.uint8, device=s.device), "per_pos": per}
-    si = SakiSpecIn()
-    si.student_logits, si.teacher_logits = s.data_ptr(), t.data_ptr()
-    si.ss_seq, si.ss_pos, si.ts_seq, si.ts_pos = s.stride(0), s.stride(1), t.stride(0), t.stride(1)
-    si.B, si.K, si.V, si.dtype = B, K1 - 1, V, _dtype_code(s)
-    si.draft, si.draft_ld = draft.data_ptr(), (draft.stride(0) if B > 1 else draft.shape[1])
-    si.eps, si.temperature, si.seed, si.seq_offset = eps, temperature, seed, seq_offset
-    so = SakiSpecOut()
-    so.n_accept, so.next_token, so.next_is_correction = (res["n_accept"].data_ptr(), res["next_token"].data_ptr(),
-                                                        res["next_is_correction"].data_ptr())
-    so.per_pos = _out_struct(per)
-    _raise(lib, lib.saki_spec_verify(C.byref(si), C.byref(so), _stream_ptr(stream)))
-    return res
+    return (_fast or _tensors()).spec(s, t, draft, eps, temperature, seed, seq_offset, _handle(stream))
 
 
 def sample_proposal(s, temperature=1.0, seed=0, row_offset=0, stream=None):
     """saki_sample_proposal: x_i ~ softmax(s_i / temperature) by Philox-keyed Gumbel-max."""
-    lib = load_library()
-    out = torch.empty(s.shape[0], dtype=torch.int32, device=s.device)
-    ld = s.stride(0) if s.shape[0] > 1 else s.shape[1]
-    _raise(lib, lib.saki_sample_proposal(s.data_ptr(), ld, s.shape[0], s.shape[1], _dtype_code(s), temperature,
-                                         seed, row_offset, out.data_ptr(), _stream_ptr(stream)))
-    return out
+    return (_fast or _tensors()).propose(s, temperature, seed, row_offset, _handle(stream))
 
 
 def check(stream=None) -> int:

@@ -1,4 +1,5 @@
-"""Builds the C-ABI CUDA library (libsaki.so) in-tree with nvcc for sm_100a.
+"""Builds the C-ABI CUDA library (libsaki.so) in-tree with nvcc for sm_100a, and the tensor side of the Python
+binding (_saki_torch.so) with the host compiler.
 
     python -m paper_2609_36601_b200.build [--verbose]
 """
@@ -11,6 +12,8 @@ import sys
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsaki.so")
+TORCH_SOURCE = os.path.join(CSRC, "saki_torch.cpp")
+TORCH_LIB = os.path.join(HERE, "_saki_torch.so")
 SOURCES = ("saki_api.cu", "saki_general.cu", "saki_cluster.cu", "saki_rowsm.cu", "saki_rowsm_half.cu", "saki_rowsm_quarter.cu", "saki_meta.cu",
            "saki_select.cu", "saki_propose.cu", "saki_vshard.cu", "saki_lmhead.cu")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -24,22 +27,41 @@ def _nvcc():
     raise RuntimeError("nvcc not found")
 
 
+def _host_command():
+    """The compiler call for the tensor side of the binding, against the installed torch."""
+    import sysconfig
+    import torch
+    from torch.utils import cpp_extension
+    inc = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
+    libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
+            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(a for d in inc for a in ("-isystem", d)),
+            TORCH_SOURCE, "-o", TORCH_LIB, f"-L{libdir}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+
+
+def _host_needs_build() -> bool:
+    deps = (TORCH_SOURCE, os.path.join(HERE, "..", "include", "saki.h"), os.path.abspath(__file__))
+    return not os.path.exists(TORCH_LIB) or any(os.path.getmtime(d) > os.path.getmtime(TORCH_LIB) for d in deps)
+
+
 def needs_build() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)] + [
+    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cu", ".cuh"))] + [
         os.path.join(HERE, "..", "include", "saki.h"), os.path.abspath(__file__)]
     return any(os.path.getmtime(d) > t for d in deps)
 
 
 def build(verbose: bool = False, force: bool = False) -> str:
-    if not force and not needs_build():
-        return LIB
     objs = []
     procs = []
+    host = force or _host_needs_build()
+    if host:
+        procs.append((TORCH_SOURCE, subprocess.Popen(_host_command(), stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)))
+    library = force or needs_build()
     flags = list(FLAGS)
-    for src in SOURCES:
+    for src in SOURCES if library else ():
         obj = os.path.join(CSRC, src.replace(".cu", ".o"))
         cmd = [_nvcc(), *flags, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
@@ -52,6 +74,8 @@ def build(verbose: bool = False, force: bool = False) -> str:
             sys.stderr.write(out)
         if p.returncode:
             raise RuntimeError(f"nvcc failed on {src}")
+    if not library:
+        return LIB
     cmd = [_nvcc(), "-shared", "-o", LIB, *objs, "-gencode", "arch=compute_100a,code=sm_100a"]
     r = subprocess.run(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
     if r.returncode:

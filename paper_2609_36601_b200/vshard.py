@@ -82,22 +82,8 @@ def route_vocab_sharded_local(slices, V: int, proposal, eps, temperature=1.0, se
     """All ranks in one process: `slices` = [(s_loc, t_loc, v0)] in rank order on one device.  Returns (out,
     [dlogits_slice per rank], waves): the stages every rank would run, the slices of all ranks in one launch per stage.
     `state_out`: a list that receives the per-row state tensor (for tests)."""
-    world = len(slices)
-    dev, N = slices[0][0].device, slices[0][0].shape[0]
-    sis = [B.vshard_in(s, t, v0, V, proposal, eps, temperature, seed, row_offset, mask, r, world)
-           for r, (s, t, v0) in enumerate(slices)]
-    state = torch.empty((N, B.VSHARD_STATE), dtype=torch.float64, device=dev)
-    gathered = torch.empty((world, N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
-    out = B.alloc_outputs(N, dev)
-    gs = [torch.empty_like(s) if backward else None for s, _, _ in slices]
-    # rank r's partial lands where the all-gather would put it
-    group = B.VshardGroup(sis, gathered.unbind(0), gs if backward else None)
-
-    def wave(stage, n_solving=None):
-        group.partial(stage, state if stage > 0 else None, stage == 2, grad_scale, stream)
-        B.vshard_combine(sis[0], stage, gathered, state, out if stage == 3 else None, n_solving, stream)
-
-    waves = _stages(wave, dev, EAGER_WAVES + 1)
+    out, gs, waves, state = B._tensors().vshard_local(slices, V, proposal, eps, temperature, seed, row_offset, mask, grad_scale,
+                                                      backward, B._handle(stream), EAGER_WAVES + 1, MAX_WAVES)
     if state_out is not None:
         state_out.append(state)
     return out, gs, waves
