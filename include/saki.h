@@ -277,12 +277,16 @@ typedef struct {
 } saki_vshard_in;
 SAKI_API int saki_vshard_partial(const saki_vshard_in* in, int stage, const double* state, double* partial,
                                  void* dlogits_slice, int64_t ld_g, float grad_scale, void* cuda_stream);
-/* The same for the n slices a process holds (several ranks' slices on one device; same rows, dtype and arguments but
- * for the slice): `in`, `partial`, `dlogits_slice` (may be NULL) and `ld_g` are HOST arrays of n entries.  One kernel
- * launch per stage and 16 slices instead of one per slice. */
-SAKI_API int saki_vshard_partial_group(const saki_vshard_in* in, int n, int stage, const double* state,
-                                       double* const* partial, void* const* dlogits_slice, const int64_t* ld_g,
-                                       float grad_scale, void* cuda_stream);
+/* One whole stage for a process that holds all ranks' slices on one device (n of them, in rank order; same rows, dtype and
+ * arguments but for the slice): the partials of every slice, in one launch per 16 slices, then the combine.  `in`,
+ * `partial`, `dlogits_slice` (may be NULL) and `ld_g` are HOST arrays of n entries; the partial pointers tile `gathered`.
+ * `counts` (device, two words, may be NULL): the number of rows that need another wave is ADDED to counts[0], the number
+ * of rows this stage marked for the float64 kernels to counts[1].  `flags`: 0, or SAKI_VSHARD_NONE_MARKED, the caller's
+ * word (from what it read there) that no row has been marked so far: the float64 kernels are then not launched for them. */
+#define SAKI_VSHARD_NONE_MARKED 1
+SAKI_API int saki_vshard_stage(const saki_vshard_in* in, int n, int stage, double* state, double* const* partial,
+                               const double* gathered, void* const* dlogits_slice, const int64_t* ld_g, float grad_scale,
+                               const saki_out* out, uint32_t* counts, int flags, void* cuda_stream);
 SAKI_API int saki_vshard_combine(const saki_vshard_in* in, int stage, const double* gathered, double* state,
                                  const saki_out* out, uint32_t* n_solving, void* cuda_stream);
 SAKI_API int saki_vshard_combine_host(const saki_vshard_in* in, int stage, const double* gathered, double* state,

@@ -17,7 +17,7 @@ LIB_PATH = os.path.join(_HERE, "libsaki.so")
 _lib = None
 _fast = None          # the module _saki_torch, bound to the library
 _BOUND = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc", "saki_route_bwd_from_meta", "saki_select_tm",
-          "saki_spec_verify", "saki_sample_proposal", "saki_vshard_partial_group", "saki_vshard_combine", "saki_last_error")
+          "saki_spec_verify", "saki_sample_proposal", "saki_vshard_stage", "saki_last_error")
 
 SAKI_F32, SAKI_BF16 = 0, 1
 ROW_SATURATED, ROW_EPS_ZERO, ROW_MASKED, ROW_NONFINITE, ROW_BAD_ID, ROW_TIMEOUT, ROW_NOT_COMPUTED = 1, 2, 4, 8, 16, 32, 64
@@ -25,7 +25,7 @@ ROW_SATURATED, ROW_EPS_ZERO, ROW_MASKED, ROW_NONFINITE, ROW_BAD_ID, ROW_TIMEOUT,
 _FLOAT_FIELDS = ("lambda", "kl", "tv", "accept_prob", "logp_x", "logq_x", "logT_x", "logp_y", "logq_y", "logT_y", "loss")
 EXPORTS = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc", "saki_route_host",
            "saki_route_bwd_from_meta", "saki_select_tm", "saki_spec_verify",
-           "saki_vshard_partial", "saki_vshard_partial_group", "saki_vshard_combine", "saki_vshard_combine_host",
+           "saki_vshard_partial", "saki_vshard_stage", "saki_vshard_combine", "saki_vshard_combine_host",
            "saki_lmhead_scratch_bytes", "saki_lmhead_lse",
            "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_redo_count",
            "saki_set_spec_early_out", "saki_spec_positions_routed", "saki_solve_evaluations", "saki_set_wait_limit", "saki_set_phase_clock", "saki_phase_cycles",
@@ -138,9 +138,6 @@ def load_library(path: str | None = None):
     lib.saki_vshard_partial.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_int64,
                                         C.c_float, C.c_void_p]
     lib.saki_vshard_partial.restype = C.c_int
-    lib.saki_vshard_partial_group.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_int, C.c_void_p, C.POINTER(C.c_void_p),
-                                              C.POINTER(C.c_void_p), C.POINTER(C.c_int64), C.c_float, C.c_void_p]
-    lib.saki_vshard_partial_group.restype = C.c_int
     lib.saki_vshard_combine.argtypes = [C.POINTER(SakiVshardIn), C.c_int, C.c_void_p, C.c_void_p, C.POINTER(SakiOut),
                                         C.c_void_p, C.c_void_p]
     lib.saki_vshard_combine.restype = C.c_int

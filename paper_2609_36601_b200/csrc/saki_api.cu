@@ -436,7 +436,7 @@ static int vshard_check(const saki_vshard_in* in, int stage) {
 }
 
 static int vshard_partials(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
-                           void* const* dlogits, const int64_t* ld_g, float grad_scale, void* cuda_stream) {
+                           void* const* dlogits, const int64_t* ld_g, float grad_scale, int flags, void* cuda_stream) {
   g_err[0] = 0;
   if (n < 0) return fail(SAKI_ERR_INVALID_ARG, "negative number of slices");
   if (n > 0 && (!in || !partial || (dlogits && !ld_g))) return fail(SAKI_ERR_INVALID_ARG, "NULL argument array");
@@ -456,7 +456,7 @@ static int vshard_partials(const saki_vshard_in* in, int n, int stage, const dou
   int rc = device_ready(&flagged);
   if (rc) return rc;
   int launches = 0;
-  cudaError_t e = launch_vshard_partial(in, n, stage, state, partial, dlogits, ld_g, grad_scale, g_kernel.load() != 1, &launches,
+  cudaError_t e = launch_vshard_partial(in, n, stage, state, partial, dlogits, ld_g, grad_scale, g_kernel.load() != 1, flags, &launches,
                                         (cudaStream_t)cuda_stream);
   if (e != cudaSuccess) return cuda_fail(e, "vocabulary-sharded partial kernel launch");
   g_launches += (uint64_t)launches;
@@ -465,12 +465,23 @@ static int vshard_partials(const saki_vshard_in* in, int n, int stage, const dou
 
 SAKI_API int saki_vshard_partial(const saki_vshard_in* in, int stage, const double* state, double* partial,
                                  void* dlogits_slice, int64_t ld_g, float grad_scale, void* cuda_stream) {
-  return vshard_partials(in, 1, stage, state, &partial, dlogits_slice ? &dlogits_slice : nullptr, &ld_g, grad_scale, cuda_stream);
+  return vshard_partials(in, 1, stage, state, &partial, dlogits_slice ? &dlogits_slice : nullptr, &ld_g, grad_scale, 0, cuda_stream);
 }
 
-SAKI_API int saki_vshard_partial_group(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
-                                       void* const* dlogits_slice, const int64_t* ld_g, float grad_scale, void* cuda_stream) {
-  return vshard_partials(in, n, stage, state, partial, dlogits_slice, ld_g, grad_scale, cuda_stream);
+SAKI_API int saki_vshard_stage(const saki_vshard_in* in, int n, int stage, double* state, double* const* partial,
+                               const double* gathered, void* const* dlogits_slice, const int64_t* ld_g, float grad_scale,
+                               const saki_out* out, uint32_t* counts, int flags, void* cuda_stream) {
+  const int rc = vshard_partials(in, n, stage, state, partial, dlogits_slice, ld_g, grad_scale, flags, cuda_stream);
+  if (rc || n == 0 || in[0].N == 0) return rc;
+  if (!gathered || !state) return fail(SAKI_ERR_INVALID_ARG, "NULL gathered or state pointer");
+  if (stage == 3 && (!out || !out->corrected || !out->token)) return fail(SAKI_ERR_INVALID_ARG, "out.corrected and out.token are required at stage 3");
+  saki_out none;
+  memset(&none, 0, sizeof(none));
+  cudaError_t e = launch_vshard_combine(in[0], stage, gathered, state, out ? *out : none, counts, counts ? counts + 1 : nullptr,
+                                        g_kernel.load() != 1, (cudaStream_t)cuda_stream);
+  if (e != cudaSuccess) return cuda_fail(e, "vocabulary-sharded combine kernel launch");
+  g_launches += 1;
+  return SAKI_OK;
 }
 
 SAKI_API int saki_vshard_combine(const saki_vshard_in* in, int stage, const double* gathered, double* state,
@@ -491,7 +502,7 @@ SAKI_API int saki_vshard_combine(const saki_vshard_in* in, int stage, const doub
   }
   saki_out none;
   memset(&none, 0, sizeof(none));
-  cudaError_t e = launch_vshard_combine(*in, stage, gathered, state, out ? *out : none, n_solving, g_kernel.load() != 1, st);
+  cudaError_t e = launch_vshard_combine(*in, stage, gathered, state, out ? *out : none, n_solving, nullptr, g_kernel.load() != 1, st);
   if (e != cudaSuccess) return cuda_fail(e, "vocabulary-sharded combine kernel launch");
   g_launches += 1;
   return SAKI_OK;

@@ -70,7 +70,14 @@ static_assert(CNT_LIVE <= CNT_LAST, "the counters of a call and of the last one 
 // here, before it touches memory, until everything in front of it has finished.
 __device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_for_predecessor() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-// Called by every block of the list-mode kernel, all threads, when it is done.
+__device__ __forceinline__ void move_counters(unsigned int* c) {
+  for (int i = threadIdx.x; i < CNT_LIVE; i += blockDim.x) {
+    c[CNT_LAST + i] = *(volatile unsigned int*)(c + i);
+    c[i] = 0u;
+  }
+}
+// Called by every block of the list-mode kernel, all threads, when it is done.  (Not where the list is empty: then one
+// block moves the counters without asking whether the others are done, which read nothing but the list's length.)
 __device__ __forceinline__ void close_counters(unsigned int* c) {
   __shared__ bool last;
   __syncthreads();
@@ -79,12 +86,7 @@ __device__ __forceinline__ void close_counters(unsigned int* c) {
     last = atomicAdd(c + CNT_DONE, 1u) == gridDim.x - 1;
   }
   __syncthreads();
-  if (last) {
-    for (int i = threadIdx.x; i < CNT_LIVE; i += blockDim.x) {
-      c[CNT_LAST + i] = *(volatile unsigned int*)(c + i);
-      c[i] = 0u;
-    }
-  }
+  if (last) move_counters(c);
 }
 // A launch that may (pdl) be set up while the kernel in front of it runs: every kernel of this library waits for its
 // predecessor before it touches memory, so that the launches of a call, and of calls that follow one another, do not leave
@@ -226,10 +228,10 @@ cudaError_t launch_propose(const void* logits, int64_t ld, int64_t N, int V, int
                            uint64_t row_offset, int32_t* out, cudaStream_t st);
 cudaError_t launch_select(const SelectParams& p, cudaStream_t st, int* n_launches);
 cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, const double* state, double* const* partial,
-                                  void* const* dlogits, const int64_t* ld_g, float grad_scale, bool allow_fast, int* n_launches,
-                                  cudaStream_t st);
+                                  void* const* dlogits, const int64_t* ld_g, float grad_scale, bool allow_fast, int flags,
+                                  int* n_launches, cudaStream_t st);
 cudaError_t launch_vshard_combine(const saki_vshard_in& in, int stage, const double* gathered, double* state, const saki_out& out,
-                                  unsigned int* n_solving, bool allow_fast, cudaStream_t st);
+                                  unsigned int* n_solving, unsigned int* n_marked, bool allow_fast, cudaStream_t st);
 int64_t lmhead_scratch_bytes(int64_t N, int32_t V);
 cudaError_t launch_lmhead(const saki_lmhead_in& in, void* logits, int64_t ld_l, float* row_max, float* lse, void* scratch,
                           cudaStream_t st, const char** why);

@@ -222,8 +222,12 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
     wait_for_predecessor();
     launch_dependents();
   }
+  if (P.from_list && *(volatile unsigned int*)P.redo_count == 0u) {      // an empty row list, as a rule
+    if (blockIdx.x == 0) move_counters(P.redo_count);
+    return;
+  }
   const int64_t n_work = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
-  if ((int64_t)(blockIdx.x / CS) >= n_work) {                // the whole cluster: nothing to do (an empty row list, as a rule)
+  if ((int64_t)(blockIdx.x / CS) >= n_work) {                // the whole cluster: nothing to do
     if (P.from_list) close_counters(P.redo_count);
     return;
   }

@@ -79,6 +79,10 @@ template <typename T>
 __global__ void __launch_bounds__(MG_THREADS) meta_general_kernel(const MetaParams P) {
   __shared__ double sh[MG_THREADS / 32];
   wait_for_predecessor();
+  if (P.from_list && *(volatile unsigned int*)P.redo_count == 0u) {      // an empty row list, as a rule
+    if (blockIdx.x == 0) move_counters(P.redo_count);
+    return;
+  }
   const int64_t n_items = P.from_list ? (int64_t)*(volatile unsigned int*)P.redo_count : P.n_rows;
   for (int64_t item = blockIdx.x; item < n_items; item += gridDim.x) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;

@@ -20,8 +20,7 @@ struct Lib {
   decltype(&saki_select_tm) select_tm;
   decltype(&saki_spec_verify) spec_verify;
   decltype(&saki_sample_proposal) sample_proposal;
-  decltype(&saki_vshard_partial_group) vshard_partial_group;
-  decltype(&saki_vshard_combine) vshard_combine;
+  decltype(&saki_vshard_stage) vshard_stage;
   decltype(&saki_last_error) last_error;
 };
 Lib lib = {};
@@ -369,42 +368,46 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
     void* const st = stream_of(a[10]);
     const int eager = (int)integer(a[11]), max_waves = (int)integer(a[12]);
     const at::Tensor state = empty({N, SAKI_VSHARD_STATE}, at::kDouble, dev), gathered = empty({world, N, SAKI_VSHARD_PARTIALS}, at::kDouble, dev);
-    const at::Tensor solving = at::zeros({eager + 1}, at::TensorOptions().dtype(at::kInt).device(dev));
+    const at::Tensor counts = at::zeros({eager + 1, 2}, at::TensorOptions().dtype(at::kInt).device(dev));
     double* const sp = (double*)state.data_ptr();
     double* const gp = (double*)gathered.data_ptr();
-    uint32_t* const np = (uint32_t*)solving.data_ptr();
+    uint32_t* const np = (uint32_t*)counts.data_ptr();
     for (int r = 0; r < world; ++r) part[(size_t)r] = gp + (int64_t)r * N * SAKI_VSHARD_PARTIALS;   // where the all-gather would put it
     saki_out so;
     Owned out(alloc_outputs(N, dev, true, &so));
-    auto stage = [&](int k, uint32_t* count) {
-      int rc = unlocked([&] {
-        const int rp = lib.vshard_partial_group(in.data(), world, k, k > 0 ? sp : nullptr, (double* const*)part.data(),
-                                                k == 2 && backward ? (void* const*)grad.data() : nullptr, ld_g.data(), scale, st);
-        return rp ? rp : lib.vshard_combine(in.data(), k, gp, sp, k == 3 ? &so : nullptr, count, st);
-      });
-      check_rc(rc);
+    auto stage = [&](int k, uint32_t* count, int flags) {
+      check_rc(unlocked([&] {
+        return lib.vshard_stage(in.data(), world, k, sp, (double* const*)part.data(), gp, k == 2 && backward ? (void* const*)grad.data() : nullptr,
+                                ld_g.data(), scale, k == 3 ? &so : nullptr, count, flags, st);
+      }));
     };
-    auto read = [&] {     // the rows still solving after stage 0 and after each wave
+    auto read = [&] {     // the rows still solving after stage 0 and after each wave, and those marked for float64
       PyThreadState* const save = PyEval_SaveThread();
-      at::Tensor h = solving.cpu();
+      at::Tensor h = counts.cpu();
       PyEval_RestoreThread(save);
       return h;
     };
     int waves = 0;
     if (N > 0) {
-      stage(0, np);
-      for (int k = 0; k < eager; ++k) stage(1, np + 1 + k);
+      constexpr int NONE = SAKI_VSHARD_NONE_MARKED;
+      stage(0, np, NONE);                                    // a wave's combine is the first that can mark a row
+      for (int k = 0; k < eager; ++k) stage(1, np + 2 * (1 + k), k == 0 ? NONE : 0);
       at::Tensor h = read();
-      const int32_t* left = (const int32_t*)h.data_ptr();
-      while (waves < eager && left[waves] > 0) ++waves;
-      while (left[eager] > 0 && waves < max_waves) {
-        stage(1, np + eager);
+      const int32_t* c = (const int32_t*)h.data_ptr();
+      while (waves < eager && c[2 * waves] > 0) ++waves;
+      int32_t sum = c[2 * eager], left = sum, marked = 0;
+      for (int k = 0; k < eager; ++k) marked += c[2 * k + 1];
+      while (left > 0 && waves < max_waves) {
+        stage(1, np + 2 * eager, 0);                         // (adds to the last pair)
         ++waves;
         h = read();
-        left = (const int32_t*)h.data_ptr();
+        c = (const int32_t*)h.data_ptr();
+        left = c[2 * eager] - sum;
+        sum = c[2 * eager];
       }
-      stage(2, nullptr);
-      stage(3, nullptr);
+      marked += c[2 * eager + 1];
+      stage(2, nullptr, marked ? 0 : NONE);
+      stage(3, nullptr, marked ? 0 : NONE);
     }
     Owned w(PyLong_FromLong(waves)), sv(THPVariable_Wrap(state));
     return PyTuple_Pack(4, out.p, gs.p, w.p, sv.p);
