@@ -201,9 +201,16 @@ struct Consts {   // per-launch constants of the scalar phases
   int V;
 };
 
-// The scalar phases run on one thread per CTA, in float64, while all other
-// threads hold the row in registers; they are kept out of line so that their
-// register needs do not add to the row loop's.
+// The scalar phases run on one thread per CTA, in float64, while all other threads wait.  In the row-per-SM kernel they
+// are inlined (SAKI_SCALARS_INLINE): a call there costs 400 to 600 cycles of stack traffic (the record of constants, the
+// saved registers of a caller that holds a hundred) through an L1 that shared memory has left little of; a row of 32000
+// elements went from 69.8 to 65.5 k cycles (four CTAs per SM).  The cluster kernel holds its row in registers and
+// keeps them out of line.
+#ifdef SAKI_SCALARS_INLINE
+#define SAKI_SCALAR_FN static __device__ __forceinline__
+#else
+#define SAKI_SCALAR_FN static __device__ __noinline__
+#endif
 
 // The coupling decision, the routed loss and the constants of pass "final".
 __device__ __forceinline__ void decide(double* bc, const Consts& K, double lam, double Glam, double G0, double G1,
@@ -271,7 +278,7 @@ static __device__ __noinline__ float anchored_guess(float b, float vd, float k3,
   return x;
 }
 
-static __device__ __noinline__ void scalar_after_lse_tail(double* bc, const double* v, Consts K, float k0f, float k1f, int x,
+SAKI_SCALAR_FN void scalar_after_lse_tail(double* bc, const double* v, Consts K, float k0f, float k1f, int x,
                                                    bool bonus, bool masked, bool row_timeout, float e_max,
                                                    bool overflow_redo, double rSs, double rSt, double G0, double G1,
                                                    const double* m4_raw = nullptr) {
@@ -359,7 +366,7 @@ static __device__ __noinline__ void scalar_after_lse(double* bc, const double* v
 // far below the resolution of the float32 sums, so one evaluation usually settles the row.  The
 // size of the last kept term (with floors against accidentally small cumulants) decides whether
 // another evaluation at the new point is needed.
-static __device__ __noinline__ void scalar_after_solve4(double* bc, const double* v, Consts K, float k0f, float k1f, int x,
+SAKI_SCALAR_FN void scalar_after_solve4(double* bc, const double* v, Consts K, float k0f, float k1f, int x,
                                                  bool bonus, bool masked) {
   const double eps = K.eps, rtau = K.rtau;
   const double G0 = bc[BC_G0], kb = bc[BC_KB];
@@ -520,7 +527,7 @@ static __device__ __noinline__ void scalar_find_owner(double* bc, const double* 
 }
 
 // tv: the row's total variation (the caller may hold it before bc[BC_TV] is written)
-static __device__ __noinline__ void write_result_tv(const double* bc, saki_out out, bool write_loss, int64_t row, int corrected,
+SAKI_SCALAR_FN void write_result_tv(const double* bc, saki_out out, bool write_loss, int64_t row, int corrected,
                                              int y, bool bonus, double c64, const __nv_bfloat16* g_s,
                                              const __nv_bfloat16* g_t, double tv) {
   RowResult r;

@@ -30,6 +30,9 @@
 //            "residual"), gradient row streamed out (Eq. "general_objective")
 // Per-element work is float32 (packed f32x2 FMAs, ex2.approx); cross-thread
 // combinations and per-row scalars are float64.
+#if defined(SAKI_ROWSM_QUARTER) || defined(SAKI_ROWSM_HALF)
+#define SAKI_SCALARS_INLINE 1       // (one CTA per SM: 1 % slower, the pass loops come out worse)
+#endif
 #include "saki_device.cuh"
 #include <mutex>
 
