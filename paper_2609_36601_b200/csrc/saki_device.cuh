@@ -19,6 +19,7 @@ constexpr double LN2 = 0.693147180559945309417232121458;
 constexpr double INV_LN2 = 1.44269504088896340735992468100;
 constexpr long long WAIT_LIMIT_CYCLES = 4000000000LL;   // ~2 s: give up on a wait
 
+constexpr int VSTAR_ELSEWHERE = -2;        // argmax index in the sums of pass "lse", token in BC_TOK: it is (will be) in BC_VSTAR
 enum { MODE_SOLVE = 0, MODE_FINAL = 1, MODE_FLAGGED = 2, MODE_REDO = 3 };
 // broadcast slots (one set per row buffer)
 enum { BC_MODE = 0, BC_BETA, BC_CB, BC_KB, BC_LO, BC_HI, BC_ITER,                    // solver
@@ -291,8 +292,9 @@ SAKI_SCALAR_FN void scalar_after_lse_tail(double* bc, const double* v, Consts K,
     status = SAKI_ROW_NONFINITE;
   }
   else if (!bonus && (x < 0 || x >= K.V)) status = SAKI_ROW_BAD_ID;
-  const int vstar = (v[6] >= 0.0 && v[6] < (double)K.V) ? (int)v[6] : 0;
-  bc[BC_VSTAR] = (double)vstar;
+  // VSTAR_ELSEWHERE: another warp is finding the argmax; it writes BC_VSTAR, and a token that is v* stays the marker
+  const int vstar = v[6] == (double)VSTAR_ELSEWHERE ? VSTAR_ELSEWHERE : (v[6] >= 0.0 && v[6] < (double)K.V) ? (int)v[6] : 0;
+  if (vstar != VSTAR_ELSEWHERE) bc[BC_VSTAR] = (double)vstar;
   if (status) { bc[BC_STATUS] = (double)status; bc[BC_MODE] = MODE_FLAGGED; return; }
   bc[BC_G0] = G0; bc[BC_G1] = G1; bc[BC_RSS] = rSs;
   bc[BC_PMAX] = fmin(1.0, (double)e_max * fmax(rSs, rSt));      // upper bound of the largest probability of either row

@@ -60,12 +60,15 @@ constexpr int KS_MAX = 208 / (RW * CTAS_PER_SM);   // steps per warp that fit in
 constexpr int MAX_STEPS = 64;            // steps per warp the draw bookkeeping can hold (V <= 64*32*8*RW)
 constexpr int RES_CHUNKS = KS_MAX * 32; // resident chunks per warp and row
 constexpr int RNV = 9;                  // doubles per partial vector
-static_assert(RW >= 14 || RW == 8 || RW == 4, "the eight gather roles go round the first eight warps; the side work has warps of its own, or is shared out");
+static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight warps, or done by warp 0; the side work has warps of its own, or is shared out");
 // Who does what beside the passes.  With 14 warps or more the row scalars that do not depend on the
-// passes (uniforms, the logits at the proposal) are fetched by warps 8-10 while warps 0-7 gather; with
-// eight warps, by warps 1-3 before the block barrier that ends pass "lse".  After the gather, while
-// thread 0 does the scalars: FIN_WARP finishes the previous row, RES_WARP reserves the next row of a
-// block verification, lane 0 of SV_WARP fetches the student's logit at the teacher's argmax.
+// passes (uniforms, the logits at the proposal) are fetched by warps 8-10 while warps 0-7 gather the warps' sums, one sum
+// each; a block barrier; then thread 0 does the scalars.  With four or eight warps warp 0 gathers all sums at once (four
+// lanes per sum) and goes straight on to the scalars: a barrier less per pass, and the eight sums are not dealt
+// twice round four warps (4096 rows of 8192 elements: 26.7 -> 25.5 k cycles a row; of 32000: 65.5 -> 65.4 k); the uniforms and the logits at the
+// proposal are fetched by warps 1-3 at the top of the row.  While thread 0 does the scalars: FIN_WARP finishes the
+// previous row, RES_WARP reserves the next row of a block verification, SV_WARP fetches the student's logit at the
+// teacher's argmax (and with four or eight warps finds the argmax).
 constexpr bool SIDE_WARPS = RW >= 14;
 constexpr int UACC_WARP = SIDE_WARPS ? 8 : 1, UDRAW_WARP = SIDE_WARPS ? 9 : 2, SX_WARP = SIDE_WARPS ? 10 : 3;
 constexpr int RES_WARP = SIDE_WARPS ? 11 : (RW == 8 ? 5 : 2), SV_WARP = SIDE_WARPS ? 13 : (RW == 8 ? 6 : 3);
@@ -117,6 +120,33 @@ __device__ __forceinline__ double warp_sum_d(double a) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   return a;
+}
+// The sums over the warp of eight values at once: lane l ends up with the total of value l / 4.  A butterfly that halves
+// the number of values in its first three steps: 9 exchanges instead of 40.
+__device__ __forceinline__ double warp_sum8(const double (&v)[8], int lane) {
+  double a[4], b[2], c;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) a[k] = (h4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, h4 ? v[k] : v[k + 4], 16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) b[k] = (h3 ? a[k + 2] : a[k]) + __shfl_xor_sync(0xffffffffu, h3 ? a[k] : a[k + 2], 8);
+  c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
+}
+// A bf16 value (as float) as an unsigned 16-bit key of the same order (-0 as +0), and back.
+__device__ __forceinline__ uint32_t bf16_key(float x) {
+  const uint32_t b = __float_as_uint(x + 0.f);
+  return ((b & 0x80000000u) ? ~b : (b | 0x80000000u)) >> 16;
+}
+__device__ __forceinline__ float bf16_of_key(uint32_t k) {
+  const uint32_t b = k << 16;
+  return __uint_as_float((b & 0x80000000u) ? (b & 0x7fffffffu) : (~b & 0xffff0000u));
+}
+__device__ __forceinline__ float ld_bf16(const __nv_bfloat16* p) {   // issued where it stands
+  unsigned short v;
+  asm volatile("ld.global.nc.u16 %0, [%1];" : "=h"(v) : "l"(p));
+  return __uint_as_float((uint32_t)v << 16);
 }
 __device__ __forceinline__ float warp_max_f(float a) {
 #pragma unroll
@@ -366,6 +396,15 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     }
     __syncthreads();
   };
+  // the same for eight values at once on warp 0 (lane l: value l / 4), which goes on alone; a barrier before, none after
+  auto gather8 = [&](auto&& term) {
+    double a = 0.0;
+#pragma unroll
+    for (int w = lane & 3; w < RW; w += 4) a += term(lane >> 2, w);
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    return a;
+  };
 
   // Block verification with early out (Section 3.5 discards what lies behind a sequence's first
   // rejection).  Positions are handed out as tickets from a device counter in position-major order
@@ -447,7 +486,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     const double tv_sum = warp_sum_d(lane < RW ? fin[lane] : 0.0);
     const double tv = (bcp[BC_LAMBDA] > 0.0) ? tv_sum : 0.0;
     const float k0p = (float)bcp[BC_K0];
-    const int tok = (int)bcp[BC_TOK];
+    const int tok0 = (int)bcp[BC_TOK], tok = tok0 == VSTAR_ELSEWHERE ? (int)bcp[BC_VSTAR] : tok0;
     if (lane == 0 && P.dlogits && tok >= 0) {   // the supervised token: gradient KG * (p - 1), over the entry its chunk's owner stored
       const float ipf = (float)bcp[BC_IP];
       const float kgf = (float)(bcp[BC_KG] * (double)ipf);
@@ -569,6 +608,13 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
         atomicMin(P.seq_stop + seq, pos);        // verification of this sequence ends here
       atomicAdd(P.seq_next + 1, 1u);             // statistic: positions routed
     };
+    // the row scalars that do not depend on the passes, on their way while pass "lse" runs
+    float sx = 0.f, tx = 0.f;
+    if (!SIDE_WARPS && lane == 0) {
+      if (warp == UACC_WARP) bc[BC_UACC] = scalar_uniform(P.seed, rid, STAGE_ACCEPT);
+      if (warp == UDRAW_WARP) bc[BC_UDRAW] = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
+      if (warp == SX_WARP && x >= 0 && x < V) { sx = ld_bf16(g_s + x); tx = ld_bf16(g_t + x); }
+    }
     if (timing && tid == 0) ph[PH_ROWS] += 1;
     RTS(PH_ROW_TOP);
     if (!dead) {
@@ -635,6 +681,69 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       // chunk order is index order; the element is found once, by the block's winner), student
       // maximum, sums
       const float2 rs2 = unpack_bf16x2(run_s);
+      int any_dead;
+      if constexpr (!SIDE_WARPS) {
+        auto tot = [](const float2 a) { return (double)a.x + (double)a.y; };
+        const double v[8] = {tot(Ss), tot(St), tot(M1), tot(M2), tot(M3), tot(N1), tot(M4), 0.0};
+        const double a = warp_sum8(v, lane);
+        // maxima as keys; the teacher's with the complement of the chunk behind it (fewer than 65535 chunks): the largest
+        // key is the largest value and the lowest chunk that holds it
+        const uint32_t skey = __reduce_max_sync(0xffffffffu, bf16_key(fmaxf(rs2.x, rs2.y)));
+        const uint32_t tkey = __reduce_max_sync(0xffffffffu, arg_c >= 0 ? (bf16_key(mt_run) << 16) | (0xffffu - (uint32_t)arg_c) : 0u);
+        uint32_t* const wm = (uint32_t*)(smem + ROFF_WMAX);
+        if ((lane & 3) == 0) {       // (the eighth value's place takes the student's shift)
+          red[(lane >> 2) * RW + warp] = lane == 28 ? (double)ksw : a;
+        }
+        if (lane == 0) { red[8 * RW + warp] = (double)ktw; wm[warp] = tkey; wm[RW + warp] = skey; }
+        if (warp == SX_WARP && lane == 0) { bc[BC_SX] = (double)sx; bc[BC_TX] = (double)tx; }
+        any_dead = __syncthreads_or(dead ? 1 : 0);
+        if (any_dead) dead = true;
+        RTS(PH_LSE_REDUCE);
+        if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);   // the previous row's draw and outputs
+        if (dyn && warp == RES_WARP) reserve_next();     // the CTA's next row (block verification)
+        pending_row = -1;
+        if (warp == SV_WARP) {       // the teacher's argmax, and the student's logit there (the supervised token of a corrected row)
+          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < RW ? wm[lane] : 0u);
+          if (lane == 0) {
+            int best = 0;
+            float sv = 0.f;
+            if (gk != 0u) {
+              const int c = (int)(0xffffu - (gk & 0xffffu));
+              const float gmt = bf16_of_key(gk >> 16);
+              const uint4 t4 = ld_l2(g_t + (size_t)c * 8, pol_last), s4 = ld_l2(g_s + (size_t)c * 8, pol_last);
+              const uint32_t tw[4] = {t4.x, t4.y, t4.z, t4.w}, sw[4] = {s4.x, s4.y, s4.z, s4.w};
+#pragma unroll
+              for (int i = 3; i >= 0; --i) {       // lowest index of the maximum inside the winning chunk
+                const float2 f2 = unpack_bf16x2(tw[i]), s2 = unpack_bf16x2(sw[i]);
+                if (f2.y == gmt) { best = c * 8 + 2 * i + 1; sv = s2.y; }
+                if (f2.x == gmt) { best = c * 8 + 2 * i; sv = s2.x; }
+              }
+            }
+            bc[BC_VSTAR] = (double)best;
+            bc[BC_SV] = (double)sv;
+          }
+        }
+        if (warp == 0) {
+          // From here on the row's shifts are those of its true maxima (the largest term of each sum has its exponent
+          // argument in (-1, 0], where float32 resolves it best); a warp's shift came from an element of the row, so it
+          // is never below the row's, and the factor is an exact power of two <= 1.
+          const float gms = bf16_of_key(__reduce_max_sync(0xffffffffu, lane < RW ? wm[RW + lane] : 0u));
+          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < RW ? wm[lane] : 0u);
+          const float gmt = gk ? bf16_of_key(gk >> 16) : -CUDART_INF_F;
+          const double krs = (double)-ceilf(c32 * fmaxf(gms, -1e30f)), krt = (double)-ceilf(c32 * fmaxf(gmt, -1e30f));
+          const double a = gather8([&](int role, int w) {
+            const bool teacher = (role == 1 || role == 5);
+            const double kw = red[(teacher ? 8 : 7) * RW + w];
+            const double f = kw < 1e29 ? (double)pow2f_exact((float)((teacher ? krt : krs) - kw)) : 0.0;
+            return role < 7 ? f * red[role * RW + w] : 0.0;
+          });
+          const int role = lane >> 2;
+          if ((lane & 3) == 0 && role < 7) gat[role < 6 ? role : 9] = a;       // gat[9]: the fourth moment
+          if (lane == 0) { gat[6] = (double)VSTAR_ELSEWHERE; gat[7] = krs; gat[8] = krt; }
+          __syncwarp();
+        }
+        RTS(PH_LSE_GATHER);
+      } else {
       const float wms = warp_max_f(fmaxf(rs2.x, rs2.y));
       float wmt = mt_run;
       int warg = arg_c >= 0 ? arg_c : 0x7fffffff;
@@ -666,8 +775,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
           bc[BC_TX] = ok ? (double)__bfloat162float(g_t[x]) : 0.0;
         }
       };
-      if (!SIDE_WARPS && lane == 0) side_work();
-      const int any_dead = __syncthreads_or(dead ? 1 : 0);
+      any_dead = __syncthreads_or(dead ? 1 : 0);
       RTS(PH_LSE_REDUCE);
       if (warp < 8) {   // block level, eight roles dealt round the first eight warps: 0-6 add up one sum each on the row's shifts, 7 finds the argmax
 #pragma unroll 1
@@ -710,7 +818,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
           }
         }
        }
-      } else if (SIDE_WARPS && lane == 0) {
+      } else if (lane == 0) {
         side_work();                             // meanwhile, on warps that would only wait
       }
       if (any_dead) dead = true;
@@ -722,6 +830,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       if (tid == SV_WARP * 32) {   // and the student's logit at the teacher's argmax (the supervised token of a corrected row)
         const int vs = (gat[6] >= 0.0 && gat[6] < (double)V) ? (int)gat[6] : 0;
         bc[BC_SV] = (double)__bfloat162float(g_s[vs]);
+      }
       }
       if (tid < 2) {   // lane 0: the student's sum, lane 1: the teacher's; then lane 0 alone
         double rS, G;
@@ -766,9 +875,21 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       }, [] {});
       RTS(PH_SOLVE);
       auto tot = [](const float2 a) { return (double)a.x + (double)a.y; };
-      const double v[5] = {warp_sum_d(tot(S0)), warp_sum_d(tot(S1)), warp_sum_d(tot(S2)), warp_sum_d(tot(S3)),
-                           warp_sum_d(tot(S4))};
-      combine(v, 5);
+      if constexpr (!SIDE_WARPS) {
+        const double v8[8] = {tot(S0), tot(S1), tot(S2), tot(S3), tot(S4), 0.0, 0.0, 0.0};
+        const double a = warp_sum8(v8, lane);
+        if ((lane & 3) == 0) red[(lane >> 2) * RW + warp] = a;
+        __syncthreads();
+        if (warp == 0) {
+          const double b = gather8([&](int role, int w) { return red[role * RW + w]; });
+          if ((lane & 3) == 0 && lane < 20) gat[lane >> 2] = b;
+          __syncwarp();
+        }
+      } else {
+        const double v[5] = {warp_sum_d(tot(S0)), warp_sum_d(tot(S1)), warp_sum_d(tot(S2)), warp_sum_d(tot(S3)),
+                             warp_sum_d(tot(S4))};
+        combine(v, 5);
+      }
       RTS(PH_SOLVE_COMBINE);
       if (tid == 0) {
         scalar_after_solve4(bc, gat, K, k0, k1, x, bonus, masked);
