@@ -27,20 +27,28 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
   return true;
 }
 
-// by_rows: a call that leaves SMs idle takes the variant with the most threads per row that still holds all its rows at
-// once (a row's passes are then a half or a quarter as long).  Measured, forward, us, 1 / 2 / 4 CTAs per SM: V = 49152,
-// 8 rows 28.8 / 30.8 / 37.1, 148 rows 28.8 / 32.5 / 38.9, 296 rows 49.5 / 39.7 / 44.9, 592 rows 86.9 / 71.0 / 67.5;
-// V = 16384, 8 rows 20.6 / 20.6 / 22.9, 296 rows 32.5 / 23.4 / 26.7, 592 rows 53.2 / 38.5 / 32.8; below V = 8192 no
-// difference.  Not where saki_set_kernel pins the kernel: then the variant goes by V alone, and pieces of a batch agree
-// with the whole to the bit.
+// by_rows: the variant that routes this number of rows soonest.  A variant with k CTAs per SM takes ceil(rows / (k SMs))
+// turns of a + b V / 1000 microseconds each (fitted to V = 2048 to 98304 and 8 to 1776 rows, within 10 %):
+//   k = 1: 6.2, 0.302     k = 2: 5.0, 0.535     k = 4: 6.0, 1.06
+// so that, e.g., 888 rows of 32000 take three turns of k = 2 (73 us) and not two of k = 4 (83 us), 296 rows of 49152 one
+// turn of k = 2 (38 us against 48 with k = 1 and 51 with k = 4); a call with a row or less per SM takes k = 1, or k = 2
+// where its inlined scalar steps outweigh the longer passes (below V = 16384: 14.1 against 16.2 us at 8192).  The limits on V above
+// hold here too, except that rows in flight that fit in L2 anyway (two per SM) may be longer.  Not where saki_set_kernel
+// pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
 cudaError_t launch_rowsm(const RowParams& p, bool by_rows, cudaStream_t st, int* n_launches, bool* served) {
-  if (by_rows && p.V >= 8192) {
+  if (by_rows) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (p.call_rows <= sms) return full_sm::launch(p, st, n_launches, served);
-    if (p.call_rows <= 2 * sms && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);
-    if (p.call_rows <= 4 * sms && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
+    const int64_t n = p.call_rows;
+    const double kv = p.V * 1e-3;
+    auto cost = [&](int k, double a, double b) { return (double)((n + (int64_t)k * sms - 1) / ((int64_t)k * sms)) * (a + b * kv); };
+    const double c1 = cost(1, 6.2, 0.302);
+    const double c2 = p.V <= HALF_MAX_V || (n <= 2 * sms && p.V <= half_sm::max_v()) ? cost(2, 5.0, 0.535) : 1e30;
+    const double c4 = p.V <= QUARTER_MAX_V ? cost(4, 6.0, 1.06) : 1e30;
+    if (n <= sms ? p.V >= 16384 : (c1 < c2 && c1 < c4)) return full_sm::launch(p, st, n_launches, served);
+    if (n <= sms || c2 < c4) return half_sm::launch(p, st, n_launches, served);
+    return quarter_sm::launch(p, st, n_launches, served);
   }
   if (p.V <= QUARTER_MAX_V && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
   if (p.V <= HALF_MAX_V && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);
