@@ -1,13 +1,11 @@
-// Register-resident cluster kernel for bf16 rows: the latency path (calls of a few long rows).
+// Cluster kernel for bf16 rows: the latency path (calls of a few long rows).
 //
-// One vocabulary row per thread-block cluster of CS CTAs x 256 threads, two
-// CTAs resident per SM.  Each CTA owns a contiguous slice of the row; each
-// thread owns 80 contiguous elements of it, held for the whole row in
-// registers as the raw packed bf16 pairs (40 + 40 registers), so the row pair
-// is read from HBM exactly once.  The single shared-memory slot of a CTA is
-// only the landing zone of the NEXT row's slice, fetched by one 1-D bulk
-// async copy per row (cp.async.bulk + mbarrier) while the current row is
-// being computed.  Passes over the registers:
+// One vocabulary row per thread-block cluster of CS CTAs x 256 threads.  Each CTA owns a contiguous slice of the row in
+// shared memory, fetched by one 1-D bulk async copy per array (cp.async.bulk + mbarrier), so the row pair is read from HBM
+// exactly once; each thread owns 80 contiguous elements of the slice.  What bounds a call here is the chain of steps of a
+// single row, and much of that was instruction fetch: with the row in registers every pass was 40 unrolled pairs of code
+// that ran once.  The passes are loops over shared memory now, and the registers that frees let the scalar steps be
+// inlined (8 rows of 151936, forward: __CL__ us).  Passes:
 //   lse      2 exponentials/element: both log-sum-exps (computed under the
 //            CTA's own maxima rounded up to whole powers of two, then moved
 //            exactly onto the row's maxima, which the CTAs exchange while the
@@ -20,8 +18,7 @@
 //            evaluation for most rows (Eqs. "bridge", "trust_region")
 //   final    2 exponentials/element: TV = sum [q-p]_+ with per-thread ordered
 //            partial sums for the inverse-CDF residual draw (Eqs. "accept",
-//            "residual"), and the gradient row written straight from
-//            registers (Eq. "general_objective")
+//            "residual"), and the gradient row (Eq. "general_objective")
 // Per-element work is float32 (packed f32x2 FMAs, ex2.approx); every
 // cross-thread combination and every per-row scalar is float64.  Per-warp
 // partial sums travel to all CTAs of the cluster as asynchronous
@@ -29,6 +26,7 @@
 // (no cluster barrier, no fence on the row loop); each CTA then forms the
 // same scalars redundantly from the same numbers in the same order, so
 // control flow is uniform across the cluster.
+#define SAKI_SCALARS_INLINE 1
 #include "saki_device.cuh"
 #include <cooperative_groups.h>
 #include <math_constants.h>
@@ -42,7 +40,6 @@ constexpr int CT = 256;                 // threads per CTA
 constexpr int CW = CT / 32;             // warps per CTA
 constexpr int CHUNKS = 10;              // 16-byte chunks (8 bf16) per thread per row
 constexpr int EPT = CHUNKS * 8;         // elements per thread
-constexpr int NPAIR = EPT / 2;          // packed registers per thread per row
 constexpr int SLICE_CAP = CT * EPT;     // elements of one row a CTA can hold
 constexpr int MAX_CS = 8;
 constexpr int NSLOT = MAX_CS * CW;      // per-warp partial slots of a cluster
@@ -56,10 +53,9 @@ constexpr int OFF_MX = OFF_RED + 2 * NV * NSLOT * 8;            // [2][MAX_CS][2
 constexpr int OFF_GAT = OFF_MX + 2 * MAX_CS * 2 * 8;            // [NV] doubles: cluster totals
 constexpr int OFF_BC = OFF_GAT + NV * 8;                        // [2][BC_DOUBLES] broadcast scalars
 constexpr int OFF_WMAX = OFF_BC + 2 * BC_DOUBLES * 8;           // [2][2][CW] floats: per-warp maxima
-constexpr int OFF_SCR = OFF_WMAX + 2 * 2 * CW * 4;              // [2][EPT] bf16: one thread's elements in index order
-constexpr int OFF_MBAR = OFF_SCR + 2 * EPT * 2;                 // copy barrier, 2 exchange barriers, 2 maxima barriers
+constexpr int OFF_MBAR = OFF_WMAX + 2 * 2 * CW * 4;             // copy barrier, 2 exchange barriers, 2 maxima barriers
 constexpr int SMEM_BYTES = OFF_MBAR + 5 * 8 + 8;
-static_assert(OFF_MBAR % 8 == 0 && OFF_SCR % 16 == 0, "alignment");
+static_assert(OFF_MBAR % 8 == 0, "alignment");
 
 template <int CS>
 __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const int n_clusters) {
@@ -91,6 +87,7 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
   K.tau = (double)P.temperature; K.rtau = 1.0 / K.tau; K.eps = (double)P.eps; K.c64 = (double)c32;
   K.rc64 = 1.0 / K.c64; K.grad_scale = (double)P.grad_scale; K.sqrt_eps = sqrtf(P.eps); K.V = V;
 
+  bool dead = false;   // a wait timed out: this CTA stops fetching and the cluster flags its rows
   auto row_ptrs = [&](int64_t row, const __nv_bfloat16*& s, const __nv_bfloat16*& t) {
     const int64_t b = row / P.K1;
     const int j = (int)(row - b * P.K1);
@@ -106,22 +103,41 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       bulk_load(smem + OFF_T, t + slice_start, slice_bytes, &mbar[0]);
     }
   };
-  // one exchange: every warp sends its N-vector to slot rank*CW+warp of red[p] in every CTA
-  auto push = [&](const double* v, int n, int p) {
-    if (lane < CS) {
-      const uint32_t dst = map_to_rank(red_s + (uint32_t)(((p * NV) * NSLOT + rank * CW + warp) * 8), lane);
-      const uint32_t bar = map_to_rank(bar_s + (uint32_t)((1 + p) * 8), lane);
+  // one exchange: every warp's totals, value lane / 4 in each lane (n of them), to slot rank*CW+warp of red[p] in every CTA
+  auto push = [&](double v, int n, int p) {
+    const int k = lane >> 2;
+    if (k < n) {
+      const uint32_t dst = red_s + (uint32_t)(((p * NV + k) * NSLOT + rank * CW + warp) * 8), bar = bar_s + (uint32_t)((1 + p) * 8);
 #pragma unroll
-      for (int k = 0; k < NV; ++k)
-        if (k < n) st_async_f64(dst + (uint32_t)(k * NSLOT * 8), v[k], bar);
+      for (int r = lane & 3; r < CS; r += 4) st_async_f64(map_to_rank(dst, r), v, map_to_rank(bar, r));
     }
   };
-  // cluster total of component k (fixed order, the same in every CTA); is_min: minimum instead of sum
-  auto gather = [&](int p, int k, bool is_min) {
-    const double* base = red + (size_t)(p * NV + k) * NSLOT;
-    double a = is_min ? CUDART_INF : 0.0;
-    for (int slot = lane; slot < CS * CW; slot += 32) a = is_min ? fmin(a, base[slot]) : a + base[slot];
-    return is_min ? warp_min(a) : warp_sum(a);
+  // warp 0: cluster total of value lane / 4 (fixed order, the same in every CTA)
+  auto gather = [&](int p) {
+    const double* base = red + (size_t)(p * NV + (lane >> 2)) * NSLOT;
+    double a = 0.0;
+#pragma unroll
+    for (int slot = lane & 3; slot < CS * CW; slot += 4) a += base[slot];
+    a += __shfl_xor_sync(0xffffffffu, a, 2);
+    a += __shfl_xor_sync(0xffffffffu, a, 1);
+    return a;
+  };
+  // this thread's chunks of the slice, in an order that keeps 128-bit shared loads free of conflicts: body(first element
+  // within the slice, student, teacher); beyond the slice's end the elements are "most negative finite"
+  auto for_chunks = [&](auto&& body) {
+#pragma unroll 2
+    for (int j = 0; j < CHUNKS; ++j) {
+      int cj = j + rot;
+      if (cj >= CHUNKS) cj -= CHUNKS;
+      const int e0 = thr_first + cj * 8;
+      uint4 a = make_uint4(SENTINEL, SENTINEL, SENTINEL, SENTINEL), b = a;
+      if (e0 < my_len && !dead) {
+        a = *reinterpret_cast<const uint4*>(slot_s + e0);
+        b = *reinterpret_cast<const uint4*>(slot_t + e0);
+      }
+      const uint32_t sw[4] = {a.x, a.y, a.z, a.w}, tw[4] = {b.x, b.y, b.z, b.w};
+      body(e0, sw, tw);
+    }
   };
 
   if (tid == 0) {
@@ -134,7 +150,6 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
   if (tid == 0 && cluster_id < P.n_rows) issue(cluster_id);
   uint32_t phase = 0, xph0 = 0, xph1 = 0, mph0 = 0, mph1 = 0;
   int parity = 0, rb = 0;
-  bool dead = false;   // a wait timed out: this CTA stops fetching and the cluster flags its rows
 
   for (int64_t row = cluster_id; row < P.n_rows; row += n_clusters, rb ^= 1) {
     double* bc = (double*)(smem + OFF_BC) + rb * BC_DOUBLES;
@@ -148,35 +163,35 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
     row_ptrs(row, g_s, g_t);
     __nv_bfloat16* g_out = P.dlogits ? (__nv_bfloat16*)P.dlogits + row * P.ld_g : nullptr;
 
-    // ------------------------------------------------ stage: shared slot -> registers
-    bool timed_out = dead;
-    if (!dead) {
-      if (!mbar_wait_bounded(&mbar[0], phase)) timed_out = true;
-      else phase ^= 1u;
-    }
-    uint32_t sr[NPAIR], tr[NPAIR];
-#pragma unroll
-    for (int j = 0; j < CHUNKS; ++j) {
-      int cj = j + rot;
-      if (cj == CHUNKS) cj = 0;
-      const int e0 = thr_first + cj * 8;
-      uint4 a = make_uint4(SENTINEL, SENTINEL, SENTINEL, SENTINEL), b = a;
-      if (e0 < my_len && !timed_out) {
-        a = *reinterpret_cast<const uint4*>(slot_s + e0);
-        b = *reinterpret_cast<const uint4*>(slot_t + e0);
+    if (row != cluster_id) {                 // the slot is free once every thread is done with the last row
+      __syncthreads();
+      if (tid == 0 && !dead) {
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        issue(row);
       }
-      sr[4 * j + 0] = a.x; sr[4 * j + 1] = a.y; sr[4 * j + 2] = a.z; sr[4 * j + 3] = a.w;
-      tr[4 * j + 0] = b.x; tr[4 * j + 1] = b.y; tr[4 * j + 2] = b.z; tr[4 * j + 3] = b.w;
+    }
+    // row scalars that do not depend on the passes, while the copy is on its way
+    if (tid == 32) bc[BC_UACC] = scalar_uniform(P.seed, rid, STAGE_ACCEPT);
+    if (tid == 64) bc[BC_UDRAW] = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
+    if (tid == 96) {
+      const bool ok = (x >= 0 && x < V);
+      bc[BC_SX] = ok ? (double)__bfloat162float(g_s[x]) : 0.0;
+      bc[BC_TX] = ok ? (double)__bfloat162float(g_t[x]) : 0.0;
+    }
+
+    // ------------------------------------------------ the slice has arrived; its maxima
+    if (!dead) {
+      if (!mbar_wait_bounded(&mbar[0], phase)) dead = true;
+      else phase ^= 1u;
     }
     // maxima of this CTA's slice (packed bf16), via shuffles and one CTA barrier
     float my_mt;
     {
-      uint32_t a = sr[0], b = tr[0];
-#pragma unroll
-      for (int i = 1; i < NPAIR; ++i) {
-        a = max_bf16x2(a, sr[i]);
-        b = max_bf16x2(b, tr[i]);
-      }
+      uint32_t a = SENTINEL, b = SENTINEL;
+      for_chunks([&](int, const uint32_t* sw, const uint32_t* tw) {
+        a = max_bf16x2(a, max_bf16x2(max_bf16x2(sw[0], sw[1]), max_bf16x2(sw[2], sw[3])));
+        b = max_bf16x2(b, max_bf16x2(max_bf16x2(tw[0], tw[1]), max_bf16x2(tw[2], tw[3])));
+      });
       const float2 fb0 = unpack_bf16x2(b);
       my_mt = fmaxf(fb0.x, fb0.y);
 #pragma unroll
@@ -190,14 +205,8 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
         wmax[(rb * 2 + 1) * CW + warp] = fmaxf(fb.x, fb.y);
       }
     }
-    const int any_timeout = __syncthreads_or(timed_out ? 1 : 0);   // also: every thread has drained the slot
-    if (any_timeout) dead = true;
+    if (__syncthreads_or(dead ? 1 : 0)) dead = true;
     if (tid == 0) {
-      const int64_t next = row + n_clusters;
-      if (!dead && next < P.n_rows) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-        issue(next);
-      }
       mbar_expect_tx(&mbar[3 + rb], (uint32_t)(CS * 16));          // maxima of all CTAs
       mbar_expect_tx(&mbar[1 + parity], (uint32_t)(CS * CW * 8 * 8));   // partials of pass "lse"
     }
@@ -217,30 +226,17 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
     // shifts differ by exact powers of two
     const float k0r = -ceilf(c32 * fmaxf(ms_r, -1e30f)), k1r = -ceilf(c32 * fmaxf(mt_r, -1e30f));
 
-    // row scalars that do not depend on the passes, fetched off the critical path
-    if (tid == 32) bc[BC_UACC] = scalar_uniform(P.seed, rid, STAGE_ACCEPT);
-    if (tid == 64) bc[BC_UDRAW] = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
-    if (tid == 96) {
-      const bool ok = (x >= 0 && x < V);
-      bc[BC_SX] = ok ? (double)__bfloat162float(g_s[x]) : 0.0;
-      bc[BC_TX] = ok ? (double)__bfloat162float(g_t[x]) : 0.0;
-    }
-
     // teacher argmax candidate of this thread (exact compare on stored values, lowest index)
-    double cand = CUDART_INF;
+    uint32_t cand = 0xffffffffu;
     if (my_mt == mt_r) {
+      for_chunks([&](int e0, const uint32_t*, const uint32_t* tw) {
 #pragma unroll
-      for (int j = 0; j < CHUNKS; ++j) {
-        int cj = j + rot;
-        if (cj == CHUNKS) cj = 0;
-        const int e0 = slice_start + thr_first + cj * 8;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const float2 f = unpack_bf16x2(tr[4 * j + k]);
-          if (f.x == mt_r) cand = fmin(cand, (double)(e0 + 2 * k));
-          if (f.y == mt_r) cand = fmin(cand, (double)(e0 + 2 * k + 1));
+        for (int k = 3; k >= 0; --k) {
+          const float2 f = unpack_bf16x2(tw[k]);
+          if (f.y == mt_r) cand = min(cand, (uint32_t)(slice_start + e0 + 2 * k + 1));
+          if (f.x == mt_r) cand = min(cand, (uint32_t)(slice_start + e0 + 2 * k));
         }
-      }
+      });
     }
 
     // ------------------------------------------------ pass "lse"
@@ -250,22 +246,24 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       float2 Ss = splat(0.f), St = splat(0.f), M1 = splat(0.f), M2 = splat(0.f), M3 = splat(0.f), M4 = splat(0.f),
              N1 = splat(0.f);
       const float2 cc = splat(c32), kk0 = splat(k0r), kk1 = splat(k1r), neg1 = splat(-1.f);
+      for_chunks([&](int, const uint32_t* sw, const uint32_t* tw) {
 #pragma unroll
-      for (int i = 0; i < NPAIR; ++i) {
-        const float2 sf = unpack_fresh(sr[i]), tf = unpack_fresh(tr[i]);
-        const float2 d = ffma2(sf, neg1, tf);
-        const float2 es = ex2f2(ffma2(sf, cc, kk0));
-        const float2 et = ex2f2(ffma2(tf, cc, kk1));
-        Ss = fadd2(Ss, es);
-        St = fadd2(St, et);
-        const float2 t1 = fmul2(es, d);
-        M1 = fadd2(M1, t1);
-        const float2 t2 = fmul2(t1, d);
-        M2 = fadd2(M2, t2);
-        M3 = ffma2(t2, d, M3);
-        M4 = ffma2(t2, fmul2(d, d), M4);
-        N1 = ffma2(et, d, N1);
-      }
+        for (int i = 0; i < 4; ++i) {
+          const float2 sf = unpack_bf16x2(sw[i]), tf = unpack_bf16x2(tw[i]);
+          const float2 d = ffma2(sf, neg1, tf);
+          const float2 es = ex2f2(ffma2(sf, cc, kk0));
+          const float2 et = ex2f2(ffma2(tf, cc, kk1));
+          Ss = fadd2(Ss, es);
+          St = fadd2(St, et);
+          const float2 t1 = fmul2(es, d);
+          M1 = fadd2(M1, t1);
+          const float2 t2 = fmul2(t1, d);
+          M2 = fadd2(M2, t2);
+          M3 = ffma2(t2, d, M3);
+          M4 = ffma2(t2, fmul2(d, d), M4);
+          N1 = ffma2(et, d, N1);
+        }
+      });
       // the row's maxima have arrived meanwhile: move the partial sums onto the row's shifts
       bool mx_timeout = false;
       if (!mbar_wait_bounded(&mbar[3 + rb], rb ? mph1 : mph0)) mx_timeout = true;
@@ -283,23 +281,30 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       k0 = -ceilf(c32 * fmaxf(gms, -1e30f)); k1 = -ceilf(c32 * fmaxf(gmt, -1e30f));
       const double fs = pow2_exact((int)(k0 - k0r)), ft = pow2_exact((int)(k1 - k1r));
       auto tot = [](const float2 a) { return (double)a.x + (double)a.y; };
-      double v[8] = {fs * tot(Ss), ft * tot(St), fs * tot(M1), fs * tot(M2), fs * tot(M3), ft * tot(N1),
-                     (mt_r == gmt) ? cand : CUDART_INF, fs * tot(M4)};
-#pragma unroll
-      for (int k = 0; k < 6; ++k) v[k] = warp_sum(v[k]);
-      v[6] = warp_min(v[6]);
-      v[7] = warp_sum(v[7]);
-      push(v, 8, parity);
-      if (warp < 8) {
+      // (the place of the argmax in the vector: its index, and the largest index where this CTA does not hold the maximum)
+      const double v[8] = {fs * tot(Ss), ft * tot(St), fs * tot(M1), fs * tot(M2), fs * tot(M3), ft * tot(N1), 0.0, fs * tot(M4)};
+      const uint32_t wc = __reduce_min_sync(0xffffffffu, mt_r == gmt ? cand : 0xffffffffu);
+      const double total = warp_sum8(v, lane);
+      push((lane >> 2) == 6 ? (double)wc : total, 8, parity);
+      if (warp == 0) {
         if (!mbar_wait_bounded(&mbar[1 + parity], parity ? xph1 : xph0)) dead = true;
-        const double g = gather(parity, warp, warp == 6);
-        if (lane == 0) gat[warp] = g;
+        const double g = gather(parity);
+        const double* const ci = red + (size_t)(parity * NV + 6) * NSLOT;
+        double am = 4294967295.0;
+        for (int slot = lane; slot < CS * CW; slot += 32) am = fmin(am, ci[slot]);
+        const uint32_t best = __reduce_min_sync(0xffffffffu, (uint32_t)am);
+        if ((lane & 3) == 0) gat[lane >> 2] = (lane >> 2) == 6 ? (double)best : g;
+        __syncwarp();
       }
       if (parity) xph1 ^= 1u; else xph0 ^= 1u;
       parity ^= 1;
-      __syncthreads();
+      if (tid < 2) {   // lane 0: the student's sum, lane 1: the teacher's; then lane 0 alone
+        double rS, G;
+        lse_of_sum(gat[lane], lane ? (double)k1 : (double)k0, rS, G);
+        const double rSt = __shfl_sync(0x3u, rS, 1), G1 = __shfl_sync(0x3u, G, 1);
+        if (tid == 0) scalar_after_lse_tail(bc, gat, K, k0, k1, x, bonus, masked, row_timeout, 1.f, false, rS, rSt, G, G1, gat + 7);
+      }
       if (tid == 0) {
-        scalar_after_lse(bc, gat, K, k0, k1, x, bonus, masked, row_timeout, gat + 7);
         if ((int)bc[BC_MODE] == MODE_SOLVE) mbar_expect_tx(&mbar[1 + parity], (uint32_t)(CS * CW * 5 * 8));
         else if ((int)bc[BC_MODE] == MODE_FINAL) mbar_expect_tx(&mbar[1 + parity], (uint32_t)(CS * CW * 3 * 8));
       }
@@ -312,31 +317,33 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       float2 S0[2] = {splat(0.f), splat(0.f)}, S1[2] = {splat(0.f), splat(0.f)}, S2[2] = {splat(0.f), splat(0.f)},
              S3[2] = {splat(0.f), splat(0.f)}, S4[2] = {splat(0.f), splat(0.f)};
       const float2 cc = splat(c32), cbb = splat(cb), kbb = splat(kb), neg1 = splat(-1.f);
+      for_chunks([&](int, const uint32_t* sw, const uint32_t* tw) {
 #pragma unroll
-      for (int i = 0; i < NPAIR; ++i) {
-        const int h = i & 1;
-        const float2 sf = unpack_fresh(sr[i]), tf = unpack_fresh(tr[i]);
-        const float2 d = ffma2(sf, neg1, tf);
-        const float2 e = ex2f2(ffma2(d, cbb, ffma2(sf, cc, kbb)));
-        S0[h] = fadd2(S0[h], e);
-        const float2 t1 = fmul2(e, d);
-        S1[h] = fadd2(S1[h], t1);
-        const float2 t2 = fmul2(t1, d);
-        S2[h] = fadd2(S2[h], t2);
-        S3[h] = ffma2(t2, d, S3[h]);
-        S4[h] = ffma2(t2, fmul2(d, d), S4[h]);
-      }
+        for (int i = 0; i < 4; ++i) {
+          const int h = i & 1;
+          const float2 sf = unpack_bf16x2(sw[i]), tf = unpack_bf16x2(tw[i]);
+          const float2 d = ffma2(sf, neg1, tf);
+          const float2 e = ex2f2(ffma2(d, cbb, ffma2(sf, cc, kbb)));
+          S0[h] = fadd2(S0[h], e);
+          const float2 t1 = fmul2(e, d);
+          S1[h] = fadd2(S1[h], t1);
+          const float2 t2 = fmul2(t1, d);
+          S2[h] = fadd2(S2[h], t2);
+          S3[h] = ffma2(t2, d, S3[h]);
+          S4[h] = ffma2(t2, fmul2(d, d), S4[h]);
+        }
+      });
       auto tot = [](const float2 (&a)[2]) { return ((double)a[0].x + (double)a[0].y) + ((double)a[1].x + (double)a[1].y); };
-      double v[5] = {warp_sum(tot(S0)), warp_sum(tot(S1)), warp_sum(tot(S2)), warp_sum(tot(S3)), warp_sum(tot(S4))};
-      push(v, 5, parity);
-      if (warp < 5) {
+      const double v[8] = {tot(S0), tot(S1), tot(S2), tot(S3), tot(S4), 0.0, 0.0, 0.0};
+      push(warp_sum8(v, lane), 5, parity);
+      if (warp == 0) {
         if (!mbar_wait_bounded(&mbar[1 + parity], parity ? xph1 : xph0)) dead = true;
-        const double g = gather(parity, warp, false);
-        if (lane == 0) gat[warp] = g;
+        const double g = gather(parity);
+        if ((lane & 3) == 0 && lane < 20) gat[lane >> 2] = g;
+        __syncwarp();
       }
       if (parity) xph1 ^= 1u; else xph0 ^= 1u;
       parity ^= 1;
-      __syncthreads();
       if (tid == 0) {
         scalar_after_solve4(bc, gat, K, k0, k1, x, bonus, masked);
         if ((int)bc[BC_MODE] == MODE_SOLVE) mbar_expect_tx(&mbar[1 + parity], (uint32_t)(CS * CW * 5 * 8));   // next evaluation
@@ -383,13 +390,12 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       float2 Sq[2] = {splat(0.f), splat(0.f)}, R[2] = {splat(0.f), splat(0.f)};
       const float2 cc = splat(c32), cll = splat(cl), kqq = splat(kq), kk0 = splat(k0), neg1 = splat(-1.f);
       const float2 iqq = splat(iq), nip = splat(-ip), kgg = splat(kg);
-#pragma unroll
-      for (int j = 0; j < CHUNKS; ++j) {
+      for_chunks([&](int e0, const uint32_t* sw, const uint32_t* tw) {
         uint32_t gp[4];
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-          const int i = 4 * j + k, h = k & 1;
-          const float2 sf = unpack_fresh(sr[i]), tf = unpack_fresh(tr[i]);
+          const int h = k & 1;
+          const float2 sf = unpack_bf16x2(sw[k]), tf = unpack_bf16x2(tw[k]);
           const float2 d = ffma2(sf, neg1, tf);
           const float2 ep = ex2f2(ffma2(sf, cc, kk0));
           const float2 eq = ex2f2(ffma2(d, cll, ffma2(sf, cc, kqq)));
@@ -400,13 +406,8 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
           const float2 gv = fmul2(ep, kgg);
           gp[k] = pack_bf16x2(gv.x, gv.y);
         }
-        if (want_g) {
-          int cj = j + rot;
-          if (cj == CHUNKS) cj = 0;
-          const int e0 = thr_first + cj * 8;
-          if (e0 < my_len) *reinterpret_cast<uint4*>(g_out + slice_start + e0) = make_uint4(gp[0], gp[1], gp[2], gp[3]);
-        }
-      }
+        if (want_g && e0 < my_len) *reinterpret_cast<uint4*>(g_out + slice_start + e0) = make_uint4(gp[0], gp[1], gp[2], gp[3]);
+      });
       const float sq_f = (Sq[0].x + Sq[0].y) + (Sq[1].x + Sq[1].y);
       const float r_f = (R[0].x + R[0].y) + (R[1].x + R[1].y);
       my_part = bonus ? sq_f * iq : r_f;
@@ -419,11 +420,11 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
           g_out[tok] = __float2bfloat16_rn(fmaf(ep, kg, -KGf));
         }
       }
-      double v[3] = {warp_sum((double)sq_f), warp_sum((double)r_f), warp_sum((double)my_part)};
-      push(v, 3, parity);
+      const double v[8] = {(double)sq_f, (double)r_f, (double)my_part, 0.0, 0.0, 0.0, 0.0, 0.0};
+      push(warp_sum8(v, lane), 3, parity);
       if (warp == 0) {
         if (!mbar_wait_bounded(&mbar[1 + parity], parity ? xph1 : xph0)) dead = true;
-        const double tv = gather(parity, 1, false);
+        const double tv = __shfl_sync(0xffffffffu, gather(parity), 4);
         if (lane == 0) {
           bc[BC_TV] = (bc[BC_LAMBDA] > 0.0) ? tv : 0.0;
           if (need_draw) scalar_find_owner(bc, red + (size_t)(parity * NV + 2) * NSLOT, CS * CW);
@@ -453,25 +454,11 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
         bool last_mode = take_last;
         if (hit) owner_lane = __ffs(hit) - 1;
         else { owner_lane = posm ? 31 - __clz(posm) : 0; last_mode = true; }
-        // the owning thread lays its 80 elements out in index order; the warp walks them together
-        uint32_t* scr_s = (uint32_t*)(smem + OFF_SCR);
-        uint32_t* scr_t = scr_s + NPAIR;
-        if (lane == owner_lane) {
-#pragma unroll
-          for (int j = 0; j < CHUNKS; ++j) {
-            int cj = j + rot;
-            if (cj == CHUNKS) cj = 0;
-            *reinterpret_cast<uint4*>(scr_s + cj * 4) = make_uint4(sr[4 * j], sr[4 * j + 1], sr[4 * j + 2], sr[4 * j + 3]);
-            *reinterpret_cast<uint4*>(scr_t + cj * 4) = make_uint4(tr[4 * j], tr[4 * j + 1], tr[4 * j + 2], tr[4 * j + 3]);
-          }
-        }
-        __syncwarp();
         double running = __shfl_sync(0xffffffffu, before + inc - (double)my_part, owner_lane);
         const int first = slice_start + (warp * 32 + owner_lane) * EPT;
         const int n_el = max(0, min(EPT, slice_start + my_len - first));
         int y = -1, last_pos = -1;
-        const __nv_bfloat16* es = (const __nv_bfloat16*)scr_s;
-        const __nv_bfloat16* et = (const __nv_bfloat16*)scr_t;
+        const __nv_bfloat16 *es = slot_s + (first - slice_start), *et = slot_t + (first - slice_start);   // the warp walks the owner's elements together
         for (int base = 0; base < n_el && y < 0; base += 32) {
           const int e = base + lane;
           float w = 0.f;

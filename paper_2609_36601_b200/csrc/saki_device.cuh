@@ -41,12 +41,6 @@ __device__ __forceinline__ float ex2f(float x) {
 __device__ __forceinline__ float2 unpack_bf16x2(uint32_t r) {
   return make_float2(__uint_as_float(r << 16), __uint_as_float(r & 0xffff0000u));
 }
-// Same, but opaque to the optimiser: each pass re-derives the floats from the
-// packed registers instead of keeping 160 unpacked values alive across passes.
-__device__ __forceinline__ float2 unpack_fresh(uint32_t r) {
-  asm volatile("" : "+r"(r));
-  return unpack_bf16x2(r);
-}
 __device__ __forceinline__ uint32_t max_bf16x2(uint32_t a, uint32_t b) {
   uint32_t d;
   asm("max.bf16x2 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(b));
@@ -190,10 +184,18 @@ __device__ __forceinline__ double warp_sum(double a) {
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   return a;
 }
-__device__ __forceinline__ double warp_min(double a) {
+// The sums over the warp of eight values at once: lane l ends up with the total of value l / 4.  A butterfly that halves
+// the number of values in its first three steps: 9 exchanges instead of 40.
+__device__ __forceinline__ double warp_sum8(const double (&v)[8], int lane) {
+  double a[4], b[2], c;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) a = fmin(a, __shfl_xor_sync(0xffffffffu, a, o));
-  return a;
+  for (int k = 0; k < 4; ++k) a[k] = (h4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, h4 ? v[k] : v[k + 4], 16);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) b[k] = (h3 ? a[k + 2] : a[k]) + __shfl_xor_sync(0xffffffffu, h3 ? a[k] : a[k + 2], 8);
+  c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
+  c += __shfl_xor_sync(0xffffffffu, c, 2);
+  return c + __shfl_xor_sync(0xffffffffu, c, 1);
 }
 
 struct Consts {   // per-launch constants of the scalar phases
@@ -348,14 +350,6 @@ SAKI_SCALAR_FN void scalar_after_lse_tail(double* bc, const double* v, Consts K,
   bc[BC_KB] = (double)(float)((1.0 - be) * k0 + be * k1);
   bc[BC_LO] = 0.0; bc[BC_HI] = 1.0; bc[BC_ITER] = 0.0; bc[BC_QSTATE] = 0.0;
   bc[BC_MODE] = MODE_SOLVE;
-}
-
-static __device__ __noinline__ void scalar_after_lse(double* bc, const double* v, Consts K, float k0f, float k1f, int x,
-                                              bool bonus, bool masked, bool row_timeout, const double* m4_raw = nullptr) {
-  double rSs, rSt, G0, G1;
-  lse_of_sum(v[0], (double)k0f, rSs, G0);
-  lse_of_sum(v[1], (double)k1f, rSt, G1);
-  scalar_after_lse_tail(bc, v, K, k0f, k1f, x, bonus, masked, row_timeout, 1.f, false, rSs, rSt, G0, G1, m4_raw);
 }
 
 // After one evaluation of pass "solve" that also carries the third and fourth moments:

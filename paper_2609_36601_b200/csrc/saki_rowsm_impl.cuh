@@ -121,19 +121,6 @@ __device__ __forceinline__ double warp_sum_d(double a) {
   for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
   return a;
 }
-// The sums over the warp of eight values at once: lane l ends up with the total of value l / 4.  A butterfly that halves
-// the number of values in its first three steps: 9 exchanges instead of 40.
-__device__ __forceinline__ double warp_sum8(const double (&v)[8], int lane) {
-  double a[4], b[2], c;
-  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) a[k] = (h4 ? v[k + 4] : v[k]) + __shfl_xor_sync(0xffffffffu, h4 ? v[k] : v[k + 4], 16);
-#pragma unroll
-  for (int k = 0; k < 2; ++k) b[k] = (h3 ? a[k + 2] : a[k]) + __shfl_xor_sync(0xffffffffu, h3 ? a[k] : a[k + 2], 8);
-  c = (h2 ? b[1] : b[0]) + __shfl_xor_sync(0xffffffffu, h2 ? b[0] : b[1], 4);
-  c += __shfl_xor_sync(0xffffffffu, c, 2);
-  return c + __shfl_xor_sync(0xffffffffu, c, 1);
-}
 // A bf16 value (as float) as an unsigned 16-bit key of the same order (-0 as +0), and back.
 __device__ __forceinline__ uint32_t bf16_key(float x) {
   const uint32_t b = __float_as_uint(x + 0.f);
