@@ -38,27 +38,28 @@ namespace saki {
 
 constexpr int CT = 256;                 // threads per CTA
 constexpr int CW = CT / 32;             // warps per CTA
-constexpr int CHUNKS = 10;              // 16-byte chunks (8 bf16) per thread per row
-constexpr int EPT = CHUNKS * 8;         // elements per thread
-constexpr int SLICE_CAP = CT * EPT;     // elements of one row a CTA can hold
-constexpr int MAX_CS = 8;
+constexpr int MAX_CHUNKS = 11;          // 16-byte chunks (8 bf16) per thread and row, at most; always an odd number: a thread's
+                                        // chunks are contiguous, and an odd stride keeps 128-bit shared loads free of conflicts
+constexpr int SLICE_CAP = CT * MAX_CHUNKS * 8;      // elements of one row a CTA can hold
+constexpr int MAX_V = 163840;
+constexpr int MAX_CS = 16;
 constexpr int NSLOT = MAX_CS * CW;      // per-warp partial slots of a cluster
 constexpr int NV = 8;                   // doubles per partial vector
 constexpr uint32_t SENTINEL = 0xFF7FFF7Fu;   // two bf16 "most negative finite": exp -> 0, difference 0
 
-constexpr int OFF_S = 0;
-constexpr int OFF_T = SLICE_CAP * 2;
-constexpr int OFF_RED = OFF_T + SLICE_CAP * 2;                  // [2][NV][NSLOT] doubles: per-warp partials
+constexpr int OFF_RED = 0;                                      // [2][NV][NSLOT] doubles: per-warp partials
 constexpr int OFF_MX = OFF_RED + 2 * NV * NSLOT * 8;            // [2][MAX_CS][2] doubles: per-CTA maxima
 constexpr int OFF_GAT = OFF_MX + 2 * MAX_CS * 2 * 8;            // [NV] doubles: cluster totals
 constexpr int OFF_BC = OFF_GAT + NV * 8;                        // [2][BC_DOUBLES] broadcast scalars
 constexpr int OFF_WMAX = OFF_BC + 2 * BC_DOUBLES * 8;           // [2][2][CW] floats: per-warp maxima
 constexpr int OFF_MBAR = OFF_WMAX + 2 * 2 * CW * 4;             // copy barrier, 2 exchange barriers, 2 maxima barriers
-constexpr int SMEM_BYTES = OFF_MBAR + 5 * 8 + 8;
+constexpr int OFF_S = (OFF_MBAR + 5 * 8 + 127) / 128 * 128;     // the slice of the student's row, then the teacher's
+static int slice_of(int V, int cs) { return ((V + cs - 1) / cs + 7) & ~7; }
+static int smem_bytes(int slice_len) { return OFF_S + 2 * ((slice_len * 2 + 127) / 128 * 128); }
 static_assert(OFF_MBAR % 8 == 0, "alignment");
 
 template <int CS>
-__global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const int n_clusters) {
+__global__ void __launch_bounds__(CT, CS > 8 ? 1 : 2) cluster_kernel(const RowParams P, const int n_clusters) {
   extern __shared__ __align__(128) unsigned char smem[];
   launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -66,7 +67,6 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
   const int cluster_id = blockIdx.x / CS;
 
   const __nv_bfloat16* slot_s = (const __nv_bfloat16*)(smem + OFF_S);
-  const __nv_bfloat16* slot_t = (const __nv_bfloat16*)(smem + OFF_T);
   double* red = (double*)(smem + OFF_RED);
   double* mx = (double*)(smem + OFF_MX);
   double* gat = (double*)(smem + OFF_GAT);
@@ -76,11 +76,13 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
 
   const int V = P.V;
   const int slice_len = ((V + CS - 1) / CS + 7) & ~7;
+  const int off_t = OFF_S + (slice_len * 2 + 127) / 128 * 128;
+  const __nv_bfloat16* slot_t = (const __nv_bfloat16*)(smem + off_t);
   const int slice_start = (int)rank * slice_len;
   const int my_len = max(0, min(slice_len, V - slice_start));
   const uint32_t slice_bytes = (uint32_t)my_len * 2u;
-  const int rot = (tid >> 2) & 1;          // chunk rotation: conflict-free 128-bit shared loads
-  const int thr_first = tid * EPT;         // first element (within the slice) of this thread
+  const int chunks = ((slice_len + 8 * CT - 1) / (8 * CT)) | 1;     // per thread
+  const int ept = chunks * 8, thr_first = tid * ept;                // elements of a thread, its first within the slice
 
   const float c32 = (float)(1.4426950408889634 / (double)P.temperature);     // log2(e)/temperature
   Consts K;
@@ -100,7 +102,7 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
     mbar_expect_tx(&mbar[0], 2u * slice_bytes);
     if (slice_bytes) {
       bulk_load(smem + OFF_S, s + slice_start, slice_bytes, &mbar[0]);
-      bulk_load(smem + OFF_T, t + slice_start, slice_bytes, &mbar[0]);
+      bulk_load(smem + off_t, t + slice_start, slice_bytes, &mbar[0]);
     }
   };
   // one exchange: every warp's totals, value lane / 4 in each lane (n of them), to slot rank*CW+warp of red[p] in every CTA
@@ -122,14 +124,44 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
     a += __shfl_xor_sync(0xffffffffu, a, 1);
     return a;
   };
-  // this thread's chunks of the slice, in an order that keeps 128-bit shared loads free of conflicts: body(first element
-  // within the slice, student, teacher); beyond the slice's end the elements are "most negative finite"
+  // warp 0, for a draw: the warp of the cluster that owns the inverse-CDF target (ordered scan of the warps' weights)
+  auto find_owner = [&](double* bc, const double* weight) {
+    constexpr int NW = CS * CW, PER = NW > 32 ? NW / 32 : 1;
+    double w[PER], mine = 0.0;
+#pragma unroll
+    for (int q = 0; q < PER; ++q) {
+      w[q] = lane * PER + q < NW ? weight[lane * PER + q] : 0.0;
+      mine += w[q];
+    }
+    double inc = mine;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const double up = __shfl_up_sync(0xffffffffu, inc, o);
+      if (lane >= o) inc += up;
+    }
+    const double target = bc[BC_UDRAW] * __shfl_sync(0xffffffffu, inc, 31);
+    const unsigned hit = __ballot_sync(0xffffffffu, inc > target), pos = __ballot_sync(0xffffffffu, mine > 0.0);
+    // rounding left no crossing: the last position with positive weight
+    if (lane == (hit ? __ffs(hit) - 1 : pos ? 31 - __clz(pos) : 0)) {
+      double before = inc - mine;
+      int owner = 0;
+#pragma unroll
+      for (int q = 0; q < PER - 1; ++q)
+        if (owner == q && (hit ? !(before + w[q] > target) : true)) { before += w[q]; ++owner; }
+      if (!hit) {
+#pragma unroll
+        for (int q = 0; q < PER; ++q) if (w[q] > 0.0) owner = q;
+        before = 0.0;
+      }
+      bc[BC_OWNER_WARP] = (double)(lane * PER + owner); bc[BC_BEFORE] = before; bc[BC_TARGET] = target; bc[BC_TAKE_LAST] = hit ? 0.0 : 1.0;
+    }
+  };
+  // this thread's chunks of the slice: body(first element within the slice, student, teacher); beyond the slice's end the
+  // elements are "most negative finite"
   auto for_chunks = [&](auto&& body) {
 #pragma unroll 2
-    for (int j = 0; j < CHUNKS; ++j) {
-      int cj = j + rot;
-      if (cj >= CHUNKS) cj -= CHUNKS;
-      const int e0 = thr_first + cj * 8;
+    for (int j = 0; j < chunks; ++j) {
+      const int e0 = thr_first + j * 8;
       uint4 a = make_uint4(SENTINEL, SENTINEL, SENTINEL, SENTINEL), b = a;
       if (e0 < my_len && !dead) {
         a = *reinterpret_cast<const uint4*>(slot_s + e0);
@@ -367,13 +399,9 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
         }
       }
       if (g_out && !redo) {
-#pragma unroll
-        for (int j = 0; j < CHUNKS; ++j) {
-          int cj = j + rot;
-          if (cj == CHUNKS) cj = 0;
-          const int e0 = thr_first + cj * 8;
-          if (e0 < my_len) *reinterpret_cast<uint4*>(g_out + slice_start + e0) = make_uint4(0, 0, 0, 0);
-        }
+#pragma unroll 1
+        for (int e0 = thr_first; e0 < min(thr_first + ept, my_len); e0 += 8)
+          *reinterpret_cast<uint4*>(g_out + slice_start + e0) = make_uint4(0, 0, 0, 0);
       }
       continue;
     }
@@ -415,7 +443,7 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       if (want_g) {
         const int tok = (int)bc[BC_TOK];
         const int loc = tok - slice_start - thr_first;
-        if (tok >= 0 && loc >= 0 && loc < EPT && tok - slice_start < my_len) {
+        if (tok >= 0 && loc >= 0 && loc < ept && tok - slice_start < my_len) {
           const float ep = ex2f(fmaf(__bfloat162float(g_s[tok]), c32, k0));
           g_out[tok] = __float2bfloat16_rn(fmaf(ep, kg, -KGf));
         }
@@ -425,10 +453,10 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
       if (warp == 0) {
         if (!mbar_wait_bounded(&mbar[1 + parity], parity ? xph1 : xph0)) dead = true;
         const double tv = __shfl_sync(0xffffffffu, gather(parity), 4);
+        if (lane == 0) bc[BC_TV] = (bc[BC_LAMBDA] > 0.0) ? tv : 0.0;
+        if (need_draw) find_owner(bc, red + (size_t)(parity * NV + 2) * NSLOT);
         if (lane == 0) {
-          bc[BC_TV] = (bc[BC_LAMBDA] > 0.0) ? tv : 0.0;
-          if (need_draw) scalar_find_owner(bc, red + (size_t)(parity * NV + 2) * NSLOT, CS * CW);
-          else if (rank == 0) write_result(bc, P.out, !P.spec, row, 0, x, false, K.c64, g_s, g_t);
+          if (!need_draw && rank == 0) write_result(bc, P.out, !P.spec, row, 0, x, false, K.c64, g_s, g_t);
         }
       }
       if (parity) xph1 ^= 1u; else xph0 ^= 1u;
@@ -455,8 +483,8 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
         if (hit) owner_lane = __ffs(hit) - 1;
         else { owner_lane = posm ? 31 - __clz(posm) : 0; last_mode = true; }
         double running = __shfl_sync(0xffffffffu, before + inc - (double)my_part, owner_lane);
-        const int first = slice_start + (warp * 32 + owner_lane) * EPT;
-        const int n_el = max(0, min(EPT, slice_start + my_len - first));
+        const int first = slice_start + (warp * 32 + owner_lane) * ept;
+        const int n_el = max(0, min(ept, slice_start + my_len - first));
         int y = -1, last_pos = -1;
         const __nv_bfloat16 *es = slot_s + (first - slice_start), *et = slot_t + (first - slice_start);   // the warp walks the owner's elements together
         for (int base = 0; base < n_el && y < 0; base += 32) {
@@ -493,15 +521,17 @@ __global__ void __launch_bounds__(CT, 2) cluster_kernel(const RowParams P, const
 }
 
 // ---------------------------------------------------------------- host side
-static int pick_cs(int V) {
+// CTAs per row: as many as a row needs (a slice fits a CTA's shared memory), and more while every CTA still has an SM to
+// itself and 4096 elements or more.
+static int pick_cs(int V, int64_t rows, int sms) {
   int cs = 1;
-  while (cs * SLICE_CAP < V) cs *= 2;
+  while (cs < MAX_CS && (cs * SLICE_CAP < V || (V >= 8192 * cs && rows * 2 * cs <= sms))) cs *= 2;
   return cs;
 }
 
 bool cluster_can_serve(const RowParams& p, int dtype) {
   if (dtype != SAKI_BF16) return false;
-  if (p.V < 2048 || p.V % 8 != 0 || p.V > MAX_CS * SLICE_CAP) return false;
+  if (p.V < 2048 || p.V % 8 != 0 || p.V > MAX_V) return false;
   if (p.n_rows > 0x7fffffffLL) return false;     // the redo list keeps row numbers in 32 bits
   auto al16 = [](const void* q) { return ((uintptr_t)q & 15) == 0; };
   if (!al16(p.s) || !al16(p.t)) return false;
@@ -512,6 +542,7 @@ bool cluster_can_serve(const RowParams& p, int dtype) {
 
 template <int CS>
 static cudaError_t launch_cs(const RowParams& p, cudaStream_t st) {
+  static_assert(CS <= MAX_CS, "partial slots");
   static std::mutex mu;
   static int cached_dev = -1, cached_clusters = 0;
   auto kern = cluster_kernel<CS>;
@@ -523,25 +554,28 @@ static cudaError_t launch_cs(const RowParams& p, cudaStream_t st) {
   at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
   at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[1].val.programmaticStreamSerializationAllowed = 1;
-  cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = SMEM_BYTES; cfg.stream = st;
+  cfg.blockDim = dim3(CT); cfg.dynamicSmemBytes = smem_bytes(SLICE_CAP); cfg.stream = st;
   cfg.attrs = at; cfg.numAttrs = 1;
   int n_clusters;
   {
     std::lock_guard<std::mutex> lock(mu);
     if (cached_dev != dev) {
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(SLICE_CAP));
+      if (e == cudaSuccess && CS > 8) e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
       cfg.gridDim = dim3(CS * 64);
       int n = 0;
       e = cudaOccupancyMaxActiveClusters(&n, kern, &cfg);
       if (e != cudaSuccess) return e;
-      if (n < 1) return cudaErrorLaunchOutOfResources;
+      if (n < 1 && CS <= 8) return cudaErrorLaunchOutOfResources;
       cached_clusters = n; cached_dev = dev;
     }
     n_clusters = cached_clusters;
   }
+  if (CS > 8 && n_clusters < p.n_rows) return launch_cs<8>(p, st);       // (clusters of 16 need that many SMs in one part of the chip)
   if ((int64_t)n_clusters > p.n_rows) n_clusters = (int)p.n_rows;
   cfg.gridDim = dim3(CS * n_clusters);
+  cfg.dynamicSmemBytes = smem_bytes(slice_of(p.V, CS));
   cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, kern, p, n_clusters);
 }
@@ -549,12 +583,16 @@ static cudaError_t launch_cs(const RowParams& p, cudaStream_t st) {
 cudaError_t launch_cluster(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
   *served = false;
   if (p.n_rows <= 0) { *served = true; return cudaSuccess; }
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaError_t e;
-  switch (pick_cs(p.V)) {
+  switch (pick_cs(p.V, p.call_rows, sms)) {
     case 1: e = launch_cs<1>(p, st); break;
     case 2: e = launch_cs<2>(p, st); break;
     case 4: e = launch_cs<4>(p, st); break;
-    default: e = launch_cs<8>(p, st); break;
+    case 8: e = launch_cs<8>(p, st); break;
+    default: e = launch_cs<16>(p, st); break;
   }
   if (e == cudaSuccess) { *served = true; if (n_launches) *n_launches += 1; }
   return e;

@@ -502,26 +502,6 @@ SAKI_SCALAR_FN void scalar_after_solve4(double* bc, const double* v, Consts K, f
   }
 }
 
-// for a draw: the warp that owns the inverse-CDF target (ordered scan of per-warp weights)
-static __device__ __noinline__ void scalar_find_owner(double* bc, const double* warp_part, int n_warps) {
-  double total = 0.0;
-  for (int w = 0; w < n_warps; ++w) total += warp_part[w];
-  const double target = bc[BC_UDRAW] * total;
-  int owner = -1;
-  double before = 0.0;
-  for (int w = 0; w < n_warps; ++w) {
-    if (before + warp_part[w] > target) { owner = w; break; }
-    before += warp_part[w];
-  }
-  double take_last = 0.0;
-  if (owner < 0) {   // rounding left no crossing: last position with positive weight
-    take_last = 1.0; before = 0.0;
-    for (int w = n_warps - 1; w >= 0; --w) if (warp_part[w] > 0.0) { owner = w; break; }
-    if (owner < 0) owner = 0;
-  }
-  bc[BC_OWNER_WARP] = (double)owner; bc[BC_BEFORE] = before; bc[BC_TARGET] = target; bc[BC_TAKE_LAST] = take_last;
-}
-
 // tv: the row's total variation (the caller may hold it before bc[BC_TV] is written)
 SAKI_SCALAR_FN void write_result_tv(const double* bc, saki_out out, bool write_loss, int64_t row, int corrected,
                                              int y, bool bonus, double c64, const __nv_bfloat16* g_s,
