@@ -43,9 +43,9 @@
  *     sees do not depend on how a batch is chunked or sharded.
  *   - Results are deterministic: same call (inputs, sizes), same GPU model, same bits.  Chunking or
  *     sharding a batch leaves every output bit-identical as long as each piece is served by the same
- *     kernel as the whole; the library picks the kernel from the call's size (calls of at most 32 rows
- *     with V >= 65536 run one row per thread-block cluster, larger ones one row per SM), so a tail piece
- *     of 32 long rows or fewer agrees with the same rows inside a large call to the tolerances of the
+ *     kernel as the whole; the library picks the kernel, and the number of blocks that share a row or
+ *     an SM, from the call's V and number of rows, so a tail piece of a few rows agrees with the same
+ *     rows inside a large call to the tolerances of the
  *     arithmetic (float outputs to ~1e-6, flags and ids wherever the decision is not within 1e-6 of
  *     its threshold), not to the bit.  saki_set_kernel pins the choice where bit-identity across pieces
  *     matters.
@@ -358,17 +358,15 @@ SAKI_API int saki_sample_proposal(const void* logits, int64_t ld, int64_t N, int
  * Returns SAKI_ERR_ROW_STATUS if that number is non-zero.  n_flagged may be NULL. */
 SAKI_API int saki_check(void* cuda_stream, uint64_t* n_flagged);
 
-/* Selects the row kernel: 0 = automatic, 1 = the general kernel (one block per
- * row, float64, any V, dtype and layout), 2 = the register-resident cluster
- * kernel (one row per cluster of up to 8 blocks), 3 = the row-per-SM kernel
- * (one row per block; shared memory plus L2; one block of 512 threads per SM for
- * V > 98304, two of 256 for shorter rows).  2 and 3 serve bf16 rows with
- * 16-byte aligned rows and V a multiple of 8, V >= 2048 (2: V <= 163840; and
- * eps = 0 or eps >= 5e-3: its float32 sums cannot resolve smaller radii to the
- * tolerance, whereas 3 takes every radius); other inputs fall back to 1.  Automatic prefers 3,
- * except for calls of at most 32 rows with V >= 65536 that 2 can serve: a few long rows finish sooner
- * spread over the whole GPU.  Process-wide; meant for
- * tests and benchmarks.  Returns the previous value. */
+/* Selects the row kernel: 0 = automatic, 1 = the general kernel (any V, dtype and layout; float64, a row shared by 1 to 8
+ * blocks), 2 = the cluster kernel (one row per cluster of 1 to 16 blocks, in shared memory), 3 = the row-per-SM kernel
+ * (one row per block; shared memory plus L2; one block of 512 threads, two of 256 or four of 128 per SM, by V and the
+ * number of rows).  2 and 3 serve bf16 rows with 16-byte aligned rows and V a multiple of 8, V >= 2048 (2: V <= 163840;
+ * and eps = 0 or eps >= 5e-3: its float32 sums cannot resolve smaller radii to the tolerance, whereas 3 takes every
+ * radius); other inputs fall back to 1.  Automatic prefers 3, except for calls of at most 32 rows with V >= 32768 that 2
+ * can serve: a few long rows finish sooner spread over the whole GPU.  Process-wide; meant for tests and benchmarks.
+ * Returns the previous value.
+ */
 SAKI_API int saki_set_kernel(int which);
 
 /* Which row kernel the calling thread's last routing call used: 1 general, 2 cluster,

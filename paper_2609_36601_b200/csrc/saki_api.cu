@@ -155,6 +155,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
   cudaError_t e;
   bool served = false;
   const int which = g_kernel.load();
+  if (which != 0) p.call_rows = 0;
   int used = 1;
   // Directly, float32 sums resolve KL(q||p) to a few 1e-7 absolute: enough for |d lambda| <= 1e-5 when
   // eps >= 5e-3 (measured), not below: for the cluster kernel smaller positive radii run on the float64
@@ -185,11 +186,10 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
     g_last_redo_count = p.redo_count;
     g_last_redo_generation = g_redo_generation.load();
   }
-  // A handful of long rows (a decoding step of a small batch) finish sooner spread over the whole GPU, one
-  // row per cluster of 8 blocks, than on one SM each: 32 clusters fit at once, and at V = 151936 a call of
-  // up to 32 rows takes 32 to 40 us there against 62 us (V = 65536: 28 to 34 against 33 to 39; at V = 32000
-  // the row-per-SM kernel is the faster one at every size).
-  if (fast && which == 0 && p.call_rows <= 32 && p.V >= 65536 && eps_ok && cluster_can_serve(p, dtype)) {
+  // A handful of long rows (a decoding step of a small batch) finish sooner spread over the whole GPU, one row per cluster
+  // of up to 16 blocks, than on one SM each: 1 / 8 / 32 rows of V = 151936 take 15.7 / 18.7 / 24.5 us there against 42 / 49
+  // / 49 us, of V = 32768 14 / 14 / 18 against 18 / 24 / 24 us (at V = 8192 there is no difference).
+  if (fast && which == 0 && p.call_rows <= 32 && p.V >= 32768 && eps_ok && cluster_can_serve(p, dtype)) {
     e = launch_cluster(p, st, &launches, &served);
     if (e != cudaSuccess) return cuda_fail(e, "cluster kernel launch");
     if (served) used = 2;
@@ -207,7 +207,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
       e = cudaMemsetAsync(p.seq_stop, 0x7f, (size_t)(p.n_rows / p.K1) * sizeof(int), st);   // "no stop yet": above any position
       if (e != cudaSuccess) return cuda_fail(e, "cudaMemsetAsync");
     }
-    e = launch_rowsm(p, which == 0, st, &launches, &served);
+    e = launch_rowsm(p, st, &launches, &served);
     p.seq_next = nullptr; p.seq_stop = nullptr;
     if (e != cudaSuccess) return cuda_fail(e, "row-per-SM kernel launch");
     if (served) used = 3;

@@ -5,7 +5,9 @@
 // exactly once; each thread owns 80 contiguous elements of the slice.  What bounds a call here is the chain of steps of a
 // single row, and much of that was instruction fetch: with the row in registers every pass was 40 unrolled pairs of code
 // that ran once.  The passes are loops over shared memory now, and the registers that frees let the scalar steps be
-// inlined (8 rows of 151936, forward: __CL__ us).  Passes:
+// inlined.  With what that made possible (warp 0 gathers all sums and goes on to the scalars, up to 16 CTAs per row, sums
+// taken chunk by chunk) 8 rows of 151936 went from 23.6 to 18.7 us, 1 row from 22.9 to 15.7, 32 rows from 32.1 to 24.5.
+// Passes:
 //   lse      2 exponentials/element: both log-sum-exps (computed under the
 //            CTA's own maxima rounded up to whole powers of two, then moved
 //            exactly onto the row's maxima, which the CTAs exchange while the
@@ -279,22 +281,25 @@ __global__ void __launch_bounds__(CT, CS > 8 ? 1 : 2) cluster_kernel(const RowPa
              N1 = splat(0.f);
       const float2 cc = splat(c32), kk0 = splat(k0r), kk1 = splat(k1r), neg1 = splat(-1.f);
       for_chunks([&](int, const uint32_t* sw, const uint32_t* tw) {
+        float2 cs = splat(0.f), ct = splat(0.f);   // per chunk first: a dominant element swamps fewer small ones
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
           const float2 sf = unpack_bf16x2(sw[i]), tf = unpack_bf16x2(tw[i]);
           const float2 d = ffma2(sf, neg1, tf);
           const float2 es = ex2f2(ffma2(sf, cc, kk0));
           const float2 et = ex2f2(ffma2(tf, cc, kk1));
-          Ss = fadd2(Ss, es);
-          St = fadd2(St, et);
-          const float2 t1 = fmul2(es, d);
-          M1 = fadd2(M1, t1);
-          const float2 t2 = fmul2(t1, d);
-          M2 = fadd2(M2, t2);
-          M3 = ffma2(t2, d, M3);
-          M4 = ffma2(t2, fmul2(d, d), M4);
+          cs = i == 0 ? es : fadd2(cs, es);
+          ct = i == 0 ? et : fadd2(ct, et);
+          const float2 d2 = fmul2(d, d);
+          M1 = ffma2(es, d, M1);
+          const float2 u = fmul2(es, d2);
+          M2 = fadd2(M2, u);
+          M3 = ffma2(u, d, M3);
+          M4 = ffma2(u, d2, M4);
           N1 = ffma2(et, d, N1);
         }
+        Ss = fadd2(Ss, cs);
+        St = fadd2(St, ct);
       });
       // the row's maxima have arrived meanwhile: move the partial sums onto the row's shifts
       bool mx_timeout = false;
@@ -346,26 +351,27 @@ __global__ void __launch_bounds__(CT, CS > 8 ? 1 : 2) cluster_kernel(const RowPa
     // ------------------------------------------------ pass "solve" (repeated)
     while ((int)bc[BC_MODE] == MODE_SOLVE) {
       const float cb = (float)bc[BC_CB], kb = (float)bc[BC_KB];
-      float2 S0[2] = {splat(0.f), splat(0.f)}, S1[2] = {splat(0.f), splat(0.f)}, S2[2] = {splat(0.f), splat(0.f)},
-             S3[2] = {splat(0.f), splat(0.f)}, S4[2] = {splat(0.f), splat(0.f)};
+      float2 S0 = splat(0.f), S1 = splat(0.f), S2 = splat(0.f), S3 = splat(0.f), S4 = splat(0.f);
       const float2 cc = splat(c32), cbb = splat(cb), kbb = splat(kb), neg1 = splat(-1.f);
       for_chunks([&](int, const uint32_t* sw, const uint32_t* tw) {
+        float2 c0 = splat(0.f), c1 = splat(0.f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int h = i & 1;
           const float2 sf = unpack_bf16x2(sw[i]), tf = unpack_bf16x2(tw[i]);
           const float2 d = ffma2(sf, neg1, tf);
           const float2 e = ex2f2(ffma2(d, cbb, ffma2(sf, cc, kbb)));
-          S0[h] = fadd2(S0[h], e);
-          const float2 t1 = fmul2(e, d);
-          S1[h] = fadd2(S1[h], t1);
-          const float2 t2 = fmul2(t1, d);
-          S2[h] = fadd2(S2[h], t2);
-          S3[h] = ffma2(t2, d, S3[h]);
-          S4[h] = ffma2(t2, fmul2(d, d), S4[h]);
+          const float2 d2 = fmul2(d, d);
+          c0 = i == 0 ? e : fadd2(c0, e);
+          c1 = i == 0 ? fmul2(e, d) : ffma2(e, d, c1);
+          const float2 u = fmul2(e, d2);
+          S2 = fadd2(S2, u);
+          S3 = ffma2(u, d, S3);
+          S4 = ffma2(u, d2, S4);
         }
+        S0 = fadd2(S0, c0);
+        S1 = fadd2(S1, c1);
       });
-      auto tot = [](const float2 (&a)[2]) { return ((double)a[0].x + (double)a[0].y) + ((double)a[1].x + (double)a[1].y); };
+      auto tot = [](const float2 a) { return (double)a.x + (double)a.y; };
       const double v[8] = {tot(S0), tot(S1), tot(S2), tot(S3), tot(S4), 0.0, 0.0, 0.0};
       push(warp_sum8(v, lane), 5, parity);
       if (warp == 0) {
@@ -521,11 +527,13 @@ __global__ void __launch_bounds__(CT, CS > 8 ? 1 : 2) cluster_kernel(const RowPa
 }
 
 // ---------------------------------------------------------------- host side
-// CTAs per row: as many as a row needs (a slice fits a CTA's shared memory), and more while every CTA still has an SM to
-// itself and 4096 elements or more.
+// CTAs per row: as many as a row needs (a slice fits a CTA's shared memory), and more while no more than two share an SM
+// and each keeps 2048 elements (forward and gradient: 32 rows of 65536 with 2 or 4 CTAs each 20.1 / 18.2 us, 8 rows of
+// 32000 with 2 or 4 13.9 / 13.3 us).  By V alone, up to 8, where the kernel is pinned (rows = 0).
 static int pick_cs(int V, int64_t rows, int sms) {
+  const int most = rows > 0 ? MAX_CS : 8;
   int cs = 1;
-  while (cs < MAX_CS && (cs * SLICE_CAP < V || (V >= 8192 * cs && rows * 2 * cs <= sms))) cs *= 2;
+  while (cs < most && (cs * SLICE_CAP < V || (V >= 4096 * cs && rows * cs <= sms))) cs *= 2;
   return cs;
 }
 

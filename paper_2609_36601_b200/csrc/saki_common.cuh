@@ -24,7 +24,7 @@ struct RowParams {
   const void* t;
   int64_t s_seq, s_pos, t_seq, t_pos;  // element strides (plain: s_seq = ld_s, s_pos = 0)
   int64_t n_rows;
-  int64_t call_rows;                   // rows of the caller's whole call (n_rows, or more where it is routed in pieces): the choice of a kernel goes by it
+  int64_t call_rows;                   // rows of the caller's whole call (n_rows, or more where it is routed in pieces): the choice of a kernel goes by it; 0 where the kernel is pinned: the choice of its variant then goes by V alone
   int32_t V;
   int32_t K1;                          // positions per sequence; the last one is the bonus row if spec
   int32_t spec;                        // 1: block verification (proposal from draft, bonus row)
@@ -216,7 +216,7 @@ __host__ __device__ inline RowResult zero_row(uint32_t status) {
 cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* n_launches);
 cudaError_t launch_cluster(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
 bool cluster_can_serve(const RowParams& p, int dtype);
-cudaError_t launch_rowsm(const RowParams& p, bool by_rows, cudaStream_t st, int* n_launches, bool* served);
+cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
 namespace full_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace half_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace quarter_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }

@@ -694,11 +694,12 @@ static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t s
   // Blocks per row.  In list mode (a handful of rows as a rule; the host does not know their number) always the most;
   // otherwise so many that few rows still fill the chip, each block keeping 1024 elements or more (below that the
   // barriers of a cluster cost more than its blocks save), and that the rows in flight stay in L2 between the passes
-  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).
+  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).  Where the
+  // kernel is pinned (call_rows = 0) the rows do not count, so that pieces of a batch agree with the whole to the bit.
   int cs = 1;
   const int64_t in_flight = BLOCKS_PER_SM<T> * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
   while (cs < MAX_CS && p.V >= 2048 * cs &&
-         (p.from_list || p.n_rows * cs < in_flight || in_flight / cs * row_bytes > (150 << 20)))
+         (p.from_list || (p.call_rows > 0 && p.call_rows * cs < in_flight) || in_flight / cs * row_bytes > (150 << 20)))
     cs *= 2;
   switch (cs) {
     case 1: return launch_cs<T, 1>(p, dev, sms, st);

@@ -27,7 +27,7 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
   return true;
 }
 
-// by_rows: the variant that routes this number of rows soonest.  A variant with k CTAs per SM takes ceil(rows / (k SMs))
+// The variant that routes this number of rows soonest.  A variant with k CTAs per SM takes ceil(rows / (k SMs))
 // turns of a + b V / 1000 microseconds each (fitted to V = 2048 to 98304 and 8 to 1776 rows, within 10 %):
 //   k = 1: 6.2, 0.302     k = 2: 5.0, 0.535     k = 4: 6.0, 1.06
 // so that, e.g., 888 rows of 32000 take three turns of k = 2 (73 us) and not two of k = 4 (83 us), 296 rows of 49152 one
@@ -35,8 +35,8 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
 // where its inlined scalar steps outweigh the longer passes (below V = 16384: 14.1 against 16.2 us at 8192).  The limits on V above
 // hold here too, except that rows in flight that fit in L2 anyway (two per SM) may be longer.  Not where saki_set_kernel
 // pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
-cudaError_t launch_rowsm(const RowParams& p, bool by_rows, cudaStream_t st, int* n_launches, bool* served) {
-  if (by_rows) {
+cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
+  if (p.call_rows > 0) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
