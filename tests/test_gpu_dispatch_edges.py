@@ -1,0 +1,71 @@
+"""Where a call goes from one form of a kernel to the next: cluster kernel with 1, 2, 4, 8 and 16 CTAs per row, the
+row-per-SM kernel with one, two or four rows per SM by the number of rows, the lm-head GEMM with one CTA or two per
+tile.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
+import numpy as np
+import pytest
+import torch
+
+import oracle as O
+import paper_2609_36601_b200 as P
+from paper_2609_36601_b200 import synth
+from parity import bf16_ulp, compare_rows, grad_check, oracle_inputs, to_np64
+
+pytestmark = pytest.mark.gpu
+DEV = "cuda:0"
+
+
+def _check(w, rows, kernel, used):
+    d = synth.generate(w, DEV)
+    prev = P.set_kernel(kernel)
+    try:
+        out, g = P.route_fwd_bwd(d["s"], d["t"], d["proposal"], w.eps, w.temperature, w.seed, grad_scale=0.25)
+        torch.cuda.synchronize()
+        assert P.last_kernel() == used
+    finally:
+        P.set_kernel(prev)
+    s64, t64 = oracle_inputs(d)
+    ref = O.route(s64, t64, d["proposal"].cpu().numpy(), w.eps, w.temperature, w.seed, grad_scale=0.25, want_grad=True,
+                  grad_dtype=w.dtype, rows=rows)
+    compare_rows(out, ref, rows)
+    same = out["corrected"].cpu().numpy()[rows] == ref["corrected"]
+    tok = np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[same]
+    grad_check(to_np64(g)[rows][same], ref["grad"][same], w.dtype, tok)
+
+
+# pinned, the number of CTAs goes by V alone (1, 1, 2, 4, 4, 8, 8); rows end in chunk remainders, and the last CTA's slice
+# is short or (8200: a chunk more than 4 x 2048) all but one chunk of a thread's share is empty
+@pytest.mark.parametrize("V,N", [(2048, 5), (4088, 5), (4096, 5), (8200, 5), (16376, 4), (16384, 4), (163840, 2)])
+def test_cluster_sizes_by_v(V, N):
+    _check(synth.Workload("t", N, V, "bf16", 0.125, 1.5, True, 401, 51, temperature=0.875), list(range(N)), 2, 2)
+
+
+# as dispatched: 16 CTAs per row up to 18 rows (148 SMs), 8 from 19 on; the shortest and the longest row of the rule
+@pytest.mark.parametrize("V,N", [(32768, 1), (32768, 18), (32776, 19), (65528, 32), (151936, 9), (163840, 18), (163840, 32)])
+def test_cluster_sizes_by_rows(V, N):
+    _check(synth.Workload("t", N, V, "bf16", 0.125, 1.5, True, 402, 52), sorted({0, N // 2, N - 1}), 0, 2)
+
+
+# the last row that fits a turn and the first that does not, for one, two and four rows per SM
+@pytest.mark.parametrize("V", [8192, 16384, 30008, 49152])
+@pytest.mark.parametrize("N", [148, 149, 296, 297, 592, 593])
+def test_rows_per_sm_by_rows(V, N):
+    _check(synth.Workload("t", N, V, "bf16", 0.125, 1.5, True, 403, 53), [0, N // 2, N - 1], 0, 3)
+
+
+@pytest.mark.parametrize("N", [1, 127, 128, 129, 255, 256, 257, 511, 513])
+@pytest.mark.parametrize("V", [264, 4096])
+def test_lmhead_tiles_by_rows(N, V):
+    d = 72
+    gen = torch.Generator(device=DEV).manual_seed(N)
+    h = torch.randn((N, d), generator=gen, device=DEV).to(torch.bfloat16)
+    w = (torch.randn((V, d), generator=gen, device=DEV) * 0.25).to(torch.bfloat16)
+    logits, row_max, lse = P.lmhead_lse(h, w, 1.0)
+    h64, w64 = to_np64(h), to_np64(w)
+    ref, _, _ = O.lmhead_lse(h64, w64, 1.0)
+    got = to_np64(logits)
+    # a bf16 step, plus the float32 accumulation of d products: d 2^-24 of the sum of their magnitudes, here under 2^-17 of it
+    assert np.all(np.abs(got - ref) <= bf16_ulp(ref) * 1.0000001 + 2.0 ** -17 * (np.abs(h64) @ np.abs(w64).T))
+    m = got.max(axis=1)
+    own = m + np.log(np.exp(got - m[:, None]).sum(axis=1))
+    assert np.array_equal(row_max.cpu().numpy().astype(np.float64), m)
+    assert np.max(np.abs(lse.cpu().numpy() - own)) <= 2e-6 * (1 + np.max(np.abs(own)))
