@@ -69,3 +69,14 @@ def test_lmhead_tiles_by_rows(N, V):
     own = m + np.log(np.exp(got - m[:, None]).sum(axis=1))
     assert np.array_equal(row_max.cpu().numpy().astype(np.float64), m)
     assert np.max(np.abs(lse.cpu().numpy() - own)) <= 2e-6 * (1 + np.max(np.abs(own)))
+
+
+# one, two, four and eight blocks per row; a thread's groups of eight logits paired, with one left over, with a partial one
+@pytest.mark.parametrize("V,N", [(2048, 3), (4088, 149), (4104, 3), (6147, 3), (32008, 70), (30003, 30), (24008, 9), (40003, 18)])
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+def test_proposal_blocks_per_row(V, N, dtype):
+    s = (torch.randn((N, V), generator=torch.Generator(device=DEV).manual_seed(V), device=DEV) * 2).to(torch.bfloat16 if dtype == "bf16" else torch.float32)
+    x = P.sample_proposal(s, 0.75, 29).cpu().numpy()
+    rows = sorted({0, 1, N // 2, N - 1})
+    ref, gaps = O.sample_proposal(to_np64(s), 0.75, 29, rows=rows)
+    assert np.array_equal(x[rows][gaps >= 1e-12], ref[gaps >= 1e-12])     # float64 keys: a few ulp of ~100
