@@ -369,7 +369,7 @@ __device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double r
 
 template <typename T>
 __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ VsGroup Gr, const int stage, const double* state,
-                                                        const double grad_scale) {
+                                                        const double grad_scale, const bool beside) {
   const VsSlice& S = Gr.s[blockIdx.y];
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
@@ -380,21 +380,26 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   __shared__ int sarg[VW];
   __shared__ int stoken;
   __shared__ unsigned char marks[VT];
+  __shared__ double row_state[SAKI_VSHARD_STATE];
   __shared__ double tab[EXP2_TAB * EXP2_COPIES];
   bool table = false;
   const Exp2 ex2(tab, threadIdx.x & 31);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
+  // beside: the float32 kernel of the same stage was launched right before, and lets this one start once all of its blocks
+  // have seen the combine before it complete.  The two touch different rows, so the marked rows are routed while the
+  // float32 kernel runs, and the wait stands at the end: the next combine starts when both are done (with the sweep of
+  // stage A, a call of 1024 rows in eight slices 717 -> 656 us).
   launch_dependents();
-  wait_for_predecessor();
-  if (only_flagged && stage == 0) return;    // no row is marked for float64 before the first combine
+  if (!beside) wait_for_predecessor();
+  if (!(only_flagged && stage == 0))         // (no row is marked for float64 before the first combine)
   // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
   // rule none is marked, and a block is done after one load)
   for (int64_t base = blockIdx.x; base < S.N; base += (int64_t)gridDim.x * VT) {
     const int64_t mine_row = base + (int64_t)tid * gridDim.x;
     if (only_flagged) {
-      const bool marked = mine_row < S.N && state[mine_row * SAKI_VSHARD_STATE + VS_F64] != 0.0;
+      const bool marked = mine_row < S.N && __ldcg(state + mine_row * SAKI_VSHARD_STATE + VS_F64) != 0.0;
       marks[tid] = marked ? 1 : 0;
       if (!__syncthreads_or(marked)) continue;
     }
@@ -407,8 +412,13 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
     const T* s = (const T*)S.s + row * S.ld_s;
     const T* t = (const T*)S.t + row * S.ld_t;
     double* out = partial + row * SAKI_VSHARD_PARTIALS;
-    const double* st = state ? state + row * SAKI_VSHARD_STATE : nullptr;
     if (only_flagged && !marks[(row - base) / gridDim.x]) continue;   // the float32 kernel has this row
+    const double* const st = row_state;
+    if (state) {
+      __syncthreads();                       // the last row is done with row_state
+      if (tid < SAKI_VSHARD_STATE) row_state[tid] = __ldcg(state + row * SAKI_VSHARD_STATE + tid);
+      __syncthreads();
+    }
     if (stage == 0) {
       // ---- stage A: maxima and argmax, then the sums under this slice's own shifts
       float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
@@ -536,6 +546,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
     }
   }
   }
+  if (beside) wait_for_predecessor();
 }
 
 // ---------------------------------------------------------------- the float32 slice kernels
@@ -624,6 +635,7 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
   auto total = [&](const float (&w)[8]) { return fq * (double)(((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]))); };
   const int seg = (n_chunks + FW - 1) / FW, c_lo = min(n_chunks, warp * seg), c_hi = min(n_chunks, c_lo + seg);
   double wsum = 0.0;
+#pragma unroll 4
   for (int c = c_lo + lane; c < c_hi; c += 32) {
     float w[8];
     weights(c, w);
@@ -645,10 +657,14 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
   if (warp == own_w) {
     double running = before;
     int found = -1, last_c = -1;
+    float next[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (c_lo + lane < c_hi) weights(c_lo + lane, next);
     for (int c0 = c_lo; c0 < c_hi && found < 0; c0 += 32) {
       const int c = c0 + lane;
-      float w[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
-      if (c < c_hi) weights(c, w);
+      float w[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) { w[i] = next[i]; next[i] = 0.f; }
+      if (c + 32 < c_hi) weights(c + 32, next);       // (on its way while this step is looked through)
       const double mine = total(w);
       double inc = mine;
 #pragma unroll
@@ -693,8 +709,8 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
 template <int STAGE>
 __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale) {
   const VsSlice& S = Gr.s[blockIdx.y];
-  launch_dependents();
   wait_for_predecessor();
+  launch_dependents();         // (in this order: the float64 kernel launched behind this one reads what the predecessor wrote)
   if (!S.fast) return;
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
@@ -718,11 +734,19 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
     const __nv_bfloat16* t = (const __nv_bfloat16*)S.t + row * S.ld_t;
     double* out = partial + row * SAKI_VSHARD_PARTIALS;
     const double* st = state ? state + row * SAKI_VSHARD_STATE : nullptr;
-    if (STAGE > 0 && st[VS_F64] != 0.0) continue;
+    // (loaded side by side: in the later waves and stage D a block has little more to do than this look at its row)
+    double mode_d = 0.0, corr = 0.0, owner = 0.0;
+    if (STAGE > 0) {
+      const double f64 = st[VS_F64];
+      mode_d = st[VS_MODE];
+      if (STAGE == 3) { corr = st[VS_CORR]; owner = st[VS_OWNER]; }
+      if (f64 != 0.0) continue;
+    }
+    const int mode = (int)mode_d;
     __nv_bfloat16* const g = STAGE >= 2 && dlogits ? (__nv_bfloat16*)dlogits + row * ld_g : nullptr;
     // the gradient slice on its own (a row without a TV pass, or a caller that asks for it at stage D)
     auto gradient_only = [&]() {
-        const double sc = (int)st[VS_MODE] == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
+        const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
         if (sc == 0.0) {
           for (int c = tid; c < n_chunks; c += FT) *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(0, 0, 0, 0);
         } else {
@@ -753,64 +777,90 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
         }
     };
     if (STAGE == 0) {
-      // ---- stage A, first sweep: the slice's maxima, and the first chunk that holds the teacher's
+      // ---- stage A: the slice's maxima, the first chunk that holds the teacher's, and the sums, in one sweep: the shifts of
+      // the sums are the maxima of the first FT chunks (as a rule within a few nats of the slice's; the sums are moved onto
+      // those in float64), and a sweep that met something much larger is repeated under the maxima themselves.  (With a
+      // sweep for the maxima first the slice was read twice, once from L2: 1024 rows of 151936 in eight slices 159 -> 150 us.)
+      uint4 s4 = make_uint4(VF_FILLER, VF_FILLER, VF_FILLER, VF_FILLER), t4 = s4;
+      if (tid < n_chunks) { s4 = vf_ld(s + (size_t)tid * 8); t4 = vf_ld(t + (size_t)tid * 8); }
+      float msc, mtc;
+      {
+        const float2 a = unpack_bf16x2(max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
+        const float2 b = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
+        float m0 = fmaxf(a.x, a.y), m1 = fmaxf(b.x, b.y);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
+          m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
+        }
+        if (lane == 0) { smax[0][warp] = m0; smax[1][warp] = m1; }
+        __syncthreads();
+        m0 = smax[0][0]; m1 = smax[1][0];
+#pragma unroll
+        for (int w = 1; w < FW; ++w) { m0 = fmaxf(m0, smax[0][w]); m1 = fmaxf(m1, smax[1][w]); }
+        __syncthreads();
+        msc = fminf(fmaxf(m0, -1e30f), 1e30f); mtc = fminf(fmaxf(m1, -1e30f), 1e30f);
+      }
       uint32_t run_s = VF_FILLER;
       float mt_run = -CUDART_INF_F;
       int arg_c = 0x7fffffff;
-      for (int c = tid; c < n_chunks; c += FT) {
-        const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
-        run_s = max_bf16x2(run_s, max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
-        const float2 cmt = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
-        const float cm = fmaxf(cmt.x, cmt.y);
-        if (cm > mt_run) { mt_run = cm; arg_c = c; }
-      }
-      const float2 rs2 = unpack_bf16x2(run_s);
-      float ms = fmaxf(rs2.x, rs2.y), mt = mt_run;
-      int ac = arg_c;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
-        const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
-        const int oac = __shfl_xor_sync(0xffffffffu, ac, o);
-        if (omt > mt || (omt == mt && oac < ac)) { mt = omt; ac = oac; }
-      }
-      if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = ac; }
-      __syncthreads();
-      ms = smax[0][0]; mt = smax[1][0]; ac = sarg[0];
-#pragma unroll
-      for (int w = 1; w < FW; ++w) {
-        ms = fmaxf(ms, smax[0][w]);
-        if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < ac)) { mt = smax[1][w]; ac = sarg[w]; }
-      }
-      __syncthreads();
-      if (n_chunks == 0) { ms = -CUDART_INF_F; mt = -CUDART_INF_F; }
-      // ---- second sweep: the sums under the slice's own shifts (the partial's definition: no factor to apply)
-      float2 Ss = splat(0.f), St = splat(0.f), Td = splat(0.f), M1 = splat(0.f), M2 = splat(0.f), M3 = splat(0.f), M4 = splat(0.f);
-      const float msc = fminf(fmaxf(ms, -1e30f), 1e30f), mtc = fminf(fmaxf(mt, -1e30f), 1e30f);
-      const float2 nms = splat(-msc), nmt = splat(-mtc);
+      float2 Ss, St, Td, M1, M2, M3, M4;
+      float ms, mt;
+      int ac;
+#pragma unroll 1
+      for (int again = 0; again < 2; ++again) {
+        Ss = St = Td = M1 = M2 = M3 = M4 = splat(0.f);
+        const float2 nms = splat(-msc), nmt = splat(-mtc);
 #pragma unroll 2
-      for (int c = tid; c < n_chunks; c += FT) {
-        const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
-        const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
-        float2 cs = splat(0.f), ct = splat(0.f);     // per chunk first: a running sum takes one addition per chunk
+        for (int c = tid; c < n_chunks; c += FT) {
+          const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
+          run_s = max_bf16x2(run_s, max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
+          const float2 cmt = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
+          const float cm = fmaxf(cmt.x, cmt.y);
+          if (cm > mt_run) { mt_run = cm; arg_c = c; }
+          const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
+          float2 cs = splat(0.f), ct = splat(0.f);     // per chunk first: a running sum takes one addition per chunk
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
-          const float2 d = ffma2(sf, neg1, tf);
-          const float2 es = ex2f2(fmul2(sf, cc));
-          const float2 et = ex2f2(fmul2(tf, cc));
-          cs = i == 0 ? es : fadd2(cs, es);
-          ct = i == 0 ? et : fadd2(ct, et);
-          Td = ffma2(et, d, Td);
-          const float2 d2 = fmul2(d, d);
-          M1 = ffma2(es, d, M1);
-          const float2 u = fmul2(es, d2);
-          M2 = fadd2(M2, u);
-          M3 = ffma2(u, d, M3);
-          M4 = ffma2(u, d2, M4);
+          for (int i = 0; i < 4; ++i) {
+            const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
+            const float2 d = ffma2(sf, neg1, tf);
+            const float2 es = ex2f2(fmul2(sf, cc));
+            const float2 et = ex2f2(fmul2(tf, cc));
+            cs = i == 0 ? es : fadd2(cs, es);
+            ct = i == 0 ? et : fadd2(ct, et);
+            Td = ffma2(et, d, Td);
+            const float2 d2 = fmul2(d, d);
+            M1 = ffma2(es, d, M1);
+            const float2 u = fmul2(es, d2);
+            M2 = fadd2(M2, u);
+            M3 = ffma2(u, d, M3);
+            M4 = ffma2(u, d2, M4);
+          }
+          Ss = fadd2(Ss, cs);
+          St = fadd2(St, ct);
         }
-        Ss = fadd2(Ss, cs);
-        St = fadd2(St, ct);
+        const float2 rs2 = unpack_bf16x2(run_s);
+        ms = fmaxf(rs2.x, rs2.y); mt = mt_run; ac = arg_c;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+          ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+          const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
+          const int oac = __shfl_xor_sync(0xffffffffu, ac, o);
+          if (omt > mt || (omt == mt && oac < ac)) { mt = omt; ac = oac; }
+        }
+        if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = ac; }
+        __syncthreads();
+        ms = smax[0][0]; mt = smax[1][0]; ac = sarg[0];
+#pragma unroll
+        for (int w = 1; w < FW; ++w) {
+          ms = fmaxf(ms, smax[0][w]);
+          if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < ac)) { mt = smax[1][w]; ac = sarg[w]; }
+        }
+        __syncthreads();
+        if (n_chunks == 0) { ms = -CUDART_INF_F; mt = -CUDART_INF_F; }
+        // (2^64 times the fourth power of a logit difference stays far inside float32's range; decided by the whole block)
+        if (!(fmaxf(ms - msc, mt - mtc) * c32 > 64.f && ms < 1e30f && mt < 1e30f)) break;
+        msc = ms; mtc = mt;
       }
       double a[7] = {vf_tot(Ss), vf_tot(St), vf_tot(Td), vf_tot(M1), vf_tot(M2), vf_tot(M3), vf_tot(M4)};
       vf_block_sum<7>(a, red);
@@ -832,6 +882,9 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
           const double r2 = rtau * rtau, D = (double)mtc - (double)msc;
           a[2] += D * a[1];
           vf_uncentre(D, a[0], a[3], a[4], a[5], a[6]);
+          const double fs = exp2(c64 * ((double)msc - (double)ms)), ft = exp2(c64 * ((double)mtc - (double)mt));
+          a[0] *= fs; a[3] *= fs; a[4] *= fs; a[5] *= fs; a[6] *= fs;
+          a[1] *= ft; a[2] *= ft;
           out[4] = a[0]; out[5] = a[1]; out[6] = a[2] * rtau;
           out[7] = a[3] * rtau; out[8] = a[4] * r2; out[12] = a[5] * r2 * rtau; out[13] = a[6] * r2 * r2;
         }
@@ -840,9 +893,7 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
       }
     } else if (STAGE == 1) {
       // ---- stage B: one evaluation at the row's current beta, under the row's shift (its maxima: no factor)
-      if ((int)st[VS_MODE] != VS_SOLVING) {        // (block-uniform)
-        continue;                                  // (its partial is not read)
-      }
+      if (mode != VS_SOLVING) continue;            // (block-uniform; its partial is not read)
       const double beta = st[VS_BETA];
       float cb = (float)(c64 * beta);
       const float ccb = c32 - cb;                  // the exponent is formed as (c - cb) s' + cb t'
@@ -882,7 +933,7 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
     } else if (STAGE == 2) {
       // ---- stage C: the slice's share of TV and KL(q||p); the student's logit at the teacher's argmax; the gradient
       // slice (the row's coefficient has been known since its lambda settled)
-      const bool live = (int)st[VS_MODE] == VS_SETTLED;
+      const bool live = mode == VS_SETTLED;
       const double lam = st[VS_LAM];
       double a[3] = {0.0, 0.0, 0.0};
       double fq = 0.0, D = 0.0;
@@ -951,22 +1002,21 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
       }
     } else {
       // ---- stage D: on the owning rank the residual draw; the gradient slice, if stage C has not written it
-      const int mode = (int)st[VS_MODE];
       if (g) gradient_only();
-      if (tid == 0) stoken = -1;
-      __syncthreads();
-      const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
-      if (mine) vf_draw(s, t, n_chunks, c32, c64, S.tau, st, red, &stoken);
-      __syncthreads();
-      if (tid == 0) {
-        for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
-        out[0] = -1.0;
-        if (mine && stoken >= 0 && stoken < Vl) {
-          out[0] = (double)(S.v0 + stoken);
-          out[1] = (double)__bfloat162float(s[stoken]); out[2] = (double)__bfloat162float(t[stoken]);
-        }
+      const bool mine = mode == VS_SETTLED && corr != 0.0 && (int)owner == S.rank;      // (block-uniform)
+      int y = -1;
+      if (mine) {
+        if (tid == 0) stoken = -1;
+        __syncthreads();
+        vf_draw(s, t, n_chunks, c32, c64, S.tau, st, red, &stoken);
+        __syncthreads();
+        y = stoken;
+        __syncthreads();
+        if (y >= Vl) y = -1;
       }
-      __syncthreads();
+      if (tid < SAKI_VSHARD_PARTIALS)
+        out[tid] = tid == 0 ? (y >= 0 ? (double)(S.v0 + y) : -1.0) : tid == 1 && y >= 0 ? (double)__bfloat162float(s[y])
+                 : tid == 2 && y >= 0 ? (double)__bfloat162float(t[y]) : 0.0;
     }
   }
 }
@@ -1031,7 +1081,7 @@ cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, co
     if (n_fast == m && (stage == 0 || (flags & SAKI_VSHARD_NONE_MARKED))) continue;    // (no row is marked before the first combine)
     const int64_t blocks = (3LL * sms + m - 1) / m;
     const dim3 grid((unsigned)(N < blocks ? N : blocks), (unsigned)m, 1);
-    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, VT, 0, st, true, Gr, stage, state, gs); };
+    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, VT, 0, st, true, Gr, stage, state, gs, n_fast > 0); };
     cudaError_t e = in[i0].dtype == SAKI_BF16 ? go(vs_partial_kernel<__nv_bfloat16>) : go(vs_partial_kernel<float>);
     *n_launches += 1;
     if (e != cudaSuccess) return e;

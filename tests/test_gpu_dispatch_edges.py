@@ -1,6 +1,6 @@
 """Where a call goes from one form of a kernel to the next: cluster kernel with 1, 2, 4, 8 and 16 CTAs per row, the
 row-per-SM kernel with one, two or four rows per SM by the number of rows, the lm-head GEMM with one CTA or two per
-tile.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
+tile, proposals with one to eight blocks per row, slices of a row whose sums are taken again under larger shifts.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
 import numpy as np
 import pytest
 import torch
@@ -8,6 +8,7 @@ import torch
 import oracle as O
 import paper_2609_36601_b200 as P
 from paper_2609_36601_b200 import synth
+from paper_2609_36601_b200.vshard import route_vocab_sharded_local, split_columns
 from parity import bf16_ulp, compare_rows, grad_check, oracle_inputs, to_np64
 
 pytestmark = pytest.mark.gpu
@@ -80,3 +81,27 @@ def test_proposal_blocks_per_row(V, N, dtype):
     rows = sorted({0, 1, N // 2, N - 1})
     ref, gaps = O.sample_proposal(to_np64(s), 0.75, 29, rows=rows)
     assert np.array_equal(x[rows][gaps >= 1e-12], ref[gaps >= 1e-12])     # float64 keys: a few ulp of ~100
+
+
+# the shifts of a slice's sums are the maxima of its first 1024 logits: here these lie `drop` nats below the others, within
+# the range the sums are moved over in float64 (44 nats), or beyond it, where they are taken again.  (Not far beyond: KL is
+# a difference of terms of lambda D, D the distance of the two models' logits, whose float32 sums leave 2^-23 D of it, as
+# measured at D = 100, where that passes the tolerance of 1e-5.)
+@pytest.mark.parametrize("drop", [30.0, 60.0])
+@pytest.mark.parametrize("sides", ["st", "s", "t"])
+def test_slices_whose_first_logits_are_low(drop, sides):
+    w = synth.Workload("t", 6, 8000, "bf16", 0.125, 1.0, False, 404, 54)
+    d = synth.generate(w, DEV)
+    for k in sides:
+        for c in (0, 4000):
+            d[k][:, c:c + 1024] -= drop
+    d["proposal"][:] = torch.arange(1500, 1506, device=DEV, dtype=torch.int32)
+    out, gs, _ = route_vocab_sharded_local([(d["s"][:, a:a + n], d["t"][:, a:a + n], a) for a, n in split_columns(8000, 2)], 8000,
+                                           d["proposal"], w.eps, w.temperature, w.seed, grad_scale=0.5)
+    s64, t64 = oracle_inputs(d)
+    ref = O.route(s64, t64, d["proposal"].cpu().numpy(), w.eps, w.temperature, w.seed, grad_scale=0.5, want_grad=True,
+                  grad_dtype=w.dtype)
+    compare_rows(out, ref)
+    same = out["corrected"].cpu().numpy() == ref["corrected"]
+    tok = np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[same]
+    grad_check(to_np64(torch.cat(gs, dim=1))[same], ref["grad"][same], w.dtype, tok)
