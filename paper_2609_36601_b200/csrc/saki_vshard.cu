@@ -620,8 +620,7 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
   const float2 cc = splat(c32), cll = splat(cl), ccll = splat(ccl), kpp = splat(-kpi), kqq = splat(-kqi);
   const float2 nms = splat(-msf), nmt = splat(-mtf);
   const float2 nrho = splat(-(float)(fp / fq));
-  auto weights = [&](int c, float (&w)[8]) {
-    const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
+  auto weights_of = [&](const uint4 s4, const uint4 t4, float (&w)[8]) {
     const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
@@ -633,13 +632,22 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
     }
   };
   auto total = [&](const float (&w)[8]) { return fq * (double)(((w[0] + w[1]) + (w[2] + w[3])) + ((w[4] + w[5]) + (w[6] + w[7]))); };
+  auto weights = [&](int c, float (&w)[8]) { weights_of(vf_ld(s + (size_t)c * 8), vf_ld(t + (size_t)c * 8), w); };
   const int seg = (n_chunks + FW - 1) / FW, c_lo = min(n_chunks, warp * seg), c_hi = min(n_chunks, c_lo + seg);
   double wsum = 0.0;
-#pragma unroll 4
-  for (int c = c_lo + lane; c < c_hi; c += 32) {
-    float w[8];
-    weights(c, w);
-    wsum += total(w);
+#pragma unroll 1
+  for (int b = c_lo + lane; b < c_hi; b += 4 * 32) {       // (four chunks on their way at a time)
+    uint4 sv[4], tv[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (b + u * 32 < c_hi) { sv[u] = vf_ld(s + (size_t)(b + u * 32) * 8); tv[u] = vf_ld(t + (size_t)(b + u * 32) * 8); }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (b + u * 32 >= c_hi) break;
+      float w[8];
+      weights_of(sv[u], tv[u], w);
+      wsum += total(w);
+    }
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xffffffffu, wsum, o);
@@ -901,26 +909,37 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
       const float msf = (float)st[VS_MS], mtf = (float)st[VS_MT];
       const float2 cbb = splat(cb), ccbb = splat(ccb), nms = splat(-msf), nmt = splat(-mtf);
       float2 S0 = splat(0.f), S1 = splat(0.f), S2 = splat(0.f), S3 = splat(0.f), S4 = splat(0.f);
-#pragma unroll 2
-      for (int c = tid; c < n_chunks; c += FT) {
-        const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
-        const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
-float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
+      // (the loads of three chunks per thread before the first is worked on, here, and of two in stage C: the waves that
+      // find few rows unsettled are the latency of one slice; 1024 rows of 151936 in eight slices 655 -> 630 us)
+#pragma unroll 1
+      for (int b = tid; b < n_chunks; b += 3 * FT) {
+        uint4 sv[3], tv[3];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
-          const float2 d = ffma2(sf, neg1, tf);
-          const float2 e = ex2f2(ffma2(tf, cbb, fmul2(sf, ccbb)));
-          const float2 d2 = fmul2(d, d);
-          c0 = i == 0 ? e : fadd2(c0, e);
-          c1 = i == 0 ? fmul2(e, d) : ffma2(e, d, c1);
-          const float2 u = fmul2(e, d2);
-          S2 = fadd2(S2, u);
-          S3 = ffma2(u, d, S3);
-          S4 = ffma2(u, d2, S4);
+        for (int u = 0; u < 3; ++u)
+          if (b + u * FT < n_chunks) { sv[u] = vf_ld(s + (size_t)(b + u * FT) * 8); tv[u] = vf_ld(t + (size_t)(b + u * FT) * 8); }
+#pragma unroll
+        for (int u = 0; u < 3; ++u) {
+          const int c = b + u * FT;
+          if (c >= n_chunks) break;
+          const uint4 s4 = sv[u], t4 = tv[u];
+          const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
+          float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
+            const float2 d = ffma2(sf, neg1, tf);
+            const float2 e = ex2f2(ffma2(tf, cbb, fmul2(sf, ccbb)));
+            const float2 d2 = fmul2(d, d);
+            c0 = i == 0 ? e : fadd2(c0, e);
+            c1 = i == 0 ? fmul2(e, d) : ffma2(e, d, c1);
+            const float2 u = fmul2(e, d2);
+            S2 = fadd2(S2, u);
+            S3 = ffma2(u, d, S3);
+            S4 = ffma2(u, d2, S4);
+          }
+          S0 = fadd2(S0, c0);
+          S1 = fadd2(S1, c1);
         }
-        S0 = fadd2(S0, c0);
-        S1 = fadd2(S1, c1);
       }
       double a[5] = {vf_tot(S0), vf_tot(S1), vf_tot(S2), vf_tot(S3), vf_tot(S4)};
       vf_block_sum<5>(a, red);
@@ -960,31 +979,40 @@ float2 c0 = splat(0.f), c1 = splat(0.f);      // the chunk's share of S0 and S1
         const float2 kgg = splat(kgf);
         const int tok = (int)st[VS_TOK] - S.v0, tok_c = (tok >= 0 && tok < Vl) ? (tok >> 3) : -1;
         float2 R = splat(0.f), Sq = splat(0.f), Sqd = splat(0.f);
-#pragma unroll 2
-        for (int c = tid; c < n_chunks; c += FT) {
-          const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
-          const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
-          float2 gv[4];
+#pragma unroll 1
+        for (int b = tid; b < n_chunks; b += 2 * FT) {
+          uint4 sv[2], tv[2];
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
-            const float2 d = ffma2(sf, neg1, tf);
-            const float2 ep = ex2f2(ffma2(sf, cc, kpp));
-            gv[i] = fmul2(ep, kgg);
-            const float2 eq = ex2f2(ffma2(tf, cll, ffma2(sf, ccll, kqq)));
-            float2 r = ffma2(ep, nrho, eq);          // (q_i - p_i) / fq
-            r.x = fmaxf(r.x, 0.f); r.y = fmaxf(r.y, 0.f);
-            R = fadd2(R, r);
-            Sq = fadd2(Sq, eq);
-            Sqd = ffma2(eq, d, Sqd);
-          }
-          if (g) {
-            if (c == tok_c) {
+          for (int u = 0; u < 2; ++u)
+            if (b + u * FT < n_chunks) { sv[u] = vf_ld(s + (size_t)(b + u * FT) * 8); tv[u] = vf_ld(t + (size_t)(b + u * FT) * 8); }
 #pragma unroll
-              for (int i = 0; i < 8; ++i) if (i == (tok & 7)) { if (i & 1) gv[i >> 1].y -= scf; else gv[i >> 1].x -= scf; }
+          for (int u = 0; u < 2; ++u) {
+            const int c = b + u * FT;
+            if (c >= n_chunks) break;
+            const uint4 s4 = sv[u], t4 = tv[u];
+            const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
+            float2 gv[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
+              const float2 d = ffma2(sf, neg1, tf);
+              const float2 ep = ex2f2(ffma2(sf, cc, kpp));
+              gv[i] = fmul2(ep, kgg);
+              const float2 eq = ex2f2(ffma2(tf, cll, ffma2(sf, ccll, kqq)));
+              float2 r = ffma2(ep, nrho, eq);          // (q_i - p_i) / fq
+              r.x = fmaxf(r.x, 0.f); r.y = fmaxf(r.y, 0.f);
+              R = fadd2(R, r);
+              Sq = fadd2(Sq, eq);
+              Sqd = ffma2(eq, d, Sqd);
             }
-            *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(pack_bf16x2(gv[0].x, gv[0].y), pack_bf16x2(gv[1].x, gv[1].y),
-                                                                      pack_bf16x2(gv[2].x, gv[2].y), pack_bf16x2(gv[3].x, gv[3].y));
+            if (g) {
+              if (c == tok_c) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) if (i == (tok & 7)) { if (i & 1) gv[i >> 1].y -= scf; else gv[i >> 1].x -= scf; }
+              }
+              *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(pack_bf16x2(gv[0].x, gv[0].y), pack_bf16x2(gv[1].x, gv[1].y),
+                                                                        pack_bf16x2(gv[2].x, gv[2].y), pack_bf16x2(gv[3].x, gv[3].y));
+            }
           }
         }
         a[0] = vf_tot(R); a[1] = vf_tot(Sq); a[2] = vf_tot(Sqd);
