@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   __syncthreads();
   const Exp2 ex2(sh.tab, lane);
   if (!P.from_list) {
-    launch_dependents();
+    if (steal) launch_dependents();
     wait_for_predecessor();
   }
 
@@ -496,6 +496,9 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       ph ^= 1;
     }
 
+    // (not earlier where the call leaves room: blocks of the next launch would take up what it leaves of each SM, unevenly;
+    // 128 fp32 rows of 1024: 18.9 -> 14.9 us)
+    if (!P.from_list && !steal) launch_dependents();
     // ---- pass "final": total variation, draw weights (of a bonus row: q itself) and the gradient
     const double li = bc[G_LAM] * INV_LN2, iz = exp(-bc[G_LOGZ]);
     const bool corrected = bc[G_CORR] != 0.0, draw = corrected || bonus;
@@ -692,14 +695,16 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
   // Blocks per row.  In list mode (a handful of rows as a rule; the host does not know their number) always the most;
-  // otherwise so many that few rows still fill the chip, each block keeping 1024 elements or more (below that the
-  // barriers of a cluster cost more than its blocks save), and that the rows in flight stay in L2 between the passes
+  // otherwise as many as are resident at once, each block keeping 2048 elements or more (below that the barriers of a
+  // cluster cost more than its blocks save: 64 fp32 rows of 2048 16.9 us with two blocks each, 14.5 with one; beyond what
+  // is resident a call takes twice the turns: 128 rows of 8192 54 us with eight, 29 with four), and so many that the rows
+  // in flight stay in L2 between the passes
   // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).  Where the
   // kernel is pinned (call_rows = 0) the rows do not count, so that pieces of a batch agree with the whole to the bit.
   int cs = 1;
   const int64_t in_flight = BLOCKS_PER_SM<T> * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
-  while (cs < MAX_CS && p.V >= 2048 * cs &&
-         (p.from_list || (p.call_rows > 0 && p.call_rows * cs < in_flight) || in_flight / cs * row_bytes > (150 << 20)))
+  while (cs < MAX_CS && p.V >= (p.from_list ? 2048 : 4096) * cs &&
+         (p.from_list || (p.call_rows > 0 && p.call_rows * 2 * cs <= in_flight) || in_flight / cs * row_bytes > (150 << 20)))
     cs *= 2;
   switch (cs) {
     case 1: return launch_cs<T, 1>(p, dev, sms, st);

@@ -1,5 +1,6 @@
 """Where a call goes from one form of a kernel to the next: cluster kernel with 1, 2, 4, 8 and 16 CTAs per row, the
-row-per-SM kernel with one, two or four rows per SM by the number of rows, the lm-head GEMM with one CTA or two per
+row-per-SM kernel with one, two or four rows per SM by the number of rows, the float64 kernel with one to eight blocks
+per row, the lm-head GEMM with one CTA or two per
 tile, proposals with one to eight blocks per row, slices of a row whose sums are taken again under larger shifts.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
 import numpy as np
 import pytest
@@ -51,6 +52,15 @@ def test_cluster_sizes_by_rows(V, N):
 @pytest.mark.parametrize("N", [148, 149, 296, 297, 592, 593])
 def test_rows_per_sm_by_rows(V, N):
     _check(synth.Workload("t", N, V, "bf16", 0.125, 1.5, True, 403, 53), [0, N // 2, N - 1], 0, 3)
+
+
+# the float64 kernel with one, two, four and eight blocks per row, by V and, at the last call size that is resident at once
+# (444 bf16 or 592 fp32 blocks on 148 SMs) and the first that is not, by the number of rows
+@pytest.mark.parametrize("V,N,dtype", [(4095, 5, "f32"), (4096, 5, "f32"), (8191, 3, "bf16"), (8193, 3, "f32"), (16387, 3, "bf16"),
+                                       (16384, 74, "f32"), (16384, 75, "f32"), (9001, 111, "bf16"), (9001, 112, "bf16"),
+                                       (5001, 222, "bf16"), (5001, 223, "bf16"), (4097, 445, "bf16"), (4100, 593, "f32")])
+def test_float64_blocks_per_row(V, N, dtype):
+    _check(synth.Workload("t", N, V, dtype, 0.125, 1.5, True, 405, 55, temperature=0.875), sorted({0, 1, N // 2, N - 1}), 0, 1)
 
 
 @pytest.mark.parametrize("N", [1, 127, 128, 129, 255, 256, 257, 511, 513])
