@@ -155,10 +155,12 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // suspend the thread for a while, so a limit shorter than the default is kept with the probe that does not.
 __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity, long long limit = WAIT_LIMIT_CYCLES) {
   if (limit < WAIT_LIMIT_CYCLES) {
+    // (the clock before the barrier: a limit of a few cycles runs out whether or not the copy has landed by the time the
+    // code that waits for it has been fetched)
     const long long t0 = clock64();
-    while (!mbar_test_wait(bar, parity)) {
+    do {
       if (clock64() - t0 > limit) return false;
-    }
+    } while (!mbar_test_wait(bar, parity));
     return true;
   }
   if (mbar_try_wait(bar, parity)) return true;
