@@ -785,90 +785,67 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
         }
     };
     if (STAGE == 0) {
-      // ---- stage A: the slice's maxima, the first chunk that holds the teacher's, and the sums, in one sweep: the shifts of
-      // the sums are the maxima of the first FT chunks (as a rule within a few nats of the slice's; the sums are moved onto
-      // those in float64), and a sweep that met something much larger is repeated under the maxima themselves.  (With a
-      // sweep for the maxima first the slice was read twice, once from L2: 1024 rows of 151936 in eight slices 159 -> 150 us.)
-      uint4 s4 = make_uint4(VF_FILLER, VF_FILLER, VF_FILLER, VF_FILLER), t4 = s4;
-      if (tid < n_chunks) { s4 = vf_ld(s + (size_t)tid * 8); t4 = vf_ld(t + (size_t)tid * 8); }
-      float msc, mtc;
-      {
-        const float2 a = unpack_bf16x2(max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
-        const float2 b = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
-        float m0 = fmaxf(a.x, a.y), m1 = fmaxf(b.x, b.y);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          m0 = fmaxf(m0, __shfl_xor_sync(0xffffffffu, m0, o));
-          m1 = fmaxf(m1, __shfl_xor_sync(0xffffffffu, m1, o));
-        }
-        if (lane == 0) { smax[0][warp] = m0; smax[1][warp] = m1; }
-        __syncthreads();
-        m0 = smax[0][0]; m1 = smax[1][0];
-#pragma unroll
-        for (int w = 1; w < FW; ++w) { m0 = fmaxf(m0, smax[0][w]); m1 = fmaxf(m1, smax[1][w]); }
-        __syncthreads();
-        msc = fminf(fmaxf(m0, -1e30f), 1e30f); mtc = fminf(fmaxf(m1, -1e30f), 1e30f);
-      }
+      // ---- stage A, first sweep: the slice's maxima, and the first chunk that holds the teacher's
       uint32_t run_s = VF_FILLER;
       float mt_run = -CUDART_INF_F;
       int arg_c = 0x7fffffff;
-      float2 Ss, St, Td, M1, M2, M3, M4;
-      float ms, mt;
-      int ac;
-#pragma unroll 1
-      for (int again = 0; again < 2; ++again) {
-        Ss = St = Td = M1 = M2 = M3 = M4 = splat(0.f);
-        const float2 nms = splat(-msc), nmt = splat(-mtc);
+      for (int c = tid; c < n_chunks; c += FT) {
+        const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
+        run_s = max_bf16x2(run_s, max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
+        const float2 cmt = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
+        const float cm = fmaxf(cmt.x, cmt.y);
+        if (cm > mt_run) { mt_run = cm; arg_c = c; }
+      }
+      const float2 rs2 = unpack_bf16x2(run_s);
+      float ms = fmaxf(rs2.x, rs2.y), mt = mt_run;
+      int ac = arg_c;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) {
+        ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+        const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
+        const int oac = __shfl_xor_sync(0xffffffffu, ac, o);
+        if (omt > mt || (omt == mt && oac < ac)) { mt = omt; ac = oac; }
+      }
+      if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = ac; }
+      __syncthreads();
+      ms = smax[0][0]; mt = smax[1][0]; ac = sarg[0];
+#pragma unroll
+      for (int w = 1; w < FW; ++w) {
+        ms = fmaxf(ms, smax[0][w]);
+        if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < ac)) { mt = smax[1][w]; ac = sarg[w]; }
+      }
+      __syncthreads();
+      if (n_chunks == 0) { ms = -CUDART_INF_F; mt = -CUDART_INF_F; }
+      // ---- second sweep: the sums under the slice's own maxima.  That is the partial's definition (no factor to apply), and
+      // the float32 products need it: the exponent argument of the largest terms is then 0 or near it, exact, where one of
+      // size a carries an error of a 2^-24.  (One sweep under the maxima of the slice's first 1024 logits takes 593 us instead
+      // of 654 for 1024 rows of 151936 in eight slices, and moves log-sum-exps by 1e-7 and with them draws.)
+      float2 Ss = splat(0.f), St = splat(0.f), Td = splat(0.f), M1 = splat(0.f), M2 = splat(0.f), M3 = splat(0.f), M4 = splat(0.f);
+      const float msc = fminf(fmaxf(ms, -1e30f), 1e30f), mtc = fminf(fmaxf(mt, -1e30f), 1e30f);
+      const float2 nms = splat(-msc), nmt = splat(-mtc);
 #pragma unroll 2
-        for (int c = tid; c < n_chunks; c += FT) {
-          const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
-          run_s = max_bf16x2(run_s, max_bf16x2(max_bf16x2(s4.x, s4.y), max_bf16x2(s4.z, s4.w)));
-          const float2 cmt = unpack_bf16x2(max_bf16x2(max_bf16x2(t4.x, t4.y), max_bf16x2(t4.z, t4.w)));
-          const float cm = fmaxf(cmt.x, cmt.y);
-          if (cm > mt_run) { mt_run = cm; arg_c = c; }
-          const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
-          float2 cs = splat(0.f), ct = splat(0.f);     // per chunk first: a running sum takes one addition per chunk
+      for (int c = tid; c < n_chunks; c += FT) {
+        const uint4 s4 = vf_ld(s + (size_t)c * 8), t4 = vf_ld(t + (size_t)c * 8);
+        const uint32_t sw[4] = {s4.x, s4.y, s4.z, s4.w}, tw[4] = {t4.x, t4.y, t4.z, t4.w};
+        float2 cs = splat(0.f), ct = splat(0.f);     // per chunk first: a running sum takes one addition per chunk
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
-            const float2 d = ffma2(sf, neg1, tf);
-            const float2 es = ex2f2(fmul2(sf, cc));
-            const float2 et = ex2f2(fmul2(tf, cc));
-            cs = i == 0 ? es : fadd2(cs, es);
-            ct = i == 0 ? et : fadd2(ct, et);
-            Td = ffma2(et, d, Td);
-            const float2 d2 = fmul2(d, d);
-            M1 = ffma2(es, d, M1);
-            const float2 u = fmul2(es, d2);
-            M2 = fadd2(M2, u);
-            M3 = ffma2(u, d, M3);
-            M4 = ffma2(u, d2, M4);
-          }
-          Ss = fadd2(Ss, cs);
-          St = fadd2(St, ct);
+        for (int i = 0; i < 4; ++i) {
+          const float2 sf = fadd2(unpack_bf16x2(sw[i]), nms), tf = fadd2(unpack_bf16x2(tw[i]), nmt);
+          const float2 d = ffma2(sf, neg1, tf);
+          const float2 es = ex2f2(fmul2(sf, cc));
+          const float2 et = ex2f2(fmul2(tf, cc));
+          cs = i == 0 ? es : fadd2(cs, es);
+          ct = i == 0 ? et : fadd2(ct, et);
+          Td = ffma2(et, d, Td);
+          const float2 d2 = fmul2(d, d);
+          M1 = ffma2(es, d, M1);
+          const float2 u = fmul2(es, d2);
+          M2 = fadd2(M2, u);
+          M3 = ffma2(u, d, M3);
+          M4 = ffma2(u, d2, M4);
         }
-        const float2 rs2 = unpack_bf16x2(run_s);
-        ms = fmaxf(rs2.x, rs2.y); mt = mt_run; ac = arg_c;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
-          const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
-          const int oac = __shfl_xor_sync(0xffffffffu, ac, o);
-          if (omt > mt || (omt == mt && oac < ac)) { mt = omt; ac = oac; }
-        }
-        if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = ac; }
-        __syncthreads();
-        ms = smax[0][0]; mt = smax[1][0]; ac = sarg[0];
-#pragma unroll
-        for (int w = 1; w < FW; ++w) {
-          ms = fmaxf(ms, smax[0][w]);
-          if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < ac)) { mt = smax[1][w]; ac = sarg[w]; }
-        }
-        __syncthreads();
-        if (n_chunks == 0) { ms = -CUDART_INF_F; mt = -CUDART_INF_F; }
-        // (2^64 times the fourth power of a logit difference stays far inside float32's range; decided by the whole block)
-        if (!(fmaxf(ms - msc, mt - mtc) * c32 > 64.f && ms < 1e30f && mt < 1e30f)) break;
-        msc = ms; mtc = mt;
+        Ss = fadd2(Ss, cs);
+        St = fadd2(St, ct);
       }
       double a[7] = {vf_tot(Ss), vf_tot(St), vf_tot(Td), vf_tot(M1), vf_tot(M2), vf_tot(M3), vf_tot(M4)};
       vf_block_sum<7>(a, red);
@@ -890,9 +867,6 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
           const double r2 = rtau * rtau, D = (double)mtc - (double)msc;
           a[2] += D * a[1];
           vf_uncentre(D, a[0], a[3], a[4], a[5], a[6]);
-          const double fs = exp2(c64 * ((double)msc - (double)ms)), ft = exp2(c64 * ((double)mtc - (double)mt));
-          a[0] *= fs; a[3] *= fs; a[4] *= fs; a[5] *= fs; a[6] *= fs;
-          a[1] *= ft; a[2] *= ft;
           out[4] = a[0]; out[5] = a[1]; out[6] = a[2] * rtau;
           out[7] = a[3] * rtau; out[8] = a[4] * r2; out[12] = a[5] * r2 * rtau; out[13] = a[6] * r2 * r2;
         }

@@ -1,7 +1,7 @@
 """Where a call goes from one form of a kernel to the next: cluster kernel with 1, 2, 4, 8 and 16 CTAs per row, the
 row-per-SM kernel with one, two or four rows per SM by the number of rows, the float64 kernel with one to eight blocks
 per row, the lm-head GEMM with one CTA or two per
-tile, proposals with one to eight blocks per row, slices of a row whose sums are taken again under larger shifts.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
+tile, proposals with one to eight blocks per row, slices whose maxima lie behind lower logits.  Against the oracle; float outputs and decisions at the tolerances of the parity tests."""
 import numpy as np
 import pytest
 import torch
@@ -93,10 +93,9 @@ def test_proposal_blocks_per_row(V, N, dtype):
     assert np.array_equal(x[rows][gaps >= 1e-12], ref[gaps >= 1e-12])     # float64 keys: a few ulp of ~100
 
 
-# the shifts of a slice's sums are the maxima of its first 1024 logits: here these lie `drop` nats below the others, within
-# the range the sums are moved over in float64 (44 nats), or beyond it, where they are taken again.  (Not far beyond: KL is
-# a difference of terms of lambda D, D the distance of the two models' logits, whose float32 sums leave 2^-23 D of it, as
-# measured at D = 100, where that passes the tolerance of 1e-5.)
+# slices whose first 1024 logits lie `drop` nats below the others.  (Not far below: KL is a difference of terms of lambda D, D
+# the distance of the two models' logits, whose float32 sums leave 2^-23 D of it, as measured at D = 100, where that passes
+# the tolerance of 1e-5.)
 @pytest.mark.parametrize("drop", [30.0, 60.0])
 @pytest.mark.parametrize("sides", ["st", "s", "t"])
 def test_slices_whose_first_logits_are_low(drop, sides):
@@ -115,3 +114,25 @@ def test_slices_whose_first_logits_are_low(drop, sides):
     same = out["corrected"].cpu().numpy() == ref["corrected"]
     tok = np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[same]
     grad_check(to_np64(torch.cat(gs, dim=1))[same], ref["grad"][same], w.dtype, tok)
+
+
+# The sums of a slice are taken under its own maxima wherever these lie, so that the exponent argument of the largest terms is
+# exact: a block of 1024 logits (a chunk for every thread) 40 nats below the others may come first or last, to the bit.  Its
+# terms, below 2^-57 of the largest, vanish in every thread's sum beside the others, which lie within 2^-25 of it; under shifts
+# taken from a slice's first logits the arguments, and with them the log-sum-exps, would move by some 1e-7.
+@pytest.mark.parametrize("sides", ["st", "s", "t"])
+def test_sums_do_not_depend_on_where_the_maxima_lie(sides):
+    V, N, world = 32768, 32, 4
+    w = synth.Workload("t", N, V, "bf16", 0.125, 1.0, False, 406, 56)
+    d = synth.generate(w, DEV)
+    got = []
+    for shift in (0, -1024):
+        rows = {k: d[k].float().clamp(-8.0, 8.0).view(N, world, V // world) for k in "st"}
+        for k in sides:
+            rows[k][:, :, :1024] -= 40.0
+        s, t = (torch.roll(rows[k], shift, dims=2).reshape(N, V).to(torch.bfloat16) for k in "st")
+        state = []
+        route_vocab_sharded_local([(s[:, a:a + n], t[:, a:a + n], a) for a, n in split_columns(V, world)], V, d["proposal"], w.eps,
+                                  w.temperature, w.seed, state_out=state)
+        got.append(state[0][:, [dict(s=5, t=6)[k] for k in sides]])          # the log-sum-exps of the lowered rows
+    assert torch.equal(got[0], got[1])
