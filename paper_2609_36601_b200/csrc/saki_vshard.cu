@@ -545,6 +545,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       }
     }
   }
+    if (only_flagged) __syncthreads();       // a warp that is through with the group overwrites its marks with the next group's
   }
   if (beside) wait_for_predecessor();
 }

@@ -153,3 +153,37 @@ def test_temperature_and_dtype_in_slices(dtype, temperature, eps):
     same = out["corrected"].cpu().numpy() == ref["corrected"]
     grad_check(to_np64(torch.cat(gs, dim=1))[same], ref["grad"][same], dtype,
                np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[same])
+
+
+def test_marked_rows_in_more_than_one_group():
+    """The float64 slice kernels look through a call's marks in groups of 512 rows per block (16 slices in one launch: 28
+    blocks per slice on 148 SMs).  More rows than a group holds, marked ones at both ends of a group and in the next one,
+    the rest in between and behind them unmarked; against the unsharded float64 kernel."""
+    V, world = 1024, 16
+    blocks = (3 * torch.cuda.get_device_properties(0).multi_processor_count + world - 1) // world
+    group = 512 * blocks
+    N = group + 3 * blocks + 5
+    w = synth.Workload("vs", N, V, "bf16", 0.02, 1.5, False, 1300, 71)
+    d = synth.generate(w, DEV)
+    marked = torch.tensor([0, 1, blocks - 1, blocks, group // 2, group - blocks, group - 1, group, group + 2 * blocks, N - 1], device=DEV)
+    for k, peak in (("s", 17.5), ("t", 11.8)):         # p = 0.99997, T = 0.992 on one token: a very flat KL(q_beta || p)
+        d[k][marked] = 0.0
+        d[k][marked, 300] = peak
+    d["proposal"][marked] = 300
+    state = []
+    out, gs, _ = route_vocab_sharded_local(_slices(d, split_columns(V, world)), V, d["proposal"], w.eps, seed=w.seed, grad_scale=0.5,
+                                           state_out=state)
+    prev = P.set_kernel(1)
+    try:
+        ref, g_ref = P.route_fwd_bwd(d["s"], d["t"], d["proposal"], w.eps, seed=w.seed, grad_scale=0.5)
+    finally:
+        P.set_kernel(prev)
+    f64 = torch.nonzero(state[0][:, 30]).flatten()
+    assert set(marked.tolist()) <= set(f64.tolist()) and len(f64) < N // 4
+    for k in ("lambda", "tv", "kl", "accept_prob", "logp_x"):
+        assert float((out[k] - ref[k]).abs().max()) <= 1e-5 * (1 + float(ref[k].abs().max())), k
+        assert float((out[k] - ref[k])[f64].abs().max()) <= 1e-6, k             # the same arithmetic to float32 rounding
+    for k in ("corrected", "token", "teacher_top1", "row_status"):
+        assert torch.equal(out[k][marked], ref[k][marked]), k
+    tok = torch.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[marked].cpu().numpy()
+    grad_check(to_np64(torch.cat(gs, dim=1)[marked]), to_np64(g_ref[marked]), w.dtype, tok)
