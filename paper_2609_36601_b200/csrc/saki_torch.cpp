@@ -5,6 +5,7 @@
 #include <Python.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
+#include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <string>
 #include <vector>
@@ -367,14 +368,18 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
     const float scale = (float)number(a[8]);
     void* const st = stream_of(a[10]);
     const int eager = (int)integer(a[11]), max_waves = (int)integer(a[12]);
+    saki_out so;
+    Owned out(alloc_outputs(N, dev, true, &so));
+    // the caller's stream is torch's current one from here on: the counters are zeroed and read in the order of the stages,
+    // and what is freed at the end of the call goes back to the allocator on the stream that used it
+    c10::cuda::OptionalCUDAStreamGuard on_stream;
+    if (a[10] != Py_None && dev.is_cuda()) on_stream.reset_stream(c10::cuda::getStreamFromExternal((cudaStream_t)st, dev.index()));
     const at::Tensor state = empty({N, SAKI_VSHARD_STATE}, at::kDouble, dev), gathered = empty({world, N, SAKI_VSHARD_PARTIALS}, at::kDouble, dev);
     const at::Tensor counts = at::zeros({eager + 1, 2}, at::TensorOptions().dtype(at::kInt).device(dev));
     double* const sp = (double*)state.data_ptr();
     double* const gp = (double*)gathered.data_ptr();
     uint32_t* const np = (uint32_t*)counts.data_ptr();
     for (int r = 0; r < world; ++r) part[(size_t)r] = gp + (int64_t)r * N * SAKI_VSHARD_PARTIALS;   // where the all-gather would put it
-    saki_out so;
-    Owned out(alloc_outputs(N, dev, true, &so));
     auto stage = [&](int k, uint32_t* count, int flags) {
       check_rc(unlocked([&] {
         return lib.vshard_stage(in.data(), world, k, sp, (double* const*)part.data(), gp, k == 2 && backward ? (void* const*)grad.data() : nullptr,

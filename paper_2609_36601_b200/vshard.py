@@ -62,18 +62,20 @@ def route_vocab_sharded(s_loc, t_loc, v0: int, V: int, proposal, eps, temperatur
     rank, world = dist.get_rank(group), dist.get_world_size(group)
     dev, N = s_loc.device, s_loc.shape[0]
     si = B.vshard_in(s_loc, t_loc, v0, V, proposal, eps, temperature, seed, row_offset, mask, rank, world)
-    state = torch.empty((N, B.VSHARD_STATE), dtype=torch.float64, device=dev)
-    part = torch.empty((N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
-    gathered = torch.empty((world, N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
     out = B.alloc_outputs(N, dev)
     g = torch.empty_like(s_loc) if backward else None
+    # the caller's stream is the current one: the exchange, the zeroing and the reading of the counters are ordered with the stages
+    with torch.cuda.stream(stream):
+        state = torch.empty((N, B.VSHARD_STATE), dtype=torch.float64, device=dev)
+        part = torch.empty((N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
+        gathered = torch.empty((world, N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
 
-    def wave(stage, n_solving=None):
-        B.vshard_partial(si, stage, state if stage > 0 else None, part, g if stage == 2 else None, grad_scale, stream)
-        dist.all_gather_into_tensor(gathered.view(-1), part.view(-1), group=group)
-        B.vshard_combine(si, stage, gathered, state, out if stage == 3 else None, n_solving, stream)
+        def wave(stage, n_solving=None):
+            B.vshard_partial(si, stage, state if stage > 0 else None, part, g if stage == 2 else None, grad_scale, stream)
+            dist.all_gather_into_tensor(gathered.view(-1), part.view(-1), group=group)
+            B.vshard_combine(si, stage, gathered, state, out if stage == 3 else None, n_solving, stream)
 
-    _stages(wave, dev, EAGER_WAVES)
+        _stages(wave, dev, EAGER_WAVES)
     return out, g
 
 

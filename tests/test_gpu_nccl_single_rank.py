@@ -39,6 +39,15 @@ try:
     for k in ref:
         assert torch.equal(out[k], ref[k]), k
     assert torch.equal(g, gs[0])
+    side = torch.cuda.Stream()                         # a stream that is not the current one, and busy
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(50_000_000)
+    out, g = route_vocab_sharded(d["s"], d["t"], 0, w.V, d["proposal"], w.eps, w.temperature, w.seed, mask=mask,
+                                 grad_scale=scale, stream=side)
+    side.synchronize()
+    for k in ref:
+        assert torch.equal(out[k], ref[k]), k
+    assert torch.equal(g, gs[0])
     whole, gw = P.route_fwd_bwd(d["s"], d["t"], d["proposal"], w.eps, w.temperature, w.seed, mask=mask, grad_scale=scale)
     torch.cuda.synchronize()
     agree = float((out["corrected"] == whole["corrected"]).float().mean().item())

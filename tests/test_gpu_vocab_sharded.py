@@ -187,3 +187,30 @@ def test_marked_rows_in_more_than_one_group():
         assert torch.equal(out[k][marked], ref[k][marked]), k
     tok = torch.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])[marked].cpu().numpy()
     grad_check(to_np64(torch.cat(gs, dim=1)[marked]), to_np64(g_ref[marked]), w.dtype, tok)
+
+
+def test_a_stream_that_is_not_the_current_one():
+    """The caller's stream, busy for a while when the call comes: counters and marks are zeroed, counted up and read in its
+    order, so that rows that take more waves and rows for the float64 kernels are routed as on the current stream."""
+    V = 4096
+    w = synth.Workload("vs", 24, V, "bf16", 0.02, 1.5, False, 1400, 81)
+    d = synth.generate(w, DEV)
+    for k, peak in (("s", 17.5), ("t", 11.8)):         # very flat rows: marked for the float64 kernels
+        d[k][::5] = 0.0
+        d[k][::5, 300] = peak
+    d["proposal"][::5] = 300
+    slices = _slices(d, split_columns(V, 4))
+    state = []
+    ref, g_ref, waves = route_vocab_sharded_local(slices, V, d["proposal"], w.eps, seed=w.seed, state_out=state)
+    assert bool((state[0][::5, 30] != 0).all()) and waves >= 2
+    torch.cuda.synchronize()
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.cuda._sleep(50_000_000)                    # some 25 ms
+    out, gs, n = route_vocab_sharded_local(slices, V, d["proposal"], w.eps, seed=w.seed, stream=side)
+    side.synchronize()
+    assert n == waves
+    for k in ref:
+        assert torch.equal(out[k], ref[k]), k
+    for a, b in zip(gs, g_ref):
+        assert torch.equal(a, b)
