@@ -138,11 +138,15 @@ void out_record(PyObject* out, saki_out* so) {
   }
 }
 
-template <typename F> int unlocked(F&& call) {       // the call itself without the interpreter lock
+struct Unlocked {      // without the interpreter lock while it lives, however its scope is left
   PyThreadState* const save = PyEval_SaveThread();
-  const int rc = call();
-  PyEval_RestoreThread(save);
-  return rc;
+  Unlocked() = default;
+  Unlocked(const Unlocked&) = delete;
+  ~Unlocked() { PyEval_RestoreThread(save); }
+};
+template <typename F> auto unlocked(F&& call) {      // a call that may take long or wait
+  const Unlocked u;
+  return call();
 }
 template <typename F> PyObject* guarded(F&& body) {
   try { return body(); }
@@ -387,10 +391,7 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
       }));
     };
     auto read = [&] {     // the rows still solving after stage 0 and after each wave, and those marked for float64
-      PyThreadState* const save = PyEval_SaveThread();
-      at::Tensor h = counts.cpu();
-      PyEval_RestoreThread(save);
-      return h;
+      return unlocked([&] { return counts.cpu(); });
     };
     int waves = 0;
     if (N > 0) {
