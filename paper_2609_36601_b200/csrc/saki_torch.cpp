@@ -3,6 +3,7 @@
 // host time through ctypes and fifteen torch.empty calls, against 25 us on the GPU).  No arithmetic: binding.py holds the
 // signatures and documentation, libsaki.so the library, whose functions are handed over by address (bind).
 #include <Python.h>
+#include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
 #include <c10/cuda/CUDAGuard.h>
@@ -148,10 +149,11 @@ template <typename F> auto unlocked(F&& call) {      // a call that may take lon
   const Unlocked u;
   return call();
 }
-template <typename F> PyObject* guarded(F&& body) {
+template <typename F> PyObject* guarded(F&& body) {  // what torch raises becomes the Python exception that torch makes of it
+  HANDLE_TH_ERRORS
   try { return body(); }
   catch (const Raised&) { return nullptr; }
-  catch (const std::exception& e) { PyErr_SetString(PyExc_RuntimeError, e.what()); return nullptr; }
+  END_HANDLE_TH_ERRORS
 }
 void n_args(Py_ssize_t got, Py_ssize_t want) {
   if (got != want) { PyErr_Format(PyExc_TypeError, "%zd arguments, got %zd", want, got); throw Raised(); }

@@ -4,6 +4,8 @@ import os
 import subprocess
 import sys
 
+import pytest
+
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 HEAD = r"""
@@ -44,3 +46,35 @@ for _ in range(3):
 assert ran == [0, 1, 1] * 3, ran
 print("done")
 """)
+
+
+def test_torch_errors_keep_their_types():
+    """An index error, an allocation that fails and a tensor without data are the exceptions that torch makes of them."""
+    _child(r"""
+def raises(kind, f, *a):
+    try:
+        f(*a)
+    except Exception as e:
+        assert type(e) is kind, (type(e), e)
+        assert "frame #" not in str(e), e          # no C++ stack in the text
+    else:
+        raise SystemExit("no error")
+u8 = torch.zeros(3, dtype=torch.uint8)
+raises(IndexError, B.select_tm, torch.tensor(3), u8, None, 0)
+raises(IndexError, B._fast.propose, torch.zeros(3), 1.0, 0, 0, 1234)           # one dimension of two
+bind(saki_vshard_stage=stage)
+s = torch.zeros(3, 8, dtype=torch.bfloat16, device="meta")
+raises(NotImplementedError, B._fast.vshard_local, [(s, s, 0)], 8, s, 0.1, 1.0, 0, 0, None, 1.0, False, 1234, 2, 5)
+raises(B.SakiError, B.route_fwd, torch.zeros(2, 3), torch.zeros(2, 4), u8, 0.1)
+raises(TypeError, B.route_fwd, [1], torch.zeros(2, 4), u8, 0.1)
+print("done")
+""")
+
+
+@pytest.mark.gpu
+def test_out_of_memory_keeps_its_type():
+    import torch
+    import paper_2609_36601_b200 as P
+    with pytest.raises(torch.OutOfMemoryError):
+        P.alloc_outputs(1 << 42, "cuda:0")             # 16 TB
+    P.alloc_outputs(16, "cuda:0")
