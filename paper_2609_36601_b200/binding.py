@@ -208,9 +208,9 @@ def alloc_outputs(n: int, device):
 
 def _alloc_pinned(n: int):
     kw = dict(device="cpu", pin_memory=True)
-    token, top1, status = torch.empty((3, n), dtype=torch.int32, **kw).unbind(0)
-    out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw), "token": token, "teacher_top1": top1, "row_status": status}
-    out.update(zip(_FLOAT_FIELDS, torch.empty((len(_FLOAT_FIELDS), n), dtype=torch.float32, **kw).unbind(0)))
+    out = {"corrected": torch.empty(n, dtype=torch.uint8, **kw)}
+    out.update((f, torch.empty(n, dtype=torch.int32, **kw)) for f in ("token", "teacher_top1", "row_status"))
+    out.update((f, torch.empty(n, dtype=torch.float32, **kw)) for f in _FLOAT_FIELDS)
     return out
 
 

@@ -36,7 +36,7 @@ def _host_command():
     libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
     return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
             f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(a for d in inc for a in ("-isystem", d)),
-            TORCH_SOURCE, "-o", TORCH_LIB, f"-L{libdir}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"]
+            TORCH_SOURCE, "-o", TORCH_LIB, f"-L{libdir}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
 
 
 def _host_needs_build() -> bool:
