@@ -332,7 +332,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
             const float d = (bt - a) - d0, e = (float)es, q = d * d;
             f1.x += e * d; f2.x += e * q; f3.x += e * d * q; f4.x += e * q * q;
             xs = fmaxf(xs, a);
-            if (bt > xt) { xt = bt; am = v; }
+            if (bt > xt || (bt == xt && v < am)) { xt = bt; am = v; }     // (the elements before the first chunk come after it here)
           });
         m1 = f1.x + f1.y; m2 = f2.x + f2.y; m3 = f3.x + f3.y; m4 = f4.x + f4.y;
 #pragma unroll

@@ -66,6 +66,23 @@ def test_maximum_far_above_the_first_elements(drop):
     _check(d, w, list(range(4)))
 
 
+@pytest.mark.parametrize("V,dtype", [(9, "bf16"), (20, "f32"), (33, "bf16"), (600, "bf16"), (2049, "f32"), (32003, "bf16")])
+@pytest.mark.parametrize("off", [1, 2, 3])
+def test_argmax_ties(V, dtype, off):
+    """The teacher's maximum several times over: among the elements before the row's first 16-byte boundary, in the chunks
+    behind it (those of the same thread and of others) and in the elements after the last chunk.  The lowest index counts."""
+    w = synth.Workload("t", 24, V, dtype, 0.125, 1.2, False, 320 + V, 18)
+    d = synth.generate(w, DEV)
+    top = d["t"].float().max() + 2.0
+    head = 16 // d["t"].element_size() - off % (16 // d["t"].element_size())
+    for r in range(w.N):
+        at = [r % 2 * V // 2, r % (head + 1), head + r % 8, min(head + 8 * 32 + r % 8, V - 1), V - 1 - r % 3]
+        for v in at[r % 3:]:
+            d["t"][r, min(v, V - 1)] = top
+    d["t"][0] = 1.0                                    # every element
+    _check(d, w, list(range(w.N)), (off, (off * 3) % 8, 0))
+
+
 @pytest.mark.parametrize("V,N,dtype,off", [(2, 5, "f32", 0), (5, 3, "bf16", 1), (1023, 4, "bf16", 3), (1024, 700, "f32", 0),
                                            (8191, 3, "bf16", 0), (8192, 3, "bf16", 2), (40003, 3, "f32", 1)])
 @pytest.mark.parametrize("scale", [1.0, 40.0])
