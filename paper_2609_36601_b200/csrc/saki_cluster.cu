@@ -339,7 +339,9 @@ __global__ void __launch_bounds__(CT, CS > 8 ? 1 : 2) cluster_kernel(const RowPa
         double rS, G;
         lse_of_sum(gat[lane], lane ? (double)k1 : (double)k0, rS, G);
         const double rSt = __shfl_sync(0x3u, rS, 1), G1 = __shfl_sync(0x3u, G, 1);
-        if (tid == 0) scalar_after_lse_tail(bc, gat, K, k0, k1, x, bonus, masked, row_timeout, 1.f, false, rS, rSt, G, G1, gat + 7);
+        // (sums that are not finite: a logit is not, or the difference of two logits, one of them masked with the type's lowest
+        // value say, has no square in float32; the float64 kernel tells the two apart and routes the second)
+        if (tid == 0) scalar_after_lse_tail(bc, gat, K, k0, k1, x, bonus, masked, row_timeout, 1.f, true, rS, rSt, G, G1, gat + 7);
       }
       if (tid == 0) {
         if ((int)bc[BC_MODE] == MODE_SOLVE) mbar_expect_tx(&mbar[1 + parity], (uint32_t)(CS * CW * 5 * 8));

@@ -254,8 +254,9 @@ __device__ __forceinline__ void decide(double* bc, const Consts& K, double lam, 
 
 // after pass "lse": v = {Ss, St, M1, M2, M3, N1, argmax index} on the row's shifts k0, k1
 // e_max: upper bound of the largest term of either sum (1 when the shifts come from the rows' maxima);
-// overflow_redo: shifts that come from an estimate of the maxima can overflow on finite rows, so
-// non-finite sums hand the row to the float64 kernel instead of flagging it.
+// overflow_redo: sums that are not finite hand the row to the float64 kernel, which flags it if a logit is not finite: under
+// shifts that come from an estimate of the maxima, and with logit differences beyond 1e19 under any shift, they overflow on
+// finite rows too
 // The reciprocal and the log-sum-exp of one row's sum S under shift k: the same instructions for the
 // student and the teacher, so two lanes of a warp can do the two rows at once.
 __device__ __forceinline__ void lse_of_sum(double S, double k, double& rS, double& G) {
