@@ -46,7 +46,7 @@ struct Shared {
   int next[2];
 };
 enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G_LO, G_HI, G_ITER, G_AM, G_OWNER, G_BEFORE,
-       G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_COUNT };
+       G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_ZERO, G_COUNT };
 static_assert(G_COUNT <= 32, "broadcast area too small");
 enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
@@ -161,6 +161,13 @@ __device__ __noinline__ double first_guess(double m1, double m2, double m3, doub
 __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps) {
   const double beta = bc[G_BETA], r0 = 1.0 / v[0], L = log(v[0]);
   const double m1 = v[1] * r0, m2 = v[2] * r0, m3 = v[3] * r0, m4 = v[4] * r0, m1s = m1 * m1;
+  if (beta == 0.0) {                                         // the moments under p, for a guess on their scale (below)
+    const double b = sqrt(2.0 * eps / (m2 - m1s)), top = 0.5 * bc[G_HI];
+    __syncwarp();
+    bc[G_BETA] = b > 0.0 && b < top ? b : top; bc[G_ZERO] = 1.0;
+    __syncwarp();
+    return false;
+  }
   const double var = fmax(m2 - m1s, 0.0), k3 = m3 - 3.0 * m2 * m1 + 2.0 * m1s * m1;
   const double k4 = m4 - 4.0 * m3 * m1 - 3.0 * m2 * m2 + 12.0 * m2 * m1s - 6.0 * m1s * m1s;
   const double kl = beta * m1 - L, slope = beta * var;
@@ -168,6 +175,9 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
   double lo = bc[G_LO], hi = bc[G_HI];
   if (kl <= eps) lo = fmax(lo, beta); else hi = fmin(hi, beta);
   const int iter = (int)bc[G_ITER] + 1;
+  // Lambda may lie on the scale of 1 / d of logits that the teacher masks (down to 1e-39 for float32's lowest value): there
+  // steps and bracket are judged relative to beta.
+  const double unit = beta < 1e-7 ? beta : 1.0;           // (below every first guess)
   // root of the fourth-order model of KL(beta + h) - eps
   const double f0 = eps - kl;
   double h = f0 / slope;
@@ -185,14 +195,17 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
   double nb = beta + h;
   bool bisected = false;
   if (!(nb > lo && nb < hi)) {
-    // a step that is nothing but rounding may end on the wrong side of the bracket; a real one is halved
-    if (fabs(h) < 1e-13) nb = fmin(fmax(nb, lo), hi);
-    else { nb = 0.5 * (lo + hi); bisected = true; }
+    // a step that is nothing but rounding may end on the wrong side of the bracket; a real one is halved (or, far apart on
+    // the scale of masked logits, the bracket's exponent is).  With nothing known yet of the side of 0, the moments at 0 tell
+    // the scale: the first guess had them in float32, where those of masked logits overflow.
+    if (fabs(h) < 1e-13 * unit) nb = fmin(fmax(nb, lo), hi);
+    else { nb = unit < 1.0 && lo > 0.0 && hi > 16.0 * lo ? sqrt(lo) * sqrt(hi) : 0.5 * (lo + hi); bisected = true; }
+    if (bisected && lo == 0.0 && bc[G_ZERO] == 0.0) nb = 0.0;
   }
   h = nb - beta;
   // the first dropped term moves lambda by (k5 / k2) h^4 / 24; with D a scale of d under q, that is D^3 h^4 / 24
   const double rv = 1.0 / var, D2 = fmax(var, fmax(k3 * rv * k3 * rv, fabs(k4) * rv)), h2 = h * h;
-  const bool done = (ok && !bisected && D2 * sqrt(D2) * h2 * h2 <= 2e-10) || fabs(h) < 1e-13 || hi - lo < 1e-15 || iter >= 100;
+  const bool done = (ok && !bisected && D2 * sqrt(D2) * h2 * h2 <= 2e-10 * unit) || fabs(h) < 1e-13 * unit || hi - lo < 1e-15 * unit || iter >= 100;
   __syncwarp();                                              // every lane has read the state
   if (done) {
     bc[G_LAM] = nb;
@@ -448,7 +461,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
             const double g0 = (double)P.redo_guess[item];
             if (g0 > 0.0 && g0 < 1.0) beta = g0;
           }
-          bc[G_BETA] = beta; bc[G_LO] = 0.0; bc[G_HI] = 1.0; bc[G_ITER] = 0.0; bc[G_MODE] = (double)G_SOLVE;
+          bc[G_BETA] = beta; bc[G_LO] = 0.0; bc[G_HI] = 1.0; bc[G_ITER] = 0.0; bc[G_ZERO] = 0.0; bc[G_MODE] = (double)G_SOLVE;
         }
       }
     }

@@ -48,3 +48,48 @@ def test_masked_student(V, N, dtype, eps):
     out = _check(w, d, list(range(4)))
     st = out["row_status"].cpu().numpy()
     assert st[0] == 8 and not np.any(st[1:4] & 8)
+
+
+def _largest_coefficient(s, t, eps):
+    """Of one row, in float64: the largest beta with KL(q_beta || p) <= eps, by bisection of its exponent (the oracle's bisection
+    ends at 1e-15; here the root may lie at 1e-39), with KL and TV there."""
+    lp, lT = (x - (x.max() + np.log(np.exp(x - x.max()).sum())) for x in (s, t))
+
+    def at(beta):
+        z = lp + beta * (lT - lp)
+        lq = z - (z.max() + np.log(np.exp(z - z.max()).sum()))
+        q = np.exp(lq)
+        return float((q * np.where(q > 0, lq - lp, 0.0)).sum()), float(np.maximum(q - np.exp(lp), 0.0).sum())
+
+    if at(1.0)[0] <= eps:
+        return 1.0, *at(1.0)
+    lo, hi = -150.0, 0.0                               # of log2
+    for _ in range(200):
+        mid = 0.5 * (lo + hi)
+        lo, hi = (mid, hi) if at(2.0 ** mid)[0] <= eps else (lo, mid)
+    return 2.0 ** lo, *at(2.0 ** lo)
+
+
+@pytest.mark.parametrize("V,N,dtype", CALLS)
+@pytest.mark.parametrize("mask,kernel", [("lowest", 0), ("lowest", 1), (-1e9, 1)])
+def test_masked_teacher(V, N, dtype, mask, kernel):
+    """The teacher's row masked where the student's is not.  Where the student has more than 1 - exp(-eps) there, every lambda
+    that moves mass away from it in earnest is beyond the radius, and the root lies at the scale of the mask (rows 0 and 1);
+    where it has less, the root is an ordinary one (rows 2 and 3)."""
+    w, d, lowest = _workload(V, N, dtype, 0.125)
+    for r, (a, b) in enumerate([(V // 4, V // 2), (0, V // 2), (V - V // 40, V), (V // 2, V // 2 + 3)]):
+        d["t"][r, a:b] = lowest if mask == "lowest" else mask
+        d["s"][r, a:b] += 2.0 if r < 2 else -6.0
+    d["proposal"][:4] = d["t"][:4].float().argmax(dim=1).to(torch.int32)
+    prev = P.set_kernel(kernel)
+    try:
+        out = P.route_fwd(d["s"], d["t"], d["proposal"], w.eps, w.temperature, w.seed)
+    finally:
+        P.set_kernel(prev)
+    s64, t64 = oracle_inputs(d, range(4))
+    got = {k: out[k].double().cpu().numpy() for k in ("lambda", "kl", "tv")}
+    for r in range(4):
+        lam, kl, tv = _largest_coefficient(s64[r], t64[r], w.eps)
+        assert (lam < 1e-7) == (r < 2), (r, lam)
+        print(f"row {r}: lambda {lam:.3e} {got['lambda'][r]:.3e} kl {kl:.6f} {got['kl'][r]:.6f} tv {tv:.6f} {got['tv'][r]:.6f}")
+        assert abs(got["lambda"][r] - lam) <= 1e-5 and abs(got["kl"][r] - kl) <= 1e-5 and abs(got["tv"][r] - tv) <= 1e-5, r
