@@ -14,6 +14,8 @@ namespace saki {
 // nearly one-hot row grows so fast over [0, beta] that the two rules agree to 1e-6 and are both 1e-4 off).
 constexpr double KL_TOL_REL = 4e-6;
 constexpr double QUAD_MAX_BETA = 0.25;
+// A sum of shifted exponentials below this has lost terms of 2^-36 of it (float32 ends at 2^-126).
+constexpr double SUM_FLOOR = 0x1p-90;
 constexpr int BC_DOUBLES = 56;             // doubles of one broadcast area
 constexpr double LN2 = 0.693147180559945309417232121458;
 constexpr double INV_LN2 = 1.44269504088896340735992468100;
@@ -371,7 +373,9 @@ SAKI_SCALAR_FN void scalar_after_solve4(double* bc, const double* v, Consts K, f
   const double G0 = bc[BC_G0], kb = bc[BC_KB];
   double lo = bc[BC_LO], hi = bc[BC_HI];
   const int iter = (int)bc[BC_ITER] + 1;
-  if (!(fabs((v[0] + v[1]) + (v[2] + v[3]) + v[4]) < CUDART_INF)) { bc[BC_BETA] = -1.0; bc[BC_MODE] = MODE_REDO; return; }   // float32 sums overflowed
+  // float32 sums overflowed, or ran out of range below: the shift is a bound from the two rows' own maxima, and where these are
+  // apart (models that disagree by hundreds of nats) all of q_beta lies far under it
+  if (!(fabs((v[0] + v[1]) + (v[2] + v[3]) + v[4]) < CUDART_INF) || v[0] < SUM_FLOOR) { bc[BC_BETA] = -1.0; bc[BC_MODE] = MODE_REDO; return; }
   // this evaluation: log-partition and cumulants of d under q at bc[BC_BETA]
   double beta = bc[BC_BETA], G, G1, G2, G3, G4;
   bool well_conditioned;
