@@ -50,6 +50,7 @@ enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G
 static_assert(G_COUNT <= 32, "broadcast area too small");
 enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
+constexpr int LOST = -2;
 
 // Dynamic rows: a block (cluster) that is done takes over the work of one that has not started yet, by cancelling its
 // launch.  The answer arrives in shared memory and completes an mbarrier.
@@ -379,10 +380,18 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         p[PA_MS] = (double)ms; p[PA_MT] = (double)mt; p[PA_AM] = inf ? -1.0 : (double)am;
       }
     }
-    if (steal && tid == 0 && crank == 0) {     // the next row, decided while pass "sums" ran
-      const bool there = mbar_wait_bounded(&sh.bar, (uint32_t)(turn & 1));
-      const int first = there ? steal_answer(sh.answer) : -1;
-      sh.next[turn & 1] = first < 0 ? -1 : first / CS;
+    if (steal && tid == 0 && crank == 0) {     // the next row, decided while pass "sums" ran: its number, -1 for none, or LOST - number
+      int next = -1;
+      if (mbar_wait_bounded(&sh.bar, (uint32_t)(turn & 1), P.wait_limit > 0 ? P.wait_limit : WAIT_LIMIT_CYCLES)) {
+        const int first = steal_answer(sh.answer);
+        next = first < 0 ? -1 : first / CS;
+      } else if (mbar_wait_bounded(&sh.bar, (uint32_t)(turn & 1))) {     // late: the row it took over, if any, is flagged and no other is asked for
+        const int first = steal_answer(sh.answer);
+        next = first < 0 ? -1 : LOST - first / CS;
+      } else {
+        atomicAdd(P.flagged, 1ull);            // no answer at all: saki_check reports that a row may have been lost
+      }
+      sh.next[turn & 1] = next;
     }
     phase_barrier();
     if (steal) {
@@ -662,6 +671,14 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       write_row(P.out, row, r, !P.spec);
     }
     ph ^= 1;
+  }
+  if (steal && nxt <= LOST) {                          // a row whose launch was cancelled by a request that was answered too late
+    const int64_t row = (int64_t)LOST - nxt;
+    if (tid == 0 && crank == 0) {
+      write_row(P.out, row, zero_row(SAKI_ROW_TIMEOUT), !P.spec);
+      atomicAdd(P.flagged, 1ull);
+    }
+    if (P.dlogits) for (int v = crank * GT + tid; v < V; v += CS * GT) st_from_float((T*)P.dlogits + row * P.ld_g, v, 0.f);
   }
   if constexpr (CS > 1) cg::this_cluster().sync();   // no block leaves while a peer may still read its shared memory
   if (P.from_list) close_counters(P.redo_count);

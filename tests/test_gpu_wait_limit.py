@@ -1,6 +1,6 @@
-"""The give-up path of the row-per-SM kernel's bounded wait, exercised without withholding anything: the
-wait limit is set to a few cycles, so the wait for a row's bulk copy runs out although the copy is on its
-way.  The kernel must return, a row is either flagged TIMEOUT with zero outputs or routed correctly,
+"""The give-up paths of the row-per-SM and the general kernel's bounded waits, exercised without withholding anything: the
+wait limit is set to a few cycles, so the wait for a row's bulk copy (for the answer to a block's request for a further
+row) runs out although it is on its way.  The kernel must return, a row is either flagged TIMEOUT with zero outputs or routed correctly,
 saki_check counts the flagged rows, and the next ordinary call is unaffected."""
 import numpy as np
 import pytest
@@ -13,16 +13,18 @@ pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
 
 
-@pytest.mark.parametrize("V,N", [(2048, 64), (32000, 700), (151936, 320)])
-def test_expired_wait_flags_rows_and_leaves_the_library_usable(V, N):
-    w = synth.Workload("limit", N, V, "bf16", 0.1, 1.5, True, 4100 + V % 97, 9)
+# the general kernel with one block per row and with clusters of two and eight (more rows than are resident at once)
+@pytest.mark.parametrize("V,N,kernel,dtype", [(2048, 64, 3, "bf16"), (32000, 700, 3, "bf16"), (151936, 320, 3, "bf16"),
+                                              (1024, 2000, 1, "f32"), (40001, 700, 1, "f32"), (151936, 400, 1, "f32")])
+def test_expired_wait_flags_rows_and_leaves_the_library_usable(V, N, kernel, dtype):
+    w = synth.Workload("limit", N, V, dtype, 0.1, 1.5, True, 4100 + V % 97, 9)
     d = synth.generate(w, DEV)
-    prev_k = P.set_kernel(3)
+    prev_k = P.set_kernel(kernel)
     P.check()                                       # clears what earlier tests may have left
     try:
         ref, g_ref = P.route_fwd_bwd(d["s"], d["t"], d["proposal"], w.eps, seed=w.seed)
         torch.cuda.synchronize()
-        assert P.last_kernel() == 3 and P.check() == 0
+        assert P.last_kernel() == kernel and P.check() == 0
         # the rows out of L2 again, so that the first copies of the limited call come from memory
         flush = torch.empty(320 << 20, dtype=torch.uint8, device=DEV)
         flush.fill_(1)
