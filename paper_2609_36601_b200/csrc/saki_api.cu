@@ -73,6 +73,18 @@ static std::atomic<uint64_t> g_redo_generation{0};
 static thread_local unsigned int* g_last_redo_count = nullptr;
 static thread_local uint64_t g_last_redo_generation = 0;
 
+// Zeroes device memory before it returns, on a stream of its own: the caller's may be under capture (one that lets memory be
+// allocated), where a memset would only happen when the graph is launched, after ordinary calls on that stream.
+static cudaError_t zero_now(void* p, size_t bytes) {
+  cudaStream_t own = nullptr;
+  cudaError_t e = cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(p, 0, bytes, own);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(own);
+  cudaStreamDestroy(own);
+  return e;
+}
+
 // g_redo_mu held by the caller
 static int redo_scratch(int64_t n_rows, cudaStream_t st, int32_t** list, unsigned int** count) {
   int dev = 0;
@@ -97,8 +109,8 @@ static int redo_scratch(int64_t n_rows, cudaStream_t st, int32_t** list, unsigne
     // row ids, the counters, and as many words again (block verification: one per sequence)
     cudaError_t e = cudaMalloc((void**)&b.list, (size_t)(2 * cap + CNT_WORDS) * sizeof(int32_t));
     if (e != cudaSuccess) { b = RedoBuf(); return cuda_fail(e, "cudaMalloc (redo list)"); }
-    e = cudaMemsetAsync(b.list + cap, 0, CNT_WORDS * sizeof(int32_t), st);
-    if (e != cudaSuccess) { cudaFree(b.list); b = RedoBuf(); return cuda_fail(e, "cudaMemsetAsync (redo list)"); }
+    e = zero_now(b.list + cap, CNT_WORDS * sizeof(int32_t));
+    if (e != cudaSuccess) { cudaFree(b.list); b = RedoBuf(); return cuda_fail(e, "zeroing the redo list's counters"); }
     b.cap = cap;
   }
   *list = b.list;
