@@ -161,6 +161,10 @@ def load_library(path: str | None = None):
               "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_redo_count",
               "saki_version"):
         getattr(lib, f).restype = C.c_int
+    from . import build
+    if os.path.exists(build.TORCH_LIB) and not build.host_matches():
+        raise SakiError(-1, f"{build.TORCH_LIB} was built for another torch or Python: build it with "
+                            "`python -m paper_2609_36601_b200.build`")
     try:
         from . import _saki_torch
     except ImportError as e:

@@ -27,6 +27,18 @@ def _nvcc():
     raise RuntimeError("nvcc not found")
 
 
+def host_tag() -> str:
+    """What the tensor side of the binding is compiled against: it is of use to no other torch or interpreter."""
+    import torch
+    return f"saki tensor side for torch {torch.__version__}, python {sys.version_info.major}.{sys.version_info.minor};"
+
+
+def host_matches() -> bool:
+    """Whether the built file is for the torch and the interpreter at hand (looked up in the file: loading it may crash)."""
+    with open(TORCH_LIB, "rb") as f:
+        return host_tag().encode() in f.read()
+
+
 def _host_command():
     """The compiler call for the tensor side of the binding, against the installed torch."""
     import sysconfig
@@ -34,14 +46,14 @@ def _host_command():
     from torch.utils import cpp_extension
     inc = [*cpp_extension.include_paths(), sysconfig.get_paths()["include"], os.path.join(os.path.dirname(os.path.dirname(_nvcc())), "include")]
     libdir = os.path.join(os.path.dirname(torch.__file__), "lib")
-    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-w",
-            f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(a for d in inc for a in ("-isystem", d)),
+    return [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", "-fvisibility=hidden", "-Wall",
+            f'-DSAKI_BUILT_FOR="{host_tag()}"', f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(a for d in inc for a in ("-isystem", d)),
             TORCH_SOURCE, "-o", TORCH_LIB, f"-L{libdir}", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-ltorch_cuda", "-lc10", "-lc10_cuda"]
 
 
 def _host_needs_build() -> bool:
     deps = (TORCH_SOURCE, os.path.join(HERE, "..", "include", "saki.h"), os.path.abspath(__file__))
-    return not os.path.exists(TORCH_LIB) or any(os.path.getmtime(d) > os.path.getmtime(TORCH_LIB) for d in deps)
+    return not os.path.exists(TORCH_LIB) or not host_matches() or any(os.path.getmtime(d) > os.path.getmtime(TORCH_LIB) for d in deps)
 
 
 def needs_build() -> bool:

@@ -429,6 +429,9 @@ PyModuleDef module = {PyModuleDef_HEAD_INIT, "_saki_torch", nullptr, -1, methods
 
 }  // namespace
 
+// the torch and the interpreter that this file was compiled against, to be found in the binary
+extern "C" __attribute__((used, visibility("default"))) const char saki_built_for[] = SAKI_BUILT_FOR;
+
 PyMODINIT_FUNC PyInit__saki_torch(void) {
   for (int k = 0; k < N_FIELDS; ++k) field_key[k] = PyUnicode_InternFromString(FIELD[k]);
   key_loss = PyUnicode_InternFromString("loss"); key_logp_tok = PyUnicode_InternFromString("logp_tok");
