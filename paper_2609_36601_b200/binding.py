@@ -378,7 +378,8 @@ def route_host(s, t, proposal, eps, temperature=1.0, seed=0, row_offset=0, mask=
 
 
 def spec_verify(s, t, draft, eps, temperature=1.0, seed=0, seq_offset=0, stream=None):
-    """saki_spec_verify on device tensors s, t: [B,K+1,V], draft: [B,K] int32."""
+    """saki_spec_verify on device tensors s, t: [B,K+1,V], draft: [B,K] int32.  (`per_pos["loss"]` is not written: block
+    verification has no loss.)"""
     return (_fast or _tensors()).spec(s, t, draft, eps, temperature, seed, seq_offset, _handle(stream))
 
 
