@@ -2,7 +2,8 @@
 //
 // One vocabulary row per thread-block cluster of CS CTAs x 256 threads.  Each CTA owns a contiguous slice of the row in
 // shared memory, fetched by one 1-D bulk async copy per array (cp.async.bulk + mbarrier), so the row pair is read from HBM
-// exactly once; each thread owns 80 contiguous elements of the slice.  What bounds a call here is the chain of steps of a
+// exactly once; each thread owns an odd number of contiguous chunks of 8 elements
+// (up to 11: 88 elements; 40 at V = 151936 with 16 CTAs).  What bounds a call here is the chain of steps of a
 // single row, and much of that was instruction fetch: with the row in registers every pass was 40 unrolled pairs of code
 // that ran once.  The passes are loops over shared memory now, and the registers that frees let the scalar steps be
 // inlined.  With what that made possible (warp 0 gathers all sums and goes on to the scalars, up to 16 CTAs per row, sums

@@ -44,7 +44,6 @@ struct RowParams {
   unsigned int* redo_count;            // scratch: the call's counters (CNT_*), zero before the first kernel of the call
   float* redo_guess;                   // scratch or NULL: what the float32 kernel made of lambda for each row of redo_list (< 0: nothing)
   int32_t from_list;                   // general kernel only: route the rows of redo_list
-
   long long wait_limit;                // SM cycles a block waits for a row's bulk copy (row-per-SM kernel) or for its next row (general kernel); <= 0: ~2 s
   unsigned long long* phase_cycles;    // row-per-SM kernel: [SAKI_PHASE_COUNTERS] cycle sums per phase (zeroed before
                                        // the launch); NULL: not wanted

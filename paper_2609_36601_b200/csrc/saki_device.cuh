@@ -208,11 +208,11 @@ struct Consts {   // per-launch constants of the scalar phases
   int V;
 };
 
-// The scalar phases run on one thread per CTA, in float64, while all other threads wait.  In the row-per-SM kernel they
-// are inlined (SAKI_SCALARS_INLINE): a call there costs 400 to 600 cycles of stack traffic (the record of constants, the
+// The scalar phases run on one thread per CTA, in float64, while all other threads wait.  In the row-per-SM kernel
+// with two and four CTAs per SM, and in the cluster kernel, they are inlined (SAKI_SCALARS_INLINE): a call costs 400 to 600 cycles of stack traffic (the record of constants, the
 // saved registers of a caller that holds a hundred) through an L1 that shared memory has left little of; a row of 32000
-// elements went from 69.8 to 65.5 k cycles (four CTAs per SM).  The cluster kernel holds its row in registers and
-// keeps them out of line.
+// elements went from 69.8 to 65.5 k cycles (four CTAs per SM).  The variant with one CTA per SM keeps them out of line: its
+// pass loops come out 1 % slower with the scalar steps among them.
 #ifdef SAKI_SCALARS_INLINE
 #define SAKI_SCALAR_FN static __device__ __forceinline__
 #else

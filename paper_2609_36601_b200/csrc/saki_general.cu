@@ -30,8 +30,11 @@ namespace {
 
 constexpr int GT = 256;        // threads per block
 constexpr int GW = GT / 32;    // warps per block
-// Blocks per SM: more of them hide one another's serial steps, fewer have the registers to interleave elements.
-// Measured (2 / 3 / 4): bf16 rows of 32003 0.275 / 0.280 / 0.309 ms, fp32 rows of 151936 0.784 / 0.786 / 0.734 ms.
+// Blocks per SM: more of them hide one another's serial steps, fewer have the registers to interleave elements.  No number is
+// the best everywhere (us, with 2 / 3 / 4): bf16 1024 rows of 32003 275 / 286 / 312, 2000 of them 516 / 505 / 515, 256 of them
+// 82 / 109 / 88, 512 rows of 100001 465 / 439 / 464, 1024 rows of 2049 52 / 47 / 48; fp32 512 rows of 151936 799 / 806 / 786, 64 of
+// them 115 / 160 / 118, 4096 rows of 1024 143 / 122 / 124, 1024 rows of 32000 304 / 355 / 340.  bf16 takes three for its long
+// calls, fp32 four for the longest rows.
 template <typename T> constexpr int BLOCKS_PER_SM = sizeof(T) == 4 ? 4 : 3;
 constexpr int MAX_CS = 8;      // blocks per row, at most
 constexpr int NPART = 12;      // doubles a warp leaves per phase
@@ -729,7 +732,10 @@ static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t s
   // cluster cost more than its blocks save: 64 fp32 rows of 2048 16.9 us with two blocks each, 14.5 with one; beyond what
   // is resident a call takes twice the turns: 128 rows of 8192 54 us with eight, 29 with four), and so many that the rows
   // in flight stay in L2 between the passes
-  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).  Where the
+  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).  The limit of 150 MB
+  // lies a little above the 126 MB of L2, as a pass behind another finds most of its rows there all the same; measured with 100 /
+  // 150 / 250 MB: 512 bf16 rows of 100001 439 / 439 / 596 us, 512 fp32 rows of 151936 785 / 786 / 739, 1024 of 32000 326 / 340 / 340.
+  // Where the
   // kernel is pinned (call_rows = 0) the rows do not count, so that pieces of a batch agree with the whole to the bit.
   int cs = 1;
   const int64_t in_flight = BLOCKS_PER_SM<T> * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);

@@ -15,8 +15,10 @@
 //   stage B  one evaluation of q_beta per wave: sum e delta^k, k = 0..4; repeated until every
 //            row's lambda has settled (two waves as a rule)
 //   stage C  the slice's share of TV = sum [q - p]_+ and of KL(q||p), the student's logit at the teacher's
-//            argmax; the combine decides acceptance and finds the rank that owns the inverse-CDF target
-//   stage D  the gradient slice, and on the owning rank the residual draw; the last combine writes the outputs
+//            argmax, and the gradient slice (acceptance is decided when lambda settles); the combine finds the rank
+//            that owns the inverse-CDF target
+//   stage D  on the owning rank the residual draw; the last combine writes the outputs (a caller that gives the
+//            gradient's buffer here instead gets it from a pass of its own)
 // Two families of slice kernels: float64 throughout (one block of 16 warps per row; any dtype, any alignment),
 // and, further down, float32 per element for aligned bf16 slices.
 #include "saki_exp2.cuh"
@@ -389,14 +391,13 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   const double rtau = 1.0 / S.tau;
   // beside: the float32 kernel of the same stage was launched right before, and lets this one start once all of its blocks
   // have seen the combine before it complete.  The two touch different rows, so the marked rows are routed while the
-  // float32 kernel runs, and the wait stands at the end: the next combine starts when both are done (with the sweep of
-  // stage A, a call of 1024 rows in eight slices 717 -> 656 us).
+  // float32 kernel runs, and the wait stands at the end: the next combine starts when both are done.
   launch_dependents();
   if (!beside) wait_for_predecessor();
-  if (!(only_flagged && stage == 0))         // (no row is marked for float64 before the first combine)
   // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
-  // rule none is marked, and a block is done after one load)
-  for (int64_t base = blockIdx.x; base < S.N; base += (int64_t)gridDim.x * VT) {
+  // rule none is marked, and a block is done after one load; before the first combine none can be)
+  const int64_t n_rows = only_flagged && stage == 0 ? 0 : S.N;
+  for (int64_t base = blockIdx.x; base < n_rows; base += (int64_t)gridDim.x * VT) {
     const int64_t mine_row = base + (int64_t)tid * gridDim.x;
     if (only_flagged) {
       const bool marked = mine_row < S.N && __ldcg(state + mine_row * SAKI_VSHARD_STATE + VS_F64) != 0.0;
@@ -408,143 +409,140 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
       __syncthreads();
       table = true;
     }
-  for (int64_t row = base; row < S.N && row < base + (int64_t)gridDim.x * VT; row += gridDim.x) {
-    const T* s = (const T*)S.s + row * S.ld_s;
-    const T* t = (const T*)S.t + row * S.ld_t;
-    double* out = partial + row * SAKI_VSHARD_PARTIALS;
-    if (only_flagged && !marks[(row - base) / gridDim.x]) continue;   // the float32 kernel has this row
-    const double* const st = row_state;
-    if (state) {
-      __syncthreads();                       // the last row is done with row_state
-      if (tid < SAKI_VSHARD_STATE) row_state[tid] = __ldcg(state + row * SAKI_VSHARD_STATE + tid);
-      __syncthreads();
-    }
-    if (stage == 0) {
-      // ---- stage A: maxima and argmax, then the sums under this slice's own shifts
-      float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
-      int am = 0x7fffffff, finite = 1;
-#pragma unroll 4
-      for (int v = tid; v < Vl; v += VT) {
-        const float a = ld_as_float(s, v), c = ld_as_float(t, v);
-        finite &= (isfinite(a) && isfinite(c)) ? 1 : 0;
-        ms = fmaxf(ms, a);
-        if (c > mt) { mt = c; am = v; }
+    for (int64_t row = base; row < S.N && row < base + (int64_t)gridDim.x * VT; row += gridDim.x) {
+      const T* s = (const T*)S.s + row * S.ld_s;
+      const T* t = (const T*)S.t + row * S.ld_t;
+      double* out = partial + row * SAKI_VSHARD_PARTIALS;
+      if (only_flagged && !marks[(row - base) / gridDim.x]) continue;   // the float32 kernel has this row
+      const double* const st = row_state;
+      if (state) {
+        __syncthreads();                       // the last row is done with row_state
+        if (tid < SAKI_VSHARD_STATE) row_state[tid] = __ldcg(state + row * SAKI_VSHARD_STATE + tid);
+        __syncthreads();
       }
+      if (stage == 0) {
+        // ---- stage A: maxima and argmax, then the sums under this slice's own shifts
+        float ms = -CUDART_INF_F, mt = -CUDART_INF_F;
+        int am = 0x7fffffff, finite = 1;
+#pragma unroll 4
+        for (int v = tid; v < Vl; v += VT) {
+          const float a = ld_as_float(s, v), c = ld_as_float(t, v);
+          finite &= (isfinite(a) && isfinite(c)) ? 1 : 0;
+          ms = fmaxf(ms, a);
+          if (c > mt) { mt = c; am = v; }
+        }
 #pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
-        const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
-        const int oam = __shfl_xor_sync(0xffffffffu, am, o);
-        if (omt > mt || (omt == mt && oam < am)) { mt = omt; am = oam; }
-      }
-      if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = am; }
-      finite = __syncthreads_and(finite);
-      ms = smax[0][0]; mt = smax[1][0]; am = sarg[0];
-      for (int w = 1; w < VW; ++w) {
-        ms = fmaxf(ms, smax[0][w]);
-        if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < am)) { mt = smax[1][w]; am = sarg[w]; }
-      }
-      __syncthreads();
-      double a[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-      if (finite && Vl > 0) {
-        const double zms = (double)ms * rtau, zmt = (double)mt * rtau;
-  #pragma unroll 4
-      for (int v = tid; v < Vl; v += VT) {
-          const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
-          const double es = ex2((zs - zms) * INV_LN2), et = ex2((zt - zmt) * INV_LN2), dl = zt - zs, ed = es * dl, ed2 = ed * dl;
-          a[0] += es; a[1] += et; a[2] += et * dl; a[3] += ed; a[4] += ed2; a[5] += ed2 * dl; a[6] += ed2 * dl * dl;
+        for (int o = 16; o > 0; o >>= 1) {
+          ms = fmaxf(ms, __shfl_xor_sync(0xffffffffu, ms, o));
+          const float omt = __shfl_xor_sync(0xffffffffu, mt, o);
+          const int oam = __shfl_xor_sync(0xffffffffu, am, o);
+          if (omt > mt || (omt == mt && oam < am)) { mt = omt; am = oam; }
         }
-      }
-      vs_block_sum<7>(a, red);
-      if (tid == 0) {
-        const int x = S.proposal[row] - S.v0;
-        const bool own = x >= 0 && x < Vl;
-        out[0] = (double)ms; out[1] = (double)mt; out[2] = am == 0x7fffffff ? 2147483647.0 : (double)(S.v0 + am);
-        out[3] = finite ? 1.0 : 0.0;
-        out[4] = a[0]; out[5] = a[1]; out[6] = a[2]; out[7] = a[3]; out[8] = a[4];
-        out[9] = own ? (double)ld_as_float(s, x) : 0.0; out[10] = own ? (double)ld_as_float(t, x) : 0.0;
-        out[11] = own ? 1.0 : 0.0;
-        out[12] = a[5]; out[13] = a[6]; out[14] = 0.0; out[15] = 0.0;
-      }
-    } else if (stage == 1) {
-      // ---- stage B: one evaluation at the row's current beta, under the row's global shift
-      double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-      if ((int)st[VS_MODE] == VS_SOLVING) {
-        const double beta = st[VS_BETA];
-        const double kb = ((1.0 - beta) * st[VS_MS] + beta * st[VS_MT]) * rtau;
-  #pragma unroll 4
-      for (int v = tid; v < Vl; v += VT) {
-          const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
-          const double dl = zt - zs, e = ex2((zs + beta * dl - kb) * INV_LN2), ed = e * dl, ed2 = ed * dl;
-          a[0] += e; a[1] += ed; a[2] += ed2; a[3] += ed2 * dl; a[4] += ed2 * dl * dl;
+        if (lane == 0) { smax[0][warp] = ms; smax[1][warp] = mt; sarg[warp] = am; }
+        finite = __syncthreads_and(finite);
+        ms = smax[0][0]; mt = smax[1][0]; am = sarg[0];
+        for (int w = 1; w < VW; ++w) {
+          ms = fmaxf(ms, smax[0][w]);
+          if (smax[1][w] > mt || (smax[1][w] == mt && sarg[w] < am)) { mt = smax[1][w]; am = sarg[w]; }
         }
-      }
-      vs_block_sum<5>(a, red);
-      if (tid == 0) {
-        for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
-        out[0] = a[0]; out[1] = a[1]; out[2] = a[2]; out[3] = a[3]; out[4] = a[4];
-      }
-    } else if (stage == 2) {
-      // ---- stage C: the slice's share of TV and KL(q||p); the student's logit at the teacher's argmax
-      double a[2] = {0.0, 0.0};
-      const bool live = (int)st[VS_MODE] == VS_SETTLED;
-      const double lam = st[VS_LAM];
-      if (live && lam > 0.0) {
-        const double lse_s = st[VS_LSE_S], lse_t = st[VS_LSE_T], logZ = st[VS_LOGZ];
-        // per-warp segments in index order, summed in warp order: close to the index-order sum of the definition
-        const int seg = (Vl + VW - 1) / VW, v_lo = warp * seg, v_hi = min(Vl, v_lo + seg);
+        __syncthreads();
+        double a[7] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        if (finite && Vl > 0) {
+          const double zms = (double)ms * rtau, zmt = (double)mt * rtau;
 #pragma unroll 4
-        for (int v = v_lo + lane; v < v_hi; v += 32) {
-          const double lp = (double)ld_as_float(s, v) * rtau - lse_s, lT = (double)ld_as_float(t, v) * rtau - lse_t;
-          const double lq = lp + lam * (lT - lp) - logZ, q = ex2(lq * INV_LN2);
-          a[0] += fmax(q - ex2(lp * INV_LN2), 0.0);
-          a[1] += q * (lq - lp);
+          for (int v = tid; v < Vl; v += VT) {
+            const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
+            const double es = ex2((zs - zms) * INV_LN2), et = ex2((zt - zmt) * INV_LN2), dl = zt - zs, ed = es * dl, ed2 = ed * dl;
+            a[0] += es; a[1] += et; a[2] += et * dl; a[3] += ed; a[4] += ed2; a[5] += ed2 * dl; a[6] += ed2 * dl * dl;
+          }
         }
-      }
-      vs_block_sum<2>(a, red);
-      if (tid == 0) {
-        for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
-        const int vs = (int)st[VS_VSTAR] - S.v0;
-        out[0] = a[0]; out[1] = a[1];
-        out[2] = (live && vs >= 0 && vs < Vl) ? (double)ld_as_float(s, vs) : 0.0;
-      }
-    } else {
-      // ---- stage D: on the owning rank the residual draw
-      const int mode = (int)st[VS_MODE];
-      if (tid == 0) stoken = -1;
-      __syncthreads();
-      const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
-      if (mine) vs_draw<T, VW>(s, t, Vl, rtau, st, red, &stoken, ex2);
-      __syncthreads();
-      if (tid == 0) {
-        for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
-        out[0] = -1.0;
-        if (mine && stoken >= 0 && stoken < Vl) {
-          out[0] = (double)(S.v0 + stoken);
-          out[1] = (double)ld_as_float(s, stoken); out[2] = (double)ld_as_float(t, stoken);
+        vs_block_sum<7>(a, red);
+        if (tid == 0) {
+          const int x = S.proposal[row] - S.v0;
+          const bool own = x >= 0 && x < Vl;
+          out[0] = (double)ms; out[1] = (double)mt; out[2] = am == 0x7fffffff ? 2147483647.0 : (double)(S.v0 + am);
+          out[3] = finite ? 1.0 : 0.0;
+          out[4] = a[0]; out[5] = a[1]; out[6] = a[2]; out[7] = a[3]; out[8] = a[4];
+          out[9] = own ? (double)ld_as_float(s, x) : 0.0; out[10] = own ? (double)ld_as_float(t, x) : 0.0;
+          out[11] = own ? 1.0 : 0.0;
+          out[12] = a[5]; out[13] = a[6]; out[14] = 0.0; out[15] = 0.0;
         }
+      } else if (stage == 1) {
+        // ---- stage B: one evaluation at the row's current beta, under the row's global shift
+        double a[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        if ((int)st[VS_MODE] == VS_SOLVING) {
+          const double beta = st[VS_BETA];
+          const double kb = ((1.0 - beta) * st[VS_MS] + beta * st[VS_MT]) * rtau;
+#pragma unroll 4
+          for (int v = tid; v < Vl; v += VT) {
+            const double zs = (double)ld_as_float(s, v) * rtau, zt = (double)ld_as_float(t, v) * rtau;
+            const double dl = zt - zs, e = ex2((zs + beta * dl - kb) * INV_LN2), ed = e * dl, ed2 = ed * dl;
+            a[0] += e; a[1] += ed; a[2] += ed2; a[3] += ed2 * dl; a[4] += ed2 * dl * dl;
+          }
+        }
+        vs_block_sum<5>(a, red);
+        if (tid == 0) {
+          for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
+          out[0] = a[0]; out[1] = a[1]; out[2] = a[2]; out[3] = a[3]; out[4] = a[4];
+        }
+      } else if (stage == 2) {
+        // ---- stage C: the slice's share of TV and KL(q||p); the student's logit at the teacher's argmax
+        double a[2] = {0.0, 0.0};
+        const bool live = (int)st[VS_MODE] == VS_SETTLED;
+        const double lam = st[VS_LAM];
+        if (live && lam > 0.0) {
+          const double lse_s = st[VS_LSE_S], lse_t = st[VS_LSE_T], logZ = st[VS_LOGZ];
+          // per-warp segments in index order, summed in warp order: close to the index-order sum of the definition
+          const int seg = (Vl + VW - 1) / VW, v_lo = warp * seg, v_hi = min(Vl, v_lo + seg);
+#pragma unroll 4
+          for (int v = v_lo + lane; v < v_hi; v += 32) {
+            const double lp = (double)ld_as_float(s, v) * rtau - lse_s, lT = (double)ld_as_float(t, v) * rtau - lse_t;
+            const double lq = lp + lam * (lT - lp) - logZ, q = ex2(lq * INV_LN2);
+            a[0] += fmax(q - ex2(lp * INV_LN2), 0.0);
+            a[1] += q * (lq - lp);
+          }
+        }
+        vs_block_sum<2>(a, red);
+        if (tid == 0) {
+          for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
+          const int vs = (int)st[VS_VSTAR] - S.v0;
+          out[0] = a[0]; out[1] = a[1];
+          out[2] = (live && vs >= 0 && vs < Vl) ? (double)ld_as_float(s, vs) : 0.0;
+        }
+      } else {
+        // ---- stage D: on the owning rank the residual draw
+        const int mode = (int)st[VS_MODE];
+        if (tid == 0) stoken = -1;
+        __syncthreads();
+        const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;
+        if (mine) vs_draw<T, VW>(s, t, Vl, rtau, st, red, &stoken, ex2);
+        __syncthreads();
+        if (tid == 0) {
+          for (int k = 0; k < SAKI_VSHARD_PARTIALS; ++k) out[k] = 0.0;
+          out[0] = -1.0;
+          if (mine && stoken >= 0 && stoken < Vl) {
+            out[0] = (double)(S.v0 + stoken);
+            out[1] = (double)ld_as_float(s, stoken); out[2] = (double)ld_as_float(t, stoken);
+          }
+        }
+        __syncthreads();
       }
-      __syncthreads();
-    }
-    if (stage >= 2 && dlogits) {
-      // ---- the gradient slice (with stage C, or with stage D)
-      const int mode = (int)st[VS_MODE];
-      T* g = (T*)dlogits + row * ld_g;
-      {
+      if (stage >= 2 && dlogits) {
+        // ---- the gradient slice (with stage C, or with stage D)
+        const int mode = (int)st[VS_MODE];
+        T* g = (T*)dlogits + row * ld_g;
         const double sc = mode == VS_FLAGGED ? 0.0 : grad_scale * st[VS_COEF] * rtau;
         const double lse_s = st[VS_LSE_S];
         const int tok = mode == VS_FLAGGED ? -1 : (int)st[VS_TOK] - S.v0;
-  #pragma unroll 4
-      for (int v = tid; v < Vl; v += VT) {
+#pragma unroll 4
+        for (int v = tid; v < Vl; v += VT) {
           double gv = 0.0;
           if (sc != 0.0) gv = sc * (ex2(((double)ld_as_float(s, v) * rtau - lse_s) * INV_LN2) - (v == tok ? 1.0 : 0.0));
-          if constexpr (sizeof(T) == 2) {
-            g[v] = __float2bfloat16_rn(to_odd(gv));
-          } else g[v] = (float)gv;
+          if constexpr (sizeof(T) == 2) g[v] = __float2bfloat16_rn(to_odd(gv));
+          else g[v] = (float)gv;
         }
       }
     }
-  }
     if (only_flagged) __syncthreads();       // a warp that is through with the group overwrites its marks with the next group's
   }
   if (beside) wait_for_predecessor();
@@ -555,7 +553,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
 // row-per-SM kernel: packed f32x2 FMAs, ex2.approx under whole-number exponent shifts (the factor between such
 // a shift and the one the partial is defined under is applied once per row, in float64), float32 sums per thread,
 // float64 across threads.  One block of four warps per row slice, several blocks per SM.  A row whose state says
-// VS_F64 is left to the float64 kernel, which is launched behind this one for those rows only.
+// VS_F64 is left to the float64 kernel, which is launched for those rows only and runs beside this one.
 constexpr int FT = 128, FW = FT / 32;
 constexpr uint32_t VF_FILLER = 0xFF7FFF7Fu;       // two bf16 of the most negative finite value
 constexpr double VF_LOG2E = 1.4426950408889634;
@@ -719,7 +717,7 @@ template <int STAGE>
 __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale) {
   const VsSlice& S = Gr.s[blockIdx.y];
   wait_for_predecessor();
-  launch_dependents();         // (in this order: the float64 kernel launched behind this one reads what the predecessor wrote)
+  launch_dependents();         // (in this order: the float64 kernel that runs beside this one reads what the predecessor wrote)
   if (!S.fast) return;
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
@@ -885,7 +883,7 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
       const float2 cbb = splat(cb), ccbb = splat(ccb), nms = splat(-msf), nmt = splat(-mtf);
       float2 S0 = splat(0.f), S1 = splat(0.f), S2 = splat(0.f), S3 = splat(0.f), S4 = splat(0.f);
       // (the loads of three chunks per thread before the first is worked on, here, and of two in stage C: the waves that
-      // find few rows unsettled are the latency of one slice; 1024 rows of 151936 in eight slices 655 -> 630 us)
+      // find few rows unsettled are the latency of one slice; 1024 rows of 151936 in eight slices 655 -> 630 us when stage A was one sweep)
 #pragma unroll 1
       for (int b = tid; b < n_chunks; b += 3 * FT) {
         uint4 sv[3], tv[3];
