@@ -303,7 +303,7 @@ def _vocab_sharded(P, synth, dev, stream, peak, rows=0):
             "bytes_sent_per_row_and_rank": stages * B.VSHARD_PARTIALS * 8, "arithmetic": "f32 per element, f64 sums and scalars",
             "roofline": {"bound": "hbm", "achieved": gbs, "peak": peak, "unit": "GB/s", "frac": gbs / peak,
                          "algorithmic_bytes": alg},
-            "note": "value = rows / wall time of all 8 ranks' kernels run one after the other on this GPU, host-side "
+            "note": "value = rows / wall time of all 8 ranks' kernels on this GPU (the slices of all ranks in one launch per stage), host-side "
                     "sequencing included (a rank's own share is ms_per_rank, the exchanges not included)"}
 
 

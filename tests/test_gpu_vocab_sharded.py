@@ -1,6 +1,6 @@
 """Vocabulary-sharded routing on the GPU: the rows' columns cut into 2, 8 and uneven slices, every slice
-reduced by its own kernel calls (one rank after the other on the one device: the same calls, in the same
-order, that one rank per GPU makes around its all-gather), against the float64 oracle on the whole rows and
+reduced as by a rank of its own (the slices of all ranks in one launch per stage: the same stages, in the same
+order, that one rank per GPU runs around its all-gather), against the float64 oracle on the whole rows and
 against the unsharded call.  Both families of slice kernels: the float32 ones (bf16 slices on 16-byte
 boundaries, eps >= 0.02; the default) and the float64 ones (everything else, and under set_kernel(1))."""
 import numpy as np
