@@ -764,9 +764,8 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       };
       any_dead = __syncthreads_or(dead ? 1 : 0);
       RTS(PH_LSE_REDUCE);
-      if (warp < 8) {   // block level, eight roles dealt round the first eight warps: 0-6 add up one sum each on the row's shifts, 7 finds the argmax
-#pragma unroll 1
-       for (int role = warp; role < 8; role += RW) {
+      if (warp < 8) {   // block level, a role for each of the first eight warps: 0-6 add up one sum each on the row's shifts, 7 finds the argmax
+        const int role = warp;
         const int wl = lane < RW ? lane : 0;       // lanes beyond the warp count carry zero weight
         const float* wm = (const float*)(smem + ROFF_WMAX);
         if (role < 7) {
@@ -804,7 +803,6 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
             gat[6] = (double)best;
           }
         }
-       }
       } else if (lane == 0) {
         side_work();                             // meanwhile, on warps that would only wait
       }
