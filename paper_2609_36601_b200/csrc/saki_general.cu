@@ -7,7 +7,7 @@
 //
 // What bounds it: the float64 pipe (64 lanes per clock and SM; a warp instruction occupies its scheduler's half of
 // it for two clocks).  Hence:
-//   - 2^y costs eight float64 operations (saki_exp2.cuh);
+//   - 2^y costs seven float64 operations (saki_exp2.cuh);
 //   - three passes over the row: "sums" (two exponentials), one or two evaluations of KL with its first four
 //     derivatives (one exponential each: the root of the fourth-order model, as in the bf16 kernels, here accepted
 //     when the dropped terms move lambda by less than about 1e-11), "final" (two exponentials; total variation, draw
@@ -525,22 +525,23 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
     // 128 fp32 rows of 1024: 18.9 -> 14.9 us)
     if (!P.from_list && !steal) launch_dependents();
     // ---- pass "final": total variation, draw weights (of a bonus row: q itself) and the gradient
-    const double li = bc[G_LAM] * INV_LN2, iz = exp(-bc[G_LOGZ]);
+    // log2 q = cq s + cl t + kq: two operations instead of the four that the logit difference d takes
+    const double lam = bc[G_LAM], cl = lam * c, cq = c - cl, kq = kp - INV_LN2 * (lam * cc + bc[G_LOGZ]);
     const bool corrected = bc[G_CORR] != 0.0, draw = corrected || bonus;
-    // p = p_v, e = Z q_v; returns q - p
-    auto diff = [&](float a, float bt, double& p, double& e) {
-      const double sd = (double)a, d = fma((double)bt - sd, rtau, -cc), lp = fma(c, sd, kp);
-      p = ex2(lp);
-      e = ex2(fma(li, d, lp));
-      return fma(e, iz, -p);
+    // p = p_v, q = q_v; returns q - p
+    auto diff = [&](float a, float bt, double& p, double& q) {
+      const double sd = (double)a;
+      p = ex2(fma(c, sd, kp));
+      q = ex2(fma(cl, (double)bt, fma(cq, sd, kq)));
+      return q - p;
     };
     double tv = 0.0, wq = 0.0;
     if (g) {
       const double sc = bc[G_SC];
       const int tok = (int)bc[G_TOK];
       auto grad = [&](float a, float bt) {
-        double p, e;
-        const double r = diff(a, bt, p, e);
+        double p, q;
+        const double r = diff(a, bt, p, q);
         if (__double2hiint(r) >= 0) tv += r;                 // (the sign, without the float64 pipe)
         return sc * p;
       };
@@ -562,9 +563,9 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         },
         [&](int v, float a, float bt) { const double gv = grad(a, bt); Chunk<T>::put(g + v, v == tok ? at_token() : gv); });
     } else if (bonus) {
-      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, e; const double r = diff(a, bt, p, e); if (__double2hiint(r) >= 0) tv += r; wq += e; });
-    } else if (li > 0.0) {
-      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, e; const double r = diff(a, bt, p, e); if (__double2hiint(r) >= 0) tv += r; });
+      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, q; const double r = diff(a, bt, p, q); if (__double2hiint(r) >= 0) tv += r; wq += q; });
+    } else if (lam > 0.0) {
+      for_elements(s, t, tvec, pt, lane, [&](int, float a, float bt) { double p, q; const double r = diff(a, bt, p, q); if (__double2hiint(r) >= 0) tv += r; });
     }
     tv = warp_sum(tv);
     if (bonus) wq = warp_sum(wq);
@@ -612,9 +613,9 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         bool last = bc[G_LAST] != 0.0;
         const int o0 = part_begin(owner), o1 = part_end(owner), sl = (((o1 - o0 + GW - 1) / GW) + 31) & ~31;
         auto weight = [&](int v) {
-          double p, e;
-          const double r = diff(ld_as_float(s, v), ld_as_float(t, v), p, e);
-          return bonus ? e : fmax(r, 0.0);
+          double p, q;
+          const double r = diff(ld_as_float(s, v), ld_as_float(t, v), p, q);
+          return bonus ? q : fmax(r, 0.0);
         };
         double w = 0.0;
         for (int v = o0 + warp * sl + lane; v < min(o1, o0 + (warp + 1) * sl); v += 32) w += weight(v);
@@ -656,7 +657,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       }
     }
     if (writer) {
-      const double lam = bc[G_LAM], lse_s = -LN2 * kp, lse_t = bc[G_LSE_T], Lam = bc[G_LOGZ], tau = (double)P.temperature;
+      const double lse_s = -LN2 * kp, lse_t = bc[G_LSE_T], Lam = bc[G_LOGZ], tau = (double)P.temperature;
       const double lp_x = bc[G_LPX], lT_x = bc[G_LTX];
       RowResult r;
       r.status = (uint32_t)bc[G_STATUS];
