@@ -6,6 +6,7 @@
 #include <torch/csrc/Exceptions.h>
 #include <torch/csrc/autograd/python_variable.h>
 #include <ATen/ATen.h>
+#include <ATen/cuda/CUDAEvent.h>
 #include <ATen/ops/empty_native.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
@@ -385,24 +386,30 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
                                 ld_g.data(), scale, k == 3 ? &so : nullptr, count, flags, st);
       }));
     };
-    auto read = [&] {     // the rows still solving after stage 0 and after each wave, and those marked for float64
-      return unlocked([&] { return counts.cpu(); });
+    // the rows still solving after stage 0 and after each wave, and those marked for float64 (page-locked: the device is idle
+    // until the host has looked at them)
+    const at::Tensor h = at::empty({eager + 1, 2}, at::TensorOptions().dtype(at::kInt).pinned_memory(dev.is_cuda()));
+    at::cuda::CUDAEvent copied;
+    auto read = [&] {
+      return unlocked([&] {
+        h.copy_(counts, true);
+        if (dev.is_cuda()) { copied.record(); copied.synchronize(); }
+        return (const int32_t*)h.data_ptr();
+      });
     };
     int waves = 0;
     if (N > 0) {
       constexpr int NONE = SAKI_VSHARD_NONE_MARKED;
       stage(0, np, NONE);                                    // a wave's combine is the first that can mark a row
       for (int k = 0; k < eager; ++k) stage(1, np + 2 * (1 + k), k == 0 ? NONE : 0);
-      at::Tensor h = read();
-      const int32_t* c = (const int32_t*)h.data_ptr();
+      const int32_t* c = read();
       while (waves < eager && c[2 * waves] > 0) ++waves;
       int32_t sum = c[2 * eager], left = sum, marked = 0;
       for (int k = 0; k < eager; ++k) marked += c[2 * k + 1];
       while (left > 0 && waves < max_waves) {
         stage(1, np + 2 * eager, 0);                         // (adds to the last pair)
         ++waves;
-        h = read();
-        c = (const int32_t*)h.data_ptr();
+        c = read();
         left = c[2 * eager] - sum;
         sum = c[2 * eager];
       }

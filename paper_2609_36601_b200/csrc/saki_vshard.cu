@@ -82,18 +82,32 @@ __host__ __device__ inline void vs_decide(const VsConsts& c, int64_t i, double* 
 }
 
 // ---------------------------------------------------------------- the combine steps (host and device)
-// `part`: [world][N][SAKI_VSHARD_PARTIALS] gathered partials; row i of rank r at part[(r * N + i) * P].
-__host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const double* part, double* st) {
-  const int P = SAKI_VSHARD_PARTIALS;
-  for (int k = 0; k < SAKI_VSHARD_STATE; ++k) st[k] = 0.0;
-  double ms = -INFINITY, mt = -INFINITY, am = 2147483647.0;
-  bool finite = true;
+// `part`: row i's partial of rank 0, of SAKI_VSHARD_PARTIALS numbers; that of rank r stands r * rs further on.
+struct VsMaxima { double ms, mt, am; bool finite; };
+__host__ __device__ inline VsMaxima vs_maxima(const VsConsts& c, const double* part, int64_t rs) {
+  VsMaxima m = {-INFINITY, -INFINITY, 2147483647.0, true};
   for (int r = 0; r < c.world; ++r) {
-    const double* p = part + ((int64_t)r * c.N + i) * P;
-    if (p[3] == 0.0) finite = false;
-    if (p[0] > ms) ms = p[0];
-    if (p[1] > mt || (p[1] == mt && p[2] < am)) { mt = p[1]; am = p[2]; }   // lowest index among ties
+    const double* p = part + r * rs;
+    if (p[3] == 0.0) m.finite = false;
+    if (p[0] > m.ms) m.ms = p[0];
+    if (p[1] > m.mt || (p[1] == m.mt && p[2] < m.am)) { m.mt = p[1]; m.am = p[2]; }   // lowest index among ties
   }
+  return m;
+}
+// a rank's sums of stage A, from its own shifts onto the row's
+enum { VA_SS = 0, VA_ST, VA_TD, VA_SD, VA_SD2, VA_SD3, VA_SD4, VA_COUNT };
+__host__ __device__ inline void vs_rescale(const VsConsts& c, const double* p, const VsMaxima& m, double* v) {
+  const double fs = p[4] > 0.0 ? exp((p[0] - m.ms) / c.tau) : 0.0, ft = p[5] > 0.0 ? exp((p[1] - m.mt) / c.tau) : 0.0;
+  v[VA_SS] = v[VA_SD] = v[VA_SD2] = v[VA_SD3] = v[VA_SD4] = v[VA_ST] = v[VA_TD] = 0.0;
+  if (p[4] > 0.0) { v[VA_SS] = fs * p[4]; v[VA_SD] = fs * p[7]; v[VA_SD2] = fs * p[8]; v[VA_SD3] = fs * p[12]; v[VA_SD4] = fs * p[13]; }
+  if (p[5] > 0.0) { v[VA_ST] = ft * p[5]; v[VA_TD] = ft * p[6]; }
+}
+// `scaled`: the ranks' records of vs_rescale, `vs` apart; null: formed here
+__host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const double* part, int64_t rs, double* st,
+                                             const VsMaxima& m, const double* scaled, int64_t vs) {
+  for (int k = 0; k < SAKI_VSHARD_STATE; ++k) st[k] = 0.0;
+  const double ms = m.ms, mt = m.mt, am = m.am;
+  const bool finite = m.finite;
   const int x = c.proposal[i];
   uint32_t status = 0;
   if (!finite || !(ms > -INFINITY) || !(mt > -INFINITY)) status = SAKI_ROW_NONFINITE;
@@ -102,10 +116,11 @@ __host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const
   if (status) { st[VS_STATUS] = (double)status; st[VS_MODE] = VS_FLAGGED; return; }
   double Ss = 0.0, St = 0.0, Td = 0.0, Sd = 0.0, Sd2 = 0.0, Sd3 = 0.0, Sd4 = 0.0, sx = 0.0, tx = 0.0;
   for (int r = 0; r < c.world; ++r) {      // rank order: the summation order is part of the protocol
-    const double* p = part + ((int64_t)r * c.N + i) * P;
-    const double fs = exp((p[0] - ms) / c.tau), ft = exp((p[1] - mt) / c.tau);
-    if (p[4] > 0.0) { Ss += fs * p[4]; Sd += fs * p[7]; Sd2 += fs * p[8]; Sd3 += fs * p[12]; Sd4 += fs * p[13]; }
-    if (p[5] > 0.0) { St += ft * p[5]; Td += ft * p[6]; }
+    const double* p = part + r * rs;
+    double own[VA_COUNT];
+    if (!scaled) vs_rescale(c, p, m, own);
+    const double* const v = scaled ? scaled + r * vs : own;
+    Ss += v[VA_SS]; St += v[VA_ST]; Td += v[VA_TD]; Sd += v[VA_SD]; Sd2 += v[VA_SD2]; Sd3 += v[VA_SD3]; Sd4 += v[VA_SD4];
     sx += p[9]; tx += p[10];
   }
   const double lse_s = ms / c.tau + log(Ss), lse_t = mt / c.tau + log(St);
@@ -151,12 +166,11 @@ __host__ __device__ inline void vs_combine_a(const VsConsts& c, int64_t i, const
 // One wave of the solver: from the sums at beta, KL(q_beta||p), the cumulants of d under q_beta and with them
 // the model  KL(beta + h) = KL(beta) + int_0^h (beta + u) (k2 + k3 u + k4 u^2 / 2) du;  h = its root at eps (Newton
 // from the first-order step), kept inside the bisection bracket.  Returns 1 if the row needs another wave.
-__host__ __device__ inline int vs_combine_b(const VsConsts& c, int64_t i, const double* part, double* st) {
+__host__ __device__ inline int vs_combine_b(const VsConsts& c, int64_t i, const double* part, int64_t rs, double* st) {
   if ((int)st[VS_MODE] != VS_SOLVING) return 0;
-  const int P = SAKI_VSHARD_PARTIALS;
   double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0, a4 = 0.0;
   for (int r = 0; r < c.world; ++r) {
-    const double* p = part + ((int64_t)r * c.N + i) * P;
+    const double* p = part + r * rs;
     a0 += p[0]; a1 += p[1]; a2 += p[2]; a3 += p[3]; a4 += p[4];
   }
   const double beta = st[VS_BETA], cc = st[VS_LSE_T] - st[VS_LSE_S];
@@ -212,12 +226,11 @@ __host__ __device__ inline int vs_combine_b(const VsConsts& c, int64_t i, const 
 }
 
 // TV, KL, the coupling decision, the routed loss and the owner of the residual draw
-__host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const double* part, double* st) {
+__host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const double* part, int64_t rs, double* st) {
   if ((int)st[VS_MODE] == VS_FLAGGED) return;
-  const int P = SAKI_VSHARD_PARTIALS;
   double tv = 0.0, kl = 0.0, sv = 0.0;
   for (int r = 0; r < c.world; ++r) {
-    const double* p = part + ((int64_t)r * c.N + i) * P;
+    const double* p = part + r * rs;
     tv += p[0]; kl += p[1]; sv += p[2];
   }
   const int x = c.proposal[i];
@@ -231,14 +244,14 @@ __host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const
     int owner = -1;
     double before = 0.0;
     for (int r = 0; r < c.world; ++r) {
-      const double w = part[((int64_t)r * c.N + i) * P];
+      const double w = part[r * rs];
       if (before + w > target) { owner = r; break; }
       before += w;
     }
     double take_last = 0.0;
     if (owner < 0) {      // rounding left no crossing: the last index with positive weight
       take_last = 1.0; before = 0.0;
-      for (int r = c.world - 1; r >= 0; --r) if (part[((int64_t)r * c.N + i) * P] > 0.0) { owner = r; break; }
+      for (int r = c.world - 1; r >= 0; --r) if (part[r * rs] > 0.0) { owner = r; break; }
       if (owner < 0) owner = c.world - 1;
     }
     st[VS_OWNER] = (double)owner; st[VS_BEFORE] = before; st[VS_TARGET] = target; st[VS_TAKE_LAST] = take_last;
@@ -248,13 +261,12 @@ __host__ __device__ inline void vs_combine_c(const VsConsts& c, int64_t i, const
 }
 
 // the drawn token and the per-position outputs
-__host__ __device__ inline void vs_combine_d(const VsConsts& c, int64_t i, const double* part, double* st, const saki_out& o) {
+__host__ __device__ inline void vs_combine_d(const VsConsts& c, int64_t i, const double* part, int64_t rs, double* st, const saki_out& o) {
   if ((int)st[VS_MODE] == VS_FLAGGED) { write_row(o, i, zero_row((uint32_t)st[VS_STATUS]), true); return; }
-  const int P = SAKI_VSHARD_PARTIALS;
   if (st[VS_CORR] != 0.0) {
     double y = -1.0, sy = 0.0, ty = 0.0;
     for (int r = 0; r < c.world; ++r) {
-      const double* p = part + ((int64_t)r * c.N + i) * P;
+      const double* p = part + r * rs;
       if (p[0] >= 0.0) { y = p[0]; sy = p[1]; ty = p[2]; }
     }
     st[VS_Y] = y; st[VS_SY] = sy; st[VS_TY] = ty;
@@ -371,7 +383,7 @@ __device__ __forceinline__ void vs_draw(const T* s, const T* t, int Vl, double r
 
 template <typename T>
 __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ VsGroup Gr, const int stage, const double* state,
-                                                        const double grad_scale, const bool beside) {
+                                                        const double grad_scale) {
   const VsSlice& S = Gr.s[blockIdx.y];
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
@@ -389,11 +401,9 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
-  // beside: the float32 kernel of the same stage was launched right before, and lets this one start once all of its blocks
-  // have seen the combine before it complete.  The two touch different rows, so the marked rows are routed while the
-  // float32 kernel runs, and the wait stands at the end: the next combine starts when both are done.
+  // (in this order: the float32 kernel of the same stage, launched right behind, starts without a wait of its own)
+  wait_for_predecessor();
   launch_dependents();
-  if (!beside) wait_for_predecessor();
   // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
   // rule none is marked, and a block is done after one load; before the first combine none can be)
   const int64_t n_rows = only_flagged && stage == 0 ? 0 : S.N;
@@ -545,7 +555,6 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
     }
     if (only_flagged) __syncthreads();       // a warp that is through with the group overwrites its marks with the next group's
   }
-  if (beside) wait_for_predecessor();
 }
 
 // ---------------------------------------------------------------- the float32 slice kernels
@@ -714,11 +723,20 @@ __device__ __forceinline__ void vf_draw(const __nv_bfloat16* s, const __nv_bfloa
 }
 
 template <int STAGE>
-__global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale) {
+__global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsGroup Gr, const double* state, const double grad_scale,
+                                                     const bool beside) {
   const VsSlice& S = Gr.s[blockIdx.y];
-  wait_for_predecessor();
-  launch_dependents();         // (in this order: the float64 kernel that runs beside this one reads what the predecessor wrote)
-  if (!S.fast) return;
+  // beside: the float64 kernel of the same stage was launched right before and lets this one start once all of its blocks
+  // have seen the combine before it complete.  The two touch different rows, so the marked rows are routed while this
+  // kernel runs, and the wait stands at the end: the next combine starts when both are done.  (With the float64 kernel
+  // behind this one it could only start with the last of these blocks, and 28 of the 31 us that it takes in stage C
+  // for 1024 rows of 151936 in eight slices came on top.)
+  if (!beside) wait_for_predecessor();
+  launch_dependents();
+  if (!S.fast) {
+    if (beside) wait_for_predecessor();
+    return;
+  }
   double* const partial = S.partial;
   void* const dlogits = S.dlogits;
   const int64_t ld_g = S.ld_g;
@@ -726,6 +744,7 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
   __shared__ float smax[2][FW];
   __shared__ int sarg[FW];
   __shared__ int stoken;
+  __shared__ double row_state[SAKI_VSHARD_STATE];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local, n_chunks = Vl >> 3;
   const double rtau = 1.0 / S.tau;
@@ -736,20 +755,22 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
   // float32 for bf16 logits): exponents are then sums of small terms, and the logit difference d' = t' - s'
   // is taken about the difference of the maxima, so float32 products keep their digits whatever offsets the two
   // models' logits carry.  Partials that are defined about zero are converted in float64, once per row.
-  for (int64_t row = blockIdx.x; row < S.N; row += gridDim.x) {
+  for (int64_t turn = blockIdx.x; turn < S.N; turn += gridDim.x) {
+    // stage B from the last row to the first: it begins with what stage A, and stage C with what stage B, has left in L2
+    const int64_t row = STAGE == 1 ? S.N - 1 - turn : turn;
     const __nv_bfloat16* s = (const __nv_bfloat16*)S.s + row * S.ld_s;
     const __nv_bfloat16* t = (const __nv_bfloat16*)S.t + row * S.ld_t;
     double* out = partial + row * SAKI_VSHARD_PARTIALS;
-    const double* st = state ? state + row * SAKI_VSHARD_STATE : nullptr;
-    // (loaded side by side: in the later waves and stage D a block has little more to do than this look at its row)
-    double mode_d = 0.0, corr = 0.0, owner = 0.0;
+    // (one load by one warp: in the later waves and stage D a block has little more to do than this look at its row.  Past
+    // L1: a launch that does not wait at its start has no claim on what another wrote)
+    const double* const st = row_state;
     if (STAGE > 0) {
-      const double f64 = st[VS_F64];
-      mode_d = st[VS_MODE];
-      if (STAGE == 3) { corr = st[VS_CORR]; owner = st[VS_OWNER]; }
-      if (f64 != 0.0) continue;
+      __syncthreads();                         // the last row is done with row_state
+      if (tid < SAKI_VSHARD_STATE) row_state[tid] = __ldcg(state + row * SAKI_VSHARD_STATE + tid);
+      __syncthreads();
+      if (st[VS_F64] != 0.0) continue;
     }
-    const int mode = (int)mode_d;
+    const int mode = STAGE > 0 ? (int)st[VS_MODE] : 0;
     __nv_bfloat16* const g = STAGE >= 2 && dlogits ? (__nv_bfloat16*)dlogits + row * ld_g : nullptr;
     // the gradient slice on its own (a row without a TV pass, or a caller that asks for it at stage D)
     auto gradient_only = [&]() {
@@ -983,8 +1004,8 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
 #pragma unroll
                 for (int i = 0; i < 8; ++i) if (i == (tok & 7)) { if (i & 1) gv[i >> 1].y -= scf; else gv[i >> 1].x -= scf; }
               }
-              *reinterpret_cast<uint4*>(g + (size_t)c * 8) = make_uint4(pack_bf16x2(gv[0].x, gv[0].y), pack_bf16x2(gv[1].x, gv[1].y),
-                                                                        pack_bf16x2(gv[2].x, gv[2].y), pack_bf16x2(gv[3].x, gv[3].y));
+              __stcs(reinterpret_cast<uint4*>(g + (size_t)c * 8), make_uint4(pack_bf16x2(gv[0].x, gv[0].y), pack_bf16x2(gv[1].x, gv[1].y),
+                                                                             pack_bf16x2(gv[2].x, gv[2].y), pack_bf16x2(gv[3].x, gv[3].y)));
             }
           }
         }
@@ -1004,7 +1025,7 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
     } else {
       // ---- stage D: on the owning rank the residual draw; the gradient slice, if stage C has not written it
       if (g) gradient_only();
-      const bool mine = mode == VS_SETTLED && corr != 0.0 && (int)owner == S.rank;      // (block-uniform)
+      const bool mine = mode == VS_SETTLED && st[VS_CORR] != 0.0 && (int)st[VS_OWNER] == S.rank;      // (block-uniform)
       int y = -1;
       if (mine) {
         if (tid == 0) stoken = -1;
@@ -1020,23 +1041,100 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
                  : tid == 2 && y >= 0 ? (double)__bfloat162float(t[y]) : 0.0;
     }
   }
+  if (beside) wait_for_predecessor();
 }
 
-__global__ void vs_combine_kernel(const VsConsts C, const int stage, const double* part, double* state, const saki_out o,
-                                  unsigned int* n_solving, unsigned int* n_marked) {
+// Stage D of a group of slices, a block per row: the draw on the slice that owns the target, if any, and the records of
+// all of them (a block per row and slice is 8192 blocks for 1024 rows in eight slices, most of which only write a record).
+__global__ void __launch_bounds__(FT, 6) vs_draw_kernel(const __grid_constant__ VsGroup Gr, const double* state, const int members, const bool beside) {
+  if (!beside) wait_for_predecessor();         // (as in vs_fast_kernel)
+  launch_dependents();
+  __shared__ double red[FW], row_state[SAKI_VSHARD_STATE];
+  __shared__ int stoken;
+  const int tid = threadIdx.x;
+  const float c32 = (float)(VF_LOG2E / Gr.s[0].tau);
+  const double c64 = (double)c32;
+  for (int64_t row = blockIdx.x; row < Gr.s[0].N; row += gridDim.x) {
+    const double* const st = row_state;
+    __syncthreads();
+    if (tid < SAKI_VSHARD_STATE) row_state[tid] = __ldcg(state + row * SAKI_VSHARD_STATE + tid);
+    __syncthreads();
+    if (st[VS_F64] != 0.0) continue;
+    int own = -1, y = -1;
+    if ((int)st[VS_MODE] == VS_SETTLED && st[VS_CORR] != 0.0)
+      for (int k = 0; k < members; ++k) if (Gr.s[k].rank == (int)st[VS_OWNER]) own = k;
+    float sy = 0.f, ty = 0.f;
+    if (own >= 0) {
+      const VsSlice& O = Gr.s[own];
+      const __nv_bfloat16* const s = (const __nv_bfloat16*)O.s + row * O.ld_s;
+      const __nv_bfloat16* const t = (const __nv_bfloat16*)O.t + row * O.ld_t;
+      if (tid == 0) stoken = -1;
+      __syncthreads();
+      vf_draw(s, t, O.V_local >> 3, c32, c64, O.tau, st, red, &stoken);
+      __syncthreads();
+      y = stoken;
+      if (y >= O.V_local) y = -1;
+      if (y >= 0) { sy = __bfloat162float(s[y]); ty = __bfloat162float(t[y]); }
+    }
+    for (int k = tid; k < members * SAKI_VSHARD_PARTIALS; k += FT) {
+      const int r = k / SAKI_VSHARD_PARTIALS, f = k % SAKI_VSHARD_PARTIALS;
+      const bool mine = r == own && y >= 0;
+      Gr.s[r].partial[row * SAKI_VSHARD_PARTIALS + f] = f == 0 ? (mine ? (double)(Gr.s[r].v0 + y) : -1.0) : f == 1 && mine ? (double)sy : f == 2 && mine ? (double)ty : 0.0;
+    }
+  }
+  if (beside) wait_for_predecessor();
+}
+
+// A row's combine is a chain of float64 scalars on one thread.  What surrounds the chain is spread over the row's VC_LANES
+// threads: partials and state come into shared memory side by side (a thread that fetched them one after the other, rank
+// by rank, waited for memory at each), the exponentials of stage A are formed one rank per thread, the state leaves as a
+// block.  The sums themselves stay in rank order.
+constexpr int VC_ROWS = 8, VC_LANES = 8, VC_THREADS = VC_ROWS * VC_LANES, VC_WORLD = 16;
+__global__ void __launch_bounds__(VC_THREADS) vs_combine_kernel(const VsConsts C, const int stage, const double* part, double* state,
+                                  const saki_out o, unsigned int* n_solving, unsigned int* n_marked) {
+  constexpr int P = SAKI_VSHARD_PARTIALS, S = SAKI_VSHARD_STATE;
+  __shared__ double sp[VC_ROWS][VC_WORLD][P + 1], sst[VC_ROWS][S + 1], scaled[VC_ROWS][VC_WORLD][VA_COUNT];
   launch_dependents();
   wait_for_predecessor();
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= C.N) return;
-  double* st = state + i * SAKI_VSHARD_STATE;
-  if (stage == 0) { vs_combine_a(C, i, part, st); if ((int)st[VS_MODE] == VS_SOLVING && n_solving) atomicAdd(n_solving, 1u); }
-  else if (stage == 1) {
-    const double was = st[VS_F64];
-    if (vs_combine_b(C, i, part, st) && n_solving) atomicAdd(n_solving, 1u);
-    if (n_marked && st[VS_F64] != was) atomicAdd(n_marked, 1u);
+  const int tid = threadIdx.x, lr = tid / VC_LANES, lane = tid % VC_LANES;
+  const int64_t row0 = (int64_t)blockIdx.x * VC_ROWS, i = row0 + lr;
+  const int rows = (int)min((int64_t)VC_ROWS, C.N - row0);
+  const bool held = C.world <= VC_WORLD;                     // (more ranks: read where they are)
+  if (held) {
+#pragma unroll 8
+    for (int k = tid; k < C.world * rows * P; k += VC_THREADS) {
+      const int r = k / (rows * P), q = k - r * rows * P;
+      sp[q / P][r][q % P] = part[((int64_t)r * C.N + row0) * P + q];
+    }
   }
-  else if (stage == 2) vs_combine_c(C, i, part, st);
-  else vs_combine_d(C, i, part, st, o);
+  if (stage > 0)
+    for (int k = tid; k < rows * S; k += VC_THREADS) sst[k / S][k % S] = state[row0 * S + k];
+  __syncthreads();
+  const double* const mine = held ? &sp[lr][0][0] : part + i * P;
+  const int64_t rs = held ? P + 1 : C.N * P;
+  VsMaxima m = {};
+  if (stage == 0) {
+    if (lr < rows) {
+      m = vs_maxima(C, mine, rs);
+      if (held) for (int r = lane; r < C.world; r += VC_LANES) vs_rescale(C, mine + r * rs, m, scaled[lr][r]);
+    }
+    __syncthreads();
+  }
+  if (lr < rows && lane == 0) {
+    double* const st = sst[lr];
+    if (stage == 0) {
+      vs_combine_a(C, i, mine, rs, st, m, held ? &scaled[lr][0][0] : nullptr, VA_COUNT);
+      if ((int)st[VS_MODE] == VS_SOLVING && n_solving) atomicAdd(n_solving, 1u);
+    } else if (stage == 1) {
+      const double was = st[VS_F64];
+      if (vs_combine_b(C, i, mine, rs, st) && n_solving) atomicAdd(n_solving, 1u);
+      if (n_marked && st[VS_F64] != was) atomicAdd(n_marked, 1u);
+    }
+    else if (stage == 2) vs_combine_c(C, i, mine, rs, st);
+    else vs_combine_d(C, i, mine, rs, st, o);
+  }
+  __syncthreads();
+  for (int k = tid; k < rows * S; k += VC_THREADS) state[row0 * S + k] = sst[k / S][k % S];
 }
 
 // the call may use the float32 slice kernels: a property of the call's arguments alone, so that every rank's
@@ -1070,22 +1168,26 @@ cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, co
     }
     const int64_t N = in[i0].N;
     const double gs = (double)grad_scale;
-    if (n_fast > 0) {
-      // (A block per row and slice, in the later waves and stage 3 too, where most rows have nothing left to do: with one
-      // per two or four rows those that have wait for one another, 715 -> 738, 753 us for 1024 rows in eight slices.)
-      const dim3 grid((unsigned)(N < 8LL * sms ? N : 8LL * sms), (unsigned)m, 1);
-      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, FT, 0, st, true, Gr, state, gs); };
-      cudaError_t e = stage == 0 ? go(vs_fast_kernel<0>) : stage == 1 ? go(vs_fast_kernel<1>) : stage == 2 ? go(vs_fast_kernel<2>) : go(vs_fast_kernel<3>);
+    const bool marks = n_fast < m || !(stage == 0 || (flags & SAKI_VSHARD_NONE_MARKED));    // (no row is marked before the first combine)
+    if (marks) {
+      const int64_t blocks = (3LL * sms + m - 1) / m;
+      const dim3 grid((unsigned)(N < blocks ? N : blocks), (unsigned)m, 1);
+      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, VT, 0, st, true, Gr, stage, state, gs); };
+      cudaError_t e = in[i0].dtype == SAKI_BF16 ? go(vs_partial_kernel<__nv_bfloat16>) : go(vs_partial_kernel<float>);
       *n_launches += 1;
       if (e != cudaSuccess) return e;
     }
-    if (n_fast == m && (stage == 0 || (flags & SAKI_VSHARD_NONE_MARKED))) continue;    // (no row is marked before the first combine)
-    const int64_t blocks = (3LL * sms + m - 1) / m;
-    const dim3 grid((unsigned)(N < blocks ? N : blocks), (unsigned)m, 1);
-    auto go = [&](auto kernel) { return launch_pdl(kernel, grid, VT, 0, st, true, Gr, stage, state, gs, n_fast > 0); };
-    cudaError_t e = in[i0].dtype == SAKI_BF16 ? go(vs_partial_kernel<__nv_bfloat16>) : go(vs_partial_kernel<float>);
-    *n_launches += 1;
-    if (e != cudaSuccess) return e;
+    if (n_fast > 0) {
+      // (A block per row and slice, in the later waves and stage 3 too, where most rows have nothing left to do: with one
+      // per two or four rows those that have wait for one another, 715 -> 738, 753 us for 1024 rows in eight slices.)
+      const bool draw = stage == 3 && n_fast == m && !dlogits;
+      const dim3 grid((unsigned)(N < 8LL * sms ? N : 8LL * sms), draw ? 1u : (unsigned)m, 1);
+      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, FT, 0, st, true, Gr, state, gs, marks); };
+      cudaError_t e = draw ? launch_pdl(vs_draw_kernel, grid, FT, 0, st, true, Gr, state, m, marks)
+                    : stage == 0 ? go(vs_fast_kernel<0>) : stage == 1 ? go(vs_fast_kernel<1>) : stage == 2 ? go(vs_fast_kernel<2>) : go(vs_fast_kernel<3>);
+      *n_launches += 1;
+      if (e != cudaSuccess) return e;
+    }
   }
   return cudaSuccess;
 }
@@ -1101,8 +1203,8 @@ static VsConsts consts_of(const saki_vshard_in& in, bool allow_fast) {
 cudaError_t launch_vshard_combine(const saki_vshard_in& in, int stage, const double* gathered, double* state, const saki_out& out,
                                   unsigned int* n_solving, unsigned int* n_marked, bool allow_fast, cudaStream_t st) {
   const VsConsts c = consts_of(in, allow_fast);
-  const int th = 32;           // one thread per row, a chain of float64 scalars: spread over the SMs
-  return launch_pdl(vs_combine_kernel, dim3((unsigned)((in.N + th - 1) / th)), th, 0, st, true, c, stage, gathered, state, out, n_solving, n_marked);
+  return launch_pdl(vs_combine_kernel, dim3((unsigned)((in.N + VC_ROWS - 1) / VC_ROWS)), VC_THREADS, 0, st, true, c, stage, gathered,
+                    state, out, n_solving, n_marked);
 }
 
 // the same combine on HOST buffers (a caller without a GPU at hand, and the multi-process tests of the exchange)
@@ -1112,10 +1214,15 @@ int vshard_combine_host(const saki_vshard_in& in, int stage, const double* gathe
   int solving = 0;
   for (int64_t i = 0; i < in.N; ++i) {
     double* st = state + i * SAKI_VSHARD_STATE;
-    if (stage == 0) { vs_combine_a(c, i, gathered, st); solving += (int)st[VS_MODE] == VS_SOLVING; }
-    else if (stage == 1) solving += vs_combine_b(c, i, gathered, st);
-    else if (stage == 2) vs_combine_c(c, i, gathered, st);
-    else vs_combine_d(c, i, gathered, st, out);
+    const double* const mine = gathered + i * SAKI_VSHARD_PARTIALS;
+    const int64_t rs = c.N * SAKI_VSHARD_PARTIALS;
+    if (stage == 0) {
+      vs_combine_a(c, i, mine, rs, st, vs_maxima(c, mine, rs), nullptr, 0);
+      solving += (int)st[VS_MODE] == VS_SOLVING;
+    }
+    else if (stage == 1) solving += vs_combine_b(c, i, mine, rs, st);
+    else if (stage == 2) vs_combine_c(c, i, mine, rs, st);
+    else vs_combine_d(c, i, mine, rs, st, out);
   }
   return solving;
 }
