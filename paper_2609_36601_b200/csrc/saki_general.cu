@@ -142,6 +142,9 @@ __device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* _
 }
 
 // The scalars between the passes, on one warp per block (all lanes alike).
+// 1 / x of a sum of exponentials: short while x is in float32's range
+__device__ __forceinline__ double rcp_sum(double x) { return x > 1e-30 && x < 1e30 ? rcp_fast(x) : 1.0 / x; }
+
 __device__ __noinline__ double first_guess(double m1, double m2, double m3, double m4, double rtau, double kl1, double eps) {
   const double var = m2 - m1 * m1, m1s = m1 * m1;
   const double c3 = m3 - 3.0 * m1 * m2 + 2.0 * m1 * m1s;
@@ -163,7 +166,7 @@ __device__ __noinline__ double first_guess(double m1, double m2, double m3, doub
 
 // One evaluation at beta: v[k] = sum p exp(beta d) d^k.  Returns true when lambda is settled (bc[G_LAM], bc[G_LOGZ], bc[G_KL]).
 __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps) {
-  const double beta = bc[G_BETA], r0 = 1.0 / v[0], L = log(v[0]);
+  const double beta = bc[G_BETA], r0 = rcp_sum(v[0]), L = LN2 * log2_fast(v[0]);
   const double m1 = v[1] * r0, m2 = v[2] * r0, m3 = v[3] * r0, m4 = v[4] * r0, m1s = m1 * m1;
   if (beta == 0.0) {                                         // the moments under p, for a guess on their scale (below)
     const double b = sqrt(2.0 * eps / (m2 - m1s)), top = 0.5 * bc[G_HI];
@@ -193,7 +196,7 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
     if (!(dv > 0.25 * slope)) { ok = false; break; }
     const double dh = pv / dv;
     h -= dh;
-    if (fabs(dh) <= 1e-15 * fabs(beta)) break;
+    if (fabs(dh) <= 1e-9 * fabs(h)) break;                   // (the next step would be the square of this one)
   }
   if (!ok) h = f0 / slope;                                   // the model bends over: Newton's step
   double nb = beta + h;
@@ -408,10 +411,10 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       double lp_x = 0.0, lT_x = 0.0, acc = 1.0;
       int corrected = 0, tok = -1;
       if (!bonus) {
-        lp_x = (double)sx / (double)P.temperature - lse_s;
-        lT_x = (double)tx / (double)P.temperature - lse_t;
+        lp_x = (double)sx * rtau - lse_s;
+        lT_x = (double)tx * rtau - lse_t;
         if (lam > 0.0) {
-          acc = exp(fmin(0.0, lam * (lT_x - lp_x) - bc[G_LOGZ]));
+          acc = exp2_fast(fmin(0.0, lam * (lT_x - lp_x) - bc[G_LOGZ]) * INV_LN2);
           corrected = (scalar_uniform(P.seed, rid, STAGE_ACCEPT) < acc) ? 0 : 1;
         }
       }
@@ -458,16 +461,16 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       bc[G_AM] = am;
       if (status) { bc[G_STATUS] = (double)status; bc[G_MODE] = (double)G_FLAG; }
       else {
-        const double lse_s = log(S) - ks * LN2, lse_t = log(St) - kt * LN2, cc = lse_t - lse_s;
+        const double lse_s = (log2_fast(S) - ks) * LN2, lse_t = (log2_fast(St) - kt) * LN2, cc = lse_t - lse_s;
         bc[G_KP] = -INV_LN2 * lse_s; bc[G_CC] = cc; bc[G_LSE_T] = lse_t;
-        const double kl1 = N1 / St * rtau - cc;               // KL(T || p)
+        const double kl1 = N1 * rcp_sum(St) * rtau - cc;      // KL(T || p)
         const bool endpoint = !(eps > 0.0) || kl1 <= eps;
         bc[G_LOGZ] = 0.0; bc[G_STATUS] = 0.0;
         bc[G_LAM] = !(eps > 0.0) ? 0.0 : 1.0; bc[G_KL] = !(eps > 0.0) ? 0.0 : kl1;
         __syncwarp();
         if (endpoint) decide_row(!(eps > 0.0) ? SAKI_ROW_EPS_ZERO : SAKI_ROW_SATURATED);
         else {
-          const double rS = 1.0 / S;
+          const double rS = rcp_sum(S);
           double beta = first_guess(M1 * rS, M2 * rS, M3 * rS, M4 * rS, rtau, kl1, eps);
           if (P.from_list && P.redo_guess) {     // the float32 kernel's value of lambda, good to ~1e-5: one evaluation from here
             const double g0 = (double)P.redo_guess[item];
