@@ -49,7 +49,7 @@ struct Shared {
   int next[2];
 };
 enum { G_STATUS = 0, G_MODE, G_BETA, G_KP, G_CC, G_LSE_T, G_LAM, G_LOGZ, G_KL, G_LO, G_HI, G_ITER, G_AM, G_OWNER, G_BEFORE,
-       G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_ZERO, G_COUNT };
+       G_TARGET, G_LAST, G_TV, G_TOK, G_SC, G_CORR, G_ACC, G_LPX, G_LTX, G_LOSS, G_ZERO, G_UACC, G_UDRAW, G_COUNT };
 static_assert(G_COUNT <= 32, "broadcast area too small");
 enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS, PA_MT, PA_AM };   // pass "sums" (AM: -1 - index if a logit is not finite)
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
@@ -194,7 +194,7 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
     const double pv = h * (slope + h * (c2 + h * (c3 + h * c4))) - f0;
     const double dv = slope + h * (2.0 * c2 + h * (3.0 * c3 + h * (4.0 * c4)));
     if (!(dv > 0.25 * slope)) { ok = false; break; }
-    const double dh = pv / dv;
+    const double dh = pv * rcp_sum(dv);
     h -= dh;
     if (fabs(dh) <= 1e-9 * fabs(h)) break;                   // (the next step would be the square of this one)
   }
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   int turn = 0, nxt = -1;
   for (int64_t item = blockIdx.x / CS; item >= 0 && item < n_work; item = steal ? (int64_t)nxt : item + stride) {
     const int64_t row = P.from_list ? (int64_t)P.redo_list[item] : item;   // list mode: rows handed over by the float32 kernels
-    const int64_t b = row / P.K1;
+    const int64_t b = P.K1 == 1 ? row : row / P.K1;
     const int j = (int)(row - b * P.K1);
     const T* const s = (const T*)P.s + b * P.s_seq + (int64_t)j * P.s_pos;
     const T* const t = (const T*)P.t + b * P.t_seq + (int64_t)j * P.t_pos;
@@ -306,6 +306,9 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
     auto part_begin = [&](int w) { return w == 0 ? 0 : head + min(nck, w * cseg) * CW; };
     auto part_end = [&](int w) { return w == NWC - 1 ? V : head + min(nck, (w + 1) * cseg) * CW; };
     if (steal && tid == 0 && crank == 0) steal_request(sh.answer, &sh.bar);
+    // the row's uniforms, on a warp that does no scalars (the last row's are read before a barrier that this warp has passed)
+    if (tid == 32) bc[G_UACC] = scalar_uniform(P.seed, rid, STAGE_ACCEPT);
+    if (tid == 64) bc[G_UDRAW] = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
     const float d0 = ld_as_float(t, 0) - ld_as_float(s, 0);  // the logit difference is taken about this one: no offset of hundreds in its moments
 
     // ---- pass "sums"
@@ -371,18 +374,15 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         ms = xs; mt = xt;
         if (!again) break;
       }
-      ss = warp_sum(ss); st = warp_sum(st); n1 = warp_sum(n1);
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        m1 += __shfl_xor_sync(0xffffffffu, m1, o); m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-        m3 += __shfl_xor_sync(0xffffffffu, m3, o); m4 += __shfl_xor_sync(0xffffffffu, m4, o);
-      }
+      const double v8[8] = {ss, st, n1, (double)m1, (double)m2, (double)m3, (double)m4, 0.0};
+      const double a = warp_sum8(v8, lane);
       // a logit that is not finite leaves n1 so (an exponential is never 0 and the difference is then infinite or NaN)
-      const bool inf = !(fabs(n1) + ss + st < CUDART_INF);
+      const bool inf = __any_sync(0xffffffffu, lane < 12 && !(fabs(a) < CUDART_INF));
+      double* const p = sh.part[ph][warp];
+      static_assert(PA_ST == PA_SS + 1 && PA_N1 == PA_SS + 2 && PA_M4 == PA_SS + 6, "seven sums side by side");
+      if ((lane & 3) == 0 && lane < 28) p[PA_SS + (lane >> 2)] = a;
       if (lane == 0) {
-        double* const p = sh.part[ph][warp];
-        p[PA_KS] = ks; p[PA_KT] = kt; p[PA_SS] = ss; p[PA_ST] = st; p[PA_N1] = n1;
-        p[PA_M1] = (double)m1; p[PA_M2] = (double)m2; p[PA_M3] = (double)m3; p[PA_M4] = (double)m4;
+        p[PA_KS] = ks; p[PA_KT] = kt;
         p[PA_MS] = (double)ms; p[PA_MT] = (double)mt; p[PA_AM] = inf ? -1.0 : (double)am;
       }
     }
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         lT_x = (double)tx * rtau - lse_t;
         if (lam > 0.0) {
           acc = exp2_fast(fmin(0.0, lam * (lT_x - lp_x) - bc[G_LOGZ]) * INV_LN2);
-          corrected = (scalar_uniform(P.seed, rid, STAGE_ACCEPT) < acc) ? 0 : 1;
+          corrected = (bc[G_UACC] < acc) ? 0 : 1;
         }
       }
       double loss = 0.0, coef = 0.0;                         // gradient = coef (p - onehot(tok)) / tau
@@ -453,8 +453,10 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         S += fs * p[PA_SS]; St += ft * p[PA_ST]; N1 += ft * p[PA_N1];
         M1 += fs * p[PA_M1]; M2 += fs * p[PA_M2]; M3 += fs * p[PA_M3]; M4 += fs * p[PA_M4];
       }
-      S = warp_sum(S); St = warp_sum(St); N1 = warp_sum(N1);
-      M1 = warp_sum(M1); M2 = warp_sum(M2); M3 = warp_sum(M3); M4 = warp_sum(M4);
+      const double v8[8] = {S, St, N1, M1, M2, M3, M4, 0.0};
+      const double a = warp_sum8(v8, lane);
+      auto total = [&](int k) { return __shfl_sync(0xffffffffu, a, 4 * k); };
+      S = total(0); St = total(1); N1 = total(2); M1 = total(3); M2 = total(4); M3 = total(5); M4 = total(6);
       uint32_t status = 0;
       if (!finite) status = SAKI_ROW_NONFINITE;
       else if (!bonus && (x < 0 || x >= V)) status = SAKI_ROW_BAD_ID;
@@ -503,11 +505,9 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         const double w1 = e * d, q = d * d, w2 = e * q;
         a0 += e; a1 += w1; a2 += w2; a3 = fma(w1, q, a3); a4 = fma(w2, q, a4);
       });
-      a0 = warp_sum(a0); a1 = warp_sum(a1); a2 = warp_sum(a2); a3 = warp_sum(a3); a4 = warp_sum(a4);
-      if (lane == 0) {
-        double* const p = sh.part[ph][warp];
-        p[0] = a0; p[1] = a1; p[2] = a2; p[3] = a3; p[4] = a4;
-      }
+      const double v8[8] = {a0, a1, a2, a3, a4, 0.0, 0.0, 0.0};
+      const double a = warp_sum8(v8, lane);
+      if ((lane & 3) == 0 && lane < 20) sh.part[ph][warp][lane >> 2] = a;
       phase_barrier();
       if (warp == 0) {
         double v[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
@@ -516,8 +516,10 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
 #pragma unroll
           for (int k = 0; k < 5; ++k) v[k] += p[k];
         }
+        const double v8[8] = {v[0], v[1], v[2], v[3], v[4], 0.0, 0.0, 0.0};
+        const double a = warp_sum8(v8, lane);
 #pragma unroll
-        for (int k = 0; k < 5; ++k) v[k] = warp_sum(v[k]);
+        for (int k = 0; k < 5; ++k) v[k] = __shfl_sync(0xffffffffu, a, 4 * k);
         if (solve_step(bc, v, eps)) decide_row(0u);
       }
       __syncthreads();
@@ -591,7 +593,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
           const double up = __shfl_up_sync(0xffffffffu, inc, o);
           if (lane >= o) inc += up;
         }
-        const double target = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL) * __shfl_sync(0xffffffffu, inc, 31);
+        const double target = bc[G_UDRAW] * __shfl_sync(0xffffffffu, inc, 31);
         const unsigned hit = __ballot_sync(0xffffffffu, inc > target), pos = __ballot_sync(0xffffffffu, wa[0] + wa[1] > 0.0);
         // rounding left no crossing: the last index with positive weight
         const int ol = hit ? __ffs(hit) - 1 : (pos ? 31 - __clz(pos) : 0);
@@ -621,6 +623,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
           return bonus ? q : fmax(r, 0.0);
         };
         double w = 0.0;
+#pragma unroll 4
         for (int v = o0 + warp * sl + lane; v < min(o1, o0 + (warp + 1) * sl); v += 32) w += weight(v);
         w = warp_sum(w);
         if (lane == 0) sh.sub[warp] = w;
@@ -638,9 +641,12 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
         if (warp == mine) {
           int last_pos = -1, found = -1;
           const int e1 = min(o1, o0 + (mine + 1) * sl);
-          for (int v0 = o0 + mine * sl; v0 < e1 && found < 0; v0 += 32) {
+          const int b1 = o0 + mine * sl;
+          double next = b1 + lane < e1 ? weight(b1 + lane) : 0.0;
+          for (int v0 = b1; v0 < e1 && found < 0; v0 += 32) {
             const int v = v0 + lane;
-            const double r = v < e1 ? weight(v) : 0.0;
+            const double r = next;
+            next = v + 32 < e1 ? weight(v + 32) : 0.0;       // (on its way while these are looked through)
             double inc = r;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -660,7 +666,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       }
     }
     if (writer) {
-      const double lse_s = -LN2 * kp, lse_t = bc[G_LSE_T], Lam = bc[G_LOGZ], tau = (double)P.temperature;
+      const double lse_s = -LN2 * kp, lse_t = bc[G_LSE_T], Lam = bc[G_LOGZ];
       const double lp_x = bc[G_LPX], lT_x = bc[G_LTX];
       RowResult r;
       r.status = (uint32_t)bc[G_STATUS];
@@ -670,11 +676,11 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
       r.accept = bonus ? 0.f : (float)bc[G_ACC];
       r.logp_x = (float)lp_x; r.logT_x = (float)lT_x;
       r.logq_x = bonus ? 0.f : (float)(lp_x + lam * (lT_x - lp_x) - Lam);
-      const double lp_y = (double)ld_as_float(s, y) / tau - lse_s, lT_y = (double)ld_as_float(t, y) / tau - lse_t;
+      const double lp_y = (double)(y == x ? sx : ld_as_float(s, y)) * rtau - lse_s, lT_y = (double)(y == x ? tx : ld_as_float(t, y)) * rtau - lse_t;
       r.logp_y = (float)lp_y; r.logT_y = (float)lT_y;
       r.logq_y = (float)(lp_y + lam * (lT_y - lp_y) - Lam);
       r.loss = (float)bc[G_LOSS];
-      if (corrected && !masked) r.loss = (float)-((double)ld_as_float(s, r.vstar) / tau - lse_s);
+      if (corrected && !masked) r.loss = (float)-((double)ld_as_float(s, r.vstar) * rtau - lse_s);
       write_row(P.out, row, r, !P.spec);
     }
     ph ^= 1;
