@@ -21,6 +21,7 @@
 #include <cooperative_groups.h>
 #include <algorithm>
 #include <atomic>
+#include <cmath>
 
 namespace cg = cooperative_groups;
 
@@ -30,12 +31,6 @@ namespace {
 
 constexpr int GT = 256;        // threads per block
 constexpr int GW = GT / 32;    // warps per block
-// Blocks per SM: more of them hide one another's serial steps, fewer have the registers to interleave elements.  No number is
-// the best everywhere (us, with 2 / 3 / 4): bf16 1024 rows of 32003 275 / 286 / 312, 2000 of them 516 / 505 / 515, 256 of them
-// 82 / 109 / 88, 512 rows of 100001 465 / 439 / 464, 1024 rows of 2049 52 / 47 / 48; fp32 512 rows of 151936 799 / 806 / 786, 64 of
-// them 115 / 160 / 118, 4096 rows of 1024 143 / 122 / 124, 1024 rows of 32000 304 / 355 / 340.  bf16 takes three for its long
-// calls, fp32 four for the longest rows.
-template <typename T> constexpr int BLOCKS_PER_SM = sizeof(T) == 4 ? 4 : 3;
 constexpr int MAX_CS = 8;      // blocks per row, at most
 constexpr int NPART = 12;      // doubles a warp leaves per phase
 
@@ -227,9 +222,9 @@ __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps)
 
 }  // namespace
 
-// CS: blocks per row (1, or a cluster of CS blocks).
-template <typename T, int CS>
-__global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const RowParams P, const int steal, const double rtau, const double c) {
+// CS: blocks per row (1, or a cluster of CS blocks); KS: blocks per SM.
+template <typename T, int CS, int KS>
+__global__ void __launch_bounds__(GT, KS) general_kernel(const RowParams P, const int steal, const double rtau, const double c) {
   __shared__ Shared sh;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int V = P.V;
@@ -697,7 +692,7 @@ __global__ void __launch_bounds__(GT, BLOCKS_PER_SM<T>) general_kernel(const Row
   if (P.from_list) close_counters(P.redo_count);
 }
 
-template <typename T, int CS>
+template <typename T, int CS, int KS>
 static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t st) {
   // blocks (clusters) that are resident at once: the grid, so that none starts after the others have finished
   static std::atomic<int> fit_of[64];
@@ -716,9 +711,9 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
     if (CS > 1) {
       cfg.gridDim = dim3(CS, 1, 1);
       at[0].val.programmaticStreamSerializationAllowed = 0;
-      e = cudaOccupancyMaxActiveClusters(&n, general_kernel<T, CS>, &cfg);
+      e = cudaOccupancyMaxActiveClusters(&n, general_kernel<T, CS, KS>, &cfg);
     } else {
-      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, general_kernel<T, CS>, GT, 0);
+      e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, general_kernel<T, CS, KS>, GT, 0);
       n *= sms;
     }
     if (e != cudaSuccess) return e;
@@ -732,31 +727,69 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
   at[0].val.programmaticStreamSerializationAllowed = 1;
   if (p.from_list) fit = std::min(fit, std::max(1, sms / CS));     // as a rule they only find the list empty
   cfg.gridDim = dim3((unsigned)(CS * (p.n_rows < fit || steal ? p.n_rows : fit)), 1, 1);
-  return cudaLaunchKernelEx(&cfg, general_kernel<T, CS>, p, (int)steal, rtau, INV_LN2 * rtau);
+  return cudaLaunchKernelEx(&cfg, general_kernel<T, CS, KS>, p, (int)steal, rtau, INV_LN2 * rtau);
+}
+
+// How a call is laid out: blocks per row (cs) and blocks per SM (k, by the registers a thread is given: 128, 80 or 64).  Two
+// blocks per SM run a row soonest, more of them hide one another's serial steps and share an SM's slots out more finely.
+//   - A call whose blocks are all resident two to an SM, and whose rows stay in L2 between the passes (200 MB: a pass behind
+//     another finds most of 126 MB of L2 all the same), takes two, and as many blocks per row as fit and keep 4000 elements or more
+//     (us, with the layout of before and now: fp32 64 rows of 1024 13.2 / 11.5, 64 of 16000 30.5 / 22.5, 148 of 50000 107 / 69;
+//     bf16 148 rows of 16001 38.5 / 29.6, 64 of 100001 84 / 64).
+//   - Of the others the one that takes the least by a cost model: turns, times what a turn takes of a row's serial steps, its
+//     elements and the rows in flight beyond L2.  Fitted to the times of fp32 rows of 1024 to 151936 and bf16 rows of 1025 to
+//     100001, 24 to 3000 of them, all layouts: the choice is 0.6 % (fp32) and 0.4 % (bf16) above the best on average, and the rule
+//     before (fp32 four to an SM, bf16 three) was 15 and 10 %.
+// The kernel pinned (call_rows = 0), the rows do not count, so that pieces of a batch agree with the whole to the bit: blocks per row
+// by V alone, so many that the rows in flight stay in L2.  In list mode (a handful of rows as a rule; the host does not know
+// their number) as many blocks per row as a row has 2048 elements for.
+struct Layout { int cs, k; };
+static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms) {
+  const int64_t row_bytes = 2 * (int64_t)V * (f32 ? 4 : 2);
+  int cs = 1;
+  if (from_list || rows <= 0) {
+    const int k = from_list ? 2 : f32 ? 4 : 3;
+    while (cs < MAX_CS && V >= (from_list ? 2048 : 4096) * cs && (from_list || (int64_t)k * sms / cs * row_bytes > (150 << 20))) cs *= 2;
+    return {cs, cs == 8 ? 2 : k};
+  }
+  if (rows <= 2 * sms && rows * row_bytes <= 200000000) {
+    while (cs < MAX_CS && rows * 2 * cs <= 2 * sms && V >= 8000 * cs) cs *= 2;
+    return {cs, 2};
+  }
+  static const Layout all[] = {{1, 2}, {1, 3}, {2, 2}, {4, 2}, {8, 2}, {1, 4}, {2, 4}, {4, 4}};     // (the last three: fp32)
+  // microseconds: a row's serial steps, 1000 elements of a block, a doubling of the blocks; the part of a turn that is waited for
+  // to its end (blocks take over rows that have not started); 126 MB in flight beyond L2
+  static const double serial[2][3] = {{10.25, 13.6, 17.0}, {7.7, 10.06, 13.0}}, element[2][3] = {{1.83, 2.62, 3.3}, {2.24, 3.4, 4.14}};
+  static const double join[2] = {0.1, 0.6}, whole[2] = {0.15, 0.2}, beyond[2] = {0.15, 0.05};
+  Layout best = all[0];
+  double least = 1e300;
+  for (int i = 0; i < (f32 ? 8 : 5); ++i) {
+    const Layout l = all[i];
+    if (l.cs > 1 && V < 4000 * l.cs) continue;
+    const double slots = (double)(l.k * sms / l.cs), turns = (double)rows / slots, in_flight = std::min((double)rows, slots) * (double)row_bytes;
+    if (l.cs == 1 && l.k > 2 && in_flight > 126e6) continue;         // (1024 fp32 rows of 32000: 316 us with four to an SM, 298 with two)
+    double t = serial[f32][l.k - 2] + element[f32][l.k - 2] * 1e-3 * V / l.cs + join[f32] * std::log2((double)l.cs);
+    t *= 1.0 + beyond[f32] * std::max(0.0, in_flight / 126e6 - 1.0);
+    if (turns > 1.0) t *= whole[f32] * std::ceil(turns) + (1.0 - whole[f32]) * (turns + 0.5);
+    if (t < least) { least = t; best = l; }
+  }
+  return best;
 }
 
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
-  // Blocks per row.  In list mode (a handful of rows as a rule; the host does not know their number) always the most;
-  // otherwise as many as are resident at once, each block keeping 2048 elements or more (below that the barriers of a
-  // cluster cost more than its blocks save: 64 fp32 rows of 2048 16.9 us with two blocks each, 14.5 with one; beyond what
-  // is resident a call takes twice the turns: 128 rows of 8192 54 us with eight, 29 with four), and so many that the rows
-  // in flight stay in L2 between the passes
-  // (fp32 rows of 151936, 1.2 MB each: 1.01 / 0.82 / 0.79 / 0.81 ms with 1 / 2 / 4 / 8 blocks per row).  The limit of 150 MB
-  // lies a little above the 126 MB of L2, as a pass behind another finds most of its rows there all the same; measured with 100 /
-  // 150 / 250 MB: 512 bf16 rows of 100001 439 / 439 / 596 us, 512 fp32 rows of 151936 785 / 786 / 739, 1024 of 32000 326 / 340 / 340.
-  // Where the
-  // kernel is pinned (call_rows = 0) the rows do not count, so that pieces of a batch agree with the whole to the bit.
-  int cs = 1;
-  const int64_t in_flight = BLOCKS_PER_SM<T> * (int64_t)sms, row_bytes = 2 * (int64_t)p.V * (int64_t)sizeof(T);
-  while (cs < MAX_CS && p.V >= (p.from_list ? 2048 : 4096) * cs &&
-         (p.from_list || (p.call_rows > 0 && p.call_rows * 2 * cs <= in_flight) || in_flight / cs * row_bytes > (150 << 20)))
-    cs *= 2;
-  switch (cs) {
-    case 1: return launch_cs<T, 1>(p, dev, sms, st);
-    case 2: return launch_cs<T, 2>(p, dev, sms, st);
-    case 4: return launch_cs<T, 4>(p, dev, sms, st);
-    default: return launch_cs<T, 8>(p, dev, sms, st);
+  const Layout l = pick_layout(p.V, p.call_rows, p.from_list != 0, sizeof(T) == 4, sms);
+  switch (l.cs * 16 + l.k) {
+    case 16 + 3: return launch_cs<T, 1, 3>(p, dev, sms, st);
+    case 16 + 4: return launch_cs<T, 1, 4>(p, dev, sms, st);
+    case 32 + 2: return launch_cs<T, 2, 2>(p, dev, sms, st);
+    case 32 + 3: return launch_cs<T, 2, 3>(p, dev, sms, st);
+    case 32 + 4: return launch_cs<T, 2, 4>(p, dev, sms, st);
+    case 64 + 2: return launch_cs<T, 4, 2>(p, dev, sms, st);
+    case 64 + 3: return launch_cs<T, 4, 3>(p, dev, sms, st);
+    case 64 + 4: return launch_cs<T, 4, 4>(p, dev, sms, st);
+    case 128 + 2: return launch_cs<T, 8, 2>(p, dev, sms, st);
+    default: return launch_cs<T, 1, 2>(p, dev, sms, st);
   }
 }
 

@@ -24,9 +24,9 @@ def _shift(x, off):
     return y
 
 
-def _check(d, w, rows, offsets=(0, 0, 0)):
+def _check(d, w, rows, offsets=(0, 0, 0), kernel=1):
     s, t, g = (_shift(x, o) for x, o in zip((d["s"], d["t"], torch.zeros_like(d["s"])), offsets))
-    prev = P.set_kernel(1)
+    prev = P.set_kernel(kernel)
     try:
         out, g = P.route_fwd_bwd(s, t, d["proposal"], w.eps, w.temperature, w.seed, grad_scale=0.25, dlogits=g)
     finally:
@@ -50,6 +50,17 @@ def test_split_edges(V, dtype, N, offsets):
     w = synth.Workload("t", N, V, dtype, 0.078125, 1.2, V > 100, 300 + V, 17, temperature=0.875)
     rows = list(range(N)) if N < 10 else list(range(0, N, 37)) + [N - 1]
     _check(synth.generate(w, DEV), w, rows, offsets)
+
+
+@pytest.mark.parametrize("N,V,dtype", [(296, 1024, "f32"), (297, 1024, "f32"), (1100, 1024, "f32"), (148, 8000, "f32"), (149, 8000, "f32"),
+                                       (148, 7999, "f32"), (74, 16000, "f32"), (37, 32001, "f32"), (160, 151936, "f32"), (700, 50000, "f32"),
+                                       (400, 2049, "bf16"), (700, 2049, "bf16"), (148, 8001, "bf16"), (37, 33001, "bf16")])
+def test_layouts(N, V, dtype):
+    """Blocks per row and per SM as an unpinned call takes them: either side of two blocks on each of 148 SMs, of 4000 elements a
+    block, of what L2 holds, and calls of more rows than are resident."""
+    w = synth.Workload("t", N, V, dtype, 0.0625, 1.2, True, 600 + N + V, 29, temperature=0.875)
+    _check(synth.generate(w, DEV), w, sorted({0, 1, N // 2, N - 2, N - 1}), kernel=0)
+    assert P.last_kernel() == 1
 
 
 @pytest.mark.parametrize("drop", [150.0, 2000.0])
