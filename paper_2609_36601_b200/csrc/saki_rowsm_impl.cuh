@@ -402,7 +402,9 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   // step discards it if it was not needed).  `seqres`: [0] the row reserved for this CTA's next turn
   // (n_rows: none left), [1], [2] the rest of a ticket range this CTA holds, [3] how many tickets it takes
   // at a time: it aims at one live ticket per range (doubles after a range without one, halves after a
-  // range with several), so late positions, where most sequences have stopped, cost few round trips.
+  // range with several), so late positions, where most sequences have stopped, cost few round trips; but never more than
+  // a quarter of its share of the tickets that are left (as far as it has seen), so that no CTA ends up with several live ones in
+  // hand while the others have none.
   const bool dyn = SPEC && P.seq_next != nullptr;
   const int n_seq = dyn ? (int)(P.n_rows / K1c) : 1;
   const int n_tickets = (int)P.n_rows;
@@ -421,9 +423,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       bool fresh = false;
       if (blo >= bhi) {
         int old = 0;
-        if (lane == 0) old = (int)min((unsigned int)n_tickets, gridDim.x + atomicAdd(P.seq_next, (unsigned int)n));
+        const int take = min(n, max(1, (n_tickets - max(bhi, (int)gridDim.x)) / (4 * (int)gridDim.x)));
+        if (lane == 0) old = (int)min((unsigned int)n_tickets, gridDim.x + atomicAdd(P.seq_next, (unsigned int)take));
         old = __shfl_sync(0xffffffffu, old, 0);
-        blo = old; bhi = min(old + n, n_tickets);
+        blo = old; bhi = min(old + take, n_tickets);
         if (blo >= bhi) break;
         fresh = true;
       }
