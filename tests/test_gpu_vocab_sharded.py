@@ -214,3 +214,20 @@ def test_a_stream_that_is_not_the_current_one():
         assert torch.equal(out[k], ref[k]), k
     for a, b in zip(gs, g_ref):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("N,world", [(1, 8), (7, 16), (9, 17), (8, 33)])
+def test_combines_at_the_edges_of_their_groups(N, world):
+    """A combine takes eight rows a block and holds the records of up to sixteen ranks at once; a launch takes sixteen slices."""
+    V = 8192
+    w = synth.Workload("vs", N, V, "bf16", 0.125, 1.5, True, 950 + world, 50 + world)
+    d = synth.generate(w, DEV)
+    out, gs, _ = route_vocab_sharded_local(_slices(d, [(8 * a, 8 * n) for a, n in split_columns(V // 8, world)]), V, d["proposal"], w.eps,
+                                           w.temperature, w.seed, grad_scale=0.5)
+    s64, t64 = oracle_inputs(d)
+    ref = O.route(s64, t64, d["proposal"].cpu().numpy(), w.eps, w.temperature, w.seed, 0, grad_scale=0.5, want_grad=True, grad_dtype=w.dtype)
+    compare_rows(out, ref)
+    same = out["corrected"].cpu().numpy() == ref["corrected"]
+    tok = np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])
+    grad_check(to_np64(torch.cat(gs, dim=1))[same], ref["grad"][same], w.dtype, tok[same])
+    assert np.max(np.abs(out["lambda"].cpu().numpy() - ref["lam"])) <= 1e-5      # what the float32 kernels are held to
