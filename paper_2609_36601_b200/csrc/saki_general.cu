@@ -692,25 +692,21 @@ __global__ void __launch_bounds__(GT, KS) general_kernel(const RowParams P, cons
   if (P.from_list) close_counters(P.redo_count);
 }
 
+// blocks (clusters) that are resident at once: the grid, so that none starts after the others have finished
 template <typename T, int CS, int KS>
-static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t st) {
-  // blocks (clusters) that are resident at once: the grid, so that none starts after the others have finished
+static cudaError_t resident_rows(int dev, int sms, int* rows) {
   static std::atomic<int> fit_of[64];
   int fit = dev < 64 ? fit_of[dev].load(std::memory_order_relaxed) : 0;
-  cudaLaunchConfig_t cfg = {};
-  cfg.blockDim = dim3(GT, 1, 1);
-  cfg.stream = st;
-  cudaLaunchAttribute at[2];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[1].id = cudaLaunchAttributeClusterDimension;
-  at[1].val.clusterDim.x = CS; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
-  cfg.attrs = at; cfg.numAttrs = CS > 1 ? 2 : 1;
   if (fit <= 0) {
     int n = 0;
     cudaError_t e;
     if (CS > 1) {
-      cfg.gridDim = dim3(CS, 1, 1);
-      at[0].val.programmaticStreamSerializationAllowed = 0;
+      cudaLaunchConfig_t cfg = {};
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = CS; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+      cfg.blockDim = dim3(GT, 1, 1); cfg.gridDim = dim3(CS, 1, 1);
+      cfg.attrs = at; cfg.numAttrs = 1;
       e = cudaOccupancyMaxActiveClusters(&n, general_kernel<T, CS, KS>, &cfg);
     } else {
       e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, general_kernel<T, CS, KS>, GT, 0);
@@ -720,6 +716,23 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
     fit = n > 0 ? n : 1;
     if (dev < 64) fit_of[dev].store(fit, std::memory_order_relaxed);
   }
+  *rows = fit;
+  return cudaSuccess;
+}
+
+template <typename T, int CS, int KS>
+static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t st) {
+  int fit = 1;
+  const cudaError_t e = resident_rows<T, CS, KS>(dev, sms, &fit);
+  if (e != cudaSuccess) return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.blockDim = dim3(GT, 1, 1);
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = CS; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = CS > 1 ? 2 : 1;
   // One cluster per row where the hardware can be asked for the next one (a row's solve takes one evaluation or two,
   // and the rows do not divide evenly); in list mode, and for more rows than a grid may have blocks, a fixed stride.
   const bool steal = !p.from_list && p.n_rows > fit && p.n_rows <= (1 << 27);
@@ -736,6 +749,9 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
 //     another finds most of 126 MB of L2 all the same), takes two, and as many blocks per row as fit and keep 4000 elements or more
 //     (us, with the layout of before and now: fp32 64 rows of 1024 13.2 / 11.5, 64 of 16000 30.5 / 22.5, 148 of 50000 107 / 69;
 //     bf16 148 rows of 16001 38.5 / 29.6, 64 of 100001 84 / 64).
+//     Where some SMs would have two blocks and others one, twice the blocks at three to an SM, if they are all resident (which
+//     launch_t sees to: clusters of four and eight do not fill every SM) and keep 5000 elements or more (8000 in clusters of eight): fp32
+//     190 rows of 50000 128 -> 108, 89 of 120000 159 -> 125, bf16 42 rows of 123205 76 -> 66.
 //   - Of the others the one that takes the least by a cost model: turns, times what a turn takes of a row's serial steps, its
 //     elements and the rows in flight beyond L2.  Fitted to the times of fp32 rows of 1024 to 151936 and bf16 rows of 1025 to
 //     100001, 24 to 3000 of them, all layouts: the choice is 0.6 % (fp32) and 0.4 % (bf16) above the best on average, and the rule
@@ -754,6 +770,8 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
   }
   if (rows <= 2 * sms && rows * row_bytes <= 200000000) {
     while (cs < MAX_CS && rows * 2 * cs <= 2 * sms && V >= 8000 * cs) cs *= 2;
+    const int wide = 2 * cs;
+    if (wide <= MAX_CS && rows * cs > sms && rows * wide <= 3 * sms && V >= (wide == 8 ? 64000 : 10000 * cs)) return {wide, 3};
     return {cs, 2};
   }
   static const Layout all[] = {{1, 2}, {1, 3}, {2, 2}, {4, 2}, {8, 2}, {1, 4}, {2, 4}, {4, 4}};     // (the last three: fp32)
@@ -778,7 +796,13 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
 
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
-  const Layout l = pick_layout(p.V, p.call_rows, p.from_list != 0, sizeof(T) == 4, sms);
+  Layout l = pick_layout(p.V, p.call_rows, p.from_list != 0, sizeof(T) == 4, sms);
+  if (l.k == 3 && l.cs > 1 && p.call_rows > 0 && !p.from_list) {
+    int fit = 0;
+    const cudaError_t e = l.cs == 2 ? resident_rows<T, 2, 3>(dev, sms, &fit) : l.cs == 4 ? resident_rows<T, 4, 3>(dev, sms, &fit) : resident_rows<T, 8, 3>(dev, sms, &fit);
+    if (e != cudaSuccess) return e;
+    if (p.call_rows > fit) l = {l.cs / 2, 2};
+  }
   switch (l.cs * 16 + l.k) {
     case 16 + 3: return launch_cs<T, 1, 3>(p, dev, sms, st);
     case 16 + 4: return launch_cs<T, 1, 4>(p, dev, sms, st);
@@ -789,6 +813,7 @@ static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t s
     case 64 + 3: return launch_cs<T, 4, 3>(p, dev, sms, st);
     case 64 + 4: return launch_cs<T, 4, 4>(p, dev, sms, st);
     case 128 + 2: return launch_cs<T, 8, 2>(p, dev, sms, st);
+    case 128 + 3: return launch_cs<T, 8, 3>(p, dev, sms, st);
     default: return launch_cs<T, 1, 2>(p, dev, sms, st);
   }
 }

@@ -53,7 +53,8 @@ def test_split_edges(V, dtype, N, offsets):
 
 
 @pytest.mark.parametrize("N,V,dtype", [(296, 1024, "f32"), (297, 1024, "f32"), (1100, 1024, "f32"), (148, 8000, "f32"), (149, 8000, "f32"),
-                                       (148, 7999, "f32"), (74, 16000, "f32"), (37, 32001, "f32"), (160, 151936, "f32"), (700, 50000, "f32"),
+                                       (148, 7999, "f32"), (222, 10000, "f32"), (223, 10000, "f32"), (99, 20000, "f32"), (100, 20001, "bf16"),
+                                       (46, 64001, "bf16"), (47, 64001, "bf16"), (74, 16000, "f32"), (37, 32001, "f32"), (160, 151936, "f32"), (700, 50000, "f32"),
                                        (400, 2049, "bf16"), (700, 2049, "bf16"), (148, 8001, "bf16"), (37, 33001, "bf16")])
 def test_layouts(N, V, dtype):
     """Blocks per row and per SM as an unpinned call takes them: either side of two blocks on each of 148 SMs, of 4000 elements a
