@@ -393,7 +393,7 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
     auto read = [&] {
       return unlocked([&] {
         h.copy_(counts, true);
-        if (dev.is_cuda()) { copied.record(); copied.synchronize(); }
+        if (dev.is_cuda()) { copied.record(c10::cuda::getCurrentCUDAStream(dev.index())); copied.synchronize(); }
         return (const int32_t*)h.data_ptr();
       });
     };
