@@ -1,8 +1,7 @@
-// 2^y in float64 at seven operations of the float64 pipe, for the kernels that work in float64 throughout.
-// y is split by a magic-number addition into n + i/256 + r; 2^(i/256) comes from a table in shared memory and 2^r from a
-// polynomial of degree three (|r| <= 1/512: its fourth-order term is replaced by the parabola that leaves an error of
-// 3.5e-14, far below what any sum over a row resolves once it is rounded to float32; a degree more costs an operation of
-// eight).  The table is stored 16 times over, one copy per
+// 2^y in float64 at eight operations of the float64 pipe, for the kernels that work in float64 throughout.
+// y is split by a magic-number addition into n + i/256 + r; 2^(i/256) comes from a table in shared memory and 2^r from its
+// Taylor polynomial (|r| <= 1/512: the first dropped term is 4e-17).  A degree less would be seen: KL is a difference of sums of
+// these of the size of 1, an error e of theirs moves lambda by e / (2 eps) of itself.  The table is stored 16 times over, one copy per
 // 64-bit bank, so the lookups of a half-warp never conflict (32 KB).
 #pragma once
 #include "saki_device.cuh"
@@ -25,8 +24,7 @@ __device__ __forceinline__ void exp2_table(double* tab, int tid, int n_threads) 
 // the exponent in and the index back in one addition.
 // The coefficients are read from the constant bank (as operands: three 64-bit immediates cost two moves each per
 // exponential once registers are short, and a float64 operation on three register operands runs at two thirds of the rate).
-// ln2^i / i!, i = 3..1; the second with ln2^4 / 4! / 512^2 added (r^4 as r^2 / 512^2)
-static __constant__ double EXP2_COEF[3] = {5.550410866482158e-02, 2.402265069591007e-01 + 9.618129107628477e-03 / 262144.0, 6.931471805599453e-01};
+static __constant__ double EXP2_COEF[4] = {9.618129107628477e-03, 5.550410866482158e-02, 2.402265069591007e-01, 6.931471805599453e-01};   // ln2^i / i!, i = 4..1
 struct Exp2 {
   uint32_t lane8;   // this lane's copy of the table: byte offset among the 16 copies of an entry
   const double* tab;
@@ -42,6 +40,7 @@ struct Exp2 {
     double T = *(const double*)((const char*)tab + ((((uint32_t)k << 7) & 0x7f80u) | lane8));
     double q = fma(r, EXP2_COEF[0], EXP2_COEF[1]);
     q = fma(r, q, EXP2_COEF[2]);
+    q = fma(r, q, EXP2_COEF[3]);
     T = __hiloint2double(__double2hiint(T) + (k << 12), __double2loint(T));
     return fma(T * r, q, T);
   }

@@ -7,7 +7,7 @@
 //
 // What bounds it: the float64 pipe (64 lanes per clock and SM; a warp instruction occupies its scheduler's half of
 // it for two clocks).  Hence:
-//   - 2^y costs seven float64 operations (saki_exp2.cuh);
+//   - 2^y costs eight float64 operations (saki_exp2.cuh);
 //   - three passes over the row: "sums" (two exponentials), one or two evaluations of KL with its first four
 //     derivatives (one exponential each: the root of the fourth-order model, as in the bf16 kernels, here accepted
 //     when the dropped terms move lambda by less than about 1e-11), "final" (two exponentials; total variation, draw
