@@ -161,7 +161,7 @@ __device__ __noinline__ double first_guess(double m1, double m2, double m3, doub
 
 // One evaluation at beta: v[k] = sum p exp(beta d) d^k.  Returns true when lambda is settled (bc[G_LAM], bc[G_LOGZ], bc[G_KL]).
 __device__ __noinline__ bool solve_step(double* bc, const double* v, double eps) {
-  const double beta = bc[G_BETA], r0 = rcp_sum(v[0]), L = LN2 * log2_fast(v[0]);
+  const double beta = bc[G_BETA], r0 = rcp_sum(v[0]), L = log(v[0]);
   const double m1 = v[1] * r0, m2 = v[2] * r0, m3 = v[3] * r0, m4 = v[4] * r0, m1s = m1 * m1;
   if (beta == 0.0) {                                         // the moments under p, for a guess on their scale (below)
     const double b = sqrt(2.0 * eps / (m2 - m1s)), top = 0.5 * bc[G_HI];
@@ -458,7 +458,8 @@ __global__ void __launch_bounds__(GT, KS) general_kernel(const RowParams P, cons
       bc[G_AM] = am;
       if (status) { bc[G_STATUS] = (double)status; bc[G_MODE] = (double)G_FLAG; }
       else {
-        const double lse_s = (log2_fast(S) - ks) * LN2, lse_t = (log2_fast(St) - kt) * LN2, cc = lse_t - lse_s;
+        // (as few roundings as there are: KL takes those of lse_s one to one, those of the short logarithm too)
+        const double lse_s = fma(-LN2, ks, log(S)), lse_t = fma(-LN2, kt, log(St)), cc = lse_t - lse_s;
         bc[G_KP] = -INV_LN2 * lse_s; bc[G_CC] = cc; bc[G_LSE_T] = lse_t;
         const double kl1 = N1 * rcp_sum(St) * rtau - cc;      // KL(T || p)
         const bool endpoint = !(eps > 0.0) || kl1 <= eps;

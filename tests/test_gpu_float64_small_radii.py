@@ -69,3 +69,26 @@ def test_lambda_to_the_last_digits(eps, V, N, kind, sharded):
     E = 2.0 ** -53 * (4.0 * np.abs(ref[:, 2]) + 8.0)
     err = np.abs(out["lambda"].cpu().numpy().astype(np.float64) - ref[:, 0])
     assert (err <= E / ref[:, 1] + 2.0 ** -24 * ref[:, 0]).all(), (err * ref[:, 1] / E).max()
+
+
+@pytest.mark.parametrize("V", [64, 1024])
+def test_log_sum_exps_of_logits_far_from_zero(V):
+    """Student logits about 1000, the teacher's about -500: KL takes the roundings of the student's log-sum-exp one to one."""
+    N, eps = 100, 2.0 ** -30
+    g = torch.Generator().manual_seed(5 + V)
+    s = 2.0 * torch.randn(N, V, generator=g)
+    t = s + torch.randn(N, V, generator=g)
+    s += 1000.0
+    t -= 500.0
+    prev = P.set_kernel(1)
+    try:
+        out = P.route_fwd_bwd(s.to(DEV), t.to(DEV), torch.zeros(N, dtype=torch.int32, device=DEV), eps, 1.0, 3)[0]
+    finally:
+        P.set_kernel(prev)
+    ref = np.array([_solve(s[i].numpy(), t[i].numpy(), eps) for i in range(N)])
+    assert (ref[:, 2] < 1024).all()
+    # The log-sum-exp, below 1024, rounded once (2^-44); log2(e) times it, below 2048, once more (2^-43 of log2); ln 2 and log2(e) as
+    # float64 numbers, each good to 2.4e-17 and used on numbers of about 1450; the bound of the test above for what has no offset.
+    E = 2.0 ** -44 + np.log(2.0) * 2.0 ** -43 + 2 * 2.4e-17 * 1450 * np.log(2.0) + 2.0 ** -53 * (4.0 * (ref[:, 2] - 1000.0) + 8.0)
+    err = np.abs(out["lambda"].cpu().numpy().astype(np.float64) - ref[:, 0])
+    assert (err <= E / ref[:, 1] + 2.0 ** -24 * ref[:, 0]).all(), (err * ref[:, 1] / E).max()
