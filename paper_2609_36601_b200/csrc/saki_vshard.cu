@@ -401,7 +401,7 @@ __global__ void __launch_bounds__(VT) vs_partial_kernel(const __grid_constant__ 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int Vl = S.V_local;
   const double rtau = 1.0 / S.tau;
-  // (in this order: the float32 kernel of the same stage, launched right behind, starts without a wait of its own)
+  // (in this order: the float32 kernel of the same stage, launched right behind, starts without a wait of its own from stage B on)
   wait_for_predecessor();
   launch_dependents();
   // rows in groups of VT, dealt out to the blocks; where only marked rows count, a thread looks at one row's mark (as a
@@ -731,6 +731,9 @@ __global__ void __launch_bounds__(FT) vs_fast_kernel(const __grid_constant__ VsG
   // kernel runs, and the wait stands at the end: the next combine starts when both are done.  (With the float64 kernel
   // behind this one it could only start with the last of these blocks, and 28 of the 31 us that it takes in stage C
   // for 1024 rows of 151936 in eight slices came on top.)
+  // Not in stage A (rows of slices of either kind): it reads the caller's logits and proposals, which the kernel in front of the
+  // call may just have written, past no wait of its own.  From stage B on those are old, and what the combine wrote is read with
+  // __ldcg.
   if (!beside) wait_for_predecessor();
   launch_dependents();
   if (!S.fast) {
@@ -1182,8 +1185,9 @@ cudaError_t launch_vshard_partial(const saki_vshard_in* in, int n, int stage, co
       // per two or four rows those that have wait for one another, 715 -> 738, 753 us for 1024 rows in eight slices.)
       const bool draw = stage == 3 && n_fast == m && !dlogits;
       const dim3 grid((unsigned)(N < 8LL * sms ? N : 8LL * sms), draw ? 1u : (unsigned)m, 1);
-      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, FT, 0, st, true, Gr, state, gs, marks); };
-      cudaError_t e = draw ? launch_pdl(vs_draw_kernel, grid, FT, 0, st, true, Gr, state, m, marks)
+      const bool beside = marks && stage > 0;
+      auto go = [&](auto kernel) { return launch_pdl(kernel, grid, FT, 0, st, true, Gr, state, gs, beside); };
+      cudaError_t e = draw ? launch_pdl(vs_draw_kernel, grid, FT, 0, st, true, Gr, state, m, beside)
                     : stage == 0 ? go(vs_fast_kernel<0>) : stage == 1 ? go(vs_fast_kernel<1>) : stage == 2 ? go(vs_fast_kernel<2>) : go(vs_fast_kernel<3>);
       *n_launches += 1;
       if (e != cudaSuccess) return e;

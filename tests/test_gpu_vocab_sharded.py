@@ -231,3 +231,32 @@ def test_combines_at_the_edges_of_their_groups(N, world):
     tok = np.where(ref["corrected"] == 1, ref["teacher_top1"], ref["token"])
     grad_check(to_np64(torch.cat(gs, dim=1))[same], ref["grad"][same], w.dtype, tok[same])
     assert np.max(np.abs(out["lambda"].cpu().numpy() - ref["lam"])) <= 1e-5      # what the float32 kernels are held to
+
+
+def test_logits_rewritten_right_in_front_of_the_call():
+    """Slices of which one is not on 16-byte boundaries (float64 beside float32), the same buffers over and over, new logits and
+    proposals copied into them by kernels that the call follows without a pause: to the bit what the call gives after a wait."""
+    V, N, sets = 32768, 300, 4
+    w = [synth.Workload("vs", N, V, "bf16", 0.125, 1.5, True, 1500 + k, 91) for k in range(sets)]
+    d = [synth.generate(x, DEV) for x in w]
+    cuts = split_columns(V, 4)
+    slices = []
+    for r, (a, n) in enumerate(cuts):
+        st = [torch.empty(N * (n + 8), dtype=torch.bfloat16, device=DEV)[r == 2:].narrow(0, 0, N * n).view(N, n) for _ in "st"]
+        slices.append((*st, a))
+    x = torch.empty(N, dtype=torch.int32, device=DEV)
+
+    def call(k, pause):
+        for (s, t, a), (_, n) in zip(slices, cuts):
+            s.copy_(d[k]["s"][:, a:a + n])
+            t.copy_(d[k]["t"][:, a:a + n])
+        x.copy_(d[k]["proposal"])
+        if pause:
+            torch.cuda.synchronize()
+        out, gs, _ = route_vocab_sharded_local(slices, V, x, w[k].eps, seed=w[k].seed)
+        return [out[f] for f in sorted(out)] + gs
+
+    ref = [call(k, True) for k in range(sets)]
+    for i in range(5 * sets):
+        for a, b in zip(call(i % sets, False), ref[i % sets]):
+            assert torch.equal(a, b)
