@@ -365,6 +365,10 @@ PyObject* py_vshard_local(PyObject*, PyObject* const* a, Py_ssize_t n) {
         PyList_SET_ITEM(gs.p, r, THPVariable_Wrap(g));
       } else PyList_SET_ITEM(gs.p, r, Py_NewRef(Py_None));
     }
+    // the slices' device is the current one from here on: without a stream from the caller, the stages, the zeroing and the reading
+    // of the counters take one and the same stream of it
+    c10::cuda::OptionalCUDAGuard on_device;
+    if (dev.is_cuda()) on_device.set_device(dev);
     const float scale = (float)number(a[8]);
     void* const st = stream_of(a[10]);
     const int eager = (int)integer(a[11]), max_waves = (int)integer(a[12]);

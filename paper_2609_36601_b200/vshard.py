@@ -64,8 +64,9 @@ def route_vocab_sharded(s_loc, t_loc, v0: int, V: int, proposal, eps, temperatur
     si = B.vshard_in(s_loc, t_loc, v0, V, proposal, eps, temperature, seed, row_offset, mask, rank, world)
     out = B.alloc_outputs(N, dev)
     g = torch.empty_like(s_loc) if backward else None
-    # the caller's stream is the current one: the exchange, the zeroing and the reading of the counters are ordered with the stages
-    with torch.cuda.stream(stream):
+    # the slice's device and the caller's stream are the current ones: the exchange, the zeroing and the reading of the counters
+    # are ordered with the stages
+    with torch.cuda.device(dev), torch.cuda.stream(stream):
         state = torch.empty((N, B.VSHARD_STATE), dtype=torch.float64, device=dev)
         part = torch.empty((N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)
         gathered = torch.empty((world, N, B.VSHARD_PARTIALS), dtype=torch.float64, device=dev)

@@ -260,3 +260,25 @@ def test_logits_rewritten_right_in_front_of_the_call():
     for i in range(5 * sets):
         for a, b in zip(call(i % sets, False), ref[i % sets]):
             assert torch.equal(a, b)
+
+
+@pytest.mark.skipif(torch.cuda.device_count() < 2, reason="needs a second GPU to be the current one")
+def test_slices_that_are_not_on_the_current_device():
+    """Without a stream from the caller the stages and their counters take the current stream of the slices' device, which is busy
+    for a while when the call comes."""
+    V = 4096
+    w = synth.Workload("vs", 24, V, "bf16", 0.02, 1.5, False, 1400, 81)
+    d = synth.generate(w, DEV)
+    slices = _slices(d, split_columns(V, 4))
+    with torch.cuda.device(0):
+        ref, g_ref, waves = route_vocab_sharded_local(slices, V, d["proposal"], w.eps, seed=w.seed)
+        torch.cuda.synchronize()
+        torch.cuda._sleep(50_000_000)                    # some 25 ms
+    with torch.cuda.device(1):
+        out, gs, n = route_vocab_sharded_local(slices, V, d["proposal"], w.eps, seed=w.seed)
+    torch.cuda.synchronize(0)
+    assert n == waves
+    for k in ref:
+        assert torch.equal(out[k], ref[k]), k
+    for a, b in zip(gs, g_ref):
+        assert torch.equal(a, b)
