@@ -374,6 +374,10 @@ SAKI_API int saki_set_kernel(int which);
  * turns off), 0 if none yet. */
 SAKI_API int saki_last_kernel(void);
 
+/* How the general kernel laid out the calling thread's last call that it served by itself: blocks per row, blocks per SM, and
+ * how many rows are resident at once that way (zeros if there was none).  For tests; NULL where not wanted. */
+SAKI_API void saki_last_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm, int32_t* resident_rows);
+
 /* Two-tier routing: the float32 kernels (2, 3) hand rows whose KL they cannot resolve to the
  * tolerance (very small eps, nearly one-hot rows) to the float64 kernel, through a row list in device
  * memory that the library allocates once per device and stream and keeps (calls on different streams

@@ -27,7 +27,7 @@ EXPORTS = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc",
            "saki_route_bwd_from_meta", "saki_select_tm", "saki_spec_verify",
            "saki_vshard_partial", "saki_vshard_stage", "saki_vshard_combine", "saki_vshard_combine_host",
            "saki_lmhead_scratch_bytes", "saki_lmhead_lse",
-           "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_redo_count",
+           "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_last_layout", "saki_redo_count",
            "saki_set_spec_early_out", "saki_spec_positions_routed", "saki_solve_evaluations", "saki_set_wait_limit", "saki_set_phase_clock", "saki_phase_cycles",
            "saki_launch_count",
            "saki_last_error", "saki_version")
@@ -155,6 +155,8 @@ def load_library(path: str | None = None):
     lib.saki_set_phase_clock.restype = C.c_int
     lib.saki_phase_cycles.argtypes = [C.c_void_p, C.POINTER(C.c_uint64)]
     lib.saki_phase_cycles.restype = C.c_int
+    lib.saki_last_layout.argtypes = [C.POINTER(C.c_int32)] * 3
+    lib.saki_last_layout.restype = None
     lib.saki_launch_count.restype = C.c_uint64
     lib.saki_last_error.restype = C.c_char_p
     for f in ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_host", "saki_spec_verify",
@@ -407,6 +409,13 @@ def last_kernel() -> int:
     """The kernel that served the calling thread's last routing call: 1 general (float64), 2 cluster, 3 row-per-SM,
     4 the streaming kernel of route_bwd_from_meta."""
     return load_library().saki_last_kernel()
+
+
+def last_layout():
+    """(blocks per row, blocks per SM, rows resident at once) of the calling thread's last call that the general kernel served."""
+    n = (C.c_int32 * 3)()
+    load_library().saki_last_layout(*(C.cast(C.byref(n, 4 * k), C.POINTER(C.c_int32)) for k in range(3)))
+    return tuple(n)
 
 
 def redo_count(stream=None) -> int:

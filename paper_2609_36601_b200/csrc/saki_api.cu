@@ -787,6 +787,14 @@ SAKI_API int saki_set_kernel(int which) {
 
 SAKI_API int saki_last_kernel(void) { return g_last_kernel; }
 
+SAKI_API void saki_last_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm, int32_t* resident_rows) {
+  int l[3];
+  general_layout(l);
+  if (blocks_per_row) *blocks_per_row = l[0];
+  if (blocks_per_sm) *blocks_per_sm = l[1];
+  if (resident_rows) *resident_rows = l[2];
+}
+
 SAKI_API int saki_redo_count(void* cuda_stream, uint64_t* n_rows) {
   g_err[0] = 0;
   if (!n_rows) return fail(SAKI_ERR_INVALID_ARG, "NULL output pointer");

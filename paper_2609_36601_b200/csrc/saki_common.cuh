@@ -213,6 +213,7 @@ __host__ __device__ inline RowResult zero_row(uint32_t status) {
 
 // host-side launchers (defined in the kernel translation units)
 cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* n_launches);
+void general_layout(int* out);      // of the calling thread's last call: blocks per row, blocks per SM, rows resident at once
 cudaError_t launch_cluster(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
 bool cluster_can_serve(const RowParams& p, int dtype);
 cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);

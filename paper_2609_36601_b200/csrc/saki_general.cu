@@ -22,6 +22,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 
 namespace cg = cooperative_groups;
 
@@ -750,8 +751,10 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
 //     another finds most of 126 MB of L2 all the same), takes two, and as many blocks per row as fit and keep 4000 elements or more
 //     (us, with the layout of before and now: fp32 64 rows of 1024 13.2 / 11.5, 64 of 16000 30.5 / 22.5, 148 of 50000 107 / 69;
 //     bf16 148 rows of 16001 38.5 / 29.6, 64 of 100001 84 / 64).
-//     Where some SMs would have two blocks and others one, twice the blocks at three to an SM, if they are all resident (which
-//     launch_t sees to: clusters of four and eight do not fill every SM) and keep 5000 elements or more (8000 in clusters of eight): fp32
+//     Clusters of four and eight do not fill every SM (71 and 33 of them are resident, not 74 and 37): what does not fit takes half
+//     the blocks per row (us, with the one or two rows of a second turn and now: fp32 34 rows of 32000 38 / 30, 72 of 64000 86 / 68, bf16 37 of 33001 46 / 33).
+//     Where that leaves SMs out, or some SMs would have two blocks and others one, twice the blocks at three to an SM, if they are all
+//     resident and keep 5000 elements or more (8000 in clusters of eight): fp32
 //     190 rows of 50000 128 -> 108, 89 of 120000 159 -> 125, bf16 42 rows of 123205 76 -> 66.
 //   - Of the others the one that takes the least by a cost model: turns, times what a turn takes of a row's serial steps, its
 //     elements and the rows in flight beyond L2.  Fitted to the times of fp32 rows of 1024 to 151936 and bf16 rows of 1025 to
@@ -761,7 +764,9 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
 // by V alone, so many that the rows in flight stay in L2.  In list mode (a handful of rows as a rule; the host does not know
 // their number) as many blocks per row as a row has 2048 elements for.
 struct Layout { int cs, k; };
-static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms) {
+// fits(l): all rows of the call are resident at once in layout l
+template <typename F>
+static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms, F&& fits) {
   const int64_t row_bytes = 2 * (int64_t)V * (f32 ? 4 : 2);
   int cs = 1;
   if (from_list || rows <= 0) {
@@ -771,8 +776,10 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
   }
   if (rows <= 2 * sms && rows * row_bytes <= 200000000) {
     while (cs < MAX_CS && rows * 2 * cs <= 2 * sms && V >= 8000 * cs) cs *= 2;
+    bool parted = false;
+    while (cs > 1 && !fits(Layout{cs, 2})) { cs /= 2; parted = true; }
     const int wide = 2 * cs;
-    if (wide <= MAX_CS && rows * cs > sms && rows * wide <= 3 * sms && V >= (wide == 8 ? 64000 : 10000 * cs)) return {wide, 3};
+    if (wide <= MAX_CS && (parted || rows * cs > sms) && V >= (wide == 8 ? 64000 : 10000 * cs) && fits(Layout{wide, 3})) return {wide, 3};
     return {cs, 2};
   }
   static const Layout all[] = {{1, 2}, {1, 3}, {2, 2}, {4, 2}, {8, 2}, {1, 4}, {2, 4}, {4, 4}};     // (the last three: fp32)
@@ -795,28 +802,44 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
   return best;
 }
 
+// f(blocks per row, blocks per SM) as constants
+template <typename F>
+static cudaError_t with_layout(Layout l, F&& f) {
+  using std::integral_constant;
+  switch (l.cs * 16 + l.k) {
+    case 16 + 3: return f(integral_constant<int, 1>{}, integral_constant<int, 3>{});
+    case 16 + 4: return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+    case 32 + 2: return f(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+    case 32 + 3: return f(integral_constant<int, 2>{}, integral_constant<int, 3>{});
+    case 32 + 4: return f(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+    case 64 + 2: return f(integral_constant<int, 4>{}, integral_constant<int, 2>{});
+    case 64 + 3: return f(integral_constant<int, 4>{}, integral_constant<int, 3>{});
+    case 64 + 4: return f(integral_constant<int, 4>{}, integral_constant<int, 4>{});
+    case 128 + 2: return f(integral_constant<int, 8>{}, integral_constant<int, 2>{});
+    case 128 + 3: return f(integral_constant<int, 8>{}, integral_constant<int, 3>{});
+    default: return f(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+  }
+}
+
+static thread_local int g_layout[3];     // of the thread's last call: blocks per row, blocks per SM, rows resident at once
+void general_layout(int* out) { std::copy(g_layout, g_layout + 3, out); }
+
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
-  Layout l = pick_layout(p.V, p.call_rows, p.from_list != 0, sizeof(T) == 4, sms);
-  if (l.k == 3 && l.cs > 1 && p.call_rows > 0 && !p.from_list) {
-    int fit = 0;
-    const cudaError_t e = l.cs == 2 ? resident_rows<T, 2, 3>(dev, sms, &fit) : l.cs == 4 ? resident_rows<T, 4, 3>(dev, sms, &fit) : resident_rows<T, 8, 3>(dev, sms, &fit);
+  auto resident = [&](Layout l, int* rows) {
+    return with_layout(l, [&](auto cs, auto k) { return resident_rows<T, cs, k>(dev, sms, rows); });
+  };
+  auto fits = [&](Layout l) {              // (an error comes again, and is returned, where the layout is launched)
+    int n = 0;
+    return resident(l, &n) != cudaSuccess || p.call_rows <= n;
+  };
+  const Layout l = pick_layout(p.V, p.call_rows, p.from_list != 0, sizeof(T) == 4, sms, fits);
+  if (!p.from_list) {
+    g_layout[0] = l.cs; g_layout[1] = l.k;
+    const cudaError_t e = resident(l, &g_layout[2]);
     if (e != cudaSuccess) return e;
-    if (p.call_rows > fit) l = {l.cs / 2, 2};
   }
-  switch (l.cs * 16 + l.k) {
-    case 16 + 3: return launch_cs<T, 1, 3>(p, dev, sms, st);
-    case 16 + 4: return launch_cs<T, 1, 4>(p, dev, sms, st);
-    case 32 + 2: return launch_cs<T, 2, 2>(p, dev, sms, st);
-    case 32 + 3: return launch_cs<T, 2, 3>(p, dev, sms, st);
-    case 32 + 4: return launch_cs<T, 2, 4>(p, dev, sms, st);
-    case 64 + 2: return launch_cs<T, 4, 2>(p, dev, sms, st);
-    case 64 + 3: return launch_cs<T, 4, 3>(p, dev, sms, st);
-    case 64 + 4: return launch_cs<T, 4, 4>(p, dev, sms, st);
-    case 128 + 2: return launch_cs<T, 8, 2>(p, dev, sms, st);
-    case 128 + 3: return launch_cs<T, 8, 3>(p, dev, sms, st);
-    default: return launch_cs<T, 1, 2>(p, dev, sms, st);
-  }
+  return with_layout(l, [&](auto cs, auto k) { return launch_cs<T, cs, k>(p, dev, sms, st); });
 }
 
 cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* n_launches) {

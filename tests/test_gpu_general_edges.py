@@ -64,6 +64,16 @@ def test_layouts(N, V, dtype):
     assert P.last_kernel() == 1
 
 
+@pytest.mark.parametrize("N,V,dtype", [(33, 32000, "f32"), (34, 32000, "f32"), (37, 64000, "f32"), (37, 33001, "bf16"), (70, 16000, "f32"),
+                                       (72, 16000, "f32"), (74, 40001, "bf16"), (104, 20000, "f32"), (111, 20000, "f32")])
+def test_rows_of_a_few_clusters_are_resident_at_once(N, V, dtype):
+    """Clusters of four and eight do not fill every SM: a call that is laid out in one turn of them has room for all its rows."""
+    w = synth.Workload("t", N, V, dtype, 0.0625, 1.2, True, 700 + N + V, 31, temperature=0.875)
+    _check(synth.generate(w, DEV), w, sorted({0, N // 2, N - 2, N - 1}), kernel=0)
+    cs, k, resident = P.last_layout()
+    assert P.last_kernel() == 1 and cs in (2, 4, 8) and k in (2, 3) and N <= resident
+
+
 @pytest.mark.parametrize("drop", [150.0, 2000.0])
 def test_maximum_far_above_the_first_elements(drop):
     """Each warp's shift comes from its first 128 elements: here every one of them is `drop` nats below the peaks."""
