@@ -137,10 +137,10 @@ __device__ __forceinline__ void for_elements(const T* __restrict__ s, const T* _
     }, element);
 }
 
-// The scalars between the passes, on one warp per block (all lanes alike).
 // 1 / x of a sum of exponentials: short while x is in float32's range
 __device__ __forceinline__ double rcp_sum(double x) { return x > 1e-30 && x < 1e30 ? rcp_fast(x) : 1.0 / x; }
 
+// The scalars between the passes, on one warp per block (all lanes alike): first_guess, solve_step.
 __device__ __noinline__ double first_guess(double m1, double m2, double m3, double m4, double rtau, double kl1, double eps) {
   const double var = m2 - m1 * m1, m1s = m1 * m1;
   const double c3 = m3 - 3.0 * m1 * m2 + 2.0 * m1 * m1s;
@@ -802,19 +802,23 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
   return best;
 }
 
-// f(blocks per row, blocks per SM) as constants
-template <typename F>
+// f(blocks per row, blocks per SM) as constants, of the layouts that pick_layout gives for T
+template <typename T, typename F>
 static cudaError_t with_layout(Layout l, F&& f) {
   using std::integral_constant;
+  if constexpr (sizeof(T) == 4) {
+    switch (l.cs * 16 + l.k) {
+      case 16 + 4: return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
+      case 32 + 4: return f(integral_constant<int, 2>{}, integral_constant<int, 4>{});
+      case 64 + 4: return f(integral_constant<int, 4>{}, integral_constant<int, 4>{});
+    }
+  }
   switch (l.cs * 16 + l.k) {
     case 16 + 3: return f(integral_constant<int, 1>{}, integral_constant<int, 3>{});
-    case 16 + 4: return f(integral_constant<int, 1>{}, integral_constant<int, 4>{});
     case 32 + 2: return f(integral_constant<int, 2>{}, integral_constant<int, 2>{});
     case 32 + 3: return f(integral_constant<int, 2>{}, integral_constant<int, 3>{});
-    case 32 + 4: return f(integral_constant<int, 2>{}, integral_constant<int, 4>{});
     case 64 + 2: return f(integral_constant<int, 4>{}, integral_constant<int, 2>{});
     case 64 + 3: return f(integral_constant<int, 4>{}, integral_constant<int, 3>{});
-    case 64 + 4: return f(integral_constant<int, 4>{}, integral_constant<int, 4>{});
     case 128 + 2: return f(integral_constant<int, 8>{}, integral_constant<int, 2>{});
     case 128 + 3: return f(integral_constant<int, 8>{}, integral_constant<int, 3>{});
     default: return f(integral_constant<int, 1>{}, integral_constant<int, 2>{});
@@ -827,7 +831,7 @@ void general_layout(int* out) { std::copy(g_layout, g_layout + 3, out); }
 template <typename T>
 static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t st) {
   auto resident = [&](Layout l, int* rows) {
-    return with_layout(l, [&](auto cs, auto k) { return resident_rows<T, cs, k>(dev, sms, rows); });
+    return with_layout<T>(l, [&](auto cs, auto k) { return resident_rows<T, cs, k>(dev, sms, rows); });
   };
   auto fits = [&](Layout l) {              // (an error comes again, and is returned, where the layout is launched)
     int n = 0;
@@ -839,7 +843,7 @@ static cudaError_t launch_t(const RowParams& p, int dev, int sms, cudaStream_t s
     const cudaError_t e = resident(l, &g_layout[2]);
     if (e != cudaSuccess) return e;
   }
-  return with_layout(l, [&](auto cs, auto k) { return launch_cs<T, cs, k>(p, dev, sms, st); });
+  return with_layout<T>(l, [&](auto cs, auto k) { return launch_cs<T, cs, k>(p, dev, sms, st); });
 }
 
 cudaError_t launch_general(const RowParams& p, int dtype, cudaStream_t st, int* n_launches) {
