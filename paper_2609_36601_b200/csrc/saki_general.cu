@@ -749,17 +749,17 @@ static cudaError_t launch_cs(const RowParams& p, int dev, int sms, cudaStream_t 
 // blocks per SM run a row soonest, more of them hide one another's serial steps and share an SM's slots out more finely.
 //   - A call whose blocks are all resident two to an SM, and whose rows stay in L2 between the passes (200 MB: a pass behind
 //     another finds most of 126 MB of L2 all the same), takes two, and as many blocks per row as fit and keep 4000 elements or more
-//     (us, with the layout of before and now: fp32 64 rows of 1024 13.2 / 11.5, 64 of 16000 30.5 / 22.5, 148 of 50000 107 / 69;
-//     bf16 148 rows of 16001 38.5 / 29.6, 64 of 100001 84 / 64).
+//     (us, against as many blocks per row as are resident at four to an SM: fp32 64 rows of 1024 12.1 / 10.9, 64 of 16000 30.4 / 21.4,
+//     148 of 50000 114 / 77; at three, bf16 148 rows of 16001 40.9 / 31.5, 64 of 100001 91 / 68).
 //     Clusters of four and eight do not fill every SM (71 and 33 of them are resident, not 74 and 37): what does not fit takes half
 //     the blocks per row (us, with the one or two rows of a second turn and now: fp32 34 rows of 32000 38 / 30, 72 of 64000 86 / 68, bf16 37 of 33001 46 / 33).
 //     Where that leaves SMs out, or some SMs would have two blocks and others one, twice the blocks at three to an SM, if they are all
 //     resident and keep 5000 elements or more (8000 in clusters of eight): fp32
-//     190 rows of 50000 128 -> 108, 89 of 120000 159 -> 125, bf16 42 rows of 123205 76 -> 66.
+//     190 rows of 50000 135 -> 113, 89 of 120000 183 -> 138, bf16 42 rows of 123205 79 -> 67.
 //   - Of the others the one that takes the least by a cost model: turns, times what a turn takes of a row's serial steps, its
-//     elements and the rows in flight beyond L2.  Fitted to the times of fp32 rows of 1024 to 151936 and bf16 rows of 1025 to
-//     100001, 24 to 3000 of them, all layouts: the choice is 0.6 % (fp32) and 0.4 % (bf16) above the best on average, and the rule
-//     before (fp32 four to an SM, bf16 three) was 15 and 10 %.
+//     elements and the rows in flight beyond L2.  Fitted to the times of 605 calls of 200 to 4000 rows of 1024 to 151937, every layout
+//     of the list: the choice is 0.9 % (fp32) and 0.6 % (bf16) above the best of them on average, 5 and 4 % or more for one call in
+//     twenty, 9 and 24 % at worst (350 fp32 rows of 32000, 350 bf16 rows of 80001).
 // The kernel pinned (call_rows = 0), the rows do not count, so that pieces of a batch agree with the whole to the bit: blocks per row
 // by V alone, so many that the rows in flight stay in L2.  In list mode (a handful of rows as a rule; the host does not know
 // their number) as many blocks per row as a row has 2048 elements for.
@@ -783,17 +783,17 @@ static Layout pick_layout(int V, int64_t rows, bool from_list, bool f32, int sms
     return {cs, 2};
   }
   static const Layout all[] = {{1, 2}, {1, 3}, {2, 2}, {4, 2}, {8, 2}, {1, 4}, {2, 4}, {4, 4}};     // (the last three: fp32)
-  // microseconds: a row's serial steps, 1000 elements of a block, a doubling of the blocks; the part of a turn that is waited for
-  // to its end (blocks take over rows that have not started); 126 MB in flight beyond L2
-  static const double serial[2][3] = {{10.25, 13.6, 17.0}, {7.7, 10.06, 13.0}}, element[2][3] = {{1.83, 2.62, 3.3}, {2.24, 3.4, 4.14}};
-  static const double join[2] = {0.1, 0.6}, whole[2] = {0.15, 0.2}, beyond[2] = {0.15, 0.05};
+  // bf16, fp32, in microseconds: a row's serial steps, 1000 elements of a block (by blocks per SM, two to four), a doubling of the
+  // blocks; the part of a turn that is waited for to its end (blocks take over rows that have not started); 126 MB in flight beyond L2
+  static const double serial[2][3] = {{15.2, 20.3}, {8.65, 10.5, 14.4}}, element[2][3] = {{2.42, 3.56}, {2.06, 3.35, 3.81}};
+  static const double join[2] = {0.67, 0.45}, whole[2] = {0.014, 0.155}, beyond[2] = {0.49, 0.002};
   Layout best = all[0];
   double least = 1e300;
   for (int i = 0; i < (f32 ? 8 : 5); ++i) {
     const Layout l = all[i];
     if (l.cs > 1 && V < 4000 * l.cs) continue;
     const double slots = (double)(l.k * sms / l.cs), turns = (double)rows / slots, in_flight = std::min((double)rows, slots) * (double)row_bytes;
-    if (l.cs == 1 && l.k > 2 && in_flight > 126e6) continue;         // (1024 fp32 rows of 32000: 316 us with four to an SM, 298 with two)
+    if (l.cs == 1 && l.k > 2 && in_flight > 126e6) continue;         // (1024 fp32 rows of 32000: 336 us with four to an SM, 293 with two)
     double t = serial[f32][l.k - 2] + element[f32][l.k - 2] * 1e-3 * V / l.cs + join[f32] * std::log2((double)l.cs);
     t *= 1.0 + beyond[f32] * std::max(0.0, in_flight / 126e6 - 1.0);
     if (turns > 1.0) t *= whole[f32] * std::ceil(turns) + (1.0 - whole[f32]) * (turns + 0.5);
