@@ -177,6 +177,22 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t local_smem_addr, uint32
   asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(local_smem_addr), "r"(rank));
   return r;
 }
+// Dynamic rows: a block (cluster) that is done takes over the work of one that has not started yet, by cancelling its
+// launch.  The answer arrives in shared memory and completes an mbarrier.
+__device__ __forceinline__ void steal_request(void* answer, uint64_t* bar) {
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the last answer has been read
+  mbar_expect_tx(bar, 16);
+  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+               ::"r"(smem_addr(answer)), "r"(smem_addr(bar)) : "memory");
+}
+__device__ __forceinline__ int steal_answer(const void* answer) {   // first block index of the cancelled cluster, or -1
+  uint32_t ok, x;
+  asm volatile("{\n\t.reg .b128 h;\n\t.reg .pred p;\n\tld.shared.b128 h, [%2];\n\t"
+               "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\tselp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t"
+               "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n\t}"
+               : "=r"(ok), "=r"(x) : "r"(smem_addr(answer)) : "memory");
+  return ok ? (int)x : -1;
+}
 // store 8 bytes into a peer CTA's shared memory; the peer's mbarrier counts the bytes
 __device__ __forceinline__ void st_async_f64(uint32_t remote_addr, double v, uint32_t remote_bar) {
   asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"

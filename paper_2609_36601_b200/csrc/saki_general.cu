@@ -51,23 +51,6 @@ enum { PA_KS = 0, PA_KT, PA_SS, PA_ST, PA_N1, PA_M1, PA_M2, PA_M3, PA_M4, PA_MS,
 enum { G_SOLVE = 0, G_FINAL = 1, G_FLAG = 2 };
 constexpr int LOST = -2;
 
-// Dynamic rows: a block (cluster) that is done takes over the work of one that has not started yet, by cancelling its
-// launch.  The answer arrives in shared memory and completes an mbarrier.
-__device__ __forceinline__ void steal_request(void* answer, uint64_t* bar) {
-  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");   // the last answer has been read
-  mbar_expect_tx(bar, 16);
-  asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
-               ::"r"(smem_addr(answer)), "r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ int steal_answer(const void* answer) {   // first block index of the cancelled cluster, or -1
-  uint32_t ok, x;
-  asm volatile("{\n\t.reg .b128 h;\n\t.reg .pred p;\n\tld.shared.b128 h, [%2];\n\t"
-               "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\tselp.u32 %0, 1, 0, p;\n\tmov.u32 %1, 0;\n\t"
-               "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %1, h;\n\t}"
-               : "=r"(ok), "=r"(x) : "r"(smem_addr(answer)) : "memory");
-  return ok ? (int)x : -1;
-}
-
 __device__ __forceinline__ double pow2_down(double n) {      // 2^n for whole n <= 0; 0 below -1000
   return n < -1000.0 ? 0.0 : __longlong_as_double((long long)(1023 + (int)n) << 52);
 }

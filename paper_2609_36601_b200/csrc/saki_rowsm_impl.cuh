@@ -67,7 +67,7 @@ static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight 
 // lanes per sum) and goes straight on to the scalars: a barrier less per pass, and the eight sums are not dealt
 // twice round four warps (4096 rows of 8192 elements: 26.7 -> 25.5 k cycles a row; of 32000: 65.5 -> 65.4 k); the uniforms and the logits at the
 // proposal are fetched by warps 1-3 at the top of the row.  While thread 0 does the scalars: FIN_WARP finishes the
-// previous row, RES_WARP reserves the next row of a block verification, SV_WARP fetches the student's logit at the
+// previous row, RES_WARP finds the next row, SV_WARP fetches the student's logit at the
 // teacher's argmax (and with four or eight warps finds the argmax).
 constexpr bool SIDE_WARPS = RW >= 14;
 constexpr int UACC_WARP = SIDE_WARPS ? 8 : 1, UDRAW_WARP = SIDE_WARPS ? 9 : 2, SX_WARP = SIDE_WARPS ? 10 : 3;
@@ -85,7 +85,9 @@ constexpr int ROFF_FIN = ROFF_STEP + RW * MAX_STEPS * 4;          // [2][2][RW] 
 constexpr int ROFF_MBAR = ROFF_FIN + 2 * 2 * RW * 8;
 constexpr int FIN_WARP = SIDE_WARPS ? 12 : (RW == 8 ? 4 : 1);   // the warp that finishes the previous row
 constexpr int ROFF_SEQ = ROFF_MBAR + 16;   // [4] ints: block verification, the CTA's reservation state
-constexpr int ROFF_PH = ROFF_SEQ + 16;     // [PH_WORDS] 64-bit words: the phase clock of thread 0
+constexpr int ROFF_ANSWER = ROFF_SEQ + 16; // 16 bytes: the answer to a request for a further row; then the mbarrier it completes
+constexpr int ROFF_PH = ROFF_ANSWER + 32;  // [PH_WORDS] 64-bit words: the phase clock of thread 0
+static_assert(ROFF_ANSWER % 16 == 0, "an answer is 16 bytes on a 16-byte boundary");
 constexpr int RSMEM_BYTES = ROFF_PH + PH_WORDS * 8;
 
 // L2 residency hints: the part of a row that is re-read from L2 in every pass is marked
@@ -295,8 +297,12 @@ __device__ __forceinline__ void for_each_chunk(const Seg& sg, int lane, const ui
 
 // SPEC: the instance that serves block verification (bonus rows, positions handed out as tickets); plain
 // routing runs an instance without that code.
+// steal: a CTA per row, of which those that run take over rows whose CTA has not started (clusterlaunchcontrol).  CTAs that
+// share an SM do not get equal shares of its schedulers: with the rows dealt out beforehand the slowest took 12 to 16 % longer
+// than the average (rows dealt out / taken over, us: 4096 rows of 32000 300 / 282, of 8192 elements 11840 rows 278 / 258, of
+// 65536 8192 rows 1082 / 1008; one CTA per SM: 16384 rows of 151936 4679 / 4626).
 template <bool SPEC>
-__global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams P) {
+__global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams P, const int steal) {
   extern __shared__ __align__(128) unsigned char smem[];
   launch_dependents();
   const int tid = threadIdx.x, lane = tid & 31;
@@ -318,6 +324,8 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   double* red = (double*)(smem + ROFF_RED);
   double* gat = (double*)(smem + ROFF_GAT);
   uint64_t* mbar = (uint64_t*)(smem + ROFF_MBAR);
+  uint64_t* answer_bar = (uint64_t*)(smem + ROFF_ANSWER + 16);
+  bool dead = false;                           // this thread's block gave up on a copy
 
   const int V = P.V;
   const int n_chunks = V / 8;
@@ -440,8 +448,26 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       seqres[1] = blo; seqres[2] = bhi; seqres[3] = n;
     }
   };
+  // Plain rows: the row of a CTA that has not started yet.  Not once this CTA has given up on a copy: what it does not take
+  // over is launched.  (lane 0 of RES_WARP)
+  uint32_t answer_phase = 0;
+  auto take_over = [&] {
+    int next = n_tickets;
+    if (!dead) {
+      steal_request(smem + ROFF_ANSWER, answer_bar);
+      if (mbar_wait_bounded(answer_bar, answer_phase)) {
+        const int first = steal_answer(smem + ROFF_ANSWER);
+        if (first >= 0) next = first;
+      } else {
+        atomicAdd(P.flagged, 1ull);      // no answer: saki_check reports that a row may have been lost
+      }
+      answer_phase ^= 1u;
+    }
+    seqres[0] = next;
+  };
   if (tid == 0) {
     mbar_init(mbar, RW);
+    mbar_init(answer_bar, 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     seqres[0] = n_tickets; seqres[1] = 0; seqres[2] = 0; seqres[3] = 1;
   }
@@ -455,7 +481,6 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     ring_prime(rg, sg, lane, n_s, n_t, pol_last);
   }
   uint32_t phase = 0;
-  bool dead = false;
   bool undrained = false;   // this thread gave up on a copy that may still be in flight
   int rb = 0;
   // Pass "final" ends without a barrier.  What is left of a row after it (the total variation, the
@@ -690,7 +715,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
         if (any_dead) dead = true;
         RTS(PH_LSE_REDUCE);
         if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);   // the previous row's draw and outputs
-        if (dyn && warp == RES_WARP) reserve_next();     // the CTA's next row (block verification)
+        if (warp == RES_WARP) {          // the CTA's next row
+          if (dyn) reserve_next();
+          else if (steal && lane == 0) take_over();
+        }
         pending_row = -1;
         if (warp == SV_WARP) {       // the teacher's argmax, and the student's logit there (the supervised token of a corrected row)
           const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < RW ? wm[lane] : 0u);
@@ -813,7 +841,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       __syncthreads();
       RTS(PH_LSE_GATHER);
       if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);   // meanwhile: the previous row's draw and outputs
-      if (dyn && warp == RES_WARP) reserve_next();     // and the CTA's next row (block verification), while thread 0 does the scalars
+      if (warp == RES_WARP) {                          // and the CTA's next row, while thread 0 does the scalars
+        if (dyn) reserve_next();
+        else if (steal && lane == 0) take_over();
+      }
       pending_row = -1;
       if (tid == SV_WARP * 32) {   // and the student's logit at the teacher's argmax (the supervised token of a corrected row)
         const int vs = (gat[6] >= 0.0 && gat[6] < (double)V) ? (int)gat[6] : 0;
@@ -887,7 +918,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       RTS(PH_SOLVE_SCALAR);
       __syncthreads();
     }
-    const int64_t next_row = dyn ? (int64_t)seqres[0] : row + gridDim.x;
+    const int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + gridDim.x;
     next_row_c = next_row;
     n_s = nullptr; n_t = nullptr;
     if (next_row < P.n_rows) row_ptrs(next_row, n_s, n_t);
@@ -1026,10 +1057,12 @@ cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* s
       cached_dev = dev;
     }
   }
+  // as many CTAs as run at once, or one per row of which they take over those that have not started
   const int64_t ctas = (int64_t)cached_sms * CTAS_PER_SM;
-  const int grid = (int)(p.n_rows < ctas ? p.n_rows : ctas);
-  const cudaError_t e = p.spec ? launch_pdl(rowsm_kernel<true>, dim3((unsigned)grid), RT, RSMEM_BYTES, st, true, p)
-                               : launch_pdl(rowsm_kernel<false>, dim3((unsigned)grid), RT, RSMEM_BYTES, st, true, p);
+  const bool steal = p.seq_next == nullptr && p.n_rows > ctas && p.n_rows <= (1 << 27);
+  const dim3 grid((unsigned)(steal || p.n_rows < ctas ? p.n_rows : ctas));
+  const cudaError_t e = p.spec ? launch_pdl(rowsm_kernel<true>, grid, RT, RSMEM_BYTES, st, true, p, (int)steal)
+                               : launch_pdl(rowsm_kernel<false>, grid, RT, RSMEM_BYTES, st, true, p, (int)steal);
   if (e == cudaSuccess) { *served = true; if (n_launches) *n_launches += 1; }
   return e;
 }
