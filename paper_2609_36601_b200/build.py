@@ -14,7 +14,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libsaki.so")
 TORCH_SOURCE = os.path.join(CSRC, "saki_torch.cpp")
 TORCH_LIB = os.path.join(HERE, "_saki_torch.so")
-SOURCES = ("saki_api.cu", "saki_general.cu", "saki_cluster.cu", "saki_rowsm.cu", "saki_rowsm_half.cu", "saki_rowsm_quarter.cu", "saki_meta.cu",
+SOURCES = ("saki_api.cu", "saki_general.cu", "saki_cluster.cu", "saki_rowsm.cu", "saki_rowsm_half.cu", "saki_rowsm_quarter.cu", "saki_rowsm_pair.cu", "saki_rowsm_wide.cu", "saki_meta.cu",
            "saki_select.cu", "saki_propose.cu", "saki_vshard.cu", "saki_lmhead.cu")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden"]

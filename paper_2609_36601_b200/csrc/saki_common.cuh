@@ -103,6 +103,22 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, int block, size_t sm
   cfg.attrs = at; cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
+// the same, programmatic, the grid in clusters of `cluster` blocks
+template <typename... KArgs, typename... Args>
+cudaError_t launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, int block, int cluster, size_t smem, cudaStream_t st, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3((unsigned)block, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  cfg.attrs = at; cfg.numAttrs = cluster > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
 #endif
 
 // Parameters of the metadata-driven backward kernels (saki_route_bwd_from_meta).
@@ -219,6 +235,8 @@ bool cluster_can_serve(const RowParams& p, int dtype);
 cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
 namespace full_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace half_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
+namespace pair_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
+namespace wide_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace quarter_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 bool rowsm_can_serve(const RowParams& p, int dtype);
 cudaError_t launch_meta_general(const MetaParams& p, int dtype, cudaStream_t st, int* n_launches);

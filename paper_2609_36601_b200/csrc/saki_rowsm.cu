@@ -1,6 +1,7 @@
-// Row-per-SM kernel, the variant with one CTA of 512 threads per SM, and the choice between the three
+// Row-per-SM kernel, the variant with one CTA of 512 threads per SM, and the choice between the five
 // variants (the implementation is saki_rowsm_impl.cuh).
 #include "saki_rowsm_impl.cuh"
+#include <cmath>
 
 namespace saki {
 
@@ -27,28 +28,42 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
   return true;
 }
 
-// The variant that routes this number of rows soonest.  A variant with k CTAs per SM takes ceil(rows / (k SMs))
-// turns of a + b V / 1000 microseconds each (fitted to V = 2048 to 98304 and 8 to 1776 rows, within 10 %):
-//   k = 1: 6.2, 0.302     k = 2: 5.0, 0.535     k = 4: 6.0, 1.06
-// so that, e.g., 888 rows of 32000 take three turns of k = 2 (73 us) and not two of k = 4 (83 us), 296 rows of 49152 one
-// turn of k = 2 (38 us against 48 with k = 1 and 51 with k = 4); a call with a row or less per SM takes k = 1, or k = 2
-// where its inlined scalar steps outweigh the longer passes (below V = 16384: 14.1 against 16.2 us at 8192).  The limits on V above
-// hold here too, except that rows in flight that fit in L2 anyway (two per SM) may be longer.  Not where saki_set_kernel
-// pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
+// The variant that routes this number of rows soonest, by 231 shapes (V = 8192 to 151936, 20 to 5000 rows, every variant timed): the
+// choice is 0.6 % above the best of them on average, 3 % or more for one shape in fifteen, 13 % at worst.
+//   - A row or less for two SMs: two CTAs of 512 threads on two SMs to a row (us, one SM per row / two: 74 rows of 151936 50.7 /
+//     33.8, of 65536 32.4 / 23.7, of 32768 22.5 / 19.0); a row or less per SM: the pair of CTAs of 256 threads (148 rows of
+//     151936 60.8 / 58.3, of 65536 33.8 / 30.1, of 24000 20.9 / 19.1).  Below V = 20000 the exchange costs what it saves: two
+//     CTAs per SM (148 rows of 16384 17.9, the pair 17.5; 20 rows 15.3, 15.4).
+//   - More: the variant that takes the least by a cost model, start + (serial + element V / 1000) turns, where a turn is waited
+//     for to its end only in part (CTAs take over rows that have not started) and costs more where the rows in flight are more than
+//     L2 holds.  The pair is what 149 to some 1000 long rows take (us, one CTA per SM / pair: 300 rows of 151936 147 / 116, 1200 395 / 372), two
+//     and four CTAs per SM shorter ones (2000 rows of 65536 314 / 267 with two; of 16384 157 / 88 with four).
+//   - Rows beyond V = 131072 by the thousands: one CTA per SM (16384 rows of 151936 4517, the pair 4550; 4096 rows 1167, 1162).
+// Not where saki_set_kernel pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
 cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
   if (p.call_rows > 0) {
     int dev = 0, sms = 148;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int64_t n = p.call_rows;
-    const double kv = p.V * 1e-3;
-    auto cost = [&](int k, double a, double b) { return (double)((n + (int64_t)k * sms - 1) / ((int64_t)k * sms)) * (a + b * kv); };
-    const double c1 = cost(1, 6.2, 0.302);
-    const double c2 = p.V <= HALF_MAX_V || (n <= 2 * sms && p.V <= half_sm::max_v()) ? cost(2, 5.0, 0.535) : 1e30;
-    const double c4 = p.V <= QUARTER_MAX_V ? cost(4, 6.0, 1.06) : 1e30;
-    if (n <= sms ? p.V >= 16384 : (c1 < c2 && c1 < c4)) return full_sm::launch(p, st, n_launches, served);
-    if (n <= sms || c2 < c4) return half_sm::launch(p, st, n_launches, served);
-    return quarter_sm::launch(p, st, n_launches, served);
+    if (n <= sms) {
+      if (p.V < 20000) return half_sm::launch(p, st, n_launches, served);
+      return 2 * n <= sms ? wide_sm::launch(p, st, n_launches, served) : pair_sm::launch(p, st, n_launches, served);
+    }
+    // per_sm: rows in flight per SM; whole: the part of a turn that is waited for to its end; late: how far into its turn an
+    // average CTA is when no row is left; beyond: for each 126 MB in flight beyond L2
+    struct Model { double per_sm, start, serial, element, whole, late, beyond; };
+    auto cost = [&](const Model& m) {
+      const double slots = m.per_sm * sms, turns = (double)n / slots, in_flight = std::min((double)n, slots) * 4.0 * p.V;
+      const double t = turns > 1.0 ? m.whole * std::ceil(turns) + (1.0 - m.whole) * (turns + m.late) : 1.0;
+      return m.start + (m.serial + m.element * 1e-3 * p.V) * std::max(1.0, t) * (1.0 + m.beyond * std::max(0.0, in_flight / 126e6 - 1.0));
+    };
+    const double full = cost({1, 4.64, 6.52, 0.2485, 0.548, 1.0, 0.05}), half = cost({2, 7.40, 3.64, 0.5366, 0.156, 0.253, 0.221}),
+                 quarter = cost({4, 5.68, 4.31, 1.0593, 0.091, 0.246, 0.131}), pair = cost({1, 4.70, 6.03, 0.2368, 0.121, 0.535, 0.05});
+    if (p.V <= QUARTER_MAX_V && quarter < half && quarter < pair) return quarter_sm::launch(p, st, n_launches, served);
+    if (p.V <= half_sm::max_v() && half < pair && half < full) return half_sm::launch(p, st, n_launches, served);
+    if (full < pair || (p.V > 131072 && n > 40 * (int64_t)sms)) return full_sm::launch(p, st, n_launches, served);
+    return pair_sm::launch(p, st, n_launches, served);
   }
   if (p.V <= QUARTER_MAX_V && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
   if (p.V <= HALF_MAX_V && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);

@@ -1,9 +1,13 @@
-// One-row-per-SM kernel for bf16 rows: the implementation, compiled twice.
+// One-row-per-SM kernel for bf16 rows: the implementation, compiled once per variant.
 //   saki_rowsm.cu       one persistent CTA of 512 threads per SM (namespace full_sm)
 //   saki_rowsm_half.cu  two persistent CTAs of 256 threads per SM (namespace half_sm, SAKI_ROWSM_HALF):
 //                       for short rows, whose passes are short against the serial phases between them,
 //                       so that one CTA's scalar phases run under the other CTA's passes
 //   saki_rowsm_quarter.cu  four of 128 threads (namespace quarter_sm, SAKI_ROWSM_QUARTER): shorter rows still
+//   saki_rowsm_pair.cu  two of 256 threads per SM, and two CTAs on two SMs (a cluster) to a row (namespace pair_sm,
+//                       SAKI_ROWSM_PAIR): long rows with one CTA's scalar phases under another's passes, as many rows in flight as SMs
+//   saki_rowsm_wide.cu  one of 512 threads per SM and two CTAs to a row (namespace wide_sm, SAKI_ROWSM_WIDE): fewer
+//                       rows than half the SMs
 //
 // A persistent CTA routes whole rows, one after the
 // other.  A row pair (student + teacher, e.g. 608 KB at V = 151936) does not
@@ -30,10 +34,11 @@
 //            "residual"), gradient row streamed out (Eq. "general_objective")
 // Per-element work is float32 (packed f32x2 FMAs, ex2.approx); cross-thread
 // combinations and per-row scalars are float64.
-#if defined(SAKI_ROWSM_QUARTER) || defined(SAKI_ROWSM_HALF)
+#if defined(SAKI_ROWSM_QUARTER) || defined(SAKI_ROWSM_HALF) || defined(SAKI_ROWSM_PAIR) || defined(SAKI_ROWSM_WIDE)
 #define SAKI_SCALARS_INLINE 1       // (one CTA per SM: 1 % slower, the pass loops come out worse)
 #endif
 #include "saki_device.cuh"
+#include <algorithm>
 #include <mutex>
 
 #if defined(SAKI_ROWSM_QUARTER)
@@ -44,10 +49,23 @@
 #define SAKI_ROWSM_NS half_sm
 #define SAKI_ROWSM_THREADS 256
 #define SAKI_ROWSM_CTAS 2
+#elif defined(SAKI_ROWSM_PAIR)
+#define SAKI_ROWSM_NS pair_sm
+#define SAKI_ROWSM_THREADS 256
+#define SAKI_ROWSM_CTAS 2
+#define SAKI_ROWSM_CLUSTER 2
+#elif defined(SAKI_ROWSM_WIDE)
+#define SAKI_ROWSM_NS wide_sm
+#define SAKI_ROWSM_THREADS 512
+#define SAKI_ROWSM_CTAS 1
+#define SAKI_ROWSM_CLUSTER 2
 #else
 #define SAKI_ROWSM_NS full_sm
 #define SAKI_ROWSM_THREADS 512
 #define SAKI_ROWSM_CTAS 1
+#endif
+#ifndef SAKI_ROWSM_CLUSTER
+#define SAKI_ROWSM_CLUSTER 1
 #endif
 
 namespace saki {
@@ -56,8 +74,11 @@ namespace SAKI_ROWSM_NS {
 constexpr int RT = SAKI_ROWSM_THREADS;  // threads per CTA
 constexpr int RW = RT / 32;             // warps per CTA
 constexpr int CTAS_PER_SM = SAKI_ROWSM_CTAS;
+constexpr int CL = SAKI_ROWSM_CLUSTER;  // CTAs per row (a cluster; its CTAs land on different SMs)
+constexpr int GW = RW * CL;             // warps per row
+static_assert(GW <= 32, "a lane per warp of the row");
 constexpr int KS_MAX = 208 / (RW * CTAS_PER_SM);   // steps per warp that fit in shared memory (a step = 32 chunks of 8 elements = 1 KB of logit pairs)
-constexpr int MAX_STEPS = 64;            // steps per warp the draw bookkeeping can hold (V <= 64*32*8*RW)
+constexpr int MAX_STEPS = GW > 16 ? 32 : 64;     // steps per warp the draw bookkeeping can hold (V <= MAX_STEPS*32*8*GW)
 constexpr int RES_CHUNKS = KS_MAX * 32; // resident chunks per warp and row
 constexpr int RNV = 9;                  // doubles per partial vector
 static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight warps, or done by warp 0; the side work has warps of its own, or is shared out");
@@ -69,26 +90,31 @@ static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight 
 // proposal are fetched by warps 1-3 at the top of the row.  While thread 0 does the scalars: FIN_WARP finishes the
 // previous row, RES_WARP finds the next row, SV_WARP fetches the student's logit at the
 // teacher's argmax (and with four or eight warps finds the argmax).
-constexpr bool SIDE_WARPS = RW >= 14;
+constexpr bool SIDE_WARPS = RW >= 14 && CL == 1;
 constexpr int UACC_WARP = SIDE_WARPS ? 8 : 1, UDRAW_WARP = SIDE_WARPS ? 9 : 2, SX_WARP = SIDE_WARPS ? 10 : 3;
-constexpr int RES_WARP = SIDE_WARPS ? 11 : (RW == 8 ? 5 : 2), SV_WARP = SIDE_WARPS ? 13 : (RW == 8 ? 6 : 3);
+constexpr int RES_WARP = SIDE_WARPS ? 11 : (RW >= 8 ? 5 : 2), SV_WARP = SIDE_WARPS ? 13 : (RW >= 8 ? 6 : 3);
 static_assert(KS_MAX - 4 >= 1, "every warp keeps at least its first step resident");
 
 constexpr int ROFF_S = 0;                                        // [RW][RES_CHUNKS] uint4
 constexpr int ROFF_T = RW * RES_CHUNKS * 16;
-constexpr int ROFF_RED = 2 * RW * RES_CHUNKS * 16;               // [RNV][RW] doubles
-constexpr int ROFF_GAT = ROFF_RED + RNV * RW * 8;                // [16] doubles: block totals
+// What the warps of a row leave for one another (red, wmax, fin) goes into the shared memory of every CTA of the row, and
+// every CTA adds it up and does the row's scalars alike: nothing has to come back.  red and wmax alternate from one row
+// barrier to the next, so that a CTA that is ahead does not write where another still reads.
+constexpr int NBUF = CL > 1 ? 2 : 1;
+constexpr int ROFF_RED = 2 * RW * RES_CHUNKS * 16;               // [NBUF][RNV][GW] doubles
+constexpr int ROFF_GAT = ROFF_RED + NBUF * RNV * GW * 8;         // [16] doubles: totals of the row
 constexpr int ROFF_BC = ROFF_GAT + 16 * 8;                       // [2][BC_DOUBLES] doubles, alternating by row
-constexpr int ROFF_WMAX = ROFF_BC + 2 * BC_DOUBLES * 8;          // [3][RW]: teacher maximum, its index, student maximum per warp
-constexpr int ROFF_STEP = ROFF_WMAX + 4 * RW * 4;                // [RW][MAX_STEPS] floats: draw weight of each step
-constexpr int ROFF_FIN = ROFF_STEP + RW * MAX_STEPS * 4;          // [2][2][RW] doubles: what pass "final" leaves per warp, by row parity
-constexpr int ROFF_MBAR = ROFF_FIN + 2 * 2 * RW * 8;
-constexpr int FIN_WARP = SIDE_WARPS ? 12 : (RW == 8 ? 4 : 1);   // the warp that finishes the previous row
+constexpr int ROFF_WMAX = ROFF_BC + 2 * BC_DOUBLES * 8;          // [NBUF][4][GW]: per warp the maxima (and the teacher's index), whether it gave up on a copy
+constexpr int ROFF_STEP = ROFF_WMAX + NBUF * 4 * GW * 4;         // [RW][MAX_STEPS] floats: draw weight of each step
+constexpr int ROFF_FIN = ROFF_STEP + RW * MAX_STEPS * 4;          // [2][2][GW] doubles: what pass "final" leaves per warp, by row parity
+constexpr int ROFF_MBAR = ROFF_FIN + 2 * 2 * GW * 8;
+constexpr int FIN_WARP = SIDE_WARPS ? 12 : (RW >= 8 ? 4 : 1);   // the warp that finishes the previous row
 constexpr int ROFF_SEQ = ROFF_MBAR + 16;   // [4] ints: block verification, the CTA's reservation state
 constexpr int ROFF_ANSWER = ROFF_SEQ + 16; // 16 bytes: the answer to a request for a further row; then the mbarrier it completes
 constexpr int ROFF_PH = ROFF_ANSWER + 32;  // [PH_WORDS] 64-bit words: the phase clock of thread 0
 static_assert(ROFF_ANSWER % 16 == 0, "an answer is 16 bytes on a 16-byte boundary");
 constexpr int RSMEM_BYTES = ROFF_PH + PH_WORDS * 8;
+static_assert((RSMEM_BYTES + 1024) * CTAS_PER_SM <= 228 * 1024, "the CTAs of an SM share 228 KB");
 
 // L2 residency hints: the part of a row that is re-read from L2 in every pass is marked
 // evict-last; everything that passes through L2 once (the shared-memory resident part, the
@@ -142,6 +168,12 @@ __device__ __forceinline__ float warp_max_f(float a) {
   for (int o = 16; o > 0; o >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
   return a;
 }
+
+// a value into the shared memory of a CTA of the cluster (addresses by mapa)
+__device__ __forceinline__ void st_cluster(uint32_t at, double v) {
+  asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(at), "l"(__double_as_longlong(v)) : "memory");
+}
+__device__ __forceinline__ void st_cluster(uint32_t at, uint32_t v) { asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(at), "r"(v) : "memory"); }
 
 struct Seg {   // this warp's share of a row, in chunks of 8 elements
   int c0, c1;          // [c0, c1)
@@ -319,9 +351,13 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     ph[PH_LAST] = clock64();
   }
   const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // broadcast: lets the compiler treat it as warp-uniform
+  // this CTA's place in its row, and the row's among those in flight
+  const int crank = CL == 1 ? 0 : (int)(blockIdx.x % CL), gwarp = crank * RW + warp;
+  const int place = (int)(blockIdx.x / CL), n_places = (int)(gridDim.x / CL);
   const uint4* res_s = reinterpret_cast<const uint4*>(smem + ROFF_S) + warp * RES_CHUNKS;
   const uint4* res_t = reinterpret_cast<const uint4*>(smem + ROFF_T) + warp * RES_CHUNKS;
   double* red = (double*)(smem + ROFF_RED);
+  uint32_t* wmax = (uint32_t*)(smem + ROFF_WMAX);
   double* gat = (double*)(smem + ROFF_GAT);
   uint64_t* mbar = (uint64_t*)(smem + ROFF_MBAR);
   uint64_t* answer_bar = (uint64_t*)(smem + ROFF_ANSWER + 16);
@@ -332,14 +368,14 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   // A row is cut into steps of 32 chunks (256 elements) and the steps are dealt out in order: every warp
   // gets steps_q of them, the first steps_r warps one more.  Whole steps: a segment that ended inside a
   // step would cost its warp a nearly empty step in every pass.
-  const int steps_all = (n_chunks + 31) / 32, steps_q = steps_all / RW, steps_r = steps_all - steps_q * RW;
+  const int steps_all = (n_chunks + 31) / 32, steps_q = steps_all / GW, steps_r = steps_all - steps_q * GW;
   auto seg_of = [&](int w, Seg& g) {
     g.steps = steps_q + (w < steps_r ? 1 : 0);
     g.c0 = min(n_chunks, 32 * (w * steps_q + min(w, steps_r)));
     g.c1 = min(n_chunks, g.c0 + 32 * g.steps);
   };
   Seg sg;
-  seg_of(warp, sg);
+  seg_of(gwarp, sg);
   // a segment that does not fit leaves NST steps to the ring, and one more where the streamed part would not be
   // a whole number of double steps
   sg.res = sg.steps <= KS_MAX ? sg.steps : KS_RES - ((sg.steps - KS_RES) & 1);
@@ -376,6 +412,18 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       bulk_load_hint((void*)res_t, t + (size_t)sg.c0 * 8, res_bytes, mbar, pol_first);
     }
   };
+  // A value for every CTA of the row, at the same place of their shared memory; theirs to read behind the next row barrier.
+  auto post = [&](auto* at, auto v) {
+    if constexpr (CL == 1) *at = v;
+    else {
+#pragma unroll
+      for (int r = 0; r < CL; ++r) st_cluster(map_to_rank(smem_addr(at), (uint32_t)r), v);
+    }
+  };
+  auto row_barrier = [&] {
+    if constexpr (CL == 1) __syncthreads();
+    else asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  };
   // n per-warp vectors -> gat[k] = sum over warps of component k; warp k adds up component k, so the
   // serial part after the barrier is one shuffle tree deep
   auto combine = [&](const double* v, int n) {
@@ -395,7 +443,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   auto gather8 = [&](auto&& term) {
     double a = 0.0;
 #pragma unroll
-    for (int w = lane & 3; w < RW; w += 4) a += term(lane >> 2, w);
+    for (int w = lane & 3; w < GW; w += 4) a += term(lane >> 2, w);
     a += __shfl_xor_sync(0xffffffffu, a, 2);
     a += __shfl_xor_sync(0xffffffffu, a, 1);
     return a;
@@ -431,8 +479,8 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       bool fresh = false;
       if (blo >= bhi) {
         int old = 0;
-        const int take = min(n, max(1, (n_tickets - max(bhi, (int)gridDim.x)) / (4 * (int)gridDim.x)));
-        if (lane == 0) old = (int)min((unsigned int)n_tickets, gridDim.x + atomicAdd(P.seq_next, (unsigned int)take));
+        const int take = min(n, max(1, (n_tickets - max(bhi, n_places)) / (4 * n_places)));
+        if (lane == 0) old = (int)min((unsigned int)n_tickets, (unsigned int)n_places + atomicAdd(P.seq_next, (unsigned int)take));
         old = __shfl_sync(0xffffffffu, old, 0);
         blo = old; bhi = min(old + take, n_tickets);
         if (blo >= bhi) break;
@@ -444,12 +492,12 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       else blo = bhi;
     }
     if (lane == 0) {
-      seqres[0] = res < n_tickets ? (int)ticket_row(res) : n_tickets;
+      post((uint32_t*)seqres, (uint32_t)(res < n_tickets ? (int)ticket_row(res) : n_tickets));
       seqres[1] = blo; seqres[2] = bhi; seqres[3] = n;
     }
   };
   // Plain rows: the row of a CTA that has not started yet.  Not once this CTA has given up on a copy: what it does not take
-  // over is launched.  (lane 0 of RES_WARP)
+  // over is launched.  (lane 0 of RES_WARP, in the row's first CTA)
   uint32_t answer_phase = 0;
   auto take_over = [&] {
     int next = n_tickets;
@@ -457,13 +505,13 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       steal_request(smem + ROFF_ANSWER, answer_bar);
       if (mbar_wait_bounded(answer_bar, answer_phase)) {
         const int first = steal_answer(smem + ROFF_ANSWER);
-        if (first >= 0) next = first;
+        if (first >= 0) next = first / CL;
       } else {
         atomicAdd(P.flagged, 1ull);      // no answer: saki_check reports that a row may have been lost
       }
       answer_phase ^= 1u;
     }
-    seqres[0] = next;
+    post((uint32_t*)seqres, (uint32_t)next);
   };
   if (tid == 0) {
     mbar_init(mbar, RW);
@@ -471,10 +519,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     seqres[0] = n_tickets; seqres[1] = 0; seqres[2] = 0; seqres[3] = 1;
   }
-  __syncthreads();
+  row_barrier();               // (the other CTAs of the row have started: their shared memory may be written)
   wait_for_predecessor();
   const __nv_bfloat16 *n_s = nullptr, *n_t = nullptr;   // the rows of the CTA's next position, if any
-  const int64_t first_row = dyn ? ticket_row((int)blockIdx.x) : (int64_t)blockIdx.x;   // grid <= n_rows
+  const int64_t first_row = dyn ? ticket_row(place) : (int64_t)place;   // n_places <= n_rows
   if (first_row < P.n_rows) {
     row_ptrs(first_row, n_s, n_t);
     if (lane == 0) issue(n_s, n_t);
@@ -482,7 +530,14 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   }
   uint32_t phase = 0;
   bool undrained = false;   // this thread gave up on a copy that may still be in flight
-  int rb = 0;
+  int rb = 0, buf = 0;
+  auto other_buffer = [&] {            // red and wmax of the coming row barrier
+    if constexpr (CL > 1) {
+      buf ^= 1;
+      red = (double*)(smem + ROFF_RED) + buf * RNV * GW;
+      wmax = (uint32_t*)(smem + ROFF_WMAX) + buf * 4 * GW;
+    }
+  };
   // Pass "final" ends without a barrier.  What is left of a row after it (the total variation, the
   // one-hot entry of the gradient, the residual draw, the outputs) is done one row later by warp
   // FIN_WARP while thread 0 does the next row's scalars: the row's broadcast buffer, the per-warp sums
@@ -491,18 +546,18 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   int64_t pending_row = -1;
   auto finish_row = [&](int64_t prow, int pb) {
     const double* bcp = (const double*)(smem + ROFF_BC) + pb * BC_DOUBLES;
-    const double* fin = (const double*)(smem + ROFF_FIN) + pb * 2 * RW;
+    const double* fin = (const double*)(smem + ROFF_FIN) + pb * 2 * GW;
     const __nv_bfloat16 *ps, *pt;
     row_ptrs(prow, ps, pt);
     const int64_t pseq = K1c == 1 ? prow : (int64_t)((uint32_t)prow / (uint32_t)K1c);
     const int ppos = (int)(prow - pseq * K1c);
     const bool pbonus = spec && (ppos == K1c - 1);
     const int xp = pbonus ? 0 : (spec ? P.proposal[pseq * P.prop_ld + ppos] : P.proposal[prow]);
-    const double tv_sum = warp_sum_d(lane < RW ? fin[lane] : 0.0);
+    const double tv_sum = warp_sum_d(lane < GW ? fin[lane] : 0.0);
     const double tv = (bcp[BC_LAMBDA] > 0.0) ? tv_sum : 0.0;
     const float k0p = (float)bcp[BC_K0];
     const int tok0 = (int)bcp[BC_TOK], tok = tok0 == VSTAR_ELSEWHERE ? (int)bcp[BC_VSTAR] : tok0;
-    if (lane == 0 && P.dlogits && tok >= 0) {   // the supervised token: gradient KG * (p - 1), over the entry its chunk's owner stored
+    if (lane == 0 && crank == 0 && P.dlogits && tok >= 0) {   // the supervised token: gradient KG * (p - 1), over the entry its chunk's owner stored
       const float ipf = (float)bcp[BC_IP];
       const float kgf = (float)(bcp[BC_KG] * (double)ipf);
       const float s_tok = (float)(tok == xp ? bcp[BC_SX] : bcp[BC_SV]);
@@ -510,20 +565,20 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       ((__nv_bfloat16*)P.dlogits + prow * P.ld_g)[tok] = __float2bfloat16_rn(fmaf(ep, kgf, -(float)bcp[BC_KG]));
     }
     if (!(pbonus || bcp[BC_CORR] != 0.0)) {
-      if (lane == 0) write_result_tv(bcp, P.out, !spec, prow, 0, xp, false, K.c64, ps, pt, tv);
+      if (lane == 0 && crank == 0) write_result_tv(bcp, P.out, !spec, prow, 0, xp, false, K.c64, ps, pt, tv);
       return;
     }
     // ---- the draw (corrected and bonus rows): the warp that owns the inverse-CDF target, by an
     // ordered scan of the per-warp weights
-    const double mine_w = lane < RW ? fin[RW + lane] : 0.0;
+    const double mine_w = lane < GW ? fin[GW + lane] : 0.0;
     double inc_w = mine_w;
 #pragma unroll
-    for (int o = 1; o < RW; o <<= 1) {
+    for (int o = 1; o < GW; o <<= 1) {
       const double up = __shfl_up_sync(0xffffffffu, inc_w, o);
       if (lane >= o) inc_w += up;
     }
-    const double target = bcp[BC_UDRAW] * __shfl_sync(0xffffffffu, inc_w, RW - 1);
-    const unsigned cross = __ballot_sync(0xffffffffu, lane < RW && inc_w > target);
+    const double target = bcp[BC_UDRAW] * __shfl_sync(0xffffffffu, inc_w, GW - 1);
+    const unsigned cross = __ballot_sync(0xffffffffu, lane < GW && inc_w > target);
     const unsigned posw = __ballot_sync(0xffffffffu, mine_w > 0.0);
     int owner;
     double running = 0.0;
@@ -535,9 +590,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       owner = posw ? 31 - __clz(posw) : 0;
       last_mode = true;
     }
+    if (CL > 1 && owner / RW != crank) return;       // (it is the CTA with the owner's step weights that draws and writes)
     Seg so;          // the owner's segment
     seg_of(owner, so);
-    const float* step_w = (const float*)(smem + ROFF_STEP) + owner * MAX_STEPS;
+    const float* step_w = (const float*)(smem + ROFF_STEP) + (owner - crank * RW) * MAX_STEPS;
     const int ns = min(so.steps, MAX_STEPS);
     // the step that holds the target (every lane walks the same few numbers)
     int ks = -1, kpos = -1;
@@ -618,7 +674,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     // thread 0, once the row's decision is known: where the CTA goes next when sequences are handed out
     auto plan_next = [&] {
       const int mode = (int)bc[BC_MODE];
-      if (!dyn || mode == MODE_SOLVE) return;
+      if (!dyn || crank != 0 || mode == MODE_SOLVE) return;
       if (!bonus && (mode == MODE_FLAGGED || (mode == MODE_FINAL && bc[BC_CORR] != 0.0)))
         atomicMin(P.seq_stop + seq, pos);        // verification of this sequence ends here
       atomicAdd(P.seq_next + 1, 1u);             // statistic: positions routed
@@ -630,6 +686,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       if (warp == UDRAW_WARP) bc[BC_UDRAW] = scalar_uniform(P.seed, rid, bonus ? STAGE_BONUS : STAGE_RESIDUAL);
       if (warp == SX_WARP && x >= 0 && x < V) { sx = ld_bf16(g_s + x); tx = ld_bf16(g_t + x); }
     }
+    other_buffer();
     if (timing && tid == 0) ph[PH_ROWS] += 1;
     RTS(PH_ROW_TOP);
     if (!dead) {
@@ -705,23 +762,29 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
         // key is the largest value and the lowest chunk that holds it
         const uint32_t skey = __reduce_max_sync(0xffffffffu, bf16_key(fmaxf(rs2.x, rs2.y)));
         const uint32_t tkey = __reduce_max_sync(0xffffffffu, arg_c >= 0 ? (bf16_key(mt_run) << 16) | (0xffffu - (uint32_t)arg_c) : 0u);
-        uint32_t* const wm = (uint32_t*)(smem + ROFF_WMAX);
+        const uint32_t* const wm = wmax;
         if ((lane & 3) == 0) {       // (the eighth value's place takes the student's shift)
-          red[(lane >> 2) * RW + warp] = lane == 28 ? (double)ksw : a;
+          post(red + (lane >> 2) * GW + gwarp, lane == 28 ? (double)ksw : a);
         }
-        if (lane == 0) { red[8 * RW + warp] = (double)ktw; wm[warp] = tkey; wm[RW + warp] = skey; }
+        if (lane == 0) { post(red + 8 * GW + gwarp, (double)ktw); post(wmax + gwarp, tkey); post(wmax + GW + gwarp, skey); }
         if (warp == SX_WARP && lane == 0) { bc[BC_SX] = (double)sx; bc[BC_TX] = (double)tx; }
-        any_dead = __syncthreads_or(dead ? 1 : 0);
+        if constexpr (CL == 1) any_dead = __syncthreads_or(dead ? 1 : 0);
+        else {
+          const int gave_up = __any_sync(0xffffffffu, dead);
+          if (lane == 0) post(wmax + 2 * GW + gwarp, (uint32_t)gave_up);
+          row_barrier();
+          any_dead = __any_sync(0xffffffffu, wm[2 * GW + (lane & (GW - 1))] != 0u);
+        }
         if (any_dead) dead = true;
         RTS(PH_LSE_REDUCE);
         if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);   // the previous row's draw and outputs
-        if (warp == RES_WARP) {          // the CTA's next row
+        if (warp == RES_WARP && crank == 0) {          // the next row
           if (dyn) reserve_next();
           else if (steal && lane == 0) take_over();
         }
         pending_row = -1;
         if (warp == SV_WARP) {       // the teacher's argmax, and the student's logit there (the supervised token of a corrected row)
-          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < RW ? wm[lane] : 0u);
+          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < GW ? wm[lane] : 0u);
           if (lane == 0) {
             int best = 0;
             float sv = 0.f;
@@ -745,15 +808,15 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
           // From here on the row's shifts are those of its true maxima (the largest term of each sum has its exponent
           // argument in (-1, 0], where float32 resolves it best); a warp's shift came from an element of the row, so it
           // is never below the row's, and the factor is an exact power of two <= 1.
-          const float gms = bf16_of_key(__reduce_max_sync(0xffffffffu, lane < RW ? wm[RW + lane] : 0u));
-          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < RW ? wm[lane] : 0u);
+          const float gms = bf16_of_key(__reduce_max_sync(0xffffffffu, lane < GW ? wm[GW + lane] : 0u));
+          const uint32_t gk = __reduce_max_sync(0xffffffffu, lane < GW ? wm[lane] : 0u);
           const float gmt = gk ? bf16_of_key(gk >> 16) : -CUDART_INF_F;
           const double krs = (double)-ceilf(c32 * fmaxf(gms, -1e30f)), krt = (double)-ceilf(c32 * fmaxf(gmt, -1e30f));
           const double a = gather8([&](int role, int w) {
             const bool teacher = (role == 1 || role == 5);
-            const double kw = red[(teacher ? 8 : 7) * RW + w];
+            const double kw = red[(teacher ? 8 : 7) * GW + w];
             const double f = kw < 1e29 ? (double)pow2f_exact((float)((teacher ? krt : krs) - kw)) : 0.0;
-            return role < 7 ? f * red[role * RW + w] : 0.0;
+            return role < 7 ? f * red[role * GW + w] : 0.0;
           });
           const int role = lane >> 2;
           if ((lane & 3) == 0 && role < 7) gat[role < 6 ? role : 9] = a;       // gat[9]: the fourth moment
@@ -865,6 +928,9 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       RTS(PH_LSE_SCALAR);
       __syncthreads();
     }
+    // the next row, which the first CTA has found meanwhile, is the others' to read behind the next row barrier: the one of the
+    // first evaluation, or one more where there is none
+    if (CL > 1 && (dyn || steal) && (int)bc[BC_MODE] != MODE_SOLVE) row_barrier();
     const float k0 = (float)bc[BC_K0], k1 = (float)bc[BC_K1];   // the row's shifts: exponent arguments <= 0
 
     // ------------------------------------------------ pass "solve" (repeated)
@@ -897,10 +963,11 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       if constexpr (!SIDE_WARPS) {
         const double v8[8] = {tot(S0), tot(S1), tot(S2), tot(S3), tot(S4), 0.0, 0.0, 0.0};
         const double a = warp_sum8(v8, lane);
-        if ((lane & 3) == 0) red[(lane >> 2) * RW + warp] = a;
-        __syncthreads();
+        other_buffer();
+        if ((lane & 3) == 0) post(red + (lane >> 2) * GW + gwarp, a);
+        row_barrier();
         if (warp == 0) {
-          const double b = gather8([&](int role, int w) { return red[role * RW + w]; });
+          const double b = gather8([&](int role, int w) { return red[role * GW + w]; });
           if ((lane & 3) == 0 && lane < 20) gat[lane >> 2] = b;
           __syncwarp();
         }
@@ -913,12 +980,12 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       if (tid == 0) {
         scalar_after_solve4(bc, gat, K, k0, k1, x, bonus, masked);
         plan_next();
-        atomicAdd(P.redo_count + 3, 1u);         // statistic: evaluation passes
+        if (crank == 0) atomicAdd(P.redo_count + 3, 1u);         // statistic: evaluation passes
       }
       RTS(PH_SOLVE_SCALAR);
       __syncthreads();
     }
-    const int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + gridDim.x;
+    const int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + n_places;
     next_row_c = next_row;
     n_s = nullptr; n_t = nullptr;
     if (next_row < P.n_rows) row_ptrs(next_row, n_s, n_t);
@@ -926,7 +993,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     // ------------------------------------------------ flagged row: zero outputs, zero gradient
     if ((int)bc[BC_MODE] == MODE_FLAGGED || (int)bc[BC_MODE] == MODE_REDO) {
       const bool redo = (int)bc[BC_MODE] == MODE_REDO;   // ill-conditioned for float32: the float64 kernel routes it
-      if (tid == 0) {
+      if (tid == 0 && crank == 0) {
         if (redo) {
           const unsigned int slot = atomicAdd(P.redo_count, 1u);
           P.redo_list[slot] = (int32_t)row;
@@ -1015,8 +1082,8 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       }
       const double v1 = warp_sum_d((double)(R.x + R.y) * (double)iq);
       if (lane == 0) {
-        double* fin = (double*)(smem + ROFF_FIN) + rb * 2 * RW;
-        fin[warp] = v1; fin[RW + warp] = part;
+        double* fin = (double*)(smem + ROFF_FIN) + rb * 2 * GW;
+        post(fin + gwarp, v1); post(fin + GW + gwarp, part);
       }
       pending_row = row;
     }
@@ -1026,11 +1093,11 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   }
 
   cp_async_wait<0>();
-  __syncthreads();
+  row_barrier();               // (and nothing is written to another CTA's shared memory behind it)
   if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);
   // a CTA that gave up on a copy still waits (bounded) for what it has in flight before leaving
   if (undrained && tid == 0) (void)mbar_wait_bounded(mbar, phase);
-  if (timing && tid == 0) {
+  if (timing && tid == 0 && crank == 0) {
     RTS(PH_TAIL);
 #pragma unroll 1
     for (int i = 0; i < PH_LAST; ++i) atomicAdd(P.phase_cycles + i, (unsigned long long)ph[i]);
@@ -1057,18 +1124,18 @@ cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* s
       cached_dev = dev;
     }
   }
-  // as many CTAs as run at once, or one per row of which they take over those that have not started
-  const int64_t ctas = (int64_t)cached_sms * CTAS_PER_SM;
-  const bool steal = p.seq_next == nullptr && p.n_rows > ctas && p.n_rows <= (1 << 27);
-  const dim3 grid((unsigned)(steal || p.n_rows < ctas ? p.n_rows : ctas));
-  const cudaError_t e = p.spec ? launch_pdl(rowsm_kernel<true>, grid, RT, RSMEM_BYTES, st, true, p, (int)steal)
-                               : launch_pdl(rowsm_kernel<false>, grid, RT, RSMEM_BYTES, st, true, p, (int)steal);
+  // CTAs (clusters) for as many rows as are in flight at once, or for every row, of which they take over those that have not started
+  const int64_t at_once = std::max<int64_t>(1, (int64_t)cached_sms * CTAS_PER_SM / CL);
+  const bool steal = p.seq_next == nullptr && p.n_rows > at_once && p.n_rows <= (1 << 27);
+  const dim3 grid((unsigned)((steal || p.n_rows < at_once ? p.n_rows : at_once) * CL));
+  const cudaError_t e = p.spec ? launch_pdl_cluster(rowsm_kernel<true>, grid, RT, CL, RSMEM_BYTES, st, p, (int)steal)
+                               : launch_pdl_cluster(rowsm_kernel<false>, grid, RT, CL, RSMEM_BYTES, st, p, (int)steal);
   if (e == cudaSuccess) { *served = true; if (n_launches) *n_launches += 1; }
   return e;
 }
 
 // largest V the variant takes (its draw bookkeeping holds MAX_STEPS steps per warp)
-int max_v() { return MAX_STEPS * 32 * 8 * RW; }
+int max_v() { return MAX_STEPS * 32 * 8 * GW; }
 
 }  // namespace SAKI_ROWSM_NS
 }  // namespace saki
