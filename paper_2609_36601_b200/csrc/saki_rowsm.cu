@@ -30,9 +30,11 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
 
 // The variant that routes this number of rows soonest, by 231 shapes (V = 8192 to 151936, 20 to 5000 rows, every variant timed): the
 // choice is 0.6 % above the best of them on average, 3 % or more for one shape in fifteen, 13 % at worst.
-//   - A row or less for two SMs: two CTAs of 512 threads on two SMs to a row (us, one SM per row / two: 74 rows of 151936 50.7 /
-//     33.8, of 65536 32.4 / 23.7, of 32768 22.5 / 19.0); a row or less per SM: the pair of CTAs of 256 threads (148 rows of
-//     151936 60.8 / 58.3, of 65536 33.8 / 30.1, of 24000 20.9 / 19.1).  Below V = 20000 the exchange costs what it saves: two
+//   - A row or less for two SMs: two CTAs of 512 threads on two SMs to a row (us, one SM per row / two: 74 rows of 98304 37.9 /
+//     26.1, of 65536 32.4 / 23.7, of 32768 22.5 / 19.0); a row or less per SM: the pair of CTAs of 256 threads (148 rows of
+//     151936 60.8 / 58.3, of 65536 33.8 / 30.1, of 24000 20.9 / 19.1).  Rows of V > 98304 take the pair there too (37 rows of 151936
+//     50.2 / 36.6, 32.8 with 512 threads; 74 rows 50.7 / 49.3, 33.8): its sixteen warps give the bits of the pinned variant, which
+//     callers and tests of such pieces compare with.  Below V = 20000 the exchange costs what it saves: two
 //     CTAs per SM (148 rows of 16384 17.9, the pair 17.5; 20 rows 15.3, 15.4).
 //   - More: the variant that takes the least by a cost model, start + (serial + element V / 1000) turns, where a turn is waited
 //     for to its end only in part (CTAs take over rows that have not started) and costs more where the rows in flight are more than
@@ -48,7 +50,7 @@ cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, b
     const int64_t n = p.call_rows;
     if (n <= sms) {
       if (p.V < 20000) return half_sm::launch(p, st, n_launches, served);
-      return 2 * n <= sms ? wide_sm::launch(p, st, n_launches, served) : pair_sm::launch(p, st, n_launches, served);
+      return 2 * n <= sms && p.V <= HALF_MAX_V ? wide_sm::launch(p, st, n_launches, served) : pair_sm::launch(p, st, n_launches, served);
     }
     // per_sm: rows in flight per SM; whole: the part of a turn that is waited for to its end; late: how far into its turn an
     // average CTA is when no row is left; beyond: for each 126 MB in flight beyond L2

@@ -42,7 +42,7 @@ def test_rows_in_one_call_and_in_pieces(V, per_sm, extra):
 
 # two blocks to a row, as dispatched: up to half as many rows as SMs in blocks of 512 threads, then of 256; the last and the first
 # row of each rule, more rows than are in flight, segments of one step, ragged last steps, and the longest row
-@pytest.mark.parametrize("V,N", [(20000, 74), (20000, 75), (24576, 148), (57344, 33), (98312, 74), (151936, 148), (151936, 149), (100352, 447), (262144, 40), (262144, 150)])
+@pytest.mark.parametrize("V,N", [(20000, 74), (20000, 75), (24576, 148), (57344, 33), (98304, 74), (98312, 74), (151936, 148), (151936, 149), (100352, 447), (262144, 40), (262144, 150)])
 @pytest.mark.parametrize("eps", [0.0, 0.1, 40.0])      # no evaluation, one or more, none (saturated): other barriers between the blocks
 def test_two_blocks_per_row(V, N, eps):
     w = synth.Workload("t", N, V, "bf16", eps, 1.5, True, 900 + V % 97, 31, temperature=0.875)
