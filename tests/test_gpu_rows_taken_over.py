@@ -6,7 +6,7 @@ import pytest
 import torch
 
 import paper_2609_36601_b200 as P
-from paper_2609_36601_b200 import synth
+from paper_2609_36601_b200 import binding as B, synth
 import oracle as O
 from parity import compare_rows, force_second_tier, grad_check, oracle_inputs, to_np64
 
@@ -60,7 +60,7 @@ def test_two_blocks_per_row(V, N, eps):
     assert P.check() == 4                  # two flagged rows, two calls
     for k in out:
         assert torch.equal(out[k], fwd[k]), k
-    assert int(out["row_status"][3]) & P.ROW_NONFINITE and int(out["row_status"][4]) & P.ROW_BAD_ID
+    assert int(out["row_status"][3]) & B.ROW_NONFINITE and int(out["row_status"][4]) & B.ROW_BAD_ID
     assert not g[3].any() and not g[4].any() and not g[5].any()
     rows = sorted({0, 1, 2, 6, N // 2, N - 2, N - 1})
     s64, t64 = oracle_inputs(d)
