@@ -199,8 +199,8 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
     g_last_redo_generation = g_redo_generation.load();
   }
   // A handful of long rows (a decoding step of a small batch) finish sooner spread over the whole GPU, one row per cluster
-  // of up to 16 blocks, than on one SM each: 1 / 8 / 32 rows of V = 151936 take 15.7 / 18.7 / 24.5 us there against 42 / 49
-  // / 49 us, of V = 32768 14 / 14 / 18 against 18 / 24 / 24 us (at V = 8192 there is no difference).
+  // of up to 16 blocks, than on one SM each: 1 / 8 / 32 rows of V = 151936 take 15.7 / 18.7 / 24.5 us there against 37 us
+  // on two SMs each, of V = 32768 14 / 14 / 18 against 18 us (at V = 8192 there is no difference).
   if (fast && which == 0 && p.call_rows <= 32 && p.V >= 32768 && eps_ok && cluster_can_serve(p, dtype)) {
     e = launch_cluster(p, st, &launches, &served);
     if (e != cudaSuccess) return cuda_fail(e, "cluster kernel launch");

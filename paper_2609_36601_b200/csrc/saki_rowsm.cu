@@ -5,7 +5,7 @@
 
 namespace saki {
 
-// Rows up to this length go to the variant with two CTAs of 256 threads per SM: their passes are short
+// Where the kernel is pinned, rows up to this length go to the variant with two CTAs of 256 threads per SM: their passes are short
 // against the serial phases between them (block reductions, float64 scalars), and a second CTA on the
 // SM runs its passes meanwhile.  Longer rows stay with one CTA per SM: with two rows in flight per SM
 // the streamed parts of all rows no longer stay in L2 between the passes.  Measured (fwd+bwd, M rows/s,

@@ -82,7 +82,7 @@ constexpr int MAX_STEPS = GW > 16 ? 32 : 64;     // steps per warp the draw book
 constexpr int RES_CHUNKS = KS_MAX * 32; // resident chunks per warp and row
 constexpr int RNV = 9;                  // doubles per partial vector
 static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight warps, or done by warp 0; the side work has warps of its own, or is shared out");
-// Who does what beside the passes.  With 14 warps or more the row scalars that do not depend on the
+// Who does what beside the passes.  With 14 warps or more, and a CTA per row, the row scalars that do not depend on the
 // passes (uniforms, the logits at the proposal) are fetched by warps 8-10 while warps 0-7 gather the warps' sums, one sum
 // each; a block barrier; then thread 0 does the scalars.  With four or eight warps warp 0 gathers all sums at once (four
 // lanes per sum) and goes straight on to the scalars: a barrier less per pass, and the eight sums are not dealt
