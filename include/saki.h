@@ -360,8 +360,8 @@ SAKI_API int saki_check(void* cuda_stream, uint64_t* n_flagged);
 
 /* Selects the row kernel: 0 = automatic, 1 = the general kernel (any V, dtype and layout; float64, a row shared by 1 to 8
  * blocks), 2 = the cluster kernel (one row per cluster of 1 to 16 blocks, in shared memory), 3 = the row-per-SM kernel
- * (one row per block; shared memory plus L2; one block of 512 threads, two of 256 or four of 128 per SM, by V and the
- * number of rows).  2 and 3 serve bf16 rows with 16-byte aligned rows and V a multiple of 8, V >= 2048 (2: V <= 163840;
+ * (one row per block; shared memory plus L2; one block of 512 threads, two of 256 or four of 128 per SM by V; automatic
+ * goes by the number of rows too, and may give a row two blocks on two SMs).  2 and 3 serve bf16 rows with 16-byte aligned rows and V a multiple of 8, V >= 2048 (2: V <= 163840;
  * and eps = 0 or eps >= 5e-3: its float32 sums cannot resolve smaller radii to the tolerance, whereas 3 takes every
  * radius); other inputs fall back to 1.  Automatic prefers 3, except for calls of at most 32 rows with V >= 32768 that 2
  * can serve: a few long rows finish sooner spread over the whole GPU.  Process-wide; meant for tests and benchmarks.
