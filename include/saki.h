@@ -393,14 +393,14 @@ SAKI_API int saki_solve_evaluations(void* cuda_stream, uint64_t* n_passes);
 
 /* Failure behaviour of the row-per-SM and general kernels (no counterpart in the paper).  A thread block of the first waits for a
  * row's bulk copy from global memory for a bounded number of SM cycles (about two seconds' worth by
- * default).  If the wait runs out the block stops fetching, flags that row and every row it still owns
- * SAKI_ROW_TIMEOUT with zero outputs, waits (full limit) for the copy it has in flight, and returns: the
- * kernel always terminates, saki_check() counts the flagged rows and later calls are unaffected.  A block of the second, in
+ * default).  If the wait runs out the block stops fetching, flags that row (in block verification every position it still
+ * takes) SAKI_ROW_TIMEOUT with zero outputs, waits (full limit) for the copy it has in flight, and returns: the
+ * kernel always terminates, saki_check() counts the flagged rows and later calls are unaffected.  A block of either kernel, in
  * calls of more rows than are resident at once, waits as long for the answer to its request for a further row; if that wait
  * runs out it waits once more at full length, flags the row that it was given SAKI_ROW_TIMEOUT and asks for no other (if there
  * is no answer then either, saki_check() counts one row that carries no flag).  This
  * call sets the limit for the routing calls that follow, from any thread (0: the default), and returns
- * the previous value; tests use a limit of a few cycles to exercise that path without withholding
+ * the previous value; tests use limits of a few to some hundred cycles to exercise those paths without withholding
  * anything. */
 SAKI_API int64_t saki_set_wait_limit(int64_t cycles);
 

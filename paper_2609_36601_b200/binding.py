@@ -439,8 +439,8 @@ PHASES = ("row_top", "copy_wait", "lse", "lse_reduce", "lse_gather", "lse_scalar
 
 
 def set_wait_limit(cycles: int) -> int:
-    """SM cycles a block of the row-per-SM kernel waits for a row's bulk copy, and one of the general kernel for its next
-    row, before it flags rows TIMEOUT (0: the default of about two seconds); returns the previous setting."""
+    """SM cycles a block of the row-per-SM kernel waits for a row's bulk copy, and one of either that or the general kernel for
+    its next row, before it flags rows TIMEOUT (0: the default of about two seconds); returns the previous setting."""
     return int(load_library().saki_set_wait_limit(int(cycles)))
 
 
