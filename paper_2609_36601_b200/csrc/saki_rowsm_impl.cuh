@@ -497,19 +497,24 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     }
   };
   // Plain rows: the row of a CTA that has not started yet.  Not once this CTA has given up on a copy: what it does not take
-  // over is launched.  An answer that is late may still have cancelled a launch, which nobody else will make up for: the row's
-  // number comes back as late_base plus the row (beyond every row, so that the row loop ends with it), and the CTAs of the row
-  // flag it on their way out.  (lane 0 of RES_WARP, in the row's first CTA)
+  // over is launched.  An answer that is late may still have cancelled a launch, which nobody else will make up for: the row comes
+  // back as late_base plus its number, and the CTAs treat it as one whose copy they gave up on.  (lane 0 of RES_WARP, in the
+  // row's first CTA)
   const int late_base = n_tickets + 1;       // (at most 2^27 rows are taken over: twice that fits)
   uint32_t answer_phase = 0;
   auto take_over = [&] {
     int next = n_tickets;
     if (!dead) {
       steal_request(smem + ROFF_ANSWER, answer_bar);
-      const bool in_time = mbar_wait_bounded(answer_bar, answer_phase, wait_limit);
-      if (in_time || mbar_wait_bounded(answer_bar, answer_phase)) {
+      const long long asked = clock64();
+      bool came, late;
+      do {
+        came = mbar_try_wait(answer_bar, answer_phase);
+        late = clock64() - asked > wait_limit;
+      } while (!came && !(late && clock64() - asked > WAIT_LIMIT_CYCLES));
+      if (came) {
         const int first = steal_answer(smem + ROFF_ANSWER);
-        if (first >= 0) next = (in_time ? 0 : late_base) + first / CL;
+        if (first >= 0) next = (late ? late_base : 0) + first / CL;
       } else {
         atomicAdd(P.flagged, 1ull);      // no answer at all: saki_check reports that a row may have been lost
       }
@@ -662,15 +667,6 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     }
     if (y < 0) y = min(V - 1, max(so.c0 * 8, so.c1 * 8 - 1));
     if (lane == 0) write_result_tv(bcp, P.out, !spec, prow, pbonus ? 0 : 1, y, pbonus, K.c64, ps, pt, tv);
-  };
-
-  auto zero_gradient = [&](int64_t row) {      // this warp's share of the gradient row of a flagged row
-    __nv_bfloat16* const g = (__nv_bfloat16*)P.dlogits + row * P.ld_g;
-#pragma unroll 1
-    for (int k = 0; k < sg.steps; ++k) {
-      const int c = sg.c0 + k * 32 + lane;
-      if (c < sg.c1) st_stream(g + (size_t)c * 8, make_uint4(0, 0, 0, 0), pol_first);
-    }
   };
 
   int64_t next_row_c = P.n_rows;
@@ -998,7 +994,8 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       RTS(PH_SOLVE_SCALAR);
       __syncthreads();
     }
-    const int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + n_places;
+    int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + n_places;
+    if (steal && next_row >= late_base) { next_row -= late_base; dead = true; }    // taken over too late: flagged, and the last
     next_row_c = next_row;
     n_s = nullptr; n_t = nullptr;
     if (next_row < P.n_rows) row_ptrs(next_row, n_s, n_t);
@@ -1017,7 +1014,13 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
           atomicAdd(P.flagged, 1ull);
         }
       }
-      if (g_out && !redo) zero_gradient(row);
+      if (g_out && !redo) {
+#pragma unroll 1
+        for (int k = 0; k < sg.steps; ++k) {
+          const int c = sg.c0 + k * 32 + lane;
+          if (c < sg.c1) st_stream(g_out + (size_t)c * 8, make_uint4(0, 0, 0, 0), pol_first);
+        }
+      }
       __syncwarp();
       if (lane == 0 && !dead && next_row < P.n_rows) {
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -1102,14 +1105,6 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
   cp_async_wait<0>();
   row_barrier();               // (and nothing is written to another CTA's shared memory behind it)
   if (warp == FIN_WARP && pending_row >= 0) finish_row(pending_row, rb ^ 1);
-  if (steal && next_row_c >= late_base) {              // a row whose launch was cancelled by a request that was answered too late
-    const int64_t row = next_row_c - late_base;
-    if (tid == 0 && crank == 0) {
-      write_row(P.out, row, zero_row(SAKI_ROW_TIMEOUT), !spec);
-      atomicAdd(P.flagged, 1ull);
-    }
-    if (P.dlogits) zero_gradient(row);
-  }
   // a CTA that gave up on a copy still waits (bounded) for what it has in flight before leaving
   if (undrained && tid == 0) (void)mbar_wait_bounded(mbar, phase);
   if (timing && tid == 0 && crank == 0) {
