@@ -439,14 +439,21 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
     }
     __syncthreads();
   };
-  // the same for eight values at once on warp 0 (lane l: value l / 4), which goes on alone; a barrier before, none after
+  // the same for eight values at once on warp 0 (lane l: value l / 4), which goes on alone; a barrier before, none after.
+  // The warps' terms are added in the order of combine's shuffle tree (the furthest apart first), so that a row of sixteen
+  // warps has the same sums on one CTA and on a pair.
   auto gather8 = [&](auto&& term) {
-    double a = 0.0;
+    double a[GW / 4];
 #pragma unroll
-    for (int w = lane & 3; w < GW; w += 4) a += term(lane >> 2, w);
-    a += __shfl_xor_sync(0xffffffffu, a, 2);
-    a += __shfl_xor_sync(0xffffffffu, a, 1);
-    return a;
+    for (int k = 0; k < GW / 4; ++k) a[k] = term(lane >> 2, 4 * k + (lane & 3));
+#pragma unroll
+    for (int h = GW / 8; h > 0; h >>= 1) {
+#pragma unroll
+      for (int k = 0; k < h; ++k) a[k] += a[k + h];
+    }
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 2);
+    a[0] += __shfl_xor_sync(0xffffffffu, a[0], 1);
+    return a[0];
   };
 
   // Block verification with early out (Section 3.5 discards what lies behind a sequence's first
