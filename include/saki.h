@@ -378,6 +378,10 @@ SAKI_API int saki_last_kernel(void);
  * how many rows are resident at once that way (zeros if there was none).  For tests; NULL where not wanted. */
 SAKI_API void saki_last_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm, int32_t* resident_rows);
 
+/* The variant of the row-per-SM kernel that served the calling thread's last routing call: blocks per row (2: on two SMs) and
+ * blocks per SM (zeros if another kernel served it).  For tests; NULL where not wanted. */
+SAKI_API void saki_last_rowsm_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm);
+
 /* Two-tier routing: the float32 kernels (2, 3) hand rows whose KL they cannot resolve to the
  * tolerance (very small eps, nearly one-hot rows) to the float64 kernel, through a row list in device
  * memory that the library allocates once per device and stream and keeps (calls on different streams

@@ -27,7 +27,7 @@ EXPORTS = ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_fwd_bwd_noalloc",
            "saki_route_bwd_from_meta", "saki_select_tm", "saki_spec_verify",
            "saki_vshard_partial", "saki_vshard_stage", "saki_vshard_combine", "saki_vshard_combine_host",
            "saki_lmhead_scratch_bytes", "saki_lmhead_lse",
-           "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_last_layout", "saki_redo_count",
+           "saki_sample_proposal", "saki_check", "saki_set_kernel", "saki_last_kernel", "saki_last_layout", "saki_last_rowsm_layout", "saki_redo_count",
            "saki_set_spec_early_out", "saki_spec_positions_routed", "saki_solve_evaluations", "saki_set_wait_limit", "saki_set_phase_clock", "saki_phase_cycles",
            "saki_launch_count",
            "saki_last_error", "saki_version")
@@ -157,6 +157,8 @@ def load_library(path: str | None = None):
     lib.saki_phase_cycles.restype = C.c_int
     lib.saki_last_layout.argtypes = [C.POINTER(C.c_int32)] * 3
     lib.saki_last_layout.restype = None
+    lib.saki_last_rowsm_layout.argtypes = [C.POINTER(C.c_int32)] * 2
+    lib.saki_last_rowsm_layout.restype = None
     lib.saki_launch_count.restype = C.c_uint64
     lib.saki_last_error.restype = C.c_char_p
     for f in ("saki_route_fwd", "saki_route_fwd_bwd", "saki_route_host", "saki_spec_verify",
@@ -415,6 +417,13 @@ def last_layout():
     """(blocks per row, blocks per SM, rows resident at once) of the calling thread's last call that the general kernel served."""
     n = (C.c_int32 * 3)()
     load_library().saki_last_layout(*(C.cast(C.byref(n, 4 * k), C.POINTER(C.c_int32)) for k in range(3)))
+    return tuple(n)
+
+
+def last_rowsm_layout():
+    """(blocks per row, blocks per SM) of the calling thread's last routing call if the row-per-SM kernel served it, else zeros."""
+    n = (C.c_int32 * 2)()
+    load_library().saki_last_rowsm_layout(*(C.cast(C.byref(n, 4 * k), C.POINTER(C.c_int32)) for k in range(2)))
     return tuple(n)
 
 

@@ -179,6 +179,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
   p.redo_list = nullptr; p.redo_count = nullptr; p.redo_guess = nullptr; p.from_list = 0;
   p.wait_limit = g_wait_limit.load();
   g_last_redo_count = nullptr;          // the counters below describe this call only
+  rowsm_layout_none();
   std::unique_lock<std::mutex> scratch_lock(g_redo_mu, std::defer_lock);
   if (fast) {
     if (scratch_list) { p.redo_list = scratch_list; p.redo_count = scratch_count; }
@@ -793,6 +794,13 @@ SAKI_API void saki_last_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm, 
   if (blocks_per_row) *blocks_per_row = l[0];
   if (blocks_per_sm) *blocks_per_sm = l[1];
   if (resident_rows) *resident_rows = l[2];
+}
+
+SAKI_API void saki_last_rowsm_layout(int32_t* blocks_per_row, int32_t* blocks_per_sm) {
+  int l[2];
+  rowsm_layout(l);
+  if (blocks_per_row) *blocks_per_row = l[0];
+  if (blocks_per_sm) *blocks_per_sm = l[1];
 }
 
 SAKI_API int saki_redo_count(void* cuda_stream, uint64_t* n_rows) {

@@ -233,6 +233,8 @@ void general_layout(int* out);      // of the calling thread's last call: blocks
 cudaError_t launch_cluster(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
 bool cluster_can_serve(const RowParams& p, int dtype);
 cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served);
+void rowsm_layout(int* out);        // of the calling thread's last routing call: blocks per row, blocks per SM (zeros: another kernel)
+void rowsm_layout_none();
 namespace full_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace half_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }
 namespace pair_sm { cudaError_t launch(const RowParams& p, cudaStream_t st, int* n_launches, bool* served); int max_v(); }

@@ -16,6 +16,8 @@ constexpr int HALF_MAX_V = 98304;
 // pass at any time.  Measured (M rows/s, two / four CTAs per SM): V = 4096 29.7 / 44.4, 8192 26.0 / 35.0,
 // 16384 19.6 / 21.7, 32000 13.1 / 14.3, 49152 9.8 / 10.0, 65536 7.8 / 7.5.
 constexpr int QUARTER_MAX_V = 49152;
+// Rows of more than this many elements do not go to two SMs in blocks of 512 threads (why: see the choice below).
+constexpr int WIDE_MAX_V = 98304;
 
 bool rowsm_can_serve(const RowParams& p, int dtype) {
   if (dtype != SAKI_BF16) return false;
@@ -27,6 +29,13 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
   if (p.dlogits && (!al16(p.dlogits) || p.ld_g % 8)) return false;
   return true;
 }
+
+struct Variant {
+  cudaError_t (*launch)(const RowParams&, cudaStream_t, int*, bool*);
+  int blocks_per_row, blocks_per_sm;
+};
+static const Variant FULL = {full_sm::launch, 1, 1}, HALF = {half_sm::launch, 1, 2}, QUARTER = {quarter_sm::launch, 1, 4},
+                     PAIR = {pair_sm::launch, 2, 2}, WIDE = {wide_sm::launch, 2, 1};
 
 // The variant that routes this number of rows soonest, by 231 shapes (V = 8192 to 151936, 20 to 5000 rows, every variant timed): the
 // choice is 0.6 % above the best of them on average, 3 % or more for one shape in fifteen, 13 % at worst.
@@ -42,34 +51,43 @@ bool rowsm_can_serve(const RowParams& p, int dtype) {
 //     and four CTAs per SM shorter ones (2000 rows of 65536 314 / 267 with two; of 16384 157 / 88 with four).
 //   - Rows beyond V = 131072 by the thousands: one CTA per SM (16384 rows of 151936 4517, the pair 4550; 4096 rows 1167, 1162).
 // Not where saki_set_kernel pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
-cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
-  if (p.call_rows > 0) {
-    int dev = 0, sms = 148;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t n = p.call_rows;
-    if (n <= sms) {
-      if (p.V < 20000) return half_sm::launch(p, st, n_launches, served);
-      return 2 * n <= sms && p.V <= HALF_MAX_V ? wide_sm::launch(p, st, n_launches, served) : pair_sm::launch(p, st, n_launches, served);
-    }
-    // per_sm: rows in flight per SM; whole: the part of a turn that is waited for to its end; late: how far into its turn an
-    // average CTA is when no row is left; beyond: for each 126 MB in flight beyond L2
-    struct Model { double per_sm, start, serial, element, whole, late, beyond; };
-    auto cost = [&](const Model& m) {
-      const double slots = m.per_sm * sms, turns = (double)n / slots, in_flight = std::min((double)n, slots) * 4.0 * p.V;
-      const double t = turns > 1.0 ? m.whole * std::ceil(turns) + (1.0 - m.whole) * (turns + m.late) : 1.0;
-      return m.start + (m.serial + m.element * 1e-3 * p.V) * std::max(1.0, t) * (1.0 + m.beyond * std::max(0.0, in_flight / 126e6 - 1.0));
-    };
-    const double full = cost({1, 4.64, 6.52, 0.2485, 0.548, 1.0, 0.05}), half = cost({2, 7.40, 3.64, 0.5366, 0.156, 0.253, 0.221}),
-                 quarter = cost({4, 5.68, 4.31, 1.0593, 0.091, 0.246, 0.131}), pair = cost({1, 4.70, 6.03, 0.2368, 0.121, 0.535, 0.05});
-    if (p.V <= QUARTER_MAX_V && quarter < half && quarter < pair) return quarter_sm::launch(p, st, n_launches, served);
-    if (p.V <= half_sm::max_v() && half < pair && half < full) return half_sm::launch(p, st, n_launches, served);
-    if (full < pair || (p.V > 131072 && n > 40 * (int64_t)sms)) return full_sm::launch(p, st, n_launches, served);
-    return pair_sm::launch(p, st, n_launches, served);
+static const Variant& pick_variant(const RowParams& p) {
+  const int64_t n = p.call_rows;
+  if (n <= 0) return p.V <= QUARTER_MAX_V ? QUARTER : p.V <= HALF_MAX_V ? HALF : FULL;
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (n <= sms) {
+    if (p.V < 20000) return HALF;
+    return 2 * n <= sms && p.V <= WIDE_MAX_V ? WIDE : PAIR;
   }
-  if (p.V <= QUARTER_MAX_V && p.V <= quarter_sm::max_v()) return quarter_sm::launch(p, st, n_launches, served);
-  if (p.V <= HALF_MAX_V && p.V <= half_sm::max_v()) return half_sm::launch(p, st, n_launches, served);
-  return full_sm::launch(p, st, n_launches, served);
+  // max_v: the longest row; per_sm: rows in flight per SM; whole: the part of a turn that is waited for to its end; late: how far into its turn an
+  // average CTA is when no row is left; beyond: for each 126 MB in flight beyond L2
+  struct Model { const Variant* v; int max_v; double per_sm, start, serial, element, whole, late, beyond; };
+  const Model models[] = {{&FULL, full_sm::max_v(), 1, 4.64, 6.52, 0.2485, 0.548, 1.0, 0.05}, {&HALF, half_sm::max_v(), 2, 7.40, 3.64, 0.5366, 0.156, 0.253, 0.221},
+                          {&QUARTER, QUARTER_MAX_V, 4, 5.68, 4.31, 1.0593, 0.091, 0.246, 0.131}, {&PAIR, pair_sm::max_v(), 1, 4.70, 6.03, 0.2368, 0.121, 0.535, 0.05}};
+  if (p.V > 131072 && n > 40 * (int64_t)sms) return FULL;
+  const Variant* best = &FULL;
+  double least = 1e300;
+  for (const Model& m : models) {
+    if (p.V > m.max_v) continue;
+    const double slots = m.per_sm * sms, turns = (double)n / slots, in_flight = std::min((double)n, slots) * 4.0 * p.V;
+    const double t = turns > 1.0 ? m.whole * std::ceil(turns) + (1.0 - m.whole) * (turns + m.late) : 1.0;
+    const double c = m.start + (m.serial + m.element * 1e-3 * p.V) * std::max(1.0, t) * (1.0 + m.beyond * std::max(0.0, in_flight / 126e6 - 1.0));
+    if (c < least) { least = c; best = m.v; }
+  }
+  return *best;
+}
+
+static thread_local int g_layout[2];      // of the thread's last routing call: blocks per row, blocks per SM
+void rowsm_layout(int* out) { std::copy(g_layout, g_layout + 2, out); }
+void rowsm_layout_none() { g_layout[0] = g_layout[1] = 0; }
+
+cudaError_t launch_rowsm(const RowParams& p, cudaStream_t st, int* n_launches, bool* served) {
+  const Variant& v = pick_variant(p);
+  const cudaError_t e = v.launch(p, st, n_launches, served);
+  if (e == cudaSuccess && *served) { g_layout[0] = v.blocks_per_row; g_layout[1] = v.blocks_per_sm; }
+  return e;
 }
 
 }  // namespace saki
