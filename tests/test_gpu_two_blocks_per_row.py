@@ -40,3 +40,28 @@ def test_pair_of_blocks_agrees_with_one_block_to_the_bit(V, eps, apart):
     for k in out:
         assert torch.equal(out[k], one[k]), k
     assert torch.equal(g, g_one)
+
+
+# (blocks per row, blocks per SM), as dispatched and with the kernel pinned
+@pytest.mark.parametrize("V,N,layout,pinned", [(8192, 100, (1, 2), (1, 4)), (8192, 2000, (1, 4), (1, 4)), (8192, 304, (1, 4), (1, 4)),
+                                               (9200, 320, (1, 4), (1, 4)), (24000, 156, (1, 2), (1, 4)), (65536, 74, (2, 1), (1, 2)), (65536, 148, (2, 2), (1, 2)),
+                                               (65536, 900, (1, 2), (1, 2)), (98304, 74, (2, 1), (1, 2)), (98312, 74, (2, 2), (1, 1)), (151936, 40, (2, 2), (1, 1)),
+                                               (151936, 447, (2, 2), (1, 1)), (262144, 150, (2, 2), (1, 1))])
+def test_layouts(V, N, layout, pinned):
+    assert torch.cuda.get_device_properties(0).multi_processor_count == 148, "the shapes are chosen for 148 SMs"
+    w = synth.Workload("layout", N, V, "bf16", 0.1, 1.5, True, 7, 7)
+    d = synth.generate(w, DEV)
+    for which, want in ((0, layout), (3, pinned)):
+        prev = P.set_kernel(which)
+        try:
+            P.route_fwd(d["s"], d["t"], d["proposal"], w.eps, seed=w.seed)
+            assert P.last_kernel() == 3 and P.last_rowsm_layout() == want, which
+        finally:
+            P.set_kernel(prev)
+    prev = P.set_kernel(1)
+    try:
+        P.route_fwd(d["s"], d["t"], d["proposal"], w.eps, seed=w.seed)
+        assert P.last_rowsm_layout() == (0, 0)
+    finally:
+        P.set_kernel(prev)
+    torch.cuda.synchronize()
