@@ -56,10 +56,11 @@ FALLBACK_HBM_GBS = 6650.0
 # routed, from an ncu capture on 2220 rows of the same workload (the kernel's ncu summary gives the
 # command); traffic grows in proportion to the rows, so a full launch is this figure times N
 TRAFFIC_BYTES_PER_POSITION = 958376
-# rows up to this length are served by the instances of the two streaming kernels that run two CTAs per SM
-# (namespace half_sm, meta_stream_kernel<16>); the names below are the ones a profiler shows
+# rows up to this length are served by the instance of the metadata backward's streaming kernel that runs two CTAs per SM
+# (meta_stream_kernel<16>); the names below are the ones a profiler shows
 TWO_CTA_MAX_V = 98304
-FOUR_CTA_MAX_V = 49152      # and the row kernel's instance with four (namespace quarter_sm) up to this length
+# the row kernel's instance (its namespace) by what the library says of the call: blocks per row, blocks per SM
+ROWSM_VARIANT = {(1, 1): "full_sm", (1, 2): "half_sm", (1, 4): "quarter_sm", (2, 2): "pair_sm", (2, 1): "wide_sm"}
 # warp-instructions the row kernel's one-CTA instance issues per 32 vocabulary elements, from the same capture
 ISSUED_PER_32_ELEMENTS = 39.09
 # the same for one meta_stream_kernel launch
@@ -416,7 +417,7 @@ def run_ours(args):
         total_ms = float(tt.item())
     ms_per_step = total_ms / args.steps
     value = world * w.N / (ms_per_step * 1e-3)
-    n_flagged = P.check()
+    kernel_used, layout_used = P.last_kernel(), P.last_rowsm_layout()
     kernel_used = P.last_kernel()
     evals_last_step = P.solve_evaluations(stream) if kernel_used == 3 else 0   # of the last timed launch
     redo_last_step = P.redo_count(stream)
@@ -550,7 +551,7 @@ def run_ours(args):
                 "peak_kind": f"of {peak_kind} (device-to-device copy, MEASURED_PEAKS.json)"
                 if peak_kind == "measured" else "of fallback",
                 "traffic": (TRAFFIC_BYTES_PER_POSITION * w.N) if TRAFFIC_BYTES_PER_POSITION else None,
-                "algorithmic_bytes_per_launch": bpp * w.N, "kernel": {3: "saki::%s::rowsm_kernel<false>" % ("quarter_sm" if w.V <= FOUR_CTA_MAX_V else "half_sm" if w.V <= TWO_CTA_MAX_V else "full_sm"),
+                "algorithmic_bytes_per_launch": bpp * w.N, "kernel": {3: "saki::%s::rowsm_kernel<false>" % ROWSM_VARIANT.get(layout_used),
                            2: "saki::cluster_kernel"}.get(kernel_used, "saki::general_kernel"),
                 "kernel_ms": kern_ms,
                 "frac_of_nominal_8TBs": achieved / 8000.0}
@@ -571,12 +572,12 @@ def run_ours(args):
         # and its other near-binding bound: issue slots (4 warp-instructions per clock per SM); the instruction
         # count per 32 elements is the profiler's (smsp__inst_executed.sum of the capture the kernel's ncu
         # summary describes, divided by the elements of that launch), not counted live
-        if w.V > TWO_CTA_MAX_V:
+        if layout_used == (1, 1):
             iss_peak = 4.0 * sm_count * mhz * 1e6 / 1e9
             iss_ach = ISSUED_PER_32_ELEMENTS * w.V * w.N / 32.0 / (kern_ms * 1e-3) / 1e9
             roofline["issue_slots"] = {"achieved": iss_ach, "peak": iss_peak, "unit": "G warp-instructions/s",
                                        "frac": iss_ach / iss_peak, "issued_per_32_elements": ISSUED_PER_32_ELEMENTS,
-                                       "source": "ncu capture on 2220 rows of this workload"}
+                                       "source": "ncu capture of the same kernel on 2220 rows of this workload"}
 
     stats = {"correction_rate": float(out["corrected"].float().mean().item()),
              "median_tv": float(out["tv"].median().item()), "mean_lambda": float(out["lambda"].mean().item()),
