@@ -417,8 +417,8 @@ def run_ours(args):
         total_ms = float(tt.item())
     ms_per_step = total_ms / args.steps
     value = world * w.N / (ms_per_step * 1e-3)
+    n_flagged = P.check()
     kernel_used, layout_used = P.last_kernel(), P.last_rowsm_layout()
-    kernel_used = P.last_kernel()
     evals_last_step = P.solve_evaluations(stream) if kernel_used == 3 else 0   # of the last timed launch
     redo_last_step = P.redo_count(stream)
     phases = None
