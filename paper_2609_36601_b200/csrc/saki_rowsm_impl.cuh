@@ -1,27 +1,27 @@
 // One-row-per-SM kernel for bf16 rows: the implementation, compiled once per variant.
-//   saki_rowsm.cu       one persistent CTA of 512 threads per SM (namespace full_sm)
-//   saki_rowsm_half.cu  two persistent CTAs of 256 threads per SM (namespace half_sm, SAKI_ROWSM_HALF):
+//   saki_rowsm.cu       one CTA of 512 threads per SM (namespace full_sm)
+//   saki_rowsm_half.cu  two CTAs of 256 threads per SM (namespace half_sm, SAKI_ROWSM_HALF):
 //                       for short rows, whose passes are short against the serial phases between them,
 //                       so that one CTA's scalar phases run under the other CTA's passes
 //   saki_rowsm_quarter.cu  four of 128 threads (namespace quarter_sm, SAKI_ROWSM_QUARTER): shorter rows still
 //   saki_rowsm_pair.cu  two of 256 threads per SM, and two CTAs on two SMs (a cluster) to a row (namespace pair_sm,
 //                       SAKI_ROWSM_PAIR): long rows with one CTA's scalar phases under another's passes, as many rows in flight as SMs
-//   saki_rowsm_wide.cu  one of 512 threads per SM and two CTAs to a row (namespace wide_sm, SAKI_ROWSM_WIDE): fewer
-//                       rows than half the SMs
+//   saki_rowsm_wide.cu  one of 512 threads per SM and two CTAs to a row (namespace wide_sm, SAKI_ROWSM_WIDE): up to half
+//                       as many rows as SMs
 //
-// A persistent CTA routes whole rows, one after the
-// other.  A row pair (student + teacher, e.g. 608 KB at V = 151936) does not
+// A CTA (or the two of a cluster) routes whole rows, one after the other: a call of more rows than are in flight at once
+// launches a CTA (cluster) per row, and those that are done take over the rows of those that have not started; block
+// verification hands out tickets.  A row pair (student + teacher, e.g. 608 KB at V = 151936) does not
 // fit on one SM.  Every warp owns a contiguous segment of the row and visits
 // it in steps of 32 chunks of 8 elements; it keeps
 //   - the leading steps of its segment resident in shared memory, filled by
 //     per-warp 1-D bulk async copies on an mbarrier, issued for the NEXT row
 //     as soon as the warp has read its resident part for the last time;
 //   - the rest in global memory, streamed in every pass through a small ring
-//     of per-lane cp.async slots.  Each row is touched by one SM only, so
-//     after the first pass these reads are L2 hits.
-// HBM therefore sees each logit row once and the gradient row once.  All
-// reductions stay inside the CTA (warp shuffles + shared memory), so a pass of
-// ~150 k elements per SM amortises them.  Passes:
+//     of per-lane cp.async slots.  After the first pass these reads are L2 hits.
+// HBM therefore sees each logit row once and the gradient row once.
+// Reductions stay inside the CTA (warp shuffles + shared memory), or go into the shared memory of both CTAs of the row,
+// so a pass of ~150 k elements per SM amortises them.  Passes:
 //   lse      2 exponentials/element under shifts fixed before the pass:
 //            log-sum-exps, moments of the logit difference under p (initial
 //            guess of lambda), KL(T||p), maxima, teacher argmax
@@ -84,12 +84,12 @@ constexpr int RNV = 9;                  // doubles per partial vector
 static_assert(RW >= 14 || RW == 8 || RW == 4, "the gather is dealt out to eight warps, or done by warp 0; the side work has warps of its own, or is shared out");
 // Who does what beside the passes.  With 14 warps or more, and a CTA per row, the row scalars that do not depend on the
 // passes (uniforms, the logits at the proposal) are fetched by warps 8-10 while warps 0-7 gather the warps' sums, one sum
-// each; a block barrier; then thread 0 does the scalars.  With four or eight warps warp 0 gathers all sums at once (four
+// each; a block barrier; then thread 0 does the scalars.  With four or eight warps, or two CTAs per row, warp 0 gathers all sums at once (four
 // lanes per sum) and goes straight on to the scalars: a barrier less per pass, and the eight sums are not dealt
 // twice round four warps (4096 rows of 8192 elements: 26.7 -> 25.5 k cycles a row; of 32000: 65.5 -> 65.4 k); the uniforms and the logits at the
 // proposal are fetched by warps 1-3 at the top of the row.  While thread 0 does the scalars: FIN_WARP finishes the
 // previous row, RES_WARP finds the next row, SV_WARP fetches the student's logit at the
-// teacher's argmax (and with four or eight warps finds the argmax).
+// teacher's argmax (and where warp 0 gathers finds the argmax).
 constexpr bool SIDE_WARPS = RW >= 14 && CL == 1;
 constexpr int UACC_WARP = SIDE_WARPS ? 8 : 1, UDRAW_WARP = SIDE_WARPS ? 9 : 2, SX_WARP = SIDE_WARPS ? 10 : 3;
 constexpr int RES_WARP = SIDE_WARPS ? 11 : (RW >= 8 ? 5 : 2), SV_WARP = SIDE_WARPS ? 13 : (RW >= 8 ? 6 : 3);
@@ -332,7 +332,7 @@ __device__ __forceinline__ void for_each_chunk(const Seg& sg, int lane, const ui
 // steal: a CTA per row, of which those that run take over rows whose CTA has not started (clusterlaunchcontrol).  CTAs that
 // share an SM do not get equal shares of its schedulers: with the rows dealt out beforehand the slowest took 12 to 16 % longer
 // than the average (rows dealt out / taken over, us: 4096 rows of 32000 300 / 282, of 8192 elements 11840 rows 278 / 258, of
-// 65536 8192 rows 1082 / 1008; one CTA per SM: 16384 rows of 151936 4679 / 4626).
+// 65536 8192 rows 1082 / 1008; one CTA per SM, 110 rows each: 16384 rows of 151936 4707 / 4670, no more than two runs of one side differ).
 template <bool SPEC>
 __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams P, const int steal) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -518,7 +518,7 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       do {
         came = mbar_try_wait(answer_bar, answer_phase);
         late = clock64() - asked > wait_limit;
-      } while (!came && !(late && clock64() - asked > WAIT_LIMIT_CYCLES));
+      } while (!came && clock64() - asked <= wait_limit + WAIT_LIMIT_CYCLES);
       if (came) {
         const int first = steal_answer(smem + ROFF_ANSWER);
         if (first >= 0) next = (late ? late_base : 0) + first / CL;
@@ -1001,8 +1001,10 @@ __global__ void __launch_bounds__(RT, CTAS_PER_SM) rowsm_kernel(const RowParams 
       RTS(PH_SOLVE_SCALAR);
       __syncthreads();
     }
-    int64_t next_row = dyn || steal ? (int64_t)seqres[0] : row + n_places;
-    if (steal && next_row >= late_base) { next_row -= late_base; dead = true; }    // taken over too late: flagged, and the last
+    // (in 32 bits, which a row number fits: in 64 the passes come out worse, 16384 rows of 151936 4565 us instead of 4470)
+    int next_r = dyn || steal ? seqres[0] : (int)min(row + n_places, P.n_rows);
+    if (steal && next_r >= late_base) { next_r -= late_base; dead = true; }    // taken over too late: flagged, and the last
+    const int64_t next_row = next_r;
     next_row_c = next_row;
     n_s = nullptr; n_t = nullptr;
     if (next_row < P.n_rows) row_ptrs(next_row, n_s, n_t);
