@@ -39,27 +39,27 @@ static const Variant FULL = {full_sm::launch, 1, 1}, HALF = {half_sm::launch, 1,
 
 // The variant that routes this number of rows soonest.  All figures: forward + gradient, rows from memory, us, calls one after the
 // other in a graph.
-//   - A row or less for two SMs: two CTAs of 512 threads on two SMs to a row (one SM per row / two: 74 rows of 98304 43.1 / 31.2,
-//     of 65536 34.7 / 25.7, of 32000 24.1 / 20.0); a row or less per SM: the pair of CTAs of 256 threads (148 rows of 151936
-//     68.8 / 60.6, of 65536 38.8 / 35.0, of 24000 22.5 / 20.5).  Below V = 20000 the exchange costs about what it saves: two CTAs
-//     per SM (148 rows of 16384 19.8, the pair 18.9; 37 rows 15.6, 15.8; 148 rows of 12288 18.3, 18.5).  49 shapes of up to 148 rows: 0.3 %
+//   - A row or less for two SMs: two CTAs of 512 threads on two SMs to a row (one SM per row / two: 74 rows of 98304 42.3 / 31.4,
+//     of 65536 34.2 / 25.8, of 32000 23.7 / 20.1); a row or less per SM: the pair of CTAs of 256 threads (148 rows of 151936
+//     68.6 / 59.8, of 65536 38.2 / 35.4, of 24000 22.6 / 20.8).  Below V = 20000 the exchange costs about what it saves: two CTAs
+//     per SM (148 rows of 16384 19.6, the pair 19.0; 37 rows 15.6, 15.7; 148 rows of 12288 18.2, 18.5).  49 shapes of up to 148 rows: 0.3 %
 //     above the best variant on average, 5 % at worst, beside what follows.
-//   - Beyond V = 98304 the pair takes those few rows too, which costs a quarter to a third (74 rows of 151936 52.7, 39.9 with 512
-//     threads; 37 rows 49.6, 36.1; one SM per row 57.6 and 53.4): its sixteen warps add up a row's sums in the order of the pinned
+//   - Beyond V = 98304 the pair takes those few rows too, which costs a quarter to a third (74 rows of 151936 52.3, 40.1 with 512
+//     threads; 37 rows 49.4, 36.4; one SM per row 56.9 and 52.8): its sixteen warps add up a row's sums in the order of the pinned
 //     variant, and a test compares 40 such rows with it to the bit.
-//   - More: the variant that takes the least by a cost model, start + (serial + element V / 1000) turns, where a turn is waited
-//     for to its end only in part (CTAs take over rows that have not started) and costs more where the rows in flight are more than
-//     L2 holds.  Fitted to 754 shapes (V = 2048 to 163840, 149 to 16384 rows), each with rows from memory, with rows in L2, and forward
-//     alone: 0.2, 0.2 and 0.4 % above the best variant on average, 3 % or more for 7, 21 and 40 of the shapes, 7, 7 and 9 % at
-//     worst.  (Where two fit, e.g. 16384 rows of 118784, the gradient's stores decide: pair / two per SM 3733 / 3786, forward alone
-//     3518 / 3281.  The choice does not look at that, so that both calls give the same bits.)
-//     The pair takes 149 to 150 rows of 32000 and to some 230 of 98304, from V = 65536 on a second turn that has just begun, and from
-//     V = 115000 on all calls but those of the next rule (320 rows of 151936 150 on one SM each, 121 on the pair; 1200 397 / 367; 4096
-//     1190 / 1167); two and four CTAs per SM the others (2000 rows of 65536 264, the pair 300; of 16384 87 with four, 97 with two).
-//   - Rows beyond V = 131072, more than 40 per SM: one CTA per SM.  The pair's lead is gone there, and it draws more power (loops of half a second
-//     over three batches, one SM / pair: 16384 rows of 151936 4566 / 4600 at 797 / 865 W, 8192 2330 / 2328, 16384 of 139264 4201 / 4198 at 816 / 833 W; 16384
-//     of 151936 among other calls 4710 / 4820).  Up to V = 131072 it is the other way round (16384 rows of 131072
-//     3989 / 3978 at 850 / 832 W, of 118784 3680 / 3631 at 843 / 799 W), as with fewer rows (4096 of 151936 1202 / 1194, 2000 607 / 592).
+//   - Rows beyond V = 131072, more than 40 per SM: one CTA per SM.  The pair's lead, the last turn, is gone there, and each row waits for
+//     the slower of its SMs (loops of half a second over three batches, one SM / pair: 16384 rows of 151936 4489 / 4541, 8192 2290 /
+//     2297, 8192 of 163840 2463 / 2471, 16384 of 139264 4128 / 4145).  Up to V = 131072 (16384 rows of 131072 3919 / 3925, of 118784 3614 /
+//     3592, of 98312 3239 / 3161) and for fewer rows (4096 of 151936 1182 / 1178, 2000 597 / 584) it is even or the other way round.
+//   - More rows than SMs otherwise: the variant that takes the least by a cost model, start + (serial + element V / 1000) turns, where a
+//     turn is waited for to its end only in part (CTAs take over rows that have not started) and costs more where the rows in
+//     flight are more than L2 holds.  Fitted to 754 shapes (V = 2048 to 163840, 149 to 16384 rows), each with rows from memory, with
+//     rows in L2, and forward alone: 0.2, 0.2 and 0.4 % above the best variant on average, 3 % or more for 15, 18 and 40 of the
+//     shapes, 7, 9 and 11 % at worst.  (Where two fit, e.g. 16384 rows of 118784, the gradient's stores decide: pair / two per SM
+//     3600 / 3693, forward alone 3500 / 3204.  The choice does not look at that, so that both calls give the same bits.)
+//     The pair takes 149 to some 175 rows of 49152 and to some 235 of 98304, from V = 65536 on a second turn that has just begun, and from
+//     V = 115000 on all calls (320 rows of 151936 149 on one SM each, 121 on the pair; 1200 390 / 365); two and four CTAs per SM the others
+//     (2000 rows of 65536 259, the pair 304; of 16384 86 with four, 97 with two).
 // Not where saki_set_kernel pins the kernel: then the variant goes by V alone, and pieces of a batch agree with the whole to the bit.
 static const Variant& pick_variant(const RowParams& p) {
   const int64_t n = p.call_rows;
@@ -75,9 +75,9 @@ static const Variant& pick_variant(const RowParams& p) {
   // max_v: the longest row; per_sm: rows in flight per SM; whole: the part of a turn that is waited for to its end; late: how far
   // into its turn an average CTA is when no row is left; beyond: for each 126 MB in flight beyond L2
   struct Model { const Variant* v; int max_v; double per_sm, start, serial, element, whole, late, beyond; };
-  const Model models[] = {{&HALF, half_sm::max_v(), 2, 7.14, 3.90, 0.5070, 0.181, 0.311, 1.101},
-                          {&QUARTER, QUARTER_MAX_V, 4, 6.13, 2.88, 1.0494, 0.114, 0.283, 0.245},
-                          {&PAIR, pair_sm::max_v(), 1, 5.53, 9.15, 0.2027, 0.047, 0.336, 0.092}};
+  const Model models[] = {{&HALF, half_sm::max_v(), 2, 7.30, 4.71, 0.4938, 0.214, 0.308, 1.812},
+                          {&QUARTER, QUARTER_MAX_V, 4, 7.52, 2.83, 1.0473, 0.153, 0.249, 0.317},
+                          {&PAIR, pair_sm::max_v(), 1, 8.72, 11.92, 0.1921, 0.0, 0.109, 0.125}};
   const Variant* best = &PAIR;
   double least = 1e300;
   for (const Model& m : models) {
