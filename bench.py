@@ -53,16 +53,16 @@ METRIC = "routed positions/sec (fwd+bwd, V=151936 bf16)"
 UNIT = "positions/s"
 FALLBACK_HBM_GBS = 6650.0
 # dram__bytes_read.sum + dram__bytes_write.sum of one rowsm_kernel launch divided by the positions it
-# routed, from an ncu capture on 2220 rows of the same workload (the kernel's ncu summary gives the
-# command); traffic grows in proportion to the rows, so a full launch is this figure times N
-TRAFFIC_BYTES_PER_POSITION = 958376
+# routed, from an ncu capture on 2220 rows of the same workload on the same variant, one CTA per SM (the kernel's ncu
+# summary gives the command); traffic grows in proportion to the rows, so a full launch is this figure times N
+TRAFFIC_BYTES_PER_POSITION = 957986
 # rows up to this length are served by the instance of the metadata backward's streaming kernel that runs two CTAs per SM
 # (meta_stream_kernel<16>); the names below are the ones a profiler shows
 TWO_CTA_MAX_V = 98304
 # the row kernel's instance (its namespace) by what the library says of the call: blocks per row, blocks per SM
 ROWSM_VARIANT = {(1, 1): "full_sm", (1, 2): "half_sm", (1, 4): "quarter_sm", (2, 2): "pair_sm", (2, 1): "wide_sm"}
 # warp-instructions the row kernel's one-CTA instance issues per 32 vocabulary elements, from the same capture
-ISSUED_PER_32_ELEMENTS = 39.09
+ISSUED_PER_32_ELEMENTS = 39.31
 # the same for one meta_stream_kernel launch
 META_TRAFFIC_BYTES_PER_POSITION = 581046
 
