@@ -177,7 +177,7 @@ static int dispatch_rows(RowParams p, int dtype, cudaStream_t st, int32_t* scrat
   const bool rowsm_ok = (which == 0 || which == 3) && rowsm_can_serve(p, dtype);
   const bool fast = (which != 1) && (rowsm_ok || (eps_ok && cluster_can_serve(p, dtype)));
   p.redo_list = nullptr; p.redo_count = nullptr; p.redo_guess = nullptr; p.from_list = 0;
-  p.wait_limit = g_wait_limit.load();
+  p.wait_limit = std::min<long long>(g_wait_limit.load(), 1LL << 61);      // (the kernels add their own limit to it)
   g_last_redo_count = nullptr;          // the counters below describe this call only
   rowsm_layout_none();
   std::unique_lock<std::mutex> scratch_lock(g_redo_mu, std::defer_lock);

@@ -67,3 +67,17 @@ def test_a_row_whose_answer_is_late_is_flagged():
     for k in ref:
         assert torch.equal(again[k], ref[k]), k
     assert torch.equal(g_again, g_ref)
+
+
+def test_a_limit_beyond_any_wait_changes_nothing():
+    w = synth.Workload("patient", 20000, 2048, "bf16", 0.1, 1.5, True, 4101, 9)          # thirty rows taken over per block
+    d = synth.generate(w, DEV)
+    prev = P.set_kernel(3)
+    P.check()
+    try:
+        ref, g_ref = P.route_fwd_bwd(d["s"], d["t"], d["proposal"], w.eps, seed=w.seed)
+        late, out, g = limited_call(d, w, 2 ** 63 - 1)
+    finally:
+        P.set_kernel(prev)
+    assert not late.any()
+    check_rows(late, out, g, ref, g_ref)
